@@ -39,18 +39,17 @@ int pitch_of(int nz) { return (nz + 31) / 32 * 32; }
 
 #include "lbm_handle.h"
 
-// The balanced one-wave grid: the fused kernel over this solve's tile plan, its
-// descriptor passed by value; the same arithmetic as inside any batch.
-cudaError_t lbm_handle_step_tiles(lbm_axi* h, int c) {
+template <typename R>
+static cudaError_t step_fused(lbm_axi* h, const Params<R>& p, int c) {
     const bool mp = h->opts.multiphase != 0, ax = h->opts.axis_terms != 0;
-    if (h->precision == 32) {
-        const lbm::BatchSolve<float> d{h->pf, (const float*)h->f[0], (float*)h->f[1], (const float*)h->hb[0],
-                                       (float*)h->hb[1]};
-        return Ops<float>::step_single(d, h->d_tiles, h->d_first, h->ncta, mp, ax, c, h->derr, h->stream, fv_of(h));
-    }
-    const lbm::BatchSolve<double> d{h->pdd, (const double*)h->f[0], (double*)h->f[1], (const double*)h->hb[0],
-                                    (double*)h->hb[1]};
-    return Ops<double>::step_single(d, h->d_tiles, h->d_first, h->ncta, mp, ax, c, h->derr, h->stream, fv_of(h));
+    const lbm::BatchSolve<R> s = lbm_handle_solve<R>(h, p, 0);
+    const lbm::LinkSets<R> hs{static_cast<const R*>(h->hb[0]), static_cast<R*>(h->hb[1])};
+    if (lbm_by_phases(h->precision, (long long)h->nz * h->nr))
+        return Ops<R>::phase_step(s, hs, mp, ax, c, h->derr, h->stream, fv_of(h));
+    return Ops<R>::step_single(s, hs, h->d_tiles, h->d_first, h->ncta, mp, ax, c, h->derr, h->stream, fv_of(h));
+}
+cudaError_t lbm_handle_step_fused(lbm_axi* h, int c) {
+    return h->precision == 32 ? step_fused<float>(h, h->pf, c) : step_fused<double>(h, h->pdd, c);
 }
 
 namespace {
@@ -100,7 +99,7 @@ cudaError_t enqueue_step(lbm_axi* h) {
     const int c = h->cur;
     cudaError_t e;
     if (h->path == LBM_PATH_FUSED && h->rows_per_cta == 0) {
-        e = lbm_handle_step_tiles(h, c);
+        e = lbm_handle_step_fused(h, c);
         h->cur = c ^ 1;
         return e;
     }
@@ -173,7 +172,7 @@ int chunk_steps(const lbm_axi* h) {
     const long long cells = (long long)h->nz * h->nr;
     long long c = (4LL << 20) / (cells > 0 ? cells : 1);
     if (c < 2) c = 2;
-    if (c > 256) c = 256;
+    if (c > 32) c = 32;
     return (int)(c & ~1LL);
 }
 
@@ -317,12 +316,13 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     h->partial = (double*)dev_alloc(4 * lbm::kReduceBlocks * sizeof(double));
     h->dred = (double*)dev_alloc(4 * sizeof(double));
     h->derr = (int*)dev_alloc(sizeof(int));
-    // tile plan of the balanced one-wave step (k_step_single, the batched kernel's single-solve form)
+    // tile plan of the marching step (wide strips, one resident wave)
     std::vector<lbm::Tile> tiles;
     std::vector<int> first;
-    {
-        const int slots = o.precision == 32 ? Ops<float>::batch_resident_ctas(lbm::kStripWide)
-                                            : Ops<double>::batch_resident_ctas(lbm::kStripWide);
+    if (lbm_by_phases(o.precision, (long long)nz * nr)) {
+        first.assign(1, 0);
+    } else {
+        const int slots = Ops<float>::batch_resident_ctas(lbm::kStripWide);
         int rc = LBM_ERR_CUDA;
         try {
             rc = slots > 0 ? lbm::plan_tiles(&nz, &nr, 1, lbm::kStripWide, slots, tiles, first, nullptr)
@@ -374,8 +374,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     if (h->precision == 32) h->pdd = make_params_out(h);
     *h->herr = 0;
     cudaError_t err = cudaSuccess;
-    {
-        // this solve's tile plan (wide strips, one resident wave)
+    if (!tiles.empty()) {
         err = cudaMemcpy(h->d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile), cudaMemcpyHostToDevice);
         if (err == cudaSuccess)
             err = cudaMemcpy(h->d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice);

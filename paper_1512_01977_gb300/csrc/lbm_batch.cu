@@ -20,6 +20,9 @@ struct lbm_axi_batch {
     std::vector<int> cur0;  // each solve's current buffer when the batch was made
     void* d_solves;         // BatchSolve<R>[n]
     lbm::BatchTable<float>* h_table;  // FP32, n <= BatchTable::N: the descriptors as one kernel argument
+    bool phases;            // this tuning steps by phases (else the marching kernel over d_tiles)
+    lbm::PhaseTile* d_ptiles;
+    int nptiles, nghost, prows;
     lbm::Tile* d_tiles;     // tile plan for (strip, grid)
     int* d_first;           // [ncta + 1]
     int ncta;
@@ -58,15 +61,19 @@ const Params<double>& params_of<double>(const lbm_axi* h) {
     return h->pdd;
 }
 
+// FP64 steps by phases at every tuning; FP32 at the default one (wide strips, grid
+// 0) while the batch is small, the marching kernel at the others.
+bool by_phases(const lbm_axi_batch* b, long long nodes) {
+    return b->precision == 64 || (b->strip == lbm::kStripWide && b->grid == 0 && lbm_by_phases(32, nodes));
+}
+
 template <typename R>
 cudaError_t upload(lbm_axi_batch* b) {
     std::vector<BatchSolve<R>> hs(b->n);
     std::vector<int> nz(b->n), nr(b->n);
     for (int i = 0; i < b->n; i++) {
         lbm_axi* h = b->solves[i];
-        hs[i].p = params_of<R>(h);
-        hs[i].f_a = static_cast<const R*>(h->f[b->cur0[i]]);
-        hs[i].f_b = static_cast<R*>(h->f[b->cur0[i] ^ 1]);
+        hs[i] = lbm_handle_solve<R>(h, params_of<R>(h), b->cur0[i]);
         nz[i] = h->nz;
         nr[i] = h->nr;
     }
@@ -74,12 +81,33 @@ cudaError_t upload(lbm_axi_batch* b) {
         if (b->h_table)
             for (int i = 0; i < b->n; i++) b->h_table->s[i] = hs[i];
     }
-    const int slots = b->grid > 0 ? b->grid : Ops<R>::batch_resident_ctas(b->strip);
-    if (slots <= 0) return cudaErrorInvalidConfiguration;
+    long long nodes = 0;
+    for (int i = 0; i < b->n; i++) nodes += (long long)nz[i] * nr[i];
+    b->phases = by_phases(b, nodes);
     std::vector<lbm::Tile> tiles;
+    std::vector<lbm::PhaseTile> ptiles;
+    size_t inner = 0;  // tiles before the ghost rows'
     std::vector<int> first;
-    if (lbm::plan_tiles(nz.data(), nr.data(), b->n, b->strip, slots, tiles, first, nullptr) != LBM_OK)
-        return cudaErrorMemoryAllocation;
+    if (b->phases) {
+        const int tz = Ops<R>::phase_tile_z();
+        b->prows = Ops<R>::phase_rows(nodes);
+        try {
+            for (int i = 0; i < b->n; i++)
+                for (int j = 0; j < nr[i]; j += b->prows)
+                    for (int k = 0; k < nz[i]; k += tz) ptiles.push_back(lbm::PhaseTile{i, k, j});
+            inner = ptiles.size();
+            for (int i = 0; i < b->n && b->ax; i++)
+                for (int k = 0; k < nz[i] && b->solves[i]->opts.top_bc != LBM_TOP_PERIODIC; k += tz)
+                    ptiles.push_back(lbm::PhaseTile{i, k, -2});
+        } catch (...) {
+            return cudaErrorMemoryAllocation;
+        }
+    } else {
+        const int slots = b->grid > 0 ? b->grid : Ops<R>::batch_resident_ctas(b->strip);
+        if (slots <= 0) return cudaErrorInvalidConfiguration;
+        if (lbm::plan_tiles(nz.data(), nr.data(), b->n, b->strip, slots, tiles, first, nullptr) != LBM_OK)
+            return cudaErrorMemoryAllocation;
+    }
     // the graph holds the old plan's pointers
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
@@ -89,23 +117,30 @@ cudaError_t upload(lbm_axi_batch* b) {
     if (e != cudaSuccess) return e;
     if (b->d_tiles) cudaFree(b->d_tiles);
     if (b->d_first) cudaFree(b->d_first);
+    if (b->d_ptiles) cudaFree(b->d_ptiles);
     b->d_tiles = nullptr;
     b->d_first = nullptr;
-    b->ncta = 0;
-    e = cudaMalloc(&b->d_tiles, tiles.size() * sizeof(lbm::Tile));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_first, first.size() * sizeof(int));
+    b->d_ptiles = nullptr;
+    b->ncta = b->nptiles = 0;
+    auto put = [&](void** d, const void* from, size_t bytes) {
+        if (e == cudaSuccess) e = cudaMalloc(d, bytes);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(*d, from, bytes, cudaMemcpyHostToDevice, b->stream);
+    };
+    if (b->phases) {
+        put((void**)&b->d_ptiles, ptiles.data(), ptiles.size() * sizeof(lbm::PhaseTile));
+    } else {
+        put((void**)&b->d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile));
+        put((void**)&b->d_first, first.data(), first.size() * sizeof(int));
+    }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->d_solves, hs.data(), sizeof(BatchSolve<R>) * b->n, cudaMemcpyHostToDevice,
                             b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile), cudaMemcpyHostToDevice,
-                            b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice,
-                            b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e == cudaSuccess) b->ncta = (int)first.size() - 1;
-    return e;
+    if (e != cudaSuccess) return e;
+    b->nptiles = (int)inner;
+    b->nghost = (int)(ptiles.size() - inner);
+    b->ncta = first.empty() ? 0 : (int)first.size() - 1;
+    return cudaSuccess;
 }
 
 cudaError_t upload_tables(lbm_axi_batch* b) {
@@ -113,14 +148,18 @@ cudaError_t upload_tables(lbm_axi_batch* b) {
 }
 
 cudaError_t launch(lbm_axi_batch* b, int parity) {
-    if (b->h_table)  // FP32, n <= BatchTable::N: parameters through the constant bank
+    if (b->precision == 64)
+        return Ops<double>::phase_step_many(static_cast<const BatchSolve<double>*>(b->d_solves), b->d_ptiles, b->nptiles,
+                                            b->nghost, b->prows, b->mp, b->ax, parity, b->d_err, b->stream);
+    const BatchSolve<float>* solves = static_cast<const BatchSolve<float>*>(b->d_solves);
+    if (b->phases)
+        return Ops<float>::phase_step_many(solves, b->d_ptiles, b->nptiles, b->nghost, b->prows, b->mp, b->ax, parity, b->d_err,
+                                           b->stream);
+    if (b->h_table)  // n <= BatchTable::N: parameters through the constant bank
         return Ops<float>::step_table(*b->h_table, b->d_tiles, b->d_first, b->ncta, b->mp, b->ax, parity, b->strip,
                                       b->d_err, b->stream);
-    if (b->precision == 32)
-        return Ops<float>::step_batch(static_cast<const BatchSolve<float>*>(b->d_solves), b->d_tiles, b->d_first,
-                                      b->ncta, b->mp, b->ax, parity, b->strip, b->d_err, b->stream);
-    return Ops<double>::step_batch(static_cast<const BatchSolve<double>*>(b->d_solves), b->d_tiles, b->d_first,
-                                   b->ncta, b->mp, b->ax, parity, b->strip, b->d_err, b->stream);
+    return Ops<float>::step_batch(solves, b->d_tiles, b->d_first, b->ncta, b->mp, b->ax, parity, b->strip, b->d_err,
+                                  b->stream);
 }
 
 int build_graph(lbm_axi_batch* b) {
@@ -159,6 +198,7 @@ void release(lbm_axi_batch* b) {
     if (b->d_solves) cudaFree(b->d_solves);
     if (b->d_tiles) cudaFree(b->d_tiles);
     if (b->d_first) cudaFree(b->d_first);
+    if (b->d_ptiles) cudaFree(b->d_ptiles);
     if (b->d_err) cudaFree(b->d_err);
     if (b->h_err) cudaFreeHost(b->h_err);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -214,6 +254,9 @@ int lbm_axi_batch_create(lbm_axi* const* solves, int n, void* stream, lbm_axi_ba
     b->device = dev;
     b->d_solves = nullptr;
     b->h_table = nullptr;
+    b->phases = false;
+    b->d_ptiles = nullptr;
+    b->nptiles = b->nghost = b->prows = 0;
     b->d_tiles = nullptr;
     b->d_first = nullptr;
     b->ncta = 0;
@@ -361,7 +404,7 @@ int lbm_axi_batch_set_tuning(lbm_axi_batch* b, const lbm_axi_batch_tuning* t) {
     if (!b || !t || (t->strip != lbm::kStripNarrow && t->strip != lbm::kStripWide) || t->grid < 0) return LBM_ERR_INVALID_ARG;
     DevGuard g(b->device);
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) return LBM_ERR_CUDA;
-    if (t->strip != b->strip || t->grid != b->grid || !b->d_tiles) {
+    if (t->strip != b->strip || t->grid != b->grid || !(b->d_tiles || b->d_ptiles)) {
         b->strip = t->strip;
         b->grid = t->grid;
         if (upload_tables(b) != cudaSuccess) return LBM_ERR_CUDA;
@@ -389,11 +432,11 @@ int lbm_axi_batch_autotune(lbm_axi_batch* b, int trials, lbm_axi_batch_tuning* c
     }
     for (int si = 0; si < 2; si++) {
         const int strip = strips[si];
-        const int resident = b->precision == 32 ? Ops<float>::batch_resident_ctas(strip)
-                                                : Ops<double>::batch_resident_ctas(strip);
-        if (resident <= 0) continue;
+        // FP64 has one form, whatever the strip and the slots
+        const int resident = b->precision == 32 ? Ops<float>::batch_resident_ctas(strip) : 0;
+        if (b->precision == 32 ? resident <= 0 : strip != lbm::kStripWide) continue;
         const int grids[2] = {0, 2 * resident};
-        for (int gi = 0; gi < 2; gi++) {
+        for (int gi = 0; gi < (resident > 0 ? 2 : 1); gi++) {
             lbm_axi_batch_tuning t = {strip, grids[gi]};
             if (lbm_axi_batch_set_tuning(b, &t) != LBM_OK) return LBM_ERR_CUDA;
             const float ms = time_launches(b->stream, trials, [&] { return launch(b, parity); });
@@ -451,7 +494,7 @@ int lbm_axi_autotune(lbm_axi* h, int trials, lbm_axi_tuning* chosen) {
         const int nrows = fv_of(h) ? 1 : 5;
         for (int q = 0; q < nrows; q++) {
             const float ms = time_launches(h->stream, trials, [&] {
-                return rows_list[q] == 0 ? lbm_handle_step_tiles(h, c) : fused(rows_list[q]);
+                return rows_list[q] == 0 ? lbm_handle_step_fused(h, c) : fused(rows_list[q]);
             });
             if (ms > 0 && (best < 0 || ms < best)) {
                 best = ms;

@@ -76,15 +76,23 @@ struct LinkPlanes {
     R* dst;
 };
 
-// One solve of a batched launch: its parameters and its two population buffers
-// (even batch steps read f_a and write f_b, odd steps the reverse), and with
-// the link-midpoint source its two sets of source planes, swapped the same way
-// (null otherwise).
+// One solve of a batched launch: its parameters, its two population buffers
+// (even batch steps read f_a and write f_b, odd steps the reverse), and the
+// scratch of the phase kernels: the field planes and the staging planes of the
+// moments pass, idle during a step.
 template <typename R>
 struct BatchSolve {
     Params<R> p;
     const R* f_a;
     R* f_b;
+    R* aux;
+    R* stage;
+};
+
+// A solve's two sets of link-midpoint source planes, swapped like f_a and f_b
+// (null when h_i is evaluated at the node).
+template <typename R>
+struct LinkSets {
     const R* h_a;
     R* h_b;
 };

@@ -69,9 +69,22 @@ inline bool fused_ok(const lbm_axi* h) {
 // Options the batched engine lacks (such a solve cannot join a batch).
 inline bool unbatchable(const lbm_axi* h) { return fv_of(h) != 0; }
 
-// One fused step of this solve over its tile plan (k_step_single, the collision
-// form fv_of(h)) reading f[c] and writing f[c^1]; enqueued on h->stream.
-cudaError_t lbm_handle_step_tiles(lbm_axi* h, int c);
+// One step of this solve in the form chosen for it (lbm_by_phases) reading
+// f[c] and writing f[c^1]; enqueued on h->stream.
+cudaError_t lbm_handle_step_fused(lbm_axi* h, int c);
+
+// The step runs as three phase launches instead of the marching kernel: FP64
+// always, FP32 up to kPhaseMaxNodes nodes in all.
+inline bool lbm_by_phases(int precision, long long nodes) {
+    return precision == 64 || nodes <= lbm::kPhaseMaxNodes;
+}
+
+// A solve as the step kernels see it, reading f[a] on even steps.
+template <typename R>
+inline lbm::BatchSolve<R> lbm_handle_solve(const lbm_axi* h, const Params<R>& p, int a) {
+    return {p, static_cast<const R*>(h->f[a]), static_cast<R*>(h->f[a ^ 1]), static_cast<R*>(h->aux),
+            reinterpret_cast<R*>(h->mout)};
+}
 
 // Step parity bookkeeping used by the batch API: after n steps run outside
 // the handle's own step loop, its current buffer flips when n is odd.

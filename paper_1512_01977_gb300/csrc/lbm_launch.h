@@ -11,6 +11,7 @@ namespace lbm {
 
 constexpr int kReduceBlocks = 304;  // 2 x 152 SMs; fixed so reductions are reproducible
 constexpr int kStepMinRows = 16;    // the single-pass kernel needs single reflections at the walls
+constexpr long long kPhaseMaxNodes = 1500000;
 // z-columns per CTA of the two compiled forms of the batched kernel (the wide
 // one is the default; the autotuner may pick the narrow one for small grids).
 // 112: with 128 threads of two columns each, stages L, D, U and C fill 124,
@@ -50,18 +51,30 @@ struct Ops {
     static int step_strip();  // z-columns per CTA of the single-pass kernel
     // Batched fused step: ncta CTAs, CTA c marching tiles first[c] .. first[c + 1] - 1
     // (device arrays planned by plan_tiles for this strip width); strip: kStripNarrow
-    // or kStripWide z-columns per CTA.  fv: FV_* collision form, nonzero only with
-    // kStripWide and mp && ax (cudaErrorInvalidValue otherwise).
+    // or kStripWide z-columns per CTA.  FP32 only (cudaErrorNotSupported in FP64, like
+    // step_single and step_table: FP64 steps by phases).
     static cudaError_t step_batch(const BatchSolve<R>* solves, const Tile* tiles, const int* first, int ncta,
-                                  bool mp, bool ax, int parity, int strip, int* err, cudaStream_t s, int fv = 0);
+                                  bool mp, bool ax, int parity, int strip, int* err, cudaStream_t s);
     // The fused step of one solve, descriptor by value (kStripWide tiles; same
-    // arithmetic as step_batch with a batch of one).
-    static cudaError_t step_single(const BatchSolve<R>& solve, const Tile* tiles, const int* first, int ncta,
-                                   bool mp, bool ax, int parity, int* err, cudaStream_t s, int fv = 0);
+    // arithmetic as step_batch with a batch of one).  fv: FV_* collision form,
+    // nonzero only with mp && ax (cudaErrorInvalidValue otherwise).
+    static cudaError_t step_single(const BatchSolve<R>& solve, const LinkSets<R>& h, const Tile* tiles,
+                                   const int* first, int ncta, bool mp, bool ax, int parity, int* err,
+                                   cudaStream_t s, int fv = 0);
     // The batched step with the descriptors as one kernel argument (FP32; n <=
     // BatchTable<R>::N solves; cudaErrorNotSupported in FP64).
     static cudaError_t step_table(const BatchTable<R>& table, const Tile* tiles, const int* first, int ncta,
                                   bool mp, bool ax, int parity, int strip, int* err, cudaStream_t s);
+    // The step as three phase launches (lbm_phase.cuh) of one solve, or of the tiles of
+    // many (device arrays; tiles of phase_tile_z() x rows nodes, rows of phase_rows).
+    static cudaError_t phase_step(const BatchSolve<R>& solve, const LinkSets<R>& h, bool mp, bool ax, int parity,
+                                  int* err, cudaStream_t s, int fv = 0);
+    // The list ends with nghost tiles at j0 = -2: the two rows beyond the axis of each
+    // solve without a periodic top (axis terms on).
+    static cudaError_t phase_step_many(const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles, int nghost,
+                                       int rows, bool mp, bool ax, int parity, int* err, cudaStream_t s);
+    static int phase_tile_z();
+    static int phase_rows(long long nodes);
     static int batch_resident_ctas(int strip);
     static size_t batch_smem(int strip);
 };

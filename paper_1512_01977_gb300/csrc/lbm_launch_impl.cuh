@@ -3,6 +3,7 @@
 
 #include "lbm_kernels.cuh"
 #include "lbm_launch.h"
+#include "lbm_phase.cuh"
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -102,12 +103,11 @@ cudaError_t Ops<R>::prepare() {
         e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR, false, true>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = set_step_attr<R>((int)step_smem());
-    // the batched kernel (also the default single-solve step): attributes and
-    // occupancy are settled here, outside any stream capture
-    if (e == cudaSuccess && (batch_resident_ctas(kStripNarrow) <= 0 || batch_resident_ctas(kStripWide) <= 0))
-        e = cudaErrorInvalidConfiguration;
-    if (e == cudaSuccess) e = single_prepare<R>();  // the single-solve form of the fused kernel
-    if constexpr (sizeof(R) == 4) {  // the argument-table form of the batched kernel
+    // the marching forms (FP32): attributes and occupancy are settled here, outside any stream capture
+    if constexpr (sizeof(R) == 4) {
+        if (e == cudaSuccess && (batch_resident_ctas(kStripNarrow) <= 0 || batch_resident_ctas(kStripWide) <= 0))
+            e = cudaErrorInvalidConfiguration;
+        if (e == cudaSuccess) e = single_prepare<R>();
         if (e == cudaSuccess) e = table_prepare<R, kStripNarrow>();
         if (e == cudaSuccess) e = table_prepare<R, kStripWide>();
     }
@@ -205,14 +205,13 @@ cudaError_t Ops<R>::pjump(const Params<R>& p, const Params<double>& pd, const R*
 
 namespace lbm {
 
-// Batched kernel forms: strip width kStripNarrow or kStripWide (the autotuner picks), force and
+// Batched marching forms (FP32): strip width kStripNarrow or kStripWide (the autotuner picks), force and
 // axis terms compiled in or out.
-// Resident CTAs per SM the launch bounds ask for: what shared memory allows at
-// each width (FP32 two columns per thread: 45.3 KB / 26.9 KB of rings; FP64
-// one column: 90.6 KB / 53.8 KB).
+// Resident CTAs per SM the launch bounds ask for: what shared memory allows at each width (45.3 KB /
+// 26.9 KB of rings).
 template <typename R, int TZ>
 struct BatchMinBlocks {
-    static constexpr int value = sizeof(R) == 4 ? (TZ == kStripWide ? 4 : 5) : (TZ == kStripWide ? 2 : 3);
+    static constexpr int value = TZ == kStripWide ? 4 : 5;
 };
 
 template <typename R, int TZ>
@@ -224,9 +223,9 @@ struct BatchTile {
     static size_t smem() { return sizeof(R) * (size_t)StepShape<TZ, RR, CP>::elems; }
 };
 
-template <typename R, int TZ, bool MP, bool AX, int FV = 0>
+template <typename R, int TZ, bool MP, bool AX>
 static auto batch_kernel() {
-    return k_step_batch<R, TZ, BatchTile<R, TZ>::RR, BatchTile<R, TZ>::CP, BatchTile<R, TZ>::MINB, MP, AX, FV>;
+    return k_step_batch<R, TZ, BatchTile<R, TZ>::RR, BatchTile<R, TZ>::CP, BatchTile<R, TZ>::MINB, MP, AX>;
 }
 
 template <typename R, bool MP, bool AX, int FV = 0>
@@ -263,17 +262,6 @@ static cudaError_t batch_prepare() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(batch_kernel<R, TZ, false, false>(),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if constexpr (TZ == kStripWide) {  // the collision variants (Guo, link source): wide strips, force + axis
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(batch_kernel<R, TZ, true, true, FV_GUO>(),
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(batch_kernel<R, TZ, true, true, FV_LINK>(),
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(batch_kernel<R, TZ, true, true, FV_GUO | FV_LINK>(),
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    }
     return e;
 }
 
@@ -329,6 +317,9 @@ size_t Ops<R>::batch_smem(int strip) {
 
 template <typename R>
 int Ops<R>::batch_resident_ctas(int strip) {
+    if constexpr (sizeof(R) == 8) {
+        return 0;  // FP64 steps by phases
+    } else {
     static int cached[2] = {0, 0};
     const int slot = strip == kStripNarrow ? 0 : 1;
     if (cached[slot] > 0) return cached[slot];
@@ -346,30 +337,14 @@ int Ops<R>::batch_resident_ctas(int strip) {
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
     cached[slot] = sms * per_sm;
     return cached[slot];
+    }
 }
 
 template <typename R, int TZ>
 static cudaError_t launch_batch(const BatchSolve<R>* solves, const Tile* tiles, const int* first, int ncta, bool mp,
-                                bool ax, int fv, int parity, int* err, cudaStream_t s) {
+                                bool ax, int parity, int* err, cudaStream_t s) {
     using T = BatchTile<R, TZ>;
     const size_t smem = T::smem();
-    if (fv != 0) {
-        if constexpr (TZ == kStripWide) {
-            if (!(mp && ax)) return cudaErrorInvalidValue;
-            if (fv == FV_GUO)
-                batch_kernel<R, TZ, true, true, FV_GUO>()<<<ncta, T::NT, smem, s>>>(solves, tiles, first, parity, err);
-            else if (fv == FV_LINK)
-                batch_kernel<R, TZ, true, true, FV_LINK>()<<<ncta, T::NT, smem, s>>>(solves, tiles, first, parity, err);
-            else if (fv == (FV_GUO | FV_LINK))
-                batch_kernel<R, TZ, true, true, FV_GUO | FV_LINK>()<<<ncta, T::NT, smem, s>>>(solves, tiles, first,
-                                                                                           parity, err);
-            else
-                return cudaErrorInvalidValue;
-            return cudaGetLastError();
-        } else {
-            return cudaErrorInvalidValue;
-        }
-    }
     if (mp && ax)
         batch_kernel<R, TZ, true, true>()<<<ncta, T::NT, smem, s>>>(solves, tiles, first, parity, err);
     else if (mp)
@@ -382,38 +357,132 @@ static cudaError_t launch_batch(const BatchSolve<R>* solves, const Tile* tiles, 
 }
 
 template <typename R>
-cudaError_t Ops<R>::step_single(const BatchSolve<R>& solve, const Tile* tiles, const int* first, int ncta, bool mp,
-                                bool ax, int parity, int* err, cudaStream_t s, int fv) {
-    using T = BatchTile<R, kStripWide>;
-    if (ncta <= 0) return cudaErrorInvalidConfiguration;
-    const size_t smem = T::smem();
-    if (fv != 0 && !(mp && ax)) return cudaErrorInvalidValue;
-    if (fv == FV_GUO)
-        single_kernel<R, true, true, FV_GUO>()<<<ncta, T::NT, smem, s>>>(solve, tiles, first, parity, err);
-    else if (fv == FV_LINK)
-        single_kernel<R, true, true, FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, tiles, first, parity, err);
-    else if (fv == (FV_GUO | FV_LINK))
-        single_kernel<R, true, true, FV_GUO | FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, tiles, first, parity, err);
-    else if (fv != 0)
-        return cudaErrorInvalidValue;
-    else if (mp && ax)
-        single_kernel<R, true, true>()<<<ncta, T::NT, smem, s>>>(solve, tiles, first, parity, err);
-    else if (mp)
-        single_kernel<R, true, false>()<<<ncta, T::NT, smem, s>>>(solve, tiles, first, parity, err);
-    else if (ax)
-        single_kernel<R, false, true>()<<<ncta, T::NT, smem, s>>>(solve, tiles, first, parity, err);
-    else
-        single_kernel<R, false, false>()<<<ncta, T::NT, smem, s>>>(solve, tiles, first, parity, err);
-    return cudaGetLastError();
+cudaError_t Ops<R>::step_single(const BatchSolve<R>& solve, const LinkSets<R>& h, const Tile* tiles, const int* first,
+                                int ncta, bool mp, bool ax, int parity, int* err, cudaStream_t s, int fv) {
+    if constexpr (sizeof(R) == 4) {
+        using T = BatchTile<R, kStripWide>;
+        if (ncta <= 0) return cudaErrorInvalidConfiguration;
+        const size_t smem = T::smem();
+        if (fv != 0 && !(mp && ax)) return cudaErrorInvalidValue;
+        if (fv == FV_GUO)
+            single_kernel<R, true, true, FV_GUO>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        else if (fv == FV_LINK)
+            single_kernel<R, true, true, FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        else if (fv == (FV_GUO | FV_LINK))
+            single_kernel<R, true, true, FV_GUO | FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity,
+                                                                                      err);
+        else if (fv != 0)
+            return cudaErrorInvalidValue;
+        else if (mp && ax)
+            single_kernel<R, true, true>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        else if (mp)
+            single_kernel<R, true, false>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        else if (ax)
+            single_kernel<R, false, true>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        else
+            single_kernel<R, false, false>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        return cudaGetLastError();
+    } else {
+        return cudaErrorNotSupported;
+    }
 }
 
 template <typename R>
 cudaError_t Ops<R>::step_batch(const BatchSolve<R>* solves, const Tile* tiles, const int* first, int ncta, bool mp,
-                               bool ax, int parity, int strip, int* err, cudaStream_t s, int fv) {
-    if (ncta <= 0) return cudaErrorInvalidConfiguration;
-    return strip == kStripNarrow
-               ? launch_batch<R, kStripNarrow>(solves, tiles, first, ncta, mp, ax, fv, parity, err, s)
-               : launch_batch<R, kStripWide>(solves, tiles, first, ncta, mp, ax, fv, parity, err, s);
+                               bool ax, int parity, int strip, int* err, cudaStream_t s) {
+    if constexpr (sizeof(R) == 4) {
+        if (ncta <= 0) return cudaErrorInvalidConfiguration;
+        return strip == kStripNarrow
+                   ? launch_batch<R, kStripNarrow>(solves, tiles, first, ncta, mp, ax, parity, err, s)
+                   : launch_batch<R, kStripWide>(solves, tiles, first, ncta, mp, ax, parity, err, s);
+    } else {
+        return cudaErrorNotSupported;
+    }
+}
+
+// ------------------------------------------------------------ phase launches --
+
+// A launch that may start while its predecessor on the stream still runs; the
+// kernel waits for it before it touches memory (griddepcontrol.wait).
+template <typename... KA, typename... A>
+static cudaError_t launch_early(void (*k)(KA...), unsigned grid, int nt, cudaStream_t s, const A&... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(nt);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, a...);
+}
+
+template <typename R, int TR, bool MP, bool AX, int FV>
+static cudaError_t phases(const PhaseOne<R>& a, unsigned grid, cudaStream_t s) {
+    const unsigned ghost = AX && a.s.p.top != TOP_PERIODIC ? a.across : 0;
+    cudaError_t e = launch_early(k_phase_l<R, TR, MP, (FV & FV_LINK) != 0>, grid, 32 * TR, s, a);
+    if (e == cudaSuccess) e = launch_early(k_phase_u<R, TR, MP, AX>, grid + ghost, 32 * TR, s, a);
+    if (e == cudaSuccess) e = launch_early(k_phase_c<R, TR, AX, FV>, grid, 32 * TR, s, a);
+    return e;
+}
+template <typename R, int TR>
+static cudaError_t phases_of(const BatchSolve<R>& v, const LinkSets<R>& h, bool mp, bool ax, int parity, int* err,
+                             cudaStream_t s, int fv) {
+    const int across = (v.p.nz + PhaseShape<R>::TZ - 1) / PhaseShape<R>::TZ;
+    const unsigned grid = (unsigned)across * (unsigned)((v.p.nr + TR - 1) / TR);
+    const PhaseOne<R> a{v, parity ? h.h_b : h.h_a, parity ? const_cast<R*>(h.h_a) : h.h_b, parity, across, err};
+    if (fv == FV_GUO && mp && ax) return phases<R, TR, true, true, FV_GUO>(a, grid, s);
+    if (fv == FV_LINK && mp && ax) return phases<R, TR, true, true, FV_LINK>(a, grid, s);
+    if (fv == (FV_GUO | FV_LINK) && mp && ax) return phases<R, TR, true, true, FV_GUO | FV_LINK>(a, grid, s);
+    if (fv != 0) return cudaErrorInvalidValue;
+    if (mp && ax) return phases<R, TR, true, true, 0>(a, grid, s);
+    if (mp) return phases<R, TR, true, false, 0>(a, grid, s);
+    if (ax) return phases<R, TR, false, true, 0>(a, grid, s);
+    return phases<R, TR, false, false, 0>(a, grid, s);
+}
+
+template <typename R, int TR, bool MP, bool AX>
+static cudaError_t phases_many(const PhaseMany<R>& a, unsigned grid, unsigned ghost, cudaStream_t s) {
+    cudaError_t e = launch_early(k_phase_l_many<R, TR, MP>, grid, 32 * TR, s, a);
+    if (e == cudaSuccess) e = launch_early(k_phase_u_many<R, TR, MP, AX>, grid + (AX ? ghost : 0), 32 * TR, s, a);
+    if (e == cudaSuccess) e = launch_early(k_phase_c_many<R, TR, AX>, grid, 32 * TR, s, a);
+    return e;
+}
+template <typename R, int TR>
+static cudaError_t phases_many_of(const PhaseMany<R>& a, unsigned grid, unsigned ghost, bool mp, bool ax,
+                                  cudaStream_t s) {
+    if (mp && ax) return phases_many<R, TR, true, true>(a, grid, ghost, s);
+    if (mp) return phases_many<R, TR, true, false>(a, grid, ghost, s);
+    if (ax) return phases_many<R, TR, false, true>(a, grid, ghost, s);
+    return phases_many<R, TR, false, false>(a, grid, ghost, s);
+}
+
+template <typename R>
+int Ops<R>::phase_tile_z() {
+    return PhaseShape<R>::TZ;
+}
+
+// Rows per tile: 8, or 4 in FP64 and while 8 would leave SMs without a tile.
+template <typename R>
+int Ops<R>::phase_rows(long long nodes) {
+    return sizeof(R) == 8 || nodes <= 152LL * 8 * PhaseShape<R>::TZ ? 4 : 8;
+}
+
+template <typename R>
+cudaError_t Ops<R>::phase_step(const BatchSolve<R>& v, const LinkSets<R>& h, bool mp, bool ax, int parity, int* err,
+                               cudaStream_t s, int fv) {
+    return phase_rows((long long)v.p.nz * v.p.nr) == 4 ? phases_of<R, 4>(v, h, mp, ax, parity, err, s, fv)
+                                                       : phases_of<R, 8>(v, h, mp, ax, parity, err, s, fv);
+}
+
+template <typename R>
+cudaError_t Ops<R>::phase_step_many(const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles, int nghost,
+                                    int rows, bool mp, bool ax, int parity, int* err, cudaStream_t s) {
+    if (ntiles <= 0) return cudaErrorInvalidConfiguration;
+    const PhaseMany<R> a{solves, tiles, parity, err};
+    return rows == 4 ? phases_many_of<R, 4>(a, (unsigned)ntiles, (unsigned)nghost, mp, ax, s)
+                     : phases_many_of<R, 8>(a, (unsigned)ntiles, (unsigned)nghost, mp, ax, s);
 }
 
 }  // namespace lbm

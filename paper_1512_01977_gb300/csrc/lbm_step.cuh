@@ -460,19 +460,23 @@ struct PairOf<double> {
 
 __device__ __forceinline__ float2 pk(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 pk(double a, double b) { return make_double2(a, b); }
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+// Packed FP32 operations, explicitly rounded.  ptxas may still fuse a product with the one sum it
+// enters, and then does so or not by kernel: where that happens the code says pfma itself.
+#define LBM_PACKED2(name, op)                                                 \
+    __device__ __forceinline__ float2 name(float2 a, float2 b) {              \
+        unsigned long long x, y, d;                                           \
+        memcpy(&x, &a, 8);                                                    \
+        memcpy(&y, &b, 8);                                                    \
+        asm(op ".rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));           \
+        float2 r;                                                             \
+        memcpy(&r, &d, 8);                                                    \
+        return r;                                                             \
+    }
+LBM_PACKED2(padd, "add")
+LBM_PACKED2(pmul, "mul")
+LBM_PACKED2(psub, "sub")  // one packed subtract, without a (-1, -1) operand pair
+#undef LBM_PACKED2
 __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b as one packed subtract (sub.rn.f32x2), without a (-1, -1) operand pair
-__device__ __forceinline__ float2 psub(float2 a, float2 b) {
-    unsigned long long x, y, d;
-    memcpy(&x, &a, 8);
-    memcpy(&y, &b, 8);
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
-    float2 r;
-    memcpy(&r, &d, 8);
-    return r;
-}
 __device__ __forceinline__ double2 padd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 pmul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
 __device__ __forceinline__ double2 pfma(double2 a, double2 b, double2 c) {
@@ -497,16 +501,14 @@ __device__ __forceinline__ Tri<T> ld3(const R* row, int c) {
     return {ld2<T>(row, c - 2), ld2<T>(row, c), ld2<T>(row, c + 2)};
 }
 
-// fd_both for the nodes at columns c and c+1 (15 pair loads instead of 32).
+// fd_both for the nodes at columns c and c+1 from the five rows' pairs (15 pair loads instead of 32).
 // Distance 1: n1z(k) = S(k+1) - S(k-1) with S the column sum of rows r-1..r+1,
 // n1r(k) = D(k-1) + D(k) + D(k+1) with D = row r+1 - row r-1.  Distance 2:
 // n2z = T(k+2) - T(k-2) with T the column sum of rows r-2, r, r+2, and
 // n2r = E(k-2) + E(k) + E(k+2) with E = row r+2 - row r-2: aligned pairs.
 template <typename R, typename T>
-__device__ __forceinline__ void fd_both2(const R* m2m, const R* mm, const R* m0, const R* mp, const R* m2p, int c,
-                                         T& dz, T& dr) {
-    const Tri<T> z0 = ld3<T>(m0, c), zm = ld3<T>(mm, c), zp = ld3<T>(mp, c);
-    const Tri<T> z2m = ld3<T>(m2m, c), z2p = ld3<T>(m2p, c);
+__device__ __forceinline__ void fd_both3(const Tri<T>& z2m, const Tri<T>& zm, const Tri<T>& z0, const Tri<T>& zp,
+                                         const Tri<T>& z2p, T& dz, T& dr) {
     const T Sa = padd(padd(z0.a, zp.a), zm.a), Sb = padd(padd(z0.b, zp.b), zm.b);
     const T Sc = padd(padd(z0.c, zp.c), zm.c);
     const T Da = psub(zp.a, zm.a), Db = psub(zp.b, zm.b), Dc = psub(zp.c, zm.c);
@@ -519,16 +521,24 @@ __device__ __forceinline__ void fd_both2(const R* m2m, const R* mm, const R* m0,
     dz = pfma(n1z, k8, pmul(n2z, k1));
     dr = pfma(n1r, k8, pmul(n2r, k1));
 }
+template <typename R, typename T>
+__device__ __forceinline__ void fd_both2(const R* m2m, const R* mm, const R* m0, const R* mp, const R* m2p, int c,
+                                         T& dz, T& dr) {
+    fd_both3<R>(ld3<T>(m2m, c), ld3<T>(mm, c), ld3<T>(m0, c), ld3<T>(mp, c), ld3<T>(m2p, c), dz, dr);
+}
 // fd_r_rows for columns c and c+1 (12 pair loads instead of 24).
 template <typename R, typename T>
-__device__ __forceinline__ T fd_r2(const R* m2m, const R* mm, const R* mp, const R* m2p, int c) {
-    const Tri<T> zm = ld3<T>(mm, c), zp = ld3<T>(mp, c), z2m = ld3<T>(m2m, c), z2p = ld3<T>(m2p, c);
+__device__ __forceinline__ T fd_r3(const Tri<T>& z2m, const Tri<T>& zm, const Tri<T>& zp, const Tri<T>& z2p) {
     const T Da = psub(zp.a, zm.a), Db = psub(zp.b, zm.b), Dc = psub(zp.c, zm.c);
     const R t = Db.x + Db.y;
     const T n1 = pk(Da.y + t, Dc.x + t);
     const T n2 = padd(padd(psub(z2p.a, z2m.a), psub(z2p.b, z2m.b)), psub(z2p.c, z2m.c));
     const T k8 = pk(R(8) / R(36), R(8) / R(36)), k1 = pk(R(-1) / R(36), R(-1) / R(36));
     return pfma(n1, k8, pmul(n2, k1));
+}
+template <typename R, typename T>
+__device__ __forceinline__ T fd_r2(const R* m2m, const R* mm, const R* mp, const R* m2p, int c) {
+    return fd_r3<R, T>(ld3<T>(m2m, c), ld3<T>(mm, c), ld3<T>(mp, c), ld3<T>(m2p, c));
 }
 // First moments of the Kupershtokh force for columns c and c+1 from psi (s1)
 // or psi^2 (s2) on rows r-1 (zm), r (z0), r+1 (zq):
@@ -589,6 +599,175 @@ __device__ __forceinline__ T kappa2(const Params<R>& p, T rho) {
     if (p.kappa == KAPPA_LATTICE) return pk(R(1) / R(9), R(1) / R(9));
     const T c2 = eos_dp2<R>(p, rho);
     return p.kappa == KAPPA_MIXED ? pmul(c2, pk(R(1) / R(3), R(1) / R(3))) : pmul(c2, c2);
+}
+
+// ------------------------------------------- the update of a node pair --
+// The arithmetic of one step for two adjacent nodes, shared by every kernel
+// that steps in FP32 (march2, the phase kernels): the same packed operations in
+// the same order, so all of them give the same bits.
+
+// rho - rho_ref, j_z, j_r of the arrived populations (la: the link source's
+// arrival planes; its halves h_i/2 have zeroth moment S0/2, first moment H/2).
+template <bool LINK, typename R, typename T>
+__device__ __forceinline__ void moments2(const T (&f)[Q], const T (&la)[3], T& drho, T& jz, T& jr) {
+    const T d1 = padd(padd(f[1], f[5]), f[7]), d2 = padd(padd(f[2], f[6]), f[8]);
+    drho = padd(padd(padd(f[0], f[3]), padd(f[4], d1)), d2);
+    jz = psub(d1, d2);
+    jr = psub(padd(padd(f[3], f[5]), f[8]), padd(padd(f[4], f[6]), f[7]));
+    if (LINK) {
+        const T half = pk(R(0.5), R(0.5));
+        drho = pfma(half, la[0], drho);
+        jz = pfma(half, la[1], jz);
+        jr = pfma(half, la[2], jr);
+    }
+}
+// psi of a pair; raises ERRBIT_PSI / ERRBIT_RHO (second lane only if v1).
+template <bool MP, typename R, typename T>
+__device__ __forceinline__ T psi2(const Params<R>& p, T drho, bool v1, int& bad) {
+    const T rho = padd(drho, pk(p.rho_ref, p.rho_ref));
+    T psi = pk(R(0), R(0));
+    if (MP) {
+        const T arg = psub(pmul(rho, pk(R(1) / R(3), R(1) / R(3))), eos_p2<R>(p, rho));
+        if (!(arg.x >= R(0)) || (v1 && !(arg.y >= R(0)))) bad |= ERRBIT_PSI;
+        psi = pk(sqrt_nonneg(arg.x), sqrt_nonneg(arg.y));
+    }
+    if (!(rho.x > R(0)) || (v1 && !(rho.y > R(0)))) bad |= ERRBIT_RHO;
+    return psi;
+}
+// Force from psi on rows r-1 (zm), r (z0), r+1 (zq): Kupershtokh, Eq. (kupershtokhforcing).
+template <typename R, typename T>
+__device__ __forceinline__ void force_k2(const Params<R>& p, const Tri<T>& zm, const Tri<T>& z0, const Tri<T>& zq,
+                                         T& fz, T& fr) {
+    const R kA = p.A, kB = R(1) - R(2) * p.A;
+    T s1z, s1r, s2z, s2r;
+    kup_moments2<R>(zm, z0, zq, s1z, s1r);
+    kup_moments2<R>(sq3(zm), sq3(z0), sq3(zq), s2z, s2r);
+    const T bk = pmul(pk(R(6) * kB, R(6) * kB), z0.b), a6k = pk(R(6) * kA, R(6) * kA);
+    fz = pfma(a6k, s2z, pfma(bk, s1z, fz));
+    fr = pfma(a6k, s2r, pfma(bk, s1r, fr));
+}
+// F_axis, Eq. (multiphasecorrections), added to (fz, fr); psi_rr = D_r(psi_r),
+// psi_rz = D_r(psi_z); rrow: the node's row, negative beyond the axis.
+template <typename R, typename T>
+__device__ __forceinline__ void force_axis2(const Params<R>& p, T rho, T psi, T psz, T psr, T prr, T prz, int rrow,
+                                            T& fz, T& fr) {
+    const R ir = rcp(R(rrow) + R(0.5));
+    const T irr = pk(ir, ir);
+    const T k3 = pmul(pk(R(3), R(3)), kappa2<R>(p, rho));
+    const R ca = p.axis_a * p.A * ir;
+    const T a6 = pmul(pk(ca, ca), psr);
+    const T pir = pmul(psi, irr);
+    fz = pfma(k3, pfma(pir, prz, pmul(a6, psz)), fz);
+    fr = pfma(k3, pfma(pir, psub(prr, pmul(psr, irr)), pmul(a6, psr)), fr);
+}
+// Physical velocity u = (j + F/2) / rho.
+template <typename R, typename T>
+__device__ __forceinline__ void velocity2(T rho, T jz, T jr, T fz, T fr, T& vz, T& vr) {
+    const T irho = prcp<R>(rho);
+    const T half = pk(R(0.5), R(0.5));
+    vz = pmul(pfma(half, fz, jz), irho);
+    vr = pmul(pfma(half, fr, jr), irho);
+}
+// Source of the axisymmetric terms: H_z, H_r and the factors of S_0 = -rho u_r / r: -1 / r and rho u_r.
+template <typename R, typename T>
+__device__ __forceinline__ void source2(const Params<R>& p, T rho, T uz, T ur, T duz_dr, T dur_dz, T dur_dr, int row,
+                                        T& Hz, T& Hr, T& mir, T& rur) {
+    const R nu = p.nu, hrs = R(p.hr_sign);
+    const R ir = rcp(R(row) + R(0.5));
+    const T irr = pk(ir, ir);
+    const T mu = pmul(rho, pk(nu, nu));
+    rur = pmul(rho, ur);
+    Hz = pmul(psub(pmul(mu, padd(duz_dr, dur_dz)), pmul(rur, uz)), irr);
+    Hr = pmul(psub(pmul(pmul(pk(R(2), R(2)), mu), pfma(pk(hrs * ir, hrs * ir), ur, dur_dr)), pmul(rur, ur)), irr);
+    mir = pk(-ir, -ir);
+}
+// EDM + BGK (or Guo) collision with the source (Hz, Hr, mir rur); store(i, v) takes the
+// new populations, store_link(q, v) this step's source planes (FV_LINK; la: the
+// previous step's).
+//   f*_i = (1 - omega) f_i + f^eq_i(u1) - (1 - omega) f^eq_i(u0) + h_i, opposite
+// directions sharing the even part (see march).
+template <int FV, typename R, typename T, typename ST, typename SL>
+__device__ __forceinline__ void collide2(const Params<R>& p, T (&fi)[Q], const T (&la)[3], T drho, T jz, T jr, T uz,
+                                         T ur, T Hz, T Hr, T mir, T rur, ST&& store, SL&& store_link) {
+    constexpr bool link = (FV & FV_LINK) != 0, guo = (FV & FV_GUO) != 0;
+    const R omega = p.tau_inv, om1 = R(1) - p.tau_inv;
+    const T rho = padd(drho, pk(p.rho_ref, p.rho_ref));
+    const T irho = prcp<R>(rho);
+    const T u0z = pmul(jz, irho), u0r = pmul(jr, irho);
+    // EDM velocity shift F / rho from u = u0 + F / (2 rho)
+    const T two = pk(R(2), R(2));
+    const T u1z = pfma(two, psub(uz, u0z), u0z), u1r = pfma(two, psub(ur, u0r), u0r);
+    const T om1p = pk(om1, om1), c15 = pk(R(1.5), R(1.5)), c45 = pk(R(4.5), R(4.5));
+    // c_i . v for the first direction of opposite pair i, i+1 (i odd)
+    auto cdot = [&](int i, T vz, T vr) {
+        const int cx = cz_of(i), cy = cr_of(i);
+        T r = cy == 0 ? vz : (cx == 0 ? vr : (cx == cy ? padd(vz, vr) : psub(vz, vr)));
+        if (cx + cy < 0) r = psub(pk(R(0), R(0)), r);  // the first direction points to -z or -r
+        return r;
+    };
+    // link-midpoint source: this node's arrival half of the previous step's h_i and
+    // the departure half of this step's; this step's S0, H kept for the next step
+    const T half = pk(R(0.5), R(0.5));
+    const T hHz = link ? pmul(half, Hz) : Hz, hHr = link ? pmul(half, Hr) : Hr;
+    // base + S_0 (its half with the link source), one fused operation: a product rounded on its own
+    // and fused or not by the compiler makes two kernels' results differ
+    auto with_s0 = [&](T base) { return link ? pfma(half, pmul(mir, rur), base) : pfma(mir, rur, base); };
+    if (link) {
+        const T m0 = pmul(mir, rur);
+        fi[0] = pfma(pk(R(0.5) * w_of<R>(0), R(0.5) * w_of<R>(0)), la[0], fi[0]);
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const int i = 2 * m + 1;
+            const R w = w_of<R>(i);
+            const T ea = pmul(pk(R(0.5) * w, R(0.5) * w), la[0]);
+            const T oa = pmul(pk(R(1.5) * w, R(1.5) * w), cdot(i, la[1], la[2]));
+            fi[i] = padd(fi[i], padd(ea, oa));
+            fi[i + 1] = padd(fi[i + 1], psub(ea, oa));
+        }
+        store_link(0, m0);
+        store_link(1, Hz);
+        store_link(2, Hr);
+    }
+    if (guo) {
+        // Guo forcing: f*_i = f_i + omega (f^eq_i(u) - f_i) + S_i + h_i with
+        // S_i = w_i (1 - omega/2) [3 (c_i - u).F + 9 (c_i.u)(c_i.F)], F = 2 rho (u - u0)
+        const T r2 = pmul(pk(R(2), R(2)), rho);
+        const T Fz = pmul(r2, psub(uz, u0z)), Fr = pmul(r2, psub(ur, u0r));
+        const T usq = pfma(uz, uz, pmul(ur, ur)), uF = pfma(uz, Fz, pmul(ur, Fr));
+        const R gpre = R(1) - R(0.5) * omega;
+        const T om = pk(omega, omega), gp = pk(gpre, gpre);
+        const T base = with_s0(
+            pfma(om, psub(drho, pmul(c15, pmul(rho, usq))), pmul(pk(R(-3) * gpre, R(-3) * gpre), uF)));
+        store(0, pfma(om1p, fi[0], pmul(pk(w_of<R>(0), w_of<R>(0)), base)));
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const int i = 2 * m + 1;
+            const R w = w_of<R>(i);
+            const T cu = cdot(i, uz, ur), cF = cdot(i, Fz, Fr), cH = cdot(i, hHz, hHr);
+            const T even = pmul(pk(w, w), padd(base, padd(pmul(pk(R(4.5) * omega, R(4.5) * omega),
+                                                               pmul(rho, pmul(cu, cu))),
+                                                          pmul(pk(R(9) * gpre, R(9) * gpre), pmul(cu, cF)))));
+            const T odd = pmul(pk(R(3) * w, R(3) * w), padd(padd(pmul(om, pmul(rho, cu)), pmul(gp, cF)), cH));
+            store(i, padd(pfma(om1p, fi[i], even), odd));
+            store(i + 1, psub(pfma(om1p, fi[i + 1], even), odd));
+        }
+    } else {
+        const T u0sq = pfma(u0z, u0z, pmul(u0r, u0r)), u1sq = pfma(u1z, u1z, pmul(u1r, u1r));
+        const T base =
+            with_s0(pfma(pk(omega, omega), drho, pmul(rho, pmul(c15, psub(pmul(om1p, u0sq), u1sq)))));
+        store(0, pfma(om1p, fi[0], pmul(pk(w_of<R>(0), w_of<R>(0)), base)));
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const int i = 2 * m + 1;  // i and i+1 are opposite
+            const R w = w_of<R>(i);
+            const T cu0 = cdot(i, u0z, u0r), cu1 = cdot(i, u1z, u1r), cH = cdot(i, hHz, hHr);
+            const T even = pmul(pk(w, w), padd(base, pmul(rho, pmul(c45, psub(pmul(cu1, cu1),
+                                                                              pmul(om1p, pmul(cu0, cu0)))))));
+            const T odd = pmul(pk(R(3) * w, R(3) * w), pfma(rho, psub(cu1, pmul(om1p, cu0)), cH));
+            store(i, padd(pfma(om1p, fi[i], even), odd));
+            store(i + 1, psub(pfma(om1p, fi[i + 1], even), odd));
+        }
+    }
 }
 
 // Pulled populations of nodes (k, j) and (k+1, j) (k, k+1 wrapped in z).
@@ -713,9 +892,7 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
     const int ck = min(k0 + cc, nz - 1);
     const bool c_contig = ck >= 1 && ck + 2 < nz && (ck & 1) == 0;
 
-    const R omega = p.tau_inv, om1 = R(1) - p.tau_inv;
-    const R kA = p.A, kB = R(1) - R(2) * p.A;
-    const R nu = p.nu, gz = p.gz, hrs = R(p.hr_sign);
+    const R gz = p.gz;
     const int uz_top = p.top == TOP_NOSLIP ? -1 : 1;
 
     auto lsrc = [&](int row, int& sgn_r) {
@@ -729,7 +906,7 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
 
     T lpf[Q], cpf[Q];  // populations gathered one iteration ahead (stage L, stage C)
     T lpa[3], cpa[3];  // link source planes, likewise (FV_LINK)
-    constexpr bool link = (FV & FV_LINK) != 0, guo = (FV & FV_GUO) != 0;
+    constexpr bool link = (FV & FV_LINK) != 0;
     if (link) {
 #pragma unroll
         for (int q = 0; q < 3; q++) lpa[q] = cpa[q] = pk(R(0), R(0));
@@ -756,24 +933,10 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
             if (l_valid(row)) {
                 int sgn_r;
                 lsrc(row, sgn_r);
-                const T d1 = padd(padd(lpf[1], lpf[5]), lpf[7]), d2 = padd(padd(lpf[2], lpf[6]), lpf[8]);
-                T drho = padd(padd(padd(lpf[0], lpf[3]), padd(lpf[4], d1)), d2);
-                T jz = psub(d1, d2);
-                T jr = psub(padd(padd(lpf[3], lpf[5]), lpf[8]), padd(padd(lpf[4], lpf[6]), lpf[7]));
-                if (link) {
-                    // arrival halves h_i(y)/2: zeroth moment S0/2, first moment H/2
-                    const T half = pk(R(0.5), R(0.5));
-                    drho = pfma(half, lpa[0], drho);
-                    jz = pfma(half, lpa[1], jz);
-                    jr = pfma(half, lpa[2], jr);
-                }
-                const T rho = padd(drho, pk(rho_ref, rho_ref));
-                if (mp) {
-                    const T arg = psub(pmul(rho, pk(R(1) / R(3), R(1) / R(3))), eos_p2<R>(p, rho));
-                    if (!(arg.x >= R(0)) || (l_v1 && !(arg.y >= R(0)))) bad |= ERRBIT_PSI;
-                    st2(sPsi + (row & (DP - 1)) * WL, lc, pk(sqrt_nonneg(arg.x), sqrt_nonneg(arg.y)));
-                }
-                if (!(rho.x > R(0)) || (l_v1 && !(rho.y > R(0)))) bad |= ERRBIT_RHO;
+                T drho, jz, jr;
+                moments2<link, R>(lpf, lpa, drho, jz, jr);
+                const T psi = psi2<mp>(p, drho, l_v1, bad);
+                if (mp) st2(sPsi + (row & (DP - 1)) * WL, lc, psi);
                 const int cu = lc - 4;
                 if (cu >= 0 && cu < WU) {
                     const int sj = (row & (DJ - 1)) * WU;
@@ -826,14 +989,7 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
                     const Tri<T> z0 = ld3<T>(sPsi + (er & (DP - 1)) * WL, c);
                     const Tri<T> zm = ld3<T>(sPsi + ((er - 1) & (DP - 1)) * WL, c);
                     const Tri<T> zq = ld3<T>(sPsi + ((er + 1) & (DP - 1)) * WL, c);
-                    // Kupershtokh force, Eq. (kupershtokhforcing)
-                    T s1z, s1r, s2z, s2r;
-                    kup_moments2<R>(zm, z0, zq, s1z, s1r);
-                    kup_moments2<R>(sq3(zm), sq3(z0), sq3(zq), s2z, s2r);
-                    const T psi = z0.b;
-                    const T bk = pmul(pk(R(6) * kB, R(6) * kB), psi), a6k = pk(R(6) * kA, R(6) * kA);
-                    fz = pfma(a6k, s2z, pfma(bk, s1z, fz));
-                    fr = pfma(a6k, s2r, pfma(bk, s1r, fr));
+                    force_k2(p, zm, z0, zq, fz, fr);
                     if (ax) {
                         // F_axis, Eq. (multiphasecorrections); psi_rr = D_r(psi_r), psi_rz = D_r(psi_z)
                         const int cd = uc + 2;
@@ -845,21 +1001,12 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
                         const T psz = ld2<T>(sPz + o0, cd), psr = ld2<T>(sPr + o0, cd);
                         int rrow = er;
                         if (periodic) rrow = row < 0 ? row + nr : (row >= nr ? row - nr : row);
-                        const R ir = rcp(R(rrow) + R(0.5));
-                        const T irr = pk(ir, ir);
-                        const T k3 = pmul(pk(R(3), R(3)), kappa2<R>(p, rho));
-                        const R ca = p.axis_a * kA * ir;
-                        const T a6 = pmul(pk(ca, ca), psr);
-                        const T pir = pmul(psi, irr);
-                        fz = pfma(k3, pfma(pir, prz, pmul(a6, psz)), fz);
-                        fr = pfma(k3, pfma(pir, psub(prr, pmul(psr, irr)), pmul(a6, psr)), fr);
+                        force_axis2(p, rho, z0.b, psz, psr, prr, prz, rrow, fz, fr);
                     }
                 }
-                const T irho = prcp<R>(rho);
-                const T half = pk(R(0.5), R(0.5));
+                T vz, vr;
+                velocity2<R>(rho, ld2<T>(sJz + sj, uc), ld2<T>(sJr + sj, uc), fz, fr, vz, vr);
                 const int ou = (row & (DU - 1)) * WU;
-                const T vz = pmul(pfma(half, fz, ld2<T>(sJz + sj, uc)), irho);
-                const T vr = pmul(pfma(half, fr, ld2<T>(sJr + sj, uc)), irho);
                 st2(sUz + ou, uc, s_uz > 0 ? vz : psub(pk(R(0), R(0)), vz));
                 st2(sUr + ou, uc, s_ur > 0 ? vr : psub(pk(R(0), R(0)), vr));
             }
@@ -884,33 +1031,17 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
                 const int sj = (row & (DJ - 1)) * WU;
                 const T drho = ld2<T>(sRho + sj, c);
                 const T rho = padd(drho, pk(rho_ref, rho_ref));
-                const T irho = prcp<R>(rho);
-                const T u0z = pmul(ld2<T>(sJz + sj, c), irho), u0r = pmul(ld2<T>(sJr + sj, c), irho);
                 const int ou = (row & (DU - 1)) * WU;
                 const T uz = ld2<T>(sUz + ou, c), ur = ld2<T>(sUr + ou, c);
-                // EDM velocity shift F / rho from u = u0 + F / (2 rho)
-                const T two = pk(R(2), R(2));
-                const T u1z = pfma(two, psub(uz, u0z), u0z), u1r = pfma(two, psub(ur, u0r), u0r);
-                T Hz = pk(R(0), R(0)), Hr = Hz, m0 = Hz;
+                T Hz = pk(R(0), R(0)), Hr = Hz, mir = Hz, rur = Hz;
                 if (ax) {
                     const int o2m = ((row - 2) & (DU - 1)) * WU, o1m = ((row - 1) & (DU - 1)) * WU;
                     const int o1p = ((row + 1) & (DU - 1)) * WU, o2p = ((row + 2) & (DU - 1)) * WU;
                     const T duz_dr = fd_r2<R, T>(sUz + o2m, sUz + o1m, sUz + o1p, sUz + o2p, c);
                     T dur_dz, dur_dr;
                     fd_both2<R>(sUr + o2m, sUr + o1m, sUr + ou, sUr + o1p, sUr + o2p, c, dur_dz, dur_dr);
-                    const R ir = rcp(R(row) + R(0.5));
-                    const T irr = pk(ir, ir);
-                    const T mu = pmul(rho, pk(nu, nu));
-                    const T rur = pmul(rho, ur);
-                    Hz = pmul(psub(pmul(mu, padd(duz_dr, dur_dz)), pmul(rur, uz)), irr);
-                    Hr = pmul(psub(pmul(pmul(pk(R(2), R(2)), mu), pfma(pk(hrs * ir, hrs * ir), ur, dur_dr)),
-                                   pmul(rur, ur)),
-                              irr);
-                    m0 = pmul(pk(-ir, -ir), rur);
+                    source2(p, rho, uz, ur, duz_dr, dur_dz, dur_dr, row, Hz, Hr, mir, rur);
                 }
-                // f*_i = (1 - omega) f_i + f^eq_i(u1) - (1 - omega) f^eq_i(u0) + h_i, opposite
-                // directions sharing the even part (see march)
-                const T om1p = pk(om1, om1), c15 = pk(R(1.5), R(1.5)), c45 = pk(R(4.5), R(4.5));
                 R* o = fout + row * pitch + k0 + cc;
                 auto store_to = [&](R* q, int i, T v) {
                     if (kStreamStore) {
@@ -925,77 +1056,10 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
                             q[i * plane] = v.x;
                     }
                 };
-                auto store = [&](int i, T v) { store_to(o, i, v); };
-                // c_i . v for the first direction of opposite pair i, i+1 (i odd)
-                auto cdot = [&](int i, T vz, T vr) {
-                    const int cx = cz_of(i), cy = cr_of(i);
-                    T r = cy == 0 ? vz : (cx == 0 ? vr : (cx == cy ? padd(vz, vr) : psub(vz, vr)));
-                    if (cx + cy < 0) r = psub(pk(R(0), R(0)), r);  // the first direction points to -z or -r
-                    return r;
-                };
-                // link-midpoint source: this node's arrival half of the previous step's h_i and
-                // the departure half of this step's; this step's S0, H kept for the next step
-                const T half = pk(R(0.5), R(0.5));
-                const T hm0 = link ? pmul(half, m0) : m0, hHz = link ? pmul(half, Hz) : Hz;
-                const T hHr = link ? pmul(half, Hr) : Hr;
-                if (link) {
-                    fi[0] = pfma(pk(R(0.5) * w_of<R>(0), R(0.5) * w_of<R>(0)), ca[0], fi[0]);
-#pragma unroll
-                    for (int m = 0; m < 4; m++) {
-                        const int i = 2 * m + 1;
-                        const R w = w_of<R>(i);
-                        const T ea = pmul(pk(R(0.5) * w, R(0.5) * w), ca[0]);
-                        const T oa = pmul(pk(R(1.5) * w, R(1.5) * w), cdot(i, ca[1], ca[2]));
-                        fi[i] = padd(fi[i], padd(ea, oa));
-                        fi[i + 1] = padd(fi[i + 1], psub(ea, oa));
-                    }
-                    R* hq = hdst + row * pitch + k0 + cc;
-                    store_to(hq, 0, m0);
-                    store_to(hq, 1, Hz);
-                    store_to(hq, 2, Hr);
-                }
-                if (guo) {
-                    // Guo forcing: f*_i = f_i + omega (f^eq_i(u) - f_i) + S_i + h_i with
-                    // S_i = w_i (1 - omega/2) [3 (c_i - u).F + 9 (c_i.u)(c_i.F)], F = 2 rho (u - u0)
-                    const T r2 = pmul(pk(R(2), R(2)), rho);
-                    const T Fz = pmul(r2, psub(uz, u0z)), Fr = pmul(r2, psub(ur, u0r));
-                    const T usq = pfma(uz, uz, pmul(ur, ur)), uF = pfma(uz, Fz, pmul(ur, Fr));
-                    const R gpre = R(1) - R(0.5) * omega;
-                    const T om = pk(omega, omega), gp = pk(gpre, gpre);
-                    const T base = padd(pfma(om, psub(drho, pmul(c15, pmul(rho, usq))),
-                                             pmul(pk(R(-3) * gpre, R(-3) * gpre), uF)),
-                                        hm0);
-                    store(0, pfma(om1p, fi[0], pmul(pk(w_of<R>(0), w_of<R>(0)), base)));
-#pragma unroll
-                    for (int m = 0; m < 4; m++) {
-                        const int i = 2 * m + 1;
-                        const R w = w_of<R>(i);
-                        const T cu = cdot(i, uz, ur), cF = cdot(i, Fz, Fr), cH = cdot(i, hHz, hHr);
-                        const T even = pmul(pk(w, w), padd(base, padd(pmul(pk(R(4.5) * omega, R(4.5) * omega),
-                                                                           pmul(rho, pmul(cu, cu))),
-                                                                      pmul(pk(R(9) * gpre, R(9) * gpre), pmul(cu, cF)))));
-                        const T odd = pmul(pk(R(3) * w, R(3) * w), padd(padd(pmul(om, pmul(rho, cu)), pmul(gp, cF)), cH));
-                        store(i, padd(pfma(om1p, fi[i], even), odd));
-                        store(i + 1, psub(pfma(om1p, fi[i + 1], even), odd));
-                    }
-                } else {
-                    const T u0sq = pfma(u0z, u0z, pmul(u0r, u0r)), u1sq = pfma(u1z, u1z, pmul(u1r, u1r));
-                    const T base =
-                        pfma(pk(omega, omega), drho, pmul(rho, pmul(c15, psub(pmul(om1p, u0sq), u1sq))));
-                    store(0, pfma(om1p, fi[0], pmul(pk(w_of<R>(0), w_of<R>(0)), padd(base, hm0))));
-#pragma unroll
-                    for (int m = 0; m < 4; m++) {
-                        const int i = 2 * m + 1;  // i and i+1 are opposite
-                        const R w = w_of<R>(i);
-                        const T cu0 = cdot(i, u0z, u0r), cu1 = cdot(i, u1z, u1r), cH = cdot(i, hHz, hHr);
-                        const T even = pmul(pk(w, w), padd(padd(base, hm0),
-                                                           pmul(rho, pmul(c45, psub(pmul(cu1, cu1),
-                                                                                    pmul(om1p, pmul(cu0, cu0)))))));
-                        const T odd = pmul(pk(R(3) * w, R(3) * w), pfma(rho, psub(cu1, pmul(om1p, cu0)), cH));
-                        store(i, padd(pfma(om1p, fi[i], even), odd));
-                        store(i + 1, psub(pfma(om1p, fi[i + 1], even), odd));
-                    }
-                }
+                R* hq = link ? hdst + row * pitch + k0 + cc : nullptr;
+                collide2<FV>(
+                    p, fi, ca, drho, ld2<T>(sJz + sj, c), ld2<T>(sJr + sj, c), uz, ur, Hz, Hr, mir, rur,
+                    [&](int i, T v) { store_to(o, i, v); }, [&](int q, T v) { store_to(hq, q, v); });
             }
         }
         __syncthreads();
@@ -1046,9 +1110,8 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB) k_step(Params
 // solve's (z-strip, row) space into tiles and deals them to the CTAs
 // (lbm_tiles.cu): CTA c marches tiles first[c] .. first[c + 1] - 1, each a row
 // range of one strip of one solve.  Even batch steps read f_a and write f_b,
-// odd steps the reverse (and the link source planes h_a / h_b likewise).  A
-// single solve runs as a batch of one.
-template <typename R, int TZ, int RR, int CP, int MINB, bool MP, bool AX, int FV = 0>
+// odd steps the reverse.  Batches larger than a BatchTable.
+template <typename R, int TZ, int RR, int CP, int MINB, bool MP, bool AX>
 __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
     k_step_batch(const BatchSolve<R>* __restrict__ solves, const Tile* __restrict__ tiles,
                  const int* __restrict__ first, int parity, int* __restrict__ err) {
@@ -1066,15 +1129,9 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
         __syncthreads();  // parameters and the skip decision are the same for the whole CTA
         const R* fin = parity ? solves[tl.solve].f_b : solves[tl.solve].f_a;
         R* fo = parity ? const_cast<R*>(solves[tl.solve].f_a) : solves[tl.solve].f_b;
-        const R* hin = nullptr;
-        R* ho = nullptr;
-        if (FV & FV_LINK) {
-            hin = parity ? solves[tl.solve].h_b : solves[tl.solve].h_a;
-            ho = parity ? const_cast<R*>(solves[tl.solve].h_a) : solves[tl.solve].h_b;
-        }
         if (!skip) {
             int bad = 0;
-            march_cp<R, TZ, RR, CP, MP, AX, FV>(sp, fin, fo, tl.strip, tl.j0, tl.jend, smem_raw, bad, hin, ho);
+            march_cp<R, TZ, RR, CP, MP, AX>(sp, fin, fo, tl.strip, tl.j0, tl.jend, smem_raw, bad);
             if (bad) atomicOr(&err[tl.solve], bad);
         }
     }
@@ -1113,8 +1170,8 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
 // and so every result, is that of k_step_batch for a batch of one).
 template <typename R, int TZ, int RR, int CP, int MINB, bool MP, bool AX, int FV = 0>
 __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
-    k_step_single(const BatchSolve<R> s, const Tile* __restrict__ tiles, const int* __restrict__ first, int parity,
-                  int* __restrict__ err) {
+    k_step_single(const BatchSolve<R> s, const LinkSets<R> hs, const Tile* __restrict__ tiles,
+                  const int* __restrict__ first, int parity, int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int skip;  // the solve already went unphysical: its populations are void, leave them
     const R* fin = parity ? s.f_b : s.f_a;
@@ -1122,8 +1179,8 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
     const R* hin = nullptr;
     R* ho = nullptr;
     if (FV & FV_LINK) {
-        hin = parity ? s.h_b : s.h_a;
-        ho = parity ? const_cast<R*>(s.h_a) : s.h_b;
+        hin = parity ? hs.h_b : hs.h_a;
+        ho = parity ? const_cast<R*>(hs.h_a) : hs.h_b;
     }
     const int t1 = first[blockIdx.x + 1];
     for (int t = first[blockIdx.x]; t < t1; t++) {

@@ -10,6 +10,11 @@ struct Tile {
     int solve, strip, j0, jend;
 };
 
+// A tile of the phase kernels: columns from k0 and rows from j0 of solve `solve`.
+struct PhaseTile {
+    int solve, k0, j0;
+};
+
 // Pipeline rows a tile costs beyond its own: 6 halo rows above it and the 12-row
 // lag between the first and the last marching stage.
 constexpr int kTileFillRows = 18;

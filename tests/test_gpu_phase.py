@@ -1,0 +1,64 @@
+"""The phase kernels (csrc/lbm_phase.cuh) at the edges of their tiles: 64 (FP32)
+or 32 (FP64) columns by 4 or 8 rows, psi halos of 4, wrapped and mirrored
+neighbours.  FP32 steps to the same bits as the marching kernel (chunked rows);
+FP64 meets the parity bar of the oracle."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1512_01977_gb300 import inputs as I
+from tests._cases import Case, component_errs, rel_err, run_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1512_01977_gb300 import build, lbm as L
+
+    build.build()
+    L.lib()
+    return L
+
+
+def _fields(c, seed):
+    rng = np.random.default_rng(seed)
+    rv, rl = c.coexistence()
+    mid = 0.5 * (rl - rv)
+    rho = rl - 0.1 * mid * rng.uniform(size=(c.nr, c.nz))  # every node its own value
+    _, uz, ur = I.random_state(c.nz, c.nr, 1.0, 0.0, 1e-3, seed)
+    return rho, uz, ur * (np.arange(c.nr) + 0.5)[:, None] / c.nr
+
+
+@pytest.mark.parametrize("top,axis", [(O.TOP_FREESLIP, 1), (O.TOP_NOSLIP, 1), (O.TOP_PERIODIC, 0)])
+@pytest.mark.parametrize("nz,nr", [(1, 16), (2, 17), (3, 19), (63, 20), (64, 21), (65, 16), (68, 24), (69, 23),
+                                   (131, 18), (516, 33), (700, 300)])
+def test_fp32_same_bits_as_marching(lbm, nz, nr, top, axis):
+    c = Case(nz, nr, T_over_Tc=0.9, top=top, axis=axis)
+    fields = _fields(c, 7 * nz + nr)
+    got = []
+    for rows in (0, 1 << 20):
+        s = c.solver(32, c.coexistence()[1])
+        lbm.lbm_axi_set_tuning(s.h, lbm.PATH_FUSED, rows)
+        s.init(*fields).step(5)
+        got.append(np.frombuffer(s.save()[192:], dtype=np.uint32))
+        s.close()
+    np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("nz,nr", [(1, 16), (2, 18), (31, 17), (32, 16), (33, 21), (65, 30)])
+@pytest.mark.parametrize("top,kappa,eos", [(O.TOP_FREESLIP, O.KAPPA_MIXED, O.EOS_VDW),
+                                           (O.TOP_NOSLIP, O.KAPPA_THERMO, O.EOS_CS)])
+def test_fp64_edges_against_the_oracle(lbm, nz, nr, top, kappa, eos):
+    c = Case(nz, nr, T_over_Tc=0.9, top=top, kappa=kappa, eos=eos)
+    fields = _fields(c, nz + nr)
+    mo = run_oracle(c, fields, 20).moments()
+    s = c.solver(64).init(*fields).step(20)
+    mg = s.moments()
+    s.close()
+    assert rel_err(mg["rho"], mo["rho"]) <= 1e-12 and rel_err(mg["p"], mo["p"]) <= 1e-12
+    assert all(e <= 1e-12 for e in component_errs(mg, mo).values())
