@@ -117,13 +117,13 @@ cudaError_t enqueue_step(lbm_axi* h) {
         const lbm::LinkPlanes<float> lk = link_planes<float>(h, c);
         e = Ops<float>::density(h->pf, (const float*)h->f[c], (float*)h->aux, h->derr, h->stream, lk);
         if (e == cudaSuccess)
-            e = Ops<float>::update(h->pf, h->pdd, (const float*)h->f[c], (float*)h->f[c ^ 1], (const float*)h->aux,
+            e = Ops<float>::update(h->pf, (const float*)h->f[c], (float*)h->f[c ^ 1], (const float*)h->aux,
                                    h->stream, lk, guo_of(h));
     } else {
         const lbm::LinkPlanes<double> lk = link_planes<double>(h, c);
         e = Ops<double>::density(h->pdd, (const double*)h->f[c], (double*)h->aux, h->derr, h->stream, lk);
         if (e == cudaSuccess)
-            e = Ops<double>::update(h->pdd, h->pdd, (const double*)h->f[c], (double*)h->f[c ^ 1],
+            e = Ops<double>::update(h->pdd, (const double*)h->f[c], (double*)h->f[c ^ 1],
                                     (const double*)h->aux, h->stream, lk, guo_of(h));
     }
     h->cur = c ^ 1;
@@ -177,24 +177,37 @@ int chunk_steps(const lbm_axi* h) {
 }
 
 int read_error(lbm_axi* h) {
-    if (cudaMemcpyAsync(h->herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
-        return LBM_ERR_CUDA;
-    if (cudaMemsetAsync(h->derr, 0, sizeof(int), h->stream) != cudaSuccess) return LBM_ERR_CUDA;
+    // one launch that writes the pinned word and clears the device's (a copy and a memset take twice as long)
+    if (Ops<float>::take_error(h->derr, h->herr, h->stream) != cudaSuccess) return LBM_ERR_CUDA;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LBM_ERR_CUDA;
     return *h->herr ? LBM_ERR_UNPHYSICAL : LBM_OK;
 }
 
-// Bare velocity of a state whose physical velocity is to be u:
-// the solve holds f^eq(rho, u) and (pz, pr) its physical velocity
-// u + F/(2 rho), so u0 = u - F/(2 rho) = 2 u - (pz, pr), written over (pz, pr).
-__global__ void __launch_bounds__(256) k_bare_from_physical(long long n, const double* __restrict__ uz,
-                                                           const double* __restrict__ ur, double* __restrict__ pz,
-                                                           double* __restrict__ pr) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    const double vz = uz ? uz[c] : 0.0, vr = ur ? ur[c] : 0.0;
-    pz[c] = vz - (pz[c] - vz);
-    pr[c] = vr - (pr[c] - vr);
+// Fields of the current state into device arrays (each may be null) and u into pitched planes (or null).
+cudaError_t enqueue_fields(lbm_axi* h, double* rho, double* uz, double* ur, double* p, void* u) {
+    if (h->precision == 32)
+        return Ops<float>::fields(lbm_handle_solve<float>(h, h->pf, 0), link_planes<float>(h, h->cur), h->pdd, h->cur,
+                                  rho, uz, ur, p, static_cast<float*>(u), h->derr, h->stream);
+    return Ops<double>::fields(lbm_handle_solve<double>(h, h->pdd, 0), link_planes<double>(h, h->cur), h->pdd, h->cur,
+                               rho, uz, ur, p, static_cast<double*>(u), h->derr, h->stream);
+}
+
+cudaError_t enqueue_init(lbm_axi* h, const double* rho, const double* uz, const double* ur, const void* phys) {
+    if (h->precision == 32)
+        return Ops<float>::init(h->pf, stored_rho_ref(h), rho, uz, ur, (float*)h->f[0], h->stream,
+                                static_cast<const float*>(phys), h->derr);
+    return Ops<double>::init(h->pdd, stored_rho_ref(h), rho, uz, ur, (double*)h->f[0], h->stream,
+                             static_cast<const double*>(phys), h->derr);
+}
+
+// Memory of this device that a kernel may write.
+bool writable_on(const void* p, int device) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
 }
 
 struct DeviceGuard {
@@ -391,22 +404,21 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     return LBM_OK;
 }
 
+// f^eq(rho, u) into buffer 0, no error and no arrival halves pending.
+static cudaError_t begin_init(lbm_axi* h, const double* rho, const double* uz, const double* ur) {
+    cudaError_t e = enqueue_init(h, rho, uz, ur, nullptr);
+    h->cur = 0;
+    // a fresh state: clear the sticky error word (a step skips a solve whose word is set)
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->derr, 0, sizeof(int), h->stream);
+    for (int q = 0; q < 2 && e == cudaSuccess && h->hb[0]; q++)
+        e = cudaMemsetAsync(h->hb[q], 0, 3 * (size_t)h->plane * (h->precision == 32 ? 4 : 8), h->stream);
+    return e;
+}
+
 int lbm_axi_init_device(lbm_axi* h, const double* rho, const double* uz, const double* ur) {
     if (!h || !rho) return LBM_ERR_INVALID_ARG;
     DeviceGuard g(h->device);
-    cudaError_t e;
-    if (h->precision == 32) {
-        e = Ops<float>::init(h->pf, stored_rho_ref(h), rho, uz, ur, (float*)h->f[0], h->stream);
-    } else {
-        e = Ops<double>::init(h->pdd, stored_rho_ref(h), rho, uz, ur, (double*)h->f[0], h->stream);
-    }
-    h->cur = 0;
-    // a fresh state: clear the sticky error word (the batched kernel skips a solve whose word is set)
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->derr, 0, sizeof(int), h->stream);
-    // no arrival halves are pending at the start
-    for (int q = 0; q < 2 && e == cudaSuccess && h->hb[0]; q++)
-        e = cudaMemsetAsync(h->hb[q], 0, 3 * (size_t)h->plane * (h->precision == 32 ? 4 : 8), h->stream);
-    if (e != cudaSuccess) return LBM_ERR_CUDA;
+    if (begin_init(h, rho, uz, ur) != cudaSuccess) return LBM_ERR_CUDA;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LBM_ERR_CUDA;
     h->initialized = true;
     h->pending = LBM_OK;
@@ -427,46 +439,35 @@ int lbm_axi_init(lbm_axi* h, const double* rho, const double* uz, const double* 
     return lbm_axi_init_device(h, d_rho, d_uz, d_ur);
 }
 
+// One stream order without a wait between: f^eq(rho, u), its fluid velocity into the field planes, then
+// f^eq(rho, u - F / (2 rho)) unless the state raised an error.
 int lbm_axi_init_physical_device(lbm_axi* h, const double* rho, const double* uz, const double* ur) {
-    int rc = lbm_axi_init_device(h, rho, uz, ur);
-    if (rc != LBM_OK) return rc;
+    if (!h || !rho) return LBM_ERR_INVALID_ARG;
     DeviceGuard g(h->device);
-    const long long n = (long long)h->nz * h->nr;
-    cudaError_t e = enqueue_density(h);
-    if (e == cudaSuccess) {
-        if (h->precision == 32)
-            e = Ops<float>::moments(h->pf, h->pdd, (const float*)h->f[h->cur], (const float*)h->aux, h->mout,
-                                    h->stream);
-        else
-            e = Ops<double>::moments(h->pdd, h->pdd, (const double*)h->f[h->cur], (const double*)h->aux, h->mout,
-                                     h->stream);
-    }
-    if (e == cudaSuccess) {
-        k_bare_from_physical<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(n, uz, ur, h->mout + n,
-                                                                                   h->mout + 2 * n);
-        e = cudaGetLastError();
-    }
+    char* phys = static_cast<char*>(h->aux) + (size_t)h->plane * (h->precision == 32 ? 4 : 8);
+    cudaError_t e = begin_init(h, rho, uz, ur);
+    if (e == cudaSuccess) e = enqueue_fields(h, nullptr, nullptr, nullptr, nullptr, phys);
+    if (e == cudaSuccess) e = enqueue_init(h, rho, uz, ur, phys);
     if (e != cudaSuccess) return LBM_ERR_CUDA;
-    rc = read_error(h);
-    if (rc != LBM_OK) return rc;
-    return lbm_axi_init_device(h, rho, h->mout + n, h->mout + 2 * n);
+    h->initialized = true;
+    h->pending = LBM_OK;
+    return read_error(h);
 }
 
 int lbm_axi_init_physical(lbm_axi* h, const double* rho, const double* uz, const double* ur) {
     if (!h || !rho) return LBM_ERR_INVALID_ARG;
     DeviceGuard g(h->device);
     const size_t n = (size_t)h->nz * h->nr;
-    double* d = nullptr;
-    if (cudaMalloc(&d, 3 * n * sizeof(double)) != cudaSuccess) return LBM_ERR_OOM;
+    double* d = h->mout;  // idle: the velocity between the two passes is in the field planes
     cudaError_t e = cudaMemcpyAsync(d, rho, n * sizeof(double), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess && uz) e = cudaMemcpyAsync(d + n, uz, n * sizeof(double), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess && ur)
         e = cudaMemcpyAsync(d + 2 * n, ur, n * sizeof(double), cudaMemcpyHostToDevice, h->stream);
-    int rc = e == cudaSuccess ? lbm_axi_init_physical_device(h, d, uz ? d + n : nullptr, ur ? d + 2 * n : nullptr)
-                              : LBM_ERR_CUDA;
-    cudaStreamSynchronize(h->stream);
-    cudaFree(d);
-    return rc;
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(h->stream);
+        return LBM_ERR_CUDA;
+    }
+    return lbm_axi_init_physical_device(h, d, uz ? d + n : nullptr, ur ? d + 2 * n : nullptr);
 }
 
 int lbm_axi_step_async(lbm_axi* h, long long n) {
@@ -539,10 +540,10 @@ int lbm_axi_time_kernels(lbm_axi* h, long long n, double* ms) {
             h->cur = c;
         } else if (e == cudaSuccess) {
             if (h->precision == 32)
-                e = Ops<float>::update(h->pf, h->pdd, (const float*)h->f[c], (float*)h->f[c ^ 1],
+                e = Ops<float>::update(h->pf, (const float*)h->f[c], (float*)h->f[c ^ 1],
                                        (const float*)h->aux, h->stream, link_planes<float>(h, c), guo_of(h));
             else
-                e = Ops<double>::update(h->pdd, h->pdd, (const double*)h->f[c], (double*)h->f[c ^ 1],
+                e = Ops<double>::update(h->pdd, (const double*)h->f[c], (double*)h->f[c ^ 1],
                                         (const double*)h->aux, h->stream, link_planes<double>(h, c), guo_of(h));
         }
         if (e == cudaSuccess) e = cudaEventRecord(ev[2], h->stream);
@@ -561,24 +562,20 @@ int lbm_axi_time_kernels(lbm_axi* h, long long n, double* ms) {
     return read_error(h);
 }
 
+// Fields to arrays a kernel may write directly, else through the staging planes.
 int lbm_axi_moments_device(lbm_axi* h, double* rho, double* uz, double* ur, double* p) {
     if (!h) return LBM_ERR_INVALID_ARG;
     if (!h->initialized) return LBM_ERR_STATE;
     DeviceGuard g(h->device);
-    cudaError_t e = enqueue_density(h);
-    if (e == cudaSuccess) {
-        if (h->precision == 32)
-            e = Ops<float>::moments(h->pf, h->pdd, (const float*)h->f[h->cur], (const float*)h->aux, h->mout,
-                                    h->stream);
-        else
-            e = Ops<double>::moments(h->pdd, h->pdd, (const double*)h->f[h->cur], (const double*)h->aux, h->mout,
-                                     h->stream);
-    }
-    if (e != cudaSuccess) return LBM_ERR_CUDA;
     const size_t n = (size_t)h->nz * h->nr;
     double* dst[4] = {rho, uz, ur, p};
+    double* to[4];
+    for (int q = 0; q < 4; q++)
+        to[q] = !dst[q] || writable_on(dst[q], h->device) ? dst[q] : h->mout + q * n;
+    cudaError_t e = enqueue_fields(h, to[0], to[1], to[2], to[3], nullptr);
     for (int q = 0; q < 4 && e == cudaSuccess; q++) {
-        if (dst[q]) e = cudaMemcpyAsync(dst[q], h->mout + q * n, n * sizeof(double), cudaMemcpyDefault, h->stream);
+        if (dst[q] && to[q] != dst[q])
+            e = cudaMemcpyAsync(dst[q], to[q], n * sizeof(double), cudaMemcpyDefault, h->stream);
     }
     if (e != cudaSuccess) return LBM_ERR_CUDA;
     return read_error(h);
@@ -716,19 +713,20 @@ int lbm_axi_mass(lbm_axi* h, double* mass_rw, double* mass_plain) {
     if (!h || !mass_rw) return LBM_ERR_INVALID_ARG;
     if (!h->initialized) return LBM_ERR_STATE;
     DeviceGuard g(h->device);
-    cudaError_t e = enqueue_density(h);
-    if (e == cudaSuccess) {
-        if (h->precision == 32)
-            e = Ops<float>::mass(h->pf, stored_rho_ref(h), (const float*)h->aux, h->partial, h->dred, h->stream);
-        else
-            e = Ops<double>::mass(h->pdd, stored_rho_ref(h), (const double*)h->aux, h->partial, h->dred, h->stream);
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->hred, h->dred, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+    cudaError_t e;
+    if (h->precision == 32)
+        e = Ops<float>::mass(h->pf, (const float*)h->f[h->cur], link_planes<float>(h, h->cur), h->partial, h->hred,
+                             h->derr, h->stream);
+    else
+        e = Ops<double>::mass(h->pdd, (const double*)h->f[h->cur], link_planes<double>(h, h->cur), h->partial, h->hred,
+                              h->derr, h->stream);
     if (e != cudaSuccess) return LBM_ERR_CUDA;
     int rc = read_error(h);
     if (rc != LBM_OK) return rc;
-    *mass_rw = h->hred[0];
-    if (mass_plain) *mass_plain = h->hred[1];
+    // the sums are over rho - rho_ref
+    const double n = (double)h->nz * h->nr, ref = stored_rho_ref(h);
+    *mass_rw = h->hred[0] + ref * (0.5 * n * h->nr);
+    if (mass_plain) *mass_plain = h->hred[1] + ref * n;
     return LBM_OK;
 }
 
@@ -736,16 +734,13 @@ int lbm_axi_pressure_jump(lbm_axi* h, double zc, double rc, double rin, double r
     if (!h || !dp || !(rin > 0) || !(rout >= rin)) return LBM_ERR_INVALID_ARG;
     if (!h->initialized) return LBM_ERR_STATE;
     DeviceGuard g(h->device);
-    cudaError_t e = enqueue_density(h);
-    if (e == cudaSuccess) {
-        if (h->precision == 32)
-            e = Ops<float>::pjump(h->pf, h->pdd, (const float*)h->aux, zc, rc, rin, rout, h->partial, h->dred,
-                                  h->stream);
-        else
-            e = Ops<double>::pjump(h->pdd, h->pdd, (const double*)h->aux, zc, rc, rin, rout, h->partial, h->dred,
-                                   h->stream);
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->hred, h->dred, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+    cudaError_t e;
+    if (h->precision == 32)
+        e = Ops<float>::pjump(h->pf, h->pdd, (const float*)h->f[h->cur], link_planes<float>(h, h->cur), zc, rc, rin,
+                              rout, h->partial, h->hred, h->derr, h->stream);
+    else
+        e = Ops<double>::pjump(h->pdd, h->pdd, (const double*)h->f[h->cur], link_planes<double>(h, h->cur), zc, rc,
+                               rin, rout, h->partial, h->hred, h->derr, h->stream);
     if (e != cudaSuccess) return LBM_ERR_CUDA;
     int rcode = read_error(h);
     if (rcode != LBM_OK) return rcode;

@@ -477,13 +477,13 @@ int lbm_axi_autotune(lbm_axi* h, int trials, lbm_axi_tuning* chosen) {
             const lbm::LinkPlanes<float> lk = link_planes<float>(h, c);
             e = Ops<float>::density(h->pf, (const float*)h->f[c], (float*)h->aux, h->derr, h->stream, lk);
             if (e == cudaSuccess)
-                e = Ops<float>::update(h->pf, h->pdd, (const float*)h->f[c], (float*)h->f[c ^ 1],
+                e = Ops<float>::update(h->pf, (const float*)h->f[c], (float*)h->f[c ^ 1],
                                        (const float*)h->aux, h->stream, lk, guo_of(h));
         } else {
             const lbm::LinkPlanes<double> lk = link_planes<double>(h, c);
             e = Ops<double>::density(h->pdd, (const double*)h->f[c], (double*)h->aux, h->derr, h->stream, lk);
             if (e == cudaSuccess)
-                e = Ops<double>::update(h->pdd, h->pdd, (const double*)h->f[c], (double*)h->f[c ^ 1],
+                e = Ops<double>::update(h->pdd, (const double*)h->f[c], (double*)h->f[c ^ 1],
                                         (const double*)h->aux, h->stream, lk, guo_of(h));
         }
         return e;

@@ -7,8 +7,8 @@
 //                       stored as deviations f_i - w_i rho_ref
 //   aux[4][nr][pitch]   rho - rho_ref, j_z, j_r, psi of the current step
 //
-// One step = k_density (kernel a) + k_update (kernel b).  Reductions (kernel
-// c) and the init/moments passes use the same maps.
+// One step of the two-kernel path = k_density (kernel a) + k_update (kernel b).
+// The init pass uses the same maps; the passes that read a solve are in lbm_read.cuh.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -16,23 +16,18 @@
 namespace lbm {
 
 // ------------------------------------------------- kernel (a): rho, j, psi --
-// Pull-gather the nine populations of node (k, j) (Sec. II.A moments:
-// rho = sum_i f_i, j = sum_i c_i f_i), evaluate psi = sqrt(rho/3 - P_k(rho))
-// (Sec. II.C) and write rho - rho_ref, j_z, j_r, psi.  Raises error bits for
-// rho <= 0, psi^2 < 0 and non-finite values; never traps.
+// rho - rho_ref, j_z, j_r of a node's arrived populations (Sec. II.A moments:
+// rho = sum_i f_i, j = sum_i c_i f_i) and psi = sqrt(rho/3 - P_k(rho)) (Sec.
+// II.C); returns error bits for rho <= 0, psi^2 < 0 and non-finite values.
 template <typename R>
-__global__ void __launch_bounds__(256) k_density(Params<R> p, const R* __restrict__ f, R* __restrict__ aux,
-                                                 int* __restrict__ err, LinkPlanes<R> lk) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (k >= p.nz || j >= p.nr) return;
-    R drho = R(0), jz = R(0), jr = R(0);
+__device__ __forceinline__ int density_node(const Params<R>& p, const R (&f)[Q], const LinkPlanes<R>& lk, int j, int k,
+                                            R& drho, R& jz, R& jr, R& psi) {
+    drho = R(0), jz = R(0), jr = R(0), psi = R(0);
 #pragma unroll
     for (int i = 0; i < Q; i++) {
-        const R fi = f[pull_slot(p, k, j, i)];
-        drho += fi;
-        jz += R(cz_of(i)) * fi;
-        jr += R(cr_of(i)) * fi;
+        drho += f[i];
+        jz += R(cz_of(i)) * f[i];
+        jr += R(cr_of(i)) * f[i];
     }
     if (lk.src) {
         // arrival halves h_i(y)/2: zeroth moment S0/2, first moment H/2
@@ -42,7 +37,6 @@ __global__ void __launch_bounds__(256) k_density(Params<R> p, const R* __restric
         jr += R(0.5) * lk.src[2 * p.plane + o];
     }
     const R rho = p.rho_ref + drho;
-    R psi = R(0);
     int bad = 0;
     if (!(rho > R(0))) bad |= ERRBIT_RHO;
     if (!isfinite(jz) || !isfinite(jr)) bad |= ERRBIT_NONFINITE;
@@ -51,6 +45,21 @@ __global__ void __launch_bounds__(256) k_density(Params<R> p, const R* __restric
         if (!(arg >= R(0))) bad |= ERRBIT_PSI;
         psi = sqrt(arg > R(0) ? arg : R(0));
     }
+    return bad;
+}
+
+// Pull-gather the nine populations of node (k, j) and write rho - rho_ref, j_z,
+// j_r, psi.  Raises error bits; never traps.
+template <typename R>
+__global__ void __launch_bounds__(256) k_density(Params<R> p, const R* __restrict__ f, R* __restrict__ aux,
+                                                 int* __restrict__ err, LinkPlanes<R> lk) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (k >= p.nz || j >= p.nr) return;
+    R fi[Q], drho, jz, jr, psi;
+#pragma unroll
+    for (int i = 0; i < Q; i++) fi[i] = f[pull_slot(p, k, j, i)];
+    const int bad = density_node(p, fi, lk, j, k, drho, jz, jr, psi);
     if (bad) atomicOr(err, bad);
     const long long o = (long long)j * p.pitch + k;
     aux[o] = drho;
@@ -93,6 +102,33 @@ __device__ __forceinline__ void kupershtokh(const R* m, R A, R& fz, R& fr) {
     fr += R(6) * (A * s2r + b * s1r);
 }
 
+// Total force and physical velocity of a node in row j from its psi tile (m, row width WP) and its
+// psi_z, psi_r tiles (width WD); u = j / rho + F / (2 rho) (Sec. II.A, half-force shift).
+template <int WP, int WD, typename R>
+__device__ __forceinline__ void velocity_node(const Params<R>& p, const R* m, const R* pz, const R* pr, int j, R drho,
+                                              R jz, R jr, bool mp, bool ax, R& fz, R& fr, R& uz, R& ur) {
+    const R rho = p.rho_ref + drho;
+    fz = rho * p.gz, fr = R(0);
+    if (mp) {
+        kupershtokh<R, WP>(m, p.A, fz, fr);
+        if (ax) {
+            // F_axis = 3 kappa [psi grad_c(psi_r / r) + (c A / r) psi_r grad_c psi],
+            // Eq. (multiphasecorrections) (c = 6 as printed, 2 from the exact expansion);
+            // psi_rr = D_r(psi_r), psi_rz = D_r(psi_z).
+            const R psi = m[0], psz = pz[0], psr = pr[0];
+            const R prr = fd_r<R, WD>(pr);
+            const R prz = fd_r<R, WD>(pz);
+            const R ir = R(1) / (R(j) + R(0.5));
+            const R k3 = R(3) * kappa_of(p, rho);
+            const R a6 = p.axis_a * p.A * ir * psr;
+            fz += k3 * (psi * prz * ir + a6 * psz);
+            fr += k3 * (psi * (prr - psr * ir) * ir + a6 * psr);
+        }
+    }
+    uz = (jz + R(0.5) * fz) / rho;
+    ur = (jr + R(0.5) * fr) / rho;
+}
+
 // ------------------------------------- kernel (b): the fused update step --
 // One CTA owns a TZ x TR tile of nodes.  Staged in shared memory:
 //   psi            tile + 6 (F on a 2-ring needs psi_rr, which needs psi_r on a 4-ring)
@@ -103,7 +139,6 @@ __device__ __forceinline__ void kupershtokh(const R* m, R A, R& fz, R& fr) {
 // Values of psi_z, psi_r and u beyond the axis or a wall are the mirror
 // images of interior values with their parity (psi, psi_z, u_z even; psi_r,
 // u_r odd; u_z odd at a no-slip wall), evaluated at the mirrored node.
-// MOMENTS = true writes rho, physical u and P_k instead of colliding.
 template <int TZ, int TR>
 struct TileShape {
     static constexpr int PW = TZ + 12, PH = TR + 12;
@@ -113,10 +148,9 @@ struct TileShape {
 };
 
 // GUO: Guo forcing (Sec. II.A) in place of the EDM shift.
-template <typename R, int TZ, int TR, bool MOMENTS, bool GUO = false>
-__global__ void __launch_bounds__(256) k_update(Params<R> p, Params<double> pd, const R* __restrict__ f,
-                                                R* __restrict__ fout, const R* __restrict__ aux,
-                                                double* __restrict__ mout, LinkPlanes<R> lk) {
+template <typename R, int TZ, int TR, bool GUO = false>
+__global__ void __launch_bounds__(256) k_update(Params<R> p, const R* __restrict__ f, R* __restrict__ fout,
+                                                const R* __restrict__ aux, LinkPlanes<R> lk) {
     using S = TileShape<TZ, TR>;
     constexpr int PW = S::PW, PH = S::PH, DW = S::DW, DH = S::DH, UW = S::UW, UH = S::UH;
     constexpr int NT = 256;
@@ -187,30 +221,10 @@ __global__ void __launch_bounds__(256) k_update(Params<R> p, Params<double> pd, 
         map_row(p, j0 - 2 + a, 1, uz_top, s_uz);
         const int jl = p.top == TOP_PERIODIC ? j0 - 2 + a : jm;  // see stage 1
         const int lu = (jl - j0 + 2) * UW + b;
-        const R drho = sRho[lu];
-        const R rho = p.rho_ref + drho;
-        R fz = rho * p.gz, fr = R(0);
-        if (mp) {
-            const R* m = sPsi + (jl - j0 + 6) * PW + (b + 4);
-            kupershtokh<R, PW>(m, p.A, fz, fr);
-            if (ax) {
-                // F_axis = 3 kappa [psi grad_c(psi_r / r) + (c A / r) psi_r grad_c psi],
-                // Eq. (multiphasecorrections) (c = 6 as printed, 2 from the exact expansion);
-                // psi_rr = D_r(psi_r), psi_rz = D_r(psi_z).
-                const int ld = (jl - j0 + 4) * DW + (b + 2);
-                const R psi = m[0], psz = sPz[ld], psr = sPr[ld];
-                const R prr = fd_r<R, DW>(sPr + ld);
-                const R prz = fd_r<R, DW>(sPz + ld);
-                const R ir = R(1) / (R(jm) + R(0.5));
-                const R k3 = R(3) * kappa_of(p, rho);
-                const R a6 = p.axis_a * p.A * ir * psr;
-                fz += k3 * (psi * prz * ir + a6 * psz);
-                fr += k3 * (psi * (prr - psr * ir) * ir + a6 * psr);
-            }
-        }
-        // u = j / rho + F / (2 rho)  (Sec. II.A, velocity with half-force shift)
-        const R uz = (sJz[lu] + R(0.5) * fz) / rho;
-        const R ur = (sJr[lu] + R(0.5) * fr) / rho;
+        R fz, fr, uz, ur;
+        const int ld = (jl - j0 + 4) * DW + (b + 2);
+        velocity_node<PW, DW>(p, sPsi + (jl - j0 + 6) * PW + (b + 4), sPz + ld, sPr + ld, jm, sRho[lu], sJz[lu], sJr[lu],
+                              mp, ax, fz, fr, uz, ur);
         sUz[idx] = R(s_uz) * uz;
         sUr[idx] = R(s_ur) * ur;
         const int ti = a - 2, tk = b - 2;
@@ -230,17 +244,6 @@ __global__ void __launch_bounds__(256) k_update(Params<R> p, Params<double> pd, 
         const R drho = sRho[lu];
         const R rho = p.rho_ref + drho;
         const R uz = sUz[lu], ur = sUr[lu];
-        if (MOMENTS) {
-            const long long o = (long long)j * p.nz + k;
-            const double rd = (double)pd.rho_ref + (double)drho;
-            if (mout) {
-                mout[o] = rd;
-                mout[(long long)p.nz * p.nr + o] = (double)uz;
-                mout[2LL * p.nz * p.nr + o] = (double)ur;
-                mout[3LL * p.nz * p.nr + o] = mp ? eos_p(pd, rd) : rd / 3.0;
-            }
-            continue;
-        }
         const R irho = R(1) / rho;
         const R u0z = sJz[lu] / rho, u0r = sJr[lu] / rho;
         const R duz = sFz[ti * TZ + tk] * irho, dur = sFr[ti * TZ + tk] * irho;
@@ -310,13 +313,22 @@ __global__ void __launch_bounds__(256) k_update(Params<R> p, Params<double> pd, 
 template <typename R>
 __global__ void __launch_bounds__(256) k_init(Params<R> p, double rho_ref, const double* __restrict__ rho,
                                               const double* __restrict__ uz, const double* __restrict__ ur,
-                                              R* __restrict__ f) {
+                                              R* __restrict__ f, const R* __restrict__ phys,
+                                              const int* __restrict__ err) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (k >= p.nz || j >= p.nr) return;
     const long long c = (long long)j * p.nz + k;
     const double d = rho[c];
-    const double vz = uz ? uz[c] : 0.0, vr = ur ? ur[c] : 0.0;
+    double vz = uz ? uz[c] : 0.0, vr = ur ? ur[c] : 0.0;
+    if (phys) {
+        // the fluid velocity is to be (vz, vr), and u + F / (2 rho) of f^eq(rho, u) is phys (two pitched
+        // planes): the bare velocity u - F / (2 rho) = u - (phys - u).  A state that raised an error stays.
+        if (*err) return;
+        const R* q = phys + ((long long)j * p.pitch + k);
+        vz = vz - ((double)q[0] - vz);
+        vr = vr - ((double)q[p.plane] - vr);
+    }
     if constexpr (sizeof(R) == 4) {
         // FP32 deviations f_i - w_i rho_ref = w_i [(rho - rho_ref) + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u.u)]:
         // rho - rho_ref in FP64, the velocity part in FP32 (FP64 arithmetic would set this kernel's time)
@@ -363,55 +375,13 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double* out) {
     }
 }
 
-// sum (j + 1/2) rho and sum rho over all nodes (blockDim.x = 256).
-template <typename R>
-__global__ void __launch_bounds__(256) k_mass(Params<R> p, double rho_ref, const R* __restrict__ aux,
-                                              double* __restrict__ partial) {
-    double v[2] = {0.0, 0.0};
-    const long long n = (long long)p.nz * p.nr;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(c / p.nz), k = (int)(c - (long long)j * p.nz);
-        const double rho = rho_ref + (double)aux[(long long)j * p.pitch + k];
-        v[0] += (j + 0.5) * rho;
-        v[1] += rho;
-    }
-    block_sum<2>(v, partial + 2 * blockIdx.x);
-}
-
-// Sums of P_k (in FP64) and node counts inside d < r_in and outside d > r_out.
-template <typename R>
-__global__ void __launch_bounds__(256) k_pjump(Params<R> p, Params<double> pd, const R* __restrict__ aux,
-                                               double zc, double rc, double rin, double rout,
-                                               double* __restrict__ partial) {
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    const long long n = (long long)p.nz * p.nr;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(c / p.nz), k = (int)(c - (long long)j * p.nz);
-        const double dz = k + 0.5 - zc, dr = j + 0.5 - rc;
-        const double d = sqrt(dz * dz + dr * dr);
-        if (d < rin || d > rout) {
-            const double rho = pd.rho_ref + (double)aux[(long long)j * p.pitch + k];
-            const double pk = p.multiphase ? eos_p(pd, rho) : rho / 3.0;
-            if (d < rin) {
-                v[0] += pk;
-                v[1] += 1.0;
-            } else {
-                v[2] += pk;
-                v[3] += 1.0;
-            }
-        }
-    }
-    block_sum<4>(v, partial + 4 * blockIdx.x);
-}
-
 // Final sum of the per-block partials by one warp (launch <<<1, 32>>>): lane l
 // adds partials l, l + 32, l + 64, ... in that order, then a shuffle tree
 // combines the lanes.  The order is fixed, so the result is bitwise
 // reproducible for a given number of partials.
 template <int N>
-__global__ void k_reduce_final(const double* __restrict__ partial, int nblocks, double* __restrict__ out) {
+__device__ __forceinline__ void reduce_partials(const double* __restrict__ partial, int nblocks,
+                                                double* __restrict__ out) {
     if (blockIdx.x != 0 || threadIdx.x >= 32) return;
     const int lane = threadIdx.x;
     double s[N];
@@ -430,6 +400,11 @@ __global__ void k_reduce_final(const double* __restrict__ partial, int nblocks, 
 #pragma unroll
         for (int q = 0; q < N; q++) out[q] = s[q];
     }
+}
+
+template <int N>
+__global__ void k_reduce_final(const double* __restrict__ partial, int nblocks, double* __restrict__ out) {
+    reduce_partials<N>(partial, nblocks, out);
 }
 
 }  // namespace lbm

@@ -27,19 +27,26 @@ struct Ops {
                                LinkPlanes<R> lk = {nullptr, nullptr});
     // kernel (b): the fused stream + force + EDM + axisymmetric source + collide step
     // (guo: Guo forcing in place of the EDM shift).
-    static cudaError_t update(const Params<R>& p, const Params<double>& pd, const R* f, R* fout, const R* aux,
-                              cudaStream_t s, LinkPlanes<R> lk = {nullptr, nullptr}, bool guo = false);
-    // rho, physical u, P_k of the current state into mout[4][nz*nr] (after density()).
-    static cudaError_t moments(const Params<R>& p, const Params<double>& pd, const R* f, const R* aux,
-                               double* mout, cudaStream_t s);
+    static cudaError_t update(const Params<R>& p, const R* f, R* fout, const R* aux, cudaStream_t s,
+                              LinkPlanes<R> lk = {nullptr, nullptr}, bool guo = false);
+    // rho, physical u, P_k of the state in v.f_a (parity 0) or v.f_b: FP64 arrays [j * nz + k] on the device,
+    // and u into two pitched planes of R (each may be null).  lk: as for density.
+    static cudaError_t fields(const BatchSolve<R>& v, LinkPlanes<R> lk, const Params<double>& pd, int parity,
+                              double* rho, double* uz, double* ur, double* pk, R* u, int* err, cudaStream_t s);
+    // f^eq(rho, u); with phys (u + F / (2 rho) of that state, two pitched planes) f^eq(rho, u - F / (2 rho))
+    // unless *err is set.
     static cudaError_t init(const Params<R>& p, double rho_ref, const double* rho, const double* uz,
-                            const double* ur, R* f, cudaStream_t s);
-    // kernel (c): out[0] = sum (j+1/2) rho, out[1] = sum rho.
-    static cudaError_t mass(const Params<R>& p, double rho_ref, const R* aux, double* partial, double* out,
+                            const double* ur, R* f, cudaStream_t s, const R* phys = nullptr,
+                            const int* err = nullptr);
+    // kernel (c): out[0] = sum (j+1/2) (rho - rho_ref), out[1] = sum (rho - rho_ref) (host-mapped or device).
+    static cudaError_t mass(const Params<R>& p, const R* f, LinkPlanes<R> lk, double* partial, double* out, int* err,
                             cudaStream_t s);
     // out[0..3] = sum P_k inside, count inside, sum P_k outside, count outside.
-    static cudaError_t pjump(const Params<R>& p, const Params<double>& pd, const R* aux, double zc, double rc,
-                             double rin, double rout, double* partial, double* out, cudaStream_t s);
+    static cudaError_t pjump(const Params<R>& p, const Params<double>& pd, const R* f, LinkPlanes<R> lk, double zc,
+                             double rc, double rin, double rout, double* partial, double* out, int* err,
+                             cudaStream_t s);
+    // *host (pinned) = *err, *err = 0.
+    static cudaError_t take_error(int* err, int* host, cudaStream_t s);
     // dynamic shared memory of one k_update CTA, bytes
     static size_t update_smem();
     // one-time kernel attributes (shared-memory opt-in); call outside stream capture

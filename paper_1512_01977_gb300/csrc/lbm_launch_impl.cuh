@@ -4,6 +4,7 @@
 #include "lbm_kernels.cuh"
 #include "lbm_launch.h"
 #include "lbm_phase.cuh"
+#include "lbm_read.cuh"
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -26,22 +27,6 @@ template <typename R>
 size_t Ops<R>::update_smem() {
     using T = UpdateTile<R>;
     return sizeof(R) * (size_t)TileShape<T::TZ, T::TR>::elems;
-}
-
-template <typename R>
-static cudaError_t launch_update(const Params<R>& p, const Params<double>& pd, const R* f, R* fout, const R* aux,
-                                 double* mout, bool moments, cudaStream_t s, LinkPlanes<R> lk, bool guo) {
-    using T = UpdateTile<R>;
-    const size_t smem = Ops<R>::update_smem();
-    dim3 grid((p.nz + T::TZ - 1) / T::TZ, (p.nr + T::TR - 1) / T::TR);
-    if (moments) {
-        k_update<R, T::TZ, T::TR, true><<<grid, 256, smem, s>>>(p, pd, f, nullptr, aux, mout, lk);
-    } else if (guo) {
-        k_update<R, T::TZ, T::TR, false, true><<<grid, 256, smem, s>>>(p, pd, f, fout, aux, nullptr, lk);
-    } else {
-        k_update<R, T::TZ, T::TR, false><<<grid, 256, smem, s>>>(p, pd, f, fout, aux, nullptr, lk);
-    }
-    return cudaGetLastError();
 }
 
 // Strip width and rows per iteration of the fused kernel per precision.
@@ -94,14 +79,9 @@ template <typename R>
 cudaError_t Ops<R>::prepare() {
     using T = UpdateTile<R>;
     const int smem = (int)update_smem();
-    cudaError_t e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR, false, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = set_step_attr<R>((int)step_smem());
     // the marching forms (FP32): attributes and occupancy are settled here, outside any stream capture
     if constexpr (sizeof(R) == 4) {
@@ -166,38 +146,46 @@ cudaError_t Ops<R>::density(const Params<R>& p, const R* f, R* aux, int* err, cu
 }
 
 template <typename R>
-cudaError_t Ops<R>::update(const Params<R>& p, const Params<double>& pd, const R* f, R* fout, const R* aux,
-                           cudaStream_t s, LinkPlanes<R> lk, bool guo) {
-    return launch_update<R>(p, pd, f, fout, aux, nullptr, false, s, lk, guo);
-}
-
-template <typename R>
-cudaError_t Ops<R>::moments(const Params<R>& p, const Params<double>& pd, const R* f, const R* aux, double* mout,
-                            cudaStream_t s) {
-    return launch_update<R>(p, pd, f, nullptr, aux, mout, true, s, LinkPlanes<R>{nullptr, nullptr}, false);
-}
-
-template <typename R>
-cudaError_t Ops<R>::init(const Params<R>& p, double rho_ref, const double* rho, const double* uz, const double* ur,
-                         R* f, cudaStream_t s) {
-    dim3 block(32, 8), grid((p.nz + 31) / 32, (p.nr + 7) / 8);
-    k_init<R><<<grid, block, 0, s>>>(p, rho_ref, rho, uz, ur, f);
+cudaError_t Ops<R>::update(const Params<R>& p, const R* f, R* fout, const R* aux, cudaStream_t s, LinkPlanes<R> lk,
+                           bool guo) {
+    using T = UpdateTile<R>;
+    const size_t smem = update_smem();
+    dim3 grid((p.nz + T::TZ - 1) / T::TZ, (p.nr + T::TR - 1) / T::TR);
+    if (guo)
+        k_update<R, T::TZ, T::TR, true><<<grid, 256, smem, s>>>(p, f, fout, aux, lk);
+    else
+        k_update<R, T::TZ, T::TR><<<grid, 256, smem, s>>>(p, f, fout, aux, lk);
     return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t Ops<R>::mass(const Params<R>& p, double rho_ref, const R* aux, double* partial, double* out,
+cudaError_t Ops<R>::init(const Params<R>& p, double rho_ref, const double* rho, const double* uz, const double* ur,
+                         R* f, cudaStream_t s, const R* phys, const int* err) {
+    dim3 block(32, 8), grid((p.nz + 31) / 32, (p.nr + 7) / 8);
+    k_init<R><<<grid, block, 0, s>>>(p, rho_ref, rho, uz, ur, f, phys, err);
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t Ops<R>::mass(const Params<R>& p, const R* f, LinkPlanes<R> lk, double* partial, double* out, int* err,
                          cudaStream_t s) {
-    k_mass<R><<<kReduceBlocks, 256, 0, s>>>(p, rho_ref, aux, partial);
+    k_mass<R><<<kReduceBlocks, 256, 0, s>>>(p, f, lk, partial, err);
     k_reduce_final<2><<<1, 32, 0, s>>>(partial, kReduceBlocks, out);
     return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t Ops<R>::pjump(const Params<R>& p, const Params<double>& pd, const R* aux, double zc, double rc,
-                          double rin, double rout, double* partial, double* out, cudaStream_t s) {
-    k_pjump<R><<<kReduceBlocks, 256, 0, s>>>(p, pd, aux, zc, rc, rin, rout, partial);
+cudaError_t Ops<R>::pjump(const Params<R>& p, const Params<double>& pd, const R* f, LinkPlanes<R> lk, double zc,
+                          double rc, double rin, double rout, double* partial, double* out, int* err,
+                          cudaStream_t s) {
+    k_pjump<R><<<kReduceBlocks, 256, 0, s>>>(p, pd, f, lk, zc, rc, rin, rout, partial, err);
     k_reduce_final<4><<<1, 32, 0, s>>>(partial, kReduceBlocks, out);
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t Ops<R>::take_error(int* err, int* host, cudaStream_t s) {
+    k_take_error<<<1, 1, 0, s>>>(err, host);
     return cudaGetLastError();
 }
 
@@ -483,6 +471,47 @@ cudaError_t Ops<R>::phase_step_many(const BatchSolve<R>* solves, const PhaseTile
     const PhaseMany<R> a{solves, tiles, parity, err};
     return rows == 4 ? phases_many_of<R, 4>(a, (unsigned)ntiles, (unsigned)nghost, mp, ax, s)
                      : phases_many_of<R, 8>(a, (unsigned)ntiles, (unsigned)nghost, mp, ax, s);
+}
+
+// -------------------------------------------------------------- field passes --
+
+template <int TR>
+static cudaError_t fields64(const BatchSolve<double>& v, const LinkPlanes<double>& lk, const Params<double>& pd,
+                            int parity, const FieldsOut<double>& out, int* err, cudaStream_t s) {
+    const int across = (v.p.nz + PhaseShape<double>::TZ - 1) / PhaseShape<double>::TZ;
+    const unsigned grid = (unsigned)across * (unsigned)((v.p.nr + TR - 1) / TR);
+    const PhaseOne<double> a{v, lk.src, lk.dst, parity, across, err};
+    const bool mp = v.p.multiphase != 0, ax = v.p.axis != 0;
+    cudaError_t e;
+    if (mp)
+        e = lk.src ? launch_early(k_phase_l<double, TR, true, true>, grid, 32 * TR, s, a)
+                   : launch_early(k_phase_l<double, TR, true, false>, grid, 32 * TR, s, a);
+    else
+        e = lk.src ? launch_early(k_phase_l<double, TR, false, true>, grid, 32 * TR, s, a)
+                   : launch_early(k_phase_l<double, TR, false, false>, grid, 32 * TR, s, a);
+    if (e != cudaSuccess) return e;
+    if (mp && ax) return launch_early(k_fields64<TR, true, true>, grid, 32 * TR, s, a, out, pd);
+    if (mp) return launch_early(k_fields64<TR, true, false>, grid, 32 * TR, s, a, out, pd);
+    return launch_early(k_fields64<TR, false, false>, grid, 32 * TR, s, a, out, pd);
+}
+
+template <typename R>
+cudaError_t Ops<R>::fields(const BatchSolve<R>& v, LinkPlanes<R> lk, const Params<double>& pd, int parity, double* rho,
+                           double* uz, double* ur, double* pk, R* u, int* err, cudaStream_t s) {
+    const FieldsOut<R> out{rho, uz, ur, pk, u};
+    if constexpr (sizeof(R) == 8) {
+        return phase_rows((long long)v.p.nz * v.p.nr) == 4 ? fields64<4>(v, lk, pd, parity, out, err, s)
+                                                           : fields64<8>(v, lk, pd, parity, out, err, s);
+    } else {
+        // 16 rows per block, 8 while that leaves SMs without one
+        const int across = (v.p.nz + 31) / 32;
+        const R* f = parity ? v.f_b : v.f_a;
+        if ((long long)v.p.nz * v.p.nr <= 2 * 152 * 512)
+            k_fields<8><<<across * ((v.p.nr + 7) / 8), 256, 0, s>>>(v.p, pd, f, lk, out, err);
+        else
+            k_fields<16><<<across * ((v.p.nr + 15) / 16), 256, 0, s>>>(v.p, pd, f, lk, out, err);
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace lbm

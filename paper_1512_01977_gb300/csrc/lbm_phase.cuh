@@ -90,10 +90,14 @@ __host__ __device__ inline long long u_plane(int nz, int nr) {
 }
 constexpr int kGhostRows = 2;
 
-// A row of psi within four rows of the grid: its mirror (even) or wrapped image.  nr >= kStepMinRows.
+// A row of psi within four rows of the grid: its mirror (even) or wrapped image.
 __device__ __forceinline__ int mirror_row(int row, int nr, bool periodic) {
-    if (row < 0) return periodic ? row + nr : -1 - row;
-    if (row >= nr) return periodic ? row - nr : 2 * nr - 1 - row;
+    while (row < 0 || row >= nr) {  // once unless nr is smaller than the halo (the field pass takes any nr)
+        if (row < 0)
+            row = periodic ? row + nr : -1 - row;
+        else
+            row = periodic ? row - nr : 2 * nr - 1 - row;
+    }
     return row;
 }
 
@@ -422,6 +426,14 @@ __device__ __forceinline__ void pull1(const Params<double>& p, const double* __r
     fi[6] = f[q.o[6] + (q.stay ? k : kp)];
 }
 
+__device__ __forceinline__ void moments1(const double (&f)[Q], double& drho, double& jz, double& jr) {
+    const double x = f[5] - f[6], y = f[7] - f[8];
+    jz = (f[1] - f[2]) + (x + y);
+    jr = (f[3] - f[4]) + (x - y);
+    drho = (f[0] + ((f[1] + f[2]) + (f[3] + f[4]))) + ((f[5] + f[6]) + (f[7] + f[8]));
+}
+__device__ __forceinline__ bool finite1(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 template <int TR, bool MP, bool LINK>
 __device__ __forceinline__ void phase_l1(const Params<double>& p, const PhaseWork<double>& w, const double* h_src,
                                          int failed) {
@@ -429,9 +441,8 @@ __device__ __forceinline__ void phase_l1(const Params<double>& p, const PhaseWor
     if (row >= p.nr || k >= p.nz) return;
     double f[Q];
     pull1(p, w.f, row, k, f);
-    const double x = f[5] - f[6], y = f[7] - f[8];
-    double jz = (f[1] - f[2]) + (x + y), jr = (f[3] - f[4]) + (x - y);
-    double drho = (f[0] + ((f[1] + f[2]) + (f[3] + f[4]))) + ((f[5] + f[6]) + (f[7] + f[8]));
+    double drho, jz, jr;
+    moments1(f, drho, jz, jr);
     if (LINK) {
         double a[3];
         link3(p, h_src, row, k, a);
@@ -440,7 +451,7 @@ __device__ __forceinline__ void phase_l1(const Params<double>& p, const PhaseWor
         jr = fma(0.5, a[2], jr);
     }
     const double rho = p.rho_ref + drho;
-    int bad = positive(rho) ? 0 : ERRBIT_RHO;
+    int bad = (positive(rho) ? 0 : ERRBIT_RHO) | (finite1(jz) && finite1(jr) ? 0 : ERRBIT_NONFINITE);
     double psi = 0.0;
     if (MP) {
         const double arg = fma(rho, 1.0 / 3.0, -eos_p3(p, rho));
@@ -464,9 +475,10 @@ struct PhaseU1 {
     static constexpr int elems = WP * (TR + 8) + 4 * WP * (TR + 4) + 2 * WD * (TR + 4);
 };
 
-template <int TR, bool MP, bool AX>
+// put(row, k, drho, u_z, u_r, 1/rho) takes the results.
+template <int TR, bool MP, bool AX, typename P>
 __device__ __forceinline__ void phase_u1(const Params<double>& p, const PhaseWork<double>& w, double* smem,
-                                         int failed) {
+                                         int failed, P&& put) {
     using S = PhaseU1<TR>;
     constexpr int TZ = S::TZ, WP = S::WP, WD = S::WD, NT = 32 * TR, NC = WP * (TR + 4);
     double* sPsi = smem;
@@ -552,11 +564,7 @@ __device__ __forceinline__ void phase_u1(const Params<double>& p, const PhaseWor
         }
     }
     const double irho = rcp3(rho);
-    double* o = w.u + ((long long)(row + kGhostRows) * u_stride<double>(nz) + k0 + c);
-    const long long n = u_plane<double>(nz, nr);
-    o[0] = mul(fma(0.5, fz, jz), irho);
-    o[n] = mul(fma(0.5, fr, row < 0 ? -jr : jr), irho);
-    o[2 * n] = irho;
+    put(row, k0 + c, drho, mul(fma(0.5, fz, jz), irho), mul(fma(0.5, fr, row < 0 ? -jr : jr), irho), irho);
 }
 
 template <int TR, bool AX, int FV>
@@ -691,7 +699,13 @@ __device__ __forceinline__ void phase_u(const Params<R>& p, const PhaseWork<R>& 
             phase_u2<TR, MP, AX, true>(p, w, smem, failed);
     } else {
         __shared__ __align__(16) R smem[PhaseU1<TR>::elems];
-        phase_u1<TR, MP, AX>(p, w, smem, failed);
+        const long long n = u_plane<double>(p.nz, p.nr);
+        phase_u1<TR, MP, AX>(p, w, smem, failed, [&](int row, int k, double, double uz, double ur, double irho) {
+            double* o = w.u + ((long long)(row + kGhostRows) * u_stride<double>(p.nz) + k);
+            o[0] = uz;
+            o[n] = ur;
+            o[2 * n] = irho;
+        });
     }
 }
 template <typename R, int TR, bool AX, int FV>
