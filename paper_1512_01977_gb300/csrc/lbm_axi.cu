@@ -46,6 +46,8 @@ static cudaError_t step_fused(lbm_axi* h, const Params<R>& p, int c) {
     const lbm::LinkSets<R> hs{static_cast<const R*>(h->hb[0]), static_cast<R*>(h->hb[1])};
     if (lbm_by_phases(h->precision, (long long)h->nz * h->nr))
         return Ops<R>::phase_step(s, hs, mp, ax, c, h->derr, h->stream, fv_of(h));
+    if constexpr (sizeof(R) == 4)
+        if (!h->hb[0]) return Ops<R>::step_warp(s, h->d_tiles, h->ncta, mp, ax, c, h->derr, h->stream, fv_of(h));
     return Ops<R>::step_single(s, hs, h->d_tiles, h->d_first, h->ncta, mp, ax, c, h->derr, h->stream, fv_of(h));
 }
 cudaError_t lbm_handle_step_fused(lbm_axi* h, int c) {
@@ -329,17 +331,21 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     h->partial = (double*)dev_alloc(4 * lbm::kReduceBlocks * sizeof(double));
     h->dred = (double*)dev_alloc(4 * sizeof(double));
     h->derr = (int*)dev_alloc(sizeof(int));
-    // tile plan of the marching step (wide strips, one resident wave)
+    // tile plan of the marching step: warps, or CTAs on wide strips with the link source
+    const bool link = o.h_eval == LBM_H_LINK_AVG && o.axis_terms;
     std::vector<lbm::Tile> tiles;
     std::vector<int> first;
     if (lbm_by_phases(o.precision, (long long)nz * nr)) {
         first.assign(1, 0);
     } else {
-        const int slots = Ops<float>::batch_resident_ctas(lbm::kStripWide);
+        const int slots = link ? Ops<float>::batch_resident_ctas(lbm::kStripWide) : Ops<float>::warp_slots();
         int rc = LBM_ERR_CUDA;
         try {
-            rc = slots > 0 ? lbm::plan_tiles(&nz, &nr, 1, lbm::kStripWide, slots, tiles, first, nullptr)
-                           : LBM_ERR_CUDA;
+            if (link)
+                rc = slots > 0 ? lbm::plan_tiles(&nz, &nr, 1, lbm::kStripWide, slots, tiles, first, nullptr) : rc;
+            else
+                rc = slots > 0 ? lbm::plan_warp_tiles(&nz, &nr, 1, slots, tiles) : rc;
+            if (!link) first.assign(1, 0);
         } catch (...) {
             rc = LBM_ERR_OOM;
         }
@@ -349,11 +355,10 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
             return rc;
         }
     }
-    h->ncta = (int)first.size() - 1;
+    h->ncta = link ? (int)first.size() - 1 : (int)tiles.size();
     h->d_tiles = (lbm::Tile*)dev_alloc(tiles.size() * sizeof(lbm::Tile));
     h->d_first = (int*)dev_alloc(first.size() * sizeof(int));
     h->bytes = lbm_axi_footprint(nz, nr, o.precision);
-    const bool link = o.h_eval == LBM_H_LINK_AVG && o.axis_terms;
     if (link) {
         h->hb[0] = dev_alloc(3 * plane_bytes);
         h->hb[1] = dev_alloc(3 * plane_bytes);

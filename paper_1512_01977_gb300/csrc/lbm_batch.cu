@@ -1,6 +1,7 @@
 // Batched stepping and the autotuners (include/lbm_axi_batch.h).
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -11,6 +12,16 @@
 using lbm::BatchSolve;
 using lbm::Ops;
 
+// How a batch steps: three launches over node tiles (lbm_phase.cuh), one warp per tile (lbm_march.cuh) or
+// the marching kernel of the chosen strip width and CTA slots (lbm_step.cuh).
+enum BatchForm { FORM_PHASES, FORM_WARPS, FORM_MARCH };
+
+// The warp march of solves [s0, ...): their descriptors (a kernel argument) and tiles [t0, t0 + nt).
+struct WarpGroup {
+    lbm::BatchTable<float> table;
+    int s0, ns, t0, nt;
+};
+
 struct lbm_axi_batch {
     int n;
     int precision;
@@ -20,7 +31,8 @@ struct lbm_axi_batch {
     std::vector<int> cur0;  // each solve's current buffer when the batch was made
     void* d_solves;         // BatchSolve<R>[n]
     lbm::BatchTable<float>* h_table;  // FP32, n <= BatchTable::N: the descriptors as one kernel argument
-    bool phases;            // this tuning steps by phases (else the marching kernel over d_tiles)
+    BatchForm form;         // of this tuning
+    std::vector<WarpGroup*> groups;
     lbm::PhaseTile* d_ptiles;
     int nptiles, nghost, prows;
     lbm::Tile* d_tiles;     // tile plan for (strip, grid)
@@ -62,9 +74,16 @@ const Params<double>& params_of<double>(const lbm_axi* h) {
 }
 
 // FP64 steps by phases at every tuning; FP32 at the default one (wide strips, grid
-// 0) while the batch is small, the marching kernel at the others.
-bool by_phases(const lbm_axi_batch* b, long long nodes) {
-    return b->precision == 64 || (b->strip == lbm::kStripWide && b->grid == 0 && lbm_by_phases(32, nodes));
+// 0) by phases while the batch is small and by warps beyond, at the others by march2.
+BatchForm form_of(const lbm_axi_batch* b, long long nodes) {
+    if (b->precision == 64) return FORM_PHASES;
+    if (b->strip != lbm::kStripWide || b->grid != 0) return FORM_MARCH;
+    return lbm_by_phases(32, nodes) ? FORM_PHASES : FORM_WARPS;
+}
+
+void drop_groups(lbm_axi_batch* b) {
+    for (WarpGroup* g : b->groups) delete g;
+    b->groups.clear();
 }
 
 template <typename R>
@@ -83,12 +102,12 @@ cudaError_t upload(lbm_axi_batch* b) {
     }
     long long nodes = 0;
     for (int i = 0; i < b->n; i++) nodes += (long long)nz[i] * nr[i];
-    b->phases = by_phases(b, nodes);
+    b->form = form_of(b, nodes);
     std::vector<lbm::Tile> tiles;
     std::vector<lbm::PhaseTile> ptiles;
     size_t inner = 0;  // tiles before the ghost rows'
     std::vector<int> first;
-    if (b->phases) {
+    if (b->form == FORM_PHASES) {
         const int tz = Ops<R>::phase_tile_z();
         b->prows = Ops<R>::phase_rows(nodes);
         try {
@@ -102,6 +121,30 @@ cudaError_t upload(lbm_axi_batch* b) {
         } catch (...) {
             return cudaErrorMemoryAllocation;
         }
+    } else if (b->form == FORM_WARPS) {
+        drop_groups(b);
+        const int slots = Ops<float>::warp_slots();
+        if (slots <= 0) return cudaErrorInvalidConfiguration;
+        try {
+            std::vector<lbm::Tile> part;
+            for (int s0 = 0; s0 < b->n; s0 += lbm::BatchTable<float>::N) {
+                const int ns = std::min(b->n - s0, (int)lbm::BatchTable<float>::N);
+                if (lbm::plan_warp_tiles(nz.data() + s0, nr.data() + s0, ns, slots, part) != LBM_OK)
+                    return cudaErrorMemoryAllocation;
+                b->groups.push_back(nullptr);
+                WarpGroup* g = b->groups.back() = new WarpGroup();
+                if constexpr (sizeof(R) == 4)
+                    for (int i = 0; i < ns; i++) g->table.s[i] = hs[s0 + i];
+                g->s0 = s0;
+                g->ns = ns;
+                g->t0 = (int)tiles.size();
+                g->nt = (int)part.size();
+                tiles.insert(tiles.end(), part.begin(), part.end());
+            }
+        } catch (...) {
+            return cudaErrorMemoryAllocation;
+        }
+        first.assign(1, 0);
     } else {
         const int slots = b->grid > 0 ? b->grid : Ops<R>::batch_resident_ctas(b->strip);
         if (slots <= 0) return cudaErrorInvalidConfiguration;
@@ -126,7 +169,7 @@ cudaError_t upload(lbm_axi_batch* b) {
         if (e == cudaSuccess) e = cudaMalloc(d, bytes);
         if (e == cudaSuccess) e = cudaMemcpyAsync(*d, from, bytes, cudaMemcpyHostToDevice, b->stream);
     };
-    if (b->phases) {
+    if (b->form == FORM_PHASES) {
         put((void**)&b->d_ptiles, ptiles.data(), ptiles.size() * sizeof(lbm::PhaseTile));
     } else {
         put((void**)&b->d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile));
@@ -152,7 +195,16 @@ cudaError_t launch(lbm_axi_batch* b, int parity) {
         return Ops<double>::phase_step_many(static_cast<const BatchSolve<double>*>(b->d_solves), b->d_ptiles, b->nptiles,
                                             b->nghost, b->prows, b->mp, b->ax, parity, b->d_err, b->stream);
     const BatchSolve<float>* solves = static_cast<const BatchSolve<float>*>(b->d_solves);
-    if (b->phases)
+    if (b->form == FORM_WARPS) {
+        cudaError_t e = cudaSuccess;
+        for (size_t i = 0; i < b->groups.size() && e == cudaSuccess; i++) {
+            const WarpGroup& g = *b->groups[i];
+            e = Ops<float>::step_warp_table(g.table, g.ns, b->d_tiles + g.t0, g.nt, b->mp, b->ax, parity, b->d_err + g.s0,
+                                            b->stream);
+        }
+        return e;
+    }
+    if (b->form == FORM_PHASES)
         return Ops<float>::phase_step_many(solves, b->d_ptiles, b->nptiles, b->nghost, b->prows, b->mp, b->ax, parity, b->d_err,
                                            b->stream);
     if (b->h_table)  // n <= BatchTable::N: parameters through the constant bank
@@ -203,6 +255,7 @@ void release(lbm_axi_batch* b) {
     if (b->h_err) cudaFreeHost(b->h_err);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b->h_table;
+    drop_groups(b);
 }
 
 // Time `trials` launches of fn on stream s (ms per launch), non-destructively.
@@ -254,7 +307,7 @@ int lbm_axi_batch_create(lbm_axi* const* solves, int n, void* stream, lbm_axi_ba
     b->device = dev;
     b->d_solves = nullptr;
     b->h_table = nullptr;
-    b->phases = false;
+    b->form = FORM_MARCH;
     b->d_ptiles = nullptr;
     b->nptiles = b->nghost = b->prows = 0;
     b->d_tiles = nullptr;

@@ -41,9 +41,9 @@ struct lbm_axi {
     int path;          // LBM_PATH_FUSED or LBM_PATH_SPLIT
     int rows_per_cta;  // fused path: 0 = balanced wave (k_step_single over the tile plan); > 0 = chunks
                        // (EDM with h_i at the node only)
-    lbm::Tile* d_tiles;  // tile plan of this solve alone (wide strips, one resident wave)
-    int* d_first;        // [ncta + 1]
-    int ncta;
+    lbm::Tile* d_tiles;  // tile plan of this solve alone (FP32 beyond the phase kernels)
+    int* d_first;        // [ncta + 1] (the link-source march)
+    int ncta;            // CTAs of that march, or tiles of the warp march
     Params<float> pf;
     Params<double> pdd;
     void* hb[2];  // h at the link midpoint: S0, H_z, H_r planes of the step that wrote f[c] (else null)
@@ -73,7 +73,7 @@ inline bool unbatchable(const lbm_axi* h) { return fv_of(h) != 0; }
 // f[c] and writing f[c^1]; enqueued on h->stream.
 cudaError_t lbm_handle_step_fused(lbm_axi* h, int c);
 
-// The step runs as three phase launches instead of the marching kernel: FP64
+// The step runs as three phase launches instead of a marching kernel: FP64
 // always, FP32 up to kPhaseMaxNodes nodes in all.
 inline bool lbm_by_phases(int precision, long long nodes) {
     return precision == 64 || nodes <= lbm::kPhaseMaxNodes;

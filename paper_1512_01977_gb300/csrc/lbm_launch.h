@@ -11,7 +11,10 @@ namespace lbm {
 
 constexpr int kReduceBlocks = 304;  // 2 x 152 SMs; fixed so reductions are reproducible
 constexpr int kStepMinRows = 16;    // the single-pass kernel needs single reflections at the walls
-constexpr long long kPhaseMaxNodes = 1500000;
+// FP32 solves and batches up to this many nodes step by phases, larger ones by warps.  us per step, phases
+// and warps: 512 x 512 13.4 and 23.1, 1024 x 768 29.7 and 30.0, 1024 x 1024 38.5 and 37.1, 2048 x 1024 82.8
+// and 51.3; batches of 510k nodes 26.7 and 29.8, of 947k 47.0 and 36.9.
+constexpr long long kPhaseMaxNodes = 800000;
 // z-columns per CTA of the two compiled forms of the batched kernel (the wide
 // one is the default; the autotuner may pick the narrow one for small grids).
 // 112: with 128 threads of two columns each, stages L, D, U and C fill 124,
@@ -62,12 +65,18 @@ struct Ops {
     // step_single and step_table: FP64 steps by phases).
     static cudaError_t step_batch(const BatchSolve<R>* solves, const Tile* tiles, const int* first, int ncta,
                                   bool mp, bool ax, int parity, int strip, int* err, cudaStream_t s);
-    // The fused step of one solve, descriptor by value (kStripWide tiles; same
-    // arithmetic as step_batch with a batch of one).  fv: FV_* collision form,
-    // nonzero only with mp && ax (cudaErrorInvalidValue otherwise).
+    // The fused step of one solve in a link-source form (fv has FV_LINK; mp && ax),
+    // descriptor by value, kStripWide tiles.
     static cudaError_t step_single(const BatchSolve<R>& solve, const LinkSets<R>& h, const Tile* tiles,
                                    const int* first, int ncta, bool mp, bool ax, int parity, int* err,
                                    cudaStream_t s, int fv = 0);
+    // The fused step by warps (lbm_march.cuh; FP32 only): tile t on block t (plan_warp_tiles for warp_slots()),
+    // of one solve (fv: 0 or FV_GUO) or of the n solves of a table.
+    static cudaError_t step_warp(const BatchSolve<R>& solve, const Tile* tiles, int ntiles, bool mp, bool ax, int parity,
+                                 int* err, cudaStream_t s, int fv);
+    static cudaError_t step_warp_table(const BatchTable<R>& table, int n, const Tile* tiles, int ntiles, bool mp,
+                                       bool ax, int parity, int* err, cudaStream_t s);
+    static int warp_slots();
     // The batched step with the descriptors as one kernel argument (FP32; n <=
     // BatchTable<R>::N solves; cudaErrorNotSupported in FP64).
     static cudaError_t step_table(const BatchTable<R>& table, const Tile* tiles, const int* first, int ncta,
@@ -85,5 +94,13 @@ struct Ops {
     static int batch_resident_ctas(int strip);
     static size_t batch_smem(int strip);
 };
+
+template <>
+int Ops<float>::warp_slots();
+template <>
+cudaError_t Ops<float>::step_warp(const BatchSolve<float>&, const Tile*, int, bool, bool, int, int*, cudaStream_t, int);
+template <>
+cudaError_t Ops<float>::step_warp_table(const BatchTable<float>&, int, const Tile*, int, bool, bool, int, int*,
+                                        cudaStream_t);
 
 }  // namespace lbm

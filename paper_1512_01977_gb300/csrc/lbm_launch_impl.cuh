@@ -216,24 +216,18 @@ static auto batch_kernel() {
     return k_step_batch<R, TZ, BatchTile<R, TZ>::RR, BatchTile<R, TZ>::CP, BatchTile<R, TZ>::MINB, MP, AX>;
 }
 
-template <typename R, bool MP, bool AX, int FV = 0>
+template <typename R, int FV>
 static auto single_kernel() {
     constexpr int TZ = kStripWide;
-    return k_step_single<R, TZ, BatchTile<R, TZ>::RR, BatchTile<R, TZ>::CP, BatchTile<R, TZ>::MINB, MP, AX, FV>;
+    return k_step_single<R, TZ, BatchTile<R, TZ>::RR, BatchTile<R, TZ>::CP, BatchTile<R, TZ>::MINB, FV>;
 }
 
 template <typename R>
 static cudaError_t single_prepare() {
     const int smem = (int)BatchTile<R, kStripWide>::smem();
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(single_kernel<R, true, true>(), a, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(single_kernel<R, true, false>(), a, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(single_kernel<R, false, true>(), a, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(single_kernel<R, false, false>(), a, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(single_kernel<R, true, true, FV_GUO>(), a, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(single_kernel<R, true, true, FV_LINK>(), a, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(single_kernel<R, true, true, FV_GUO | FV_LINK>(), a, smem);
-    return e;
+    const cudaError_t e = cudaFuncSetAttribute(single_kernel<R, FV_LINK>(), a, smem);
+    return e == cudaSuccess ? cudaFuncSetAttribute(single_kernel<R, FV_GUO | FV_LINK>(), a, smem) : e;
 }
 
 template <typename R, int TZ>
@@ -351,24 +345,11 @@ cudaError_t Ops<R>::step_single(const BatchSolve<R>& solve, const LinkSets<R>& h
         using T = BatchTile<R, kStripWide>;
         if (ncta <= 0) return cudaErrorInvalidConfiguration;
         const size_t smem = T::smem();
-        if (fv != 0 && !(mp && ax)) return cudaErrorInvalidValue;
-        if (fv == FV_GUO)
-            single_kernel<R, true, true, FV_GUO>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
-        else if (fv == FV_LINK)
-            single_kernel<R, true, true, FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
-        else if (fv == (FV_GUO | FV_LINK))
-            single_kernel<R, true, true, FV_GUO | FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity,
-                                                                                      err);
-        else if (fv != 0)
-            return cudaErrorInvalidValue;
-        else if (mp && ax)
-            single_kernel<R, true, true>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
-        else if (mp)
-            single_kernel<R, true, false>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
-        else if (ax)
-            single_kernel<R, false, true>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        if (!(fv & FV_LINK) || !(mp && ax)) return cudaErrorInvalidValue;
+        if (fv == FV_LINK)
+            single_kernel<R, FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
         else
-            single_kernel<R, false, false>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+            single_kernel<R, FV_GUO | FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
         return cudaGetLastError();
     } else {
         return cudaErrorNotSupported;

@@ -2,7 +2,7 @@
 // is cut into tiles (rows [j0, jend) of one strip of one solve) and the tiles
 // are dealt to the CTAs of one launch, largest first, each to the CTA with the
 // smallest load so far (longest-processing-time scheduling).  A tile costs its
-// rows plus kTileFillRows rows of pipeline fill: the kernel marches 6 halo rows
+// rows plus `fill` rows of pipeline fill (march2: kTileFillRows): the kernel marches 6 halo rows
 // above the tile and its last stage trails the first by 12 rows.  Host code.
 #include <algorithm>
 #include <new>
@@ -48,7 +48,7 @@ long long count_tiles(const int* nz, const int* nr, int n, int strip, int h) {
     return t;
 }
 
-void deal(std::vector<Tile>& tiles, int slots, Cand& c) {
+void deal(std::vector<Tile>& tiles, int slots, int fill, Cand& c) {
     std::vector<int> order(tiles.size());
     for (size_t i = 0; i < order.size(); i++) order[i] = (int)i;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
@@ -65,7 +65,7 @@ void deal(std::vector<Tile>& tiles, int slots, Cand& c) {
         L top = heap.top();
         heap.pop();
         owner[i] = top.second;
-        top.first += tiles[i].jend - tiles[i].j0 + kTileFillRows;
+        top.first += tiles[i].jend - tiles[i].j0 + fill;
         load[top.second] = top.first;
         heap.push(top);
     }
@@ -85,7 +85,7 @@ void deal(std::vector<Tile>& tiles, int slots, Cand& c) {
 }  // namespace
 
 int plan_tiles(const int* nz, const int* nr, int n, int strip, int slots, std::vector<Tile>& tiles,
-               std::vector<int>& first, long long* makespan) {
+               std::vector<int>& first, long long* makespan, int fill) {
     if (!nz || !nr || n < 1 || strip < 1 || slots < 1) return LBM_ERR_INVALID_ARG;
     int max_nr = 0;
     for (int s = 0; s < n; s++) {
@@ -111,7 +111,7 @@ int plan_tiles(const int* nz, const int* nr, int n, int strip, int slots, std::v
         for (int h : heights) {
             cut(nz, nr, n, strip, h, cutv);
             Cand c;
-            deal(cutv, slots, c);
+            deal(cutv, slots, fill, c);
             if (best.makespan < 0 || c.makespan < best.makespan ||
                 (c.makespan == best.makespan && c.tiles.size() < best.tiles.size()))
                 best = std::move(c);
@@ -119,6 +119,19 @@ int plan_tiles(const int* nz, const int* nr, int n, int strip, int slots, std::v
         tiles = std::move(best.tiles);
         first = std::move(best.first);
         if (makespan) *makespan = best.makespan;
+    } catch (const std::bad_alloc&) {
+        return LBM_ERR_OOM;
+    }
+    return LBM_OK;
+}
+
+int plan_warp_tiles(const int* nz, const int* nr, int n, int slots, std::vector<Tile>& tiles) {
+    std::vector<int> first;
+    const int rc = plan_tiles(nz, nr, n, kWarpStrip, slots, tiles, first, nullptr, kWarpFillRows);
+    if (rc != LBM_OK) return rc;
+    try {
+        std::stable_sort(tiles.begin(), tiles.end(),
+                         [](const Tile& a, const Tile& b) { return a.jend - a.j0 > b.jend - b.j0; });
     } catch (const std::bad_alloc&) {
         return LBM_ERR_OOM;
     }

@@ -18,11 +18,18 @@ struct PhaseTile {
 // Pipeline rows a tile costs beyond its own: 6 halo rows above it and the 12-row
 // lag between the first and the last marching stage.
 constexpr int kTileFillRows = 18;
+// The same of the warp march (lbm_march.cuh), and the columns a warp stores.
+constexpr int kWarpFillRows = 13, kWarpStrip = 52;
 
 // Plan for n solves (nz[i] x nr[i]), z-strips of `strip` columns, `slots` CTAs:
 // tiles in CTA order, first[c] .. first[c + 1] those of CTA c (first has one entry
 // per CTA with work, plus one).  Returns LBM_OK, LBM_ERR_INVALID_ARG or LBM_ERR_OOM.
+// fill: pipeline rows a tile costs beyond its own.
 int plan_tiles(const int* nz, const int* nr, int n, int strip, int slots, std::vector<Tile>& tiles,
-               std::vector<int>& first, long long* makespan);
+               std::vector<int>& first, long long* makespan, int fill = kTileFillRows);
+
+// Tiles of the warp march for `slots` resident warps, one block each, the tallest first (the hardware
+// starts a block wherever one ends, which deals them as plan_tiles does).
+int plan_warp_tiles(const int* nz, const int* nr, int n, int slots, std::vector<Tile>& tiles);
 
 }  // namespace lbm

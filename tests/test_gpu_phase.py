@@ -1,6 +1,7 @@
 """The phase kernels (csrc/lbm_phase.cuh) at the edges of their tiles: 64 (FP32)
 or 32 (FP64) columns by 4 or 8 rows, psi halos of 4, wrapped and mirrored
-neighbours.  FP32 steps to the same bits as the marching kernel (chunked rows);
+neighbours; and the warp march (csrc/lbm_march.cuh) that takes larger FP32 grids,
+in strips of 52 columns.  FP32 steps to the same bits as march2 (chunked rows);
 FP64 meets the parity bar of the oracle."""
 import numpy as np
 import pytest
@@ -36,7 +37,9 @@ def _fields(c, seed):
 
 @pytest.mark.parametrize("top,axis", [(O.TOP_FREESLIP, 1), (O.TOP_NOSLIP, 1), (O.TOP_PERIODIC, 0)])
 @pytest.mark.parametrize("nz,nr", [(1, 16), (2, 17), (3, 19), (63, 20), (64, 21), (65, 16), (68, 24), (69, 23),
-                                   (131, 18), (516, 33), (700, 300)])
+                                   (131, 18), (516, 33), (700, 300),
+                                   # beyond the phase kernels: whole, odd and ragged strips, short columns
+                                   (1040, 800), (1041, 801), (1093, 799), (40000, 21), (60, 14000)])
 def test_fp32_same_bits_as_marching(lbm, nz, nr, top, axis):
     c = Case(nz, nr, T_over_Tc=0.9, top=top, axis=axis)
     fields = _fields(c, 7 * nz + nr)
@@ -48,6 +51,43 @@ def test_fp32_same_bits_as_marching(lbm, nz, nr, top, axis):
         got.append(np.frombuffer(s.save()[192:], dtype=np.uint32))
         s.close()
     np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("eos,kappa", [(O.EOS_CS, O.KAPPA_LATTICE), (O.EOS_VDW, O.KAPPA_THERMO),
+                                       (O.EOS_VDW, O.KAPPA_MIXED)])
+def test_warp_march_knows_its_solve(lbm, eos, kappa):
+    """The compiled kinds of the warp march (EOS, kappa), and a body force."""
+    c = Case(1040, 800, T_over_Tc=0.9, eos=eos, kappa=kappa, gz=1e-6)
+    fields = _fields(c, 5)
+    got = []
+    for rows in (0, 1 << 20):
+        s = c.solver(32, c.coexistence()[1])
+        lbm.lbm_axi_set_tuning(s.h, lbm.PATH_FUSED, rows)
+        s.init(*fields).step(3)
+        got.append(np.frombuffer(s.save()[192:], dtype=np.uint32))
+        s.close()
+    np.testing.assert_array_equal(got[0], got[1])
+
+
+def test_warp_batch_of_mixed_solves_equals_alone(lbm):
+    """300 solves of both EOS and kappa readings, beyond the phase kernels and one table: each the bits of
+    its run alone (by phases)."""
+    rng = np.random.default_rng(3)
+    cases = [Case(int(rng.integers(17, 140)), int(rng.integers(16, 90)), T_over_Tc=0.9,
+                  eos=O.EOS_CS if i % 2 else O.EOS_VDW, kappa=O.KAPPA_THERMO if i % 3 else O.KAPPA_LATTICE,
+                  top=O.TOP_NOSLIP if i % 5 == 0 else O.TOP_FREESLIP) for i in range(300)]
+    assert sum(c.nz * c.nr for c in cases) > 800000
+    fields = [_fields(c, i) for i, c in enumerate(cases)]
+    solvers = [c.solver(32, c.coexistence()[1]).init(*f) for c, f in zip(cases, fields)]
+    b = lbm.Batch(solvers)
+    assert b.step(5) == lbm.OK
+    b.close()
+    for i in range(0, 300, 23):
+        s = cases[i].solver(32, cases[i].coexistence()[1]).init(*fields[i]).step(5)
+        assert solvers[i].save() == s.save()
+        s.close()
+    for s in solvers:
+        s.close()
 
 
 @pytest.mark.parametrize("nz,nr", [(1, 16), (2, 18), (31, 17), (32, 16), (33, 21), (65, 30)])
