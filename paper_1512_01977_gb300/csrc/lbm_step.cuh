@@ -181,7 +181,7 @@ __device__ __forceinline__ void march(const Params<R>& p, const R* __restrict__ 
 
     // Every thread owns one item (row offset, column) in each stage, the same
     // in every iteration; inactive items get a row offset far out of range.
-    constexpr int OFF = -100000;
+    constexpr int OFF = -(1 << 28);  // beyond any row: nr < 2^23
     const int lr = tid / WL, lc = tid - (tid / WL) * WL;
     const int l_rr = (tid < RR * WL && lc < kn + 12) ? lr : OFF;
     const int dr_ = tid / WD, dc = tid - (tid / WD) * WD;
@@ -862,7 +862,7 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
     // warps: no warp straddles two ring rows, whose loads would replay as bank
     // conflicts (a reader stage's row is narrower than the ring's stride);
     // measured 2 % faster.  Otherwise the items of a stage are packed row after row.
-    constexpr int OFF = -100000;
+    constexpr int OFF = -(1 << 28);  // beyond any row: nr < 2^23
     constexpr bool kWarpRows = S::NT == 128 && RR == 2 && HL <= 64;
     int lr, lc, dr_, dc, ur_, uc, cr_, cc;
     bool la, da, ua, ca;

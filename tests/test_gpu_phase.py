@@ -39,7 +39,7 @@ def _fields(c, seed):
 @pytest.mark.parametrize("nz,nr", [(1, 16), (2, 17), (3, 19), (63, 20), (64, 21), (65, 16), (68, 24), (69, 23),
                                    (131, 18), (516, 33), (700, 300),
                                    # beyond the phase kernels: whole, odd and ragged strips, short columns
-                                   (1040, 800), (1041, 801), (1093, 799), (40000, 21), (60, 14000)])
+                                   (1040, 800), (1041, 801), (1093, 799), (40000, 21), (60, 14000), (2, 400001)])
 def test_fp32_same_bits_as_marching(lbm, nz, nr, top, axis):
     c = Case(nz, nr, T_over_Tc=0.9, top=top, axis=axis)
     fields = _fields(c, 7 * nz + nr)
