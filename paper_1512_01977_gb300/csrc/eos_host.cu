@@ -69,6 +69,7 @@ static double bisect_root(const lbm_eos& e, double T, double lo, double hi, doub
     double flo = f(lo);
     for (int it = 0; it < 300; it++) {
         const double mid = 0.5 * (lo + hi);
+        if (mid == lo || mid == hi) break;  // neighbours: further halving changes nothing
         const double fm = f(mid);
         if ((fm > 0) == (flo > 0)) {
             lo = mid;
@@ -79,6 +80,14 @@ static double bisect_root(const lbm_eos& e, double T, double lo, double hi, doub
         if (hi - lo <= 1e-17 * hi) break;
     }
     return 0.5 * (lo + hi);
+}
+
+// Antiderivative of (P_k - ps) / rho^2: vdW lambda [(8T/3) ln(rho/(3 - rho)) - 3 rho] + ps / rho; CS
+// RT [ln rho + (4e - 3e^2)/(1 - e)^2] - a rho + ps / rho, e = b rho / 4.
+static double area(const lbm_eos& e, double T, double rho, double ps) {
+    if (e.kind == LBM_EOS_VDW) return e.lambda * (8.0 * T / 3.0 * log(rho / (3.0 - rho)) - 3.0 * rho) + ps / rho;
+    const double x = e.b * rho * 0.25, om = 1.0 - x;
+    return e.R * T * (log(rho) + x * (4.0 - 3.0 * x) / (om * om)) - e.a * rho + ps / rho;
 }
 
 // integral_{rv}^{rl} (P_k - ps) / rho^2 drho, in s = ln(rho): integrand (P_k - ps)/rho,
@@ -113,15 +122,32 @@ bool coexistence(const lbm_eos& e, double T, double* rv_out, double* rl_out) {
     const double pa = eos_p_at(e, T, ra), pb = eos_p_at(e, T, rb);
     double lo = pb > 1e-12 * pa ? pb : 1e-12 * pa, hi = pa;
     double rv = 0, rl = 0;
-    for (int it = 0; it < 200; it++) {
-        const double ps = 0.5 * (lo + hi);
+    auto densities = [&](double ps) {
         rv = bisect_root(e, T, 0.0, ra, ps, false);
         rl = bisect_root(e, T, rb, rmax, ps, false);
-        // the residual decreases with ps
-        if (equal_area_residual(e, T, rv, rl, ps) > 0) lo = ps; else hi = ps;
-        if (hi - lo <= 1e-16 * hi) break;
+    };
+    // bisection on the closed form of the area (it decreases with ps) ...
+    const double lo0 = lo, hi0 = hi;
+    for (int it = 0; it < 200; it++) {
+        const double ps = 0.5 * (lo + hi);
+        densities(ps);
+        if (area(e, T, rl, ps) - area(e, T, rv, ps) > 0) lo = ps; else hi = ps;
+        if (hi - lo <= 1e-15 * hi) break;
     }
-    const double ps = 0.5 * (lo + hi);
+    // ... and Newton steps on the quadrature, which keeps its relative precision near the critical point,
+    // where the closed form's two values cancel; d/dps of the area is 1/rho_l - 1/rho_v.  (Bisection on
+    // the quadrature alone took 4.7 ms, this 0.3 ms.)
+    double ps = 0.5 * (lo + hi);
+    for (int it = 0; it < 4; it++) {
+        densities(ps);
+        const double slope = 1.0 / rl - 1.0 / rv;
+        if (!(slope < 0)) break;
+        const double next = ps - equal_area_residual(e, T, rv, rl, ps) / slope;
+        if (!(next > lo0 && next < hi0) || next == ps) break;
+        const bool done = fabs(next - ps) <= 1e-16 * ps;
+        ps = next;
+        if (done) break;
+    }
     *rv_out = bisect_root(e, T, 0.0, ra, ps, false);
     *rl_out = bisect_root(e, T, rb, rmax, ps, false);
     return true;
