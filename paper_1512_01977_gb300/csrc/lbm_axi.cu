@@ -44,6 +44,8 @@ static cudaError_t step_fused(lbm_axi* h, const Params<R>& p, int c) {
     const bool mp = h->opts.multiphase != 0, ax = h->opts.axis_terms != 0;
     const lbm::BatchSolve<R> s = lbm_handle_solve<R>(h, p, 0);
     const lbm::LinkSets<R> hs{static_cast<const R*>(h->hb[0]), static_cast<R*>(h->hb[1])};
+    if constexpr (sizeof(R) == 4)
+        if (h->tile != lbm::TILE_NONE) return Ops<R>::tile_step(h->tile, s, ax, c, h->derr, h->stream, fv_of(h));
     if (lbm_by_phases(h->precision, (long long)h->nz * h->nr))
         return Ops<R>::phase_step(s, hs, mp, ax, c, h->derr, h->stream, fv_of(h));
     if constexpr (sizeof(R) == 4)
@@ -388,6 +390,8 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     h->pf = make_params<float>(h);
     h->pdd = make_params<double>(h);
     h->path = fused_ok(h) ? LBM_PATH_FUSED : LBM_PATH_SPLIT;
+    h->tile = o.precision == 32 ? lbm::tile_form(&nz, &nr, 1, o.multiphase != 0, o.axis_terms != 0, fv_of(h))
+                                : lbm::TILE_NONE;
     h->rows_per_cta = 0;  // balanced single wave
     if (h->precision == 32) h->pdd = make_params_out(h);
     *h->herr = 0;

@@ -12,9 +12,9 @@
 using lbm::BatchSolve;
 using lbm::Ops;
 
-// How a batch steps: three launches over node tiles (lbm_phase.cuh), one warp per tile (lbm_march.cuh) or
+// How a batch steps: one or three launches over node tiles (lbm_tile.cuh, lbm_phase.cuh), one warp per tile (lbm_march.cuh) or
 // the marching kernel of the chosen strip width and CTA slots (lbm_step.cuh).
-enum BatchForm { FORM_PHASES, FORM_WARPS, FORM_MARCH };
+enum BatchForm { FORM_TILES, FORM_PHASES, FORM_WARPS, FORM_MARCH };
 
 // The warp march of solves [s0, ...): their descriptors (a kernel argument) and tiles [t0, t0 + nt).
 struct WarpGroup {
@@ -32,6 +32,7 @@ struct lbm_axi_batch {
     void* d_solves;         // BatchSolve<R>[n]
     lbm::BatchTable<float>* h_table;  // FP32, n <= BatchTable::N: the descriptors as one kernel argument
     BatchForm form;         // of this tuning
+    lbm::TileForm tile;
     std::vector<WarpGroup*> groups;
     lbm::PhaseTile* d_ptiles;
     int nptiles, nghost, prows;
@@ -44,7 +45,8 @@ struct lbm_axi_batch {
     bool own_stream;
     long long steps;  // batch steps taken; parity = steps & 1
     int strip, grid;
-    cudaGraphExec_t graph;  // two steps, parity 0 then 1
+    cudaGraphExec_t graph;  // an even number of steps from parity 0
+    int graph_steps;
     int graph_strip, graph_grid;
     int pending;
 };
@@ -74,10 +76,11 @@ const Params<double>& params_of<double>(const lbm_axi* h) {
 }
 
 // FP64 steps by phases at every tuning; FP32 at the default one (wide strips, grid
-// 0) by phases while the batch is small and by warps beyond, at the others by march2.
+// 0) by tiles or phases while the batch is small and by warps beyond, at the others by march2.
 BatchForm form_of(const lbm_axi_batch* b, long long nodes) {
     if (b->precision == 64) return FORM_PHASES;
     if (b->strip != lbm::kStripWide || b->grid != 0) return FORM_MARCH;
+    if (b->tile != lbm::TILE_NONE) return FORM_TILES;
     return lbm_by_phases(32, nodes) ? FORM_PHASES : FORM_WARPS;
 }
 
@@ -102,20 +105,23 @@ cudaError_t upload(lbm_axi_batch* b) {
     }
     long long nodes = 0;
     for (int i = 0; i < b->n; i++) nodes += (long long)nz[i] * nr[i];
+    b->tile = b->precision == 32 ? lbm::tile_form(nz.data(), nr.data(), b->n, b->mp, b->ax, 0) : lbm::TILE_NONE;
     b->form = form_of(b, nodes);
     std::vector<lbm::Tile> tiles;
     std::vector<lbm::PhaseTile> ptiles;
     size_t inner = 0;  // tiles before the ghost rows'
     std::vector<int> first;
-    if (b->form == FORM_PHASES) {
-        const int tz = Ops<R>::phase_tile_z();
+    const bool node_tiles = b->form == FORM_PHASES || b->form == FORM_TILES;
+    if (node_tiles) {
+        int tz = Ops<R>::phase_tile_z();
         b->prows = Ops<R>::phase_rows(nodes);
+        if (b->form == FORM_TILES) lbm::tile_size(b->tile, &tz, &b->prows);
         try {
             for (int i = 0; i < b->n; i++)
                 for (int j = 0; j < nr[i]; j += b->prows)
                     for (int k = 0; k < nz[i]; k += tz) ptiles.push_back(lbm::PhaseTile{i, k, j});
             inner = ptiles.size();
-            for (int i = 0; i < b->n && b->ax; i++)
+            for (int i = 0; i < b->n && b->ax && b->form == FORM_PHASES; i++)
                 for (int k = 0; k < nz[i] && b->solves[i]->opts.top_bc != LBM_TOP_PERIODIC; k += tz)
                     ptiles.push_back(lbm::PhaseTile{i, k, -2});
         } catch (...) {
@@ -169,7 +175,7 @@ cudaError_t upload(lbm_axi_batch* b) {
         if (e == cudaSuccess) e = cudaMalloc(d, bytes);
         if (e == cudaSuccess) e = cudaMemcpyAsync(*d, from, bytes, cudaMemcpyHostToDevice, b->stream);
     };
-    if (b->form == FORM_PHASES) {
+    if (node_tiles) {
         put((void**)&b->d_ptiles, ptiles.data(), ptiles.size() * sizeof(lbm::PhaseTile));
     } else {
         put((void**)&b->d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile));
@@ -204,6 +210,8 @@ cudaError_t launch(lbm_axi_batch* b, int parity) {
         }
         return e;
     }
+    if (b->form == FORM_TILES)
+        return Ops<float>::tile_step_many(b->tile, solves, b->d_ptiles, b->nptiles, b->ax, parity, b->d_err, b->stream);
     if (b->form == FORM_PHASES)
         return Ops<float>::phase_step_many(solves, b->d_ptiles, b->nptiles, b->nghost, b->prows, b->mp, b->ax, parity, b->d_err,
                                            b->stream);
@@ -214,6 +222,9 @@ cudaError_t launch(lbm_axi_batch* b, int parity) {
                                   b->stream);
 }
 
+// Steps per graph replay: small batches take a few us per step, which a replay would otherwise spend on itself.
+int graph_steps_of(const lbm_axi_batch* b) { return b->form == FORM_TILES || b->form == FORM_PHASES ? 16 : 2; }
+
 int build_graph(lbm_axi_batch* b) {
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
@@ -221,8 +232,9 @@ int build_graph(lbm_axi_batch* b) {
     }
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LBM_ERR_CUDA;
-    cudaError_t e = launch(b, 0);
-    if (e == cudaSuccess) e = launch(b, 1);
+    b->graph_steps = graph_steps_of(b);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < b->graph_steps && e == cudaSuccess; i++) e = launch(b, i & 1);
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess || !g) {
         if (g) cudaGraphDestroy(g);
@@ -308,6 +320,7 @@ int lbm_axi_batch_create(lbm_axi* const* solves, int n, void* stream, lbm_axi_ba
     b->d_solves = nullptr;
     b->h_table = nullptr;
     b->form = FORM_MARCH;
+    b->tile = lbm::TILE_NONE;
     b->d_ptiles = nullptr;
     b->nptiles = b->nghost = b->prows = 0;
     b->d_tiles = nullptr;
@@ -321,6 +334,7 @@ int lbm_axi_batch_create(lbm_axi* const* solves, int n, void* stream, lbm_axi_ba
     b->strip = lbm::kStripWide;
     b->grid = 0;
     b->graph = nullptr;
+    b->graph_steps = 0;
     b->graph_strip = b->graph_grid = -1;
     b->pending = LBM_OK;
     try {
@@ -385,20 +399,21 @@ int lbm_axi_batch_step_async(lbm_axi_batch* b, long long nsteps) {
         b->steps++;
         nsteps--;
     }
-    if (e == cudaSuccess && nsteps >= 2) {
+    if (e == cudaSuccess && nsteps >= graph_steps_of(b)) {
         if (!b->graph || b->graph_strip != b->strip || b->graph_grid != b->grid) {
             int rc = build_graph(b);
             if (rc != LBM_OK) return rc;
         }
-        while (nsteps >= 2 && e == cudaSuccess) {
+        while (nsteps >= b->graph_steps && e == cudaSuccess) {
             e = cudaGraphLaunch(b->graph, b->stream);
-            b->steps += 2;
-            nsteps -= 2;
+            b->steps += b->graph_steps;
+            nsteps -= b->graph_steps;
         }
     }
-    if (e == cudaSuccess && nsteps == 1) {
-        e = launch(b, 0);
+    while (e == cudaSuccess && nsteps > 0) {
+        e = launch(b, (int)(b->steps & 1));
         b->steps++;
+        nsteps--;
     }
     sync_handles(b);
     if (e != cudaSuccess) {

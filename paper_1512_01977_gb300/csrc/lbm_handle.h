@@ -41,6 +41,7 @@ struct lbm_axi {
     int path;          // LBM_PATH_FUSED or LBM_PATH_SPLIT
     int rows_per_cta;  // fused path: 0 = balanced wave (k_step_single over the tile plan); > 0 = chunks
                        // (EDM with h_i at the node only)
+    lbm::TileForm tile;  // FP32: the one-launch step of small grids (TILE_NONE: phases or a marching kernel)
     lbm::Tile* d_tiles;  // tile plan of this solve alone (FP32 beyond the phase kernels)
     int* d_first;        // [ncta + 1] (the link-source march)
     int ncta;            // CTAs of that march, or tiles of the warp march

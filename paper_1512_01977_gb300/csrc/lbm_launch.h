@@ -22,6 +22,12 @@ constexpr long long kPhaseMaxNodes = 800000;
 // fastest of the even widths 96 ... 116 on the 4096 x 2048 wave.
 constexpr int kStripNarrow = 64, kStripWide = 112;
 
+// Forms of the one-launch tile step (lbm_tile.cuh, FP32 with the force on) for n solves together, by their
+// sizes; TILE_NONE: another kernel is faster or the form is not compiled.  tile_size: nodes of a tile.
+enum TileForm { TILE_NONE, TILE_A, TILE_B, TILE_C, TILE_D };
+TileForm tile_form(const int* nz, const int* nr, int n, bool mp, bool ax, int fv);
+void tile_size(TileForm f, int* tz, int* tr);
+
 template <typename R>
 struct Ops {
     // kernel (a): gather, rho/j, psi; raises bits in *err.
@@ -89,12 +95,21 @@ struct Ops {
     // solve without a periodic top (axis terms on).
     static cudaError_t phase_step_many(const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles, int nghost,
                                        int rows, bool mp, bool ax, int parity, int* err, cudaStream_t s);
+    static cudaError_t tile_step(TileForm f, const BatchSolve<R>& solve, bool ax, int parity, int* err, cudaStream_t s,
+                                 int fv = 0);
+    static cudaError_t tile_step_many(TileForm f, const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles,
+                                      bool ax, int parity, int* err, cudaStream_t s);
     static int phase_tile_z();
     static int phase_rows(long long nodes);
     static int batch_resident_ctas(int strip);
     static size_t batch_smem(int strip);
 };
 
+template <>
+cudaError_t Ops<float>::tile_step(TileForm, const BatchSolve<float>&, bool, int, int*, cudaStream_t, int);
+template <>
+cudaError_t Ops<float>::tile_step_many(TileForm, const BatchSolve<float>*, const PhaseTile*, int, bool, int, int*,
+                                       cudaStream_t);
 template <>
 int Ops<float>::warp_slots();
 template <>

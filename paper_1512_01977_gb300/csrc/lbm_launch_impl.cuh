@@ -1,6 +1,7 @@
 // Definitions of Ops<R>; included once per precision.
 #pragma once
 
+#include "lbm_early.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_launch.h"
 #include "lbm_phase.cuh"
@@ -370,22 +371,6 @@ cudaError_t Ops<R>::step_batch(const BatchSolve<R>* solves, const Tile* tiles, c
 }
 
 // ------------------------------------------------------------ phase launches --
-
-// A launch that may start while its predecessor on the stream still runs; the
-// kernel waits for it before it touches memory (griddepcontrol.wait).
-template <typename... KA, typename... A>
-static cudaError_t launch_early(void (*k)(KA...), unsigned grid, int nt, cudaStream_t s, const A&... a) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(nt);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, a...);
-}
 
 template <typename R, int TR, bool MP, bool AX, int FV>
 static cudaError_t phases(const PhaseOne<R>& a, unsigned grid, cudaStream_t s) {

@@ -1,6 +1,7 @@
 """The phase kernels (csrc/lbm_phase.cuh) at the edges of their tiles: 64 (FP32)
 or 32 (FP64) columns by 4 or 8 rows, psi halos of 4, wrapped and mirrored
-neighbours; and the warp march (csrc/lbm_march.cuh) that takes larger FP32 grids,
+neighbours; the one-launch tile step of small FP32 grids (csrc/lbm_tile.cuh), its
+tiles of 16 x 8 to 32 x 16 nodes; and the warp march (csrc/lbm_march.cuh) that takes larger FP32 grids,
 in strips of 52 columns.  FP32 steps to the same bits as march2 (chunked rows);
 FP64 meets the parity bar of the oracle."""
 import numpy as np
@@ -37,7 +38,9 @@ def _fields(c, seed):
 
 @pytest.mark.parametrize("top,axis", [(O.TOP_FREESLIP, 1), (O.TOP_NOSLIP, 1), (O.TOP_PERIODIC, 0)])
 @pytest.mark.parametrize("nz,nr", [(1, 16), (2, 17), (3, 19), (63, 20), (64, 21), (65, 16), (68, 24), (69, 23),
-                                   (131, 18), (516, 33), (700, 300),
+                                   (131, 18), (516, 33), (255, 131), (461, 301),
+                                   # the phase kernels
+                                   (513, 401), (65, 3301), (640, 320),
                                    # beyond the phase kernels: whole, odd and ragged strips, short columns
                                    (1040, 800), (1041, 801), (1093, 799), (40000, 21), (60, 14000), (2, 400001)])
 def test_fp32_same_bits_as_marching(lbm, nz, nr, top, axis):
