@@ -375,36 +375,21 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double* out) {
     }
 }
 
-// Final sum of the per-block partials by one warp (launch <<<1, 32>>>): lane l
-// adds partials l, l + 32, l + 64, ... in that order, then a shuffle tree
-// combines the lanes.  The order is fixed, so the result is bitwise
-// reproducible for a given number of partials.
+// Final sum of the per-block partials by one block (launch <<<1, 256>>>): thread t
+// adds partials t, t + 256, ... in that order, then block_sum combines the
+// threads.  The order is fixed, so the result is bitwise reproducible for a
+// given number of partials.
 template <int N>
-__device__ __forceinline__ void reduce_partials(const double* __restrict__ partial, int nblocks,
-                                                double* __restrict__ out) {
-    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
-    const int lane = threadIdx.x;
+__global__ void __launch_bounds__(256) k_reduce_final(const double* __restrict__ partial, int nblocks,
+                                                      double* __restrict__ out) {
     double s[N];
 #pragma unroll
     for (int q = 0; q < N; q++) s[q] = 0.0;
-    for (int b = lane; b < nblocks; b += 32) {
+    for (int b = threadIdx.x; b < nblocks; b += 256) {
 #pragma unroll
         for (int q = 0; q < N; q++) s[q] += partial[N * b + q];
     }
-#pragma unroll
-    for (int q = 0; q < N; q++) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_down_sync(0xffffffffu, s[q], o);
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < N; q++) out[q] = s[q];
-    }
-}
-
-template <int N>
-__global__ void k_reduce_final(const double* __restrict__ partial, int nblocks, double* __restrict__ out) {
-    reduce_partials<N>(partial, nblocks, out);
+    block_sum<N>(s, out);
 }
 
 }  // namespace lbm

@@ -9,7 +9,7 @@
 
 namespace lbm {
 
-constexpr int kReduceBlocks = 304;  // 2 x 152 SMs; fixed so reductions are reproducible
+constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs (all that fit); fixed so reductions are reproducible
 constexpr int kStepMinRows = 16;    // the single-pass kernel needs single reflections at the walls
 // FP32 solves and batches up to this many nodes step by phases, larger ones by warps.  us per step, phases
 // and warps: 512 x 512 13.4 and 23.1, 1024 x 768 29.7 and 30.0, 1024 x 1024 38.5 and 37.1, 2048 x 1024 82.8

@@ -171,7 +171,7 @@ template <typename R>
 cudaError_t Ops<R>::mass(const Params<R>& p, const R* f, LinkPlanes<R> lk, double* partial, double* out, int* err,
                          cudaStream_t s) {
     k_mass<R><<<kReduceBlocks, 256, 0, s>>>(p, f, lk, partial, err);
-    k_reduce_final<2><<<1, 32, 0, s>>>(partial, kReduceBlocks, out);
+    k_reduce_final<2><<<1, 256, 0, s>>>(partial, kReduceBlocks, out);
     return cudaGetLastError();
 }
 
@@ -180,14 +180,13 @@ cudaError_t Ops<R>::pjump(const Params<R>& p, const Params<double>& pd, const R*
                           double rc, double rin, double rout, double* partial, double* out, int* err,
                           cudaStream_t s) {
     k_pjump<R><<<kReduceBlocks, 256, 0, s>>>(p, pd, f, lk, zc, rc, rin, rout, partial, err);
-    k_reduce_final<4><<<1, 32, 0, s>>>(partial, kReduceBlocks, out);
+    k_reduce_final<4><<<1, 256, 0, s>>>(partial, kReduceBlocks, out);
     return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t Ops<R>::take_error(int* err, int* host, cudaStream_t s) {
-    k_take_error<<<1, 1, 0, s>>>(err, host);
-    return cudaGetLastError();
+    return launch_early(k_take_error, 1, 1, s, err, host);
 }
 
 }  // namespace lbm
@@ -375,9 +374,12 @@ cudaError_t Ops<R>::step_batch(const BatchSolve<R>* solves, const Tile* tiles, c
 template <typename R, int TR, bool MP, bool AX, int FV>
 static cudaError_t phases(const PhaseOne<R>& a, unsigned grid, cudaStream_t s) {
     const unsigned ghost = AX && a.s.p.top != TOP_PERIODIC ? a.across : 0;
-    cudaError_t e = launch_early(k_phase_l<R, TR, MP, (FV & FV_LINK) != 0>, grid, 32 * TR, s, a);
+    // the gather and the collision read no halo of their own rows: 4 rows per block keep more warps resident
+    // (1023 x 511 Guo 21.6 -> 20.3 us)
+    const unsigned grid4 = a.across * (unsigned)((a.s.p.nr + 3) / 4);
+    cudaError_t e = launch_early(k_phase_l<R, 4, MP, (FV & FV_LINK) != 0>, grid4, 128, s, a);
     if (e == cudaSuccess) e = launch_early(k_phase_u<R, TR, MP, AX>, grid + ghost, 32 * TR, s, a);
-    if (e == cudaSuccess) e = launch_early(k_phase_c<R, TR, AX, FV>, grid, 32 * TR, s, a);
+    if (e == cudaSuccess) e = launch_early(k_phase_c<R, 4, AX, FV>, grid4, 128, s, a);
     return e;
 }
 template <typename R, int TR>
@@ -417,10 +419,12 @@ int Ops<R>::phase_tile_z() {
     return PhaseShape<R>::TZ;
 }
 
-// Rows per tile: 8, or 4 in FP64 and while 8 would leave SMs without a tile.
+// Rows per tile: 8, or 4 while 8 would leave SMs without a tile or, in FP64, unevenly loaded (its blocks are
+// bound by their SM's arithmetic rate, and 8 rows compute less halo: 500 x 250 70 us per step with 4 rows and
+// 78 with 8, 512 x 512 147 and 143, 1024 x 512 282 and 275).
 template <typename R>
 int Ops<R>::phase_rows(long long nodes) {
-    return sizeof(R) == 8 || nodes <= 152LL * 8 * PhaseShape<R>::TZ ? 4 : 8;
+    return nodes <= 152LL * 8 * PhaseShape<R>::TZ * (sizeof(R) == 8 ? 4 : 1) ? 4 : 8;
 }
 
 template <typename R>
@@ -473,10 +477,10 @@ cudaError_t Ops<R>::fields(const BatchSolve<R>& v, LinkPlanes<R> lk, const Param
         const int across = (v.p.nz + 31) / 32;
         const R* f = parity ? v.f_b : v.f_a;
         if ((long long)v.p.nz * v.p.nr <= 2 * 152 * 512)
-            k_fields<8><<<across * ((v.p.nr + 7) / 8), 256, 0, s>>>(v.p, pd, f, lk, out, err);
-        else
-            k_fields<16><<<across * ((v.p.nr + 15) / 16), 256, 0, s>>>(v.p, pd, f, lk, out, err);
-        return cudaGetLastError();
+            return launch_early(k_fields<8>, across * ((v.p.nr + 7) / 8), 256, s, v.p, pd, f, lk, out, err);
+        if ((long long)v.p.nz * v.p.nr > 1000000)
+            return launch_early(k_fields<32>, across * ((v.p.nr + 31) / 32), 256, s, v.p, pd, f, lk, out, err);
+        return launch_early(k_fields<16>, across * ((v.p.nr + 15) / 16), 256, s, v.p, pd, f, lk, out, err);
     }
 }
 

@@ -127,12 +127,13 @@ __global__ void __launch_bounds__(256) k_fields(Params<float> p, Params<double> 
     const int tid = threadIdx.x, across = (p.nz + TZ - 1) / TZ, ti = blockIdx.x / across;
     const int k0 = (blockIdx.x - ti * across) * TZ, j0 = ti * TR;
     const int kn = min(TZ, p.nz - k0), jn = min(TR, p.nr - j0);
-    const bool mp = p.multiphase != 0, ax = p.axis != 0;
+    const bool mp = p.multiphase != 0, ax = p.axis != 0, want_u = out.uz || out.ur || out.u;
     int bad = 0;
+    phase_wait();
     for (int i = tid; i < WP * (TR + 8); i += NT) {
         const int a = i / WP, b = i - a * WP, tj = a - 4, tk = b - 4;
         const bool own = tj >= 0 && tj < jn && tk >= 0 && tk < kn;
-        if (a >= jn + 8 || b >= kn + 8 || !(mp || own)) continue;
+        if (a >= jn + 8 || b >= kn + 8 || !((mp && want_u) || own)) continue;
         int s;
         const int jm = map_row(p, j0 + tj, 1, 1, s), km = wrap_any(k0 + tk, p.nz);
         float drho, jz, jr, psi;
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(256) k_fields(Params<float> p, Params<double> 
     }
     if (bad) atomicOr(err, bad);
     __syncthreads();
-    if (!(out.uz || out.ur || out.u)) {
+    if (!want_u) {
         for (int i = tid; i < TZ * TR; i += NT) {
             const int tj = i / TZ, tk = i - tj * TZ;
             if (tj < jn && tk < kn) put_fields(out, p, pd, j0 + tj, k0 + tk, sRho[i], 0.0f, 0.0f);
@@ -255,6 +256,7 @@ __global__ void __launch_bounds__(256) k_pjump(Params<R> p, Params<double> pd, c
 
 // The error word to the host, cleared on the device.
 static __global__ void k_take_error(int* __restrict__ err, int* __restrict__ host) {
+    phase_wait();
     *host = *err;
     *err = 0;
 }

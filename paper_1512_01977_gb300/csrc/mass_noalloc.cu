@@ -76,6 +76,6 @@ extern "C" int lbm_axi_mass_field_noalloc(const double* d_rho, int nz, int nr, d
     const int blocks = (int)((n + kNodesPerBlock - 1) / kNodesPerBlock);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     k_mass_partials<<<blocks, kThreads, 0, s>>>(d_rho, nz, n, partial);
-    lbm::k_reduce_final<2><<<1, 32, 0, s>>>(partial, blocks, d_out);
+    lbm::k_reduce_final<2><<<1, 256, 0, s>>>(partial, blocks, d_out);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
