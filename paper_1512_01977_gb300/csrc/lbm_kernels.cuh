@@ -352,26 +352,26 @@ __global__ void __launch_bounds__(256) k_init(Params<R> p, double rho_ref, const
 }
 
 // --------------------------------------------- kernel (c): reductions --
-// Warp-shuffle sums in FP64; one partial per block, summed by k_reduce_final
-// in a fixed order, so results are bitwise reproducible for a given grid.
+// FP64 sums; one partial per block, summed by k_reduce_final in a fixed order, so results are bitwise
+// reproducible for a given grid.  block_sum adds over a block of 256 threads: one warp per value, 7
+// additions and 5 shuffle steps for 256 terms.  (Five shuffle steps in each of 8 warps for every value take
+// three times the FP64 pipe, which bounds the sums: mass of 2048 x 1024 45 us that way, 38 this way; the
+// pressure jump 105 and 83.)
 template <int N>
 __device__ __forceinline__ void block_sum(double (&v)[N], double* out) {
-    __shared__ double red[N][8];
+    static_assert(N <= 8, "one warp per value");
+    __shared__ double all[N][256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < N; q++) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
-        if (lane == 0) red[q][warp] = v[q];
-    }
+    for (int q = 0; q < N; q++) all[q][threadIdx.x] = v[q];
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp < N) {
+        double s = all[warp][lane];
 #pragma unroll
-        for (int q = 0; q < N; q++) {
-            double s = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[q][w];
-            out[q] = s;
-        }
+        for (int i = 1; i < 8; i++) s += all[warp][lane + 32 * i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) out[warp] = s;
     }
 }
 
