@@ -204,14 +204,14 @@ cudaError_t enqueue_init(lbm_axi* h, const double* rho, const double* uz, const 
                              static_cast<const double*>(phys), h->derr);
 }
 
-// Memory of this device that a kernel may write.
+// Memory of this device that a kernel may write as doubles (a copy takes any address).
 bool writable_on(const void* p, int device) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return a.type == cudaMemoryTypeDevice && a.device == device;
+    return a.type == cudaMemoryTypeDevice && a.device == device && reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
 }
 
 struct DeviceGuard {
@@ -232,7 +232,6 @@ void release_all(lbm_axi* h) {
     dev_free(h->aux, h->via_hook, h->hook_ctx, h->hook_release);
     dev_free(h->mout, h->via_hook, h->hook_ctx, h->hook_release);
     dev_free(h->partial, h->via_hook, h->hook_ctx, h->hook_release);
-    dev_free(h->dred, h->via_hook, h->hook_ctx, h->hook_release);
     dev_free(h->derr, h->via_hook, h->hook_ctx, h->hook_release);
     dev_free(h->d_tiles, h->via_hook, h->hook_ctx, h->hook_release);
     dev_free(h->d_first, h->via_hook, h->hook_ctx, h->hook_release);
@@ -331,7 +330,6 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     h->aux = dev_alloc(4 * plane_bytes);
     h->mout = (double*)dev_alloc(4 * (size_t)nz * nr * sizeof(double));
     h->partial = (double*)dev_alloc(4 * lbm::kReduceBlocks * sizeof(double));
-    h->dred = (double*)dev_alloc(4 * sizeof(double));
     h->derr = (int*)dev_alloc(sizeof(int));
     // tile plan of the marching step: warps, or CTAs on wide strips with the link source
     const bool link = o.h_eval == LBM_H_LINK_AVG && o.axis_terms;
@@ -366,7 +364,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
         h->hb[1] = dev_alloc(3 * plane_bytes);
         h->bytes += 6 * plane_bytes;
     }
-    bool ok = h->f[0] && h->f[1] && h->aux && h->mout && h->partial && h->dred && h->derr &&
+    bool ok = h->f[0] && h->f[1] && h->aux && h->mout && h->partial && h->derr &&
               h->d_tiles && h->d_first && (!link || (h->hb[0] && h->hb[1]));
     ok = ok && cudaMallocHost(&h->herr, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMallocHost(&h->hred, 4 * sizeof(double)) == cudaSuccess;
@@ -392,7 +390,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     h->path = fused_ok(h) ? LBM_PATH_FUSED : LBM_PATH_SPLIT;
     h->tile = o.precision == 32 ? lbm::tile_form(&nz, &nr, 1, o.multiphase != 0, o.axis_terms != 0, fv_of(h))
                                 : lbm::TILE_NONE;
-    h->rows_per_cta = 0;  // balanced single wave
+    h->rows_per_cta = 0;  // the form the size chooses (step_fused)
     if (h->precision == 32) h->pdd = make_params_out(h);
     *h->herr = 0;
     cudaError_t err = cudaSuccess;

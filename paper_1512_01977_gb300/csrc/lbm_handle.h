@@ -24,7 +24,6 @@ struct lbm_axi {
     void* aux;
     double* mout;     // 4 planes of nz*nr doubles (moments / init staging)
     double* partial;  // reduction partials
-    double* dred;     // reduction results (4 doubles)
     int* derr;        // sticky device error word
     int* herr;        // pinned copy
     double* hred;     // pinned reduction results
@@ -39,7 +38,7 @@ struct lbm_axi {
     int pending;  // error status carried to the next sync
     size_t bytes;
     int path;          // LBM_PATH_FUSED or LBM_PATH_SPLIT
-    int rows_per_cta;  // fused path: 0 = balanced wave (k_step_single over the tile plan); > 0 = chunks
+    int rows_per_cta;  // fused path: 0 = the form its size chooses (step_fused); > 0 = chunks
                        // (EDM with h_i at the node only)
     lbm::TileForm tile;  // FP32: the one-launch step of small grids (TILE_NONE: phases or a marching kernel)
     lbm::Tile* d_tiles;  // tile plan of this solve alone (FP32 beyond the phase kernels)

@@ -7,7 +7,7 @@
 // lanes per clock and SM: 14 us per operation and node of a 4096 x 2048 solve),
 // so P_k is evaluated in 9 operations (30 with its division), FP32 values
 // are widened by their bits and distances are compared in FP32 where that
-// decides.  us per call, before -> now: see k_fields and the kernels below.
+// decides.  What each read took and takes stands at its kernel, host call included.
 #pragma once
 
 #include "lbm_phase.cuh"
@@ -43,13 +43,11 @@ template <typename R>
 __device__ __forceinline__ void put_fields(const FieldsOut<R>& o, const Params<R>& p, const Params<double>& pd, int j,
                                            int k, R drho, R uz, R ur) {
     const long long c = (long long)j * p.nz + k;
-    if (o.rho || o.p) {
-        const double rho = pd.rho_ref + widen(drho);
-        if (o.rho) o.rho[c] = rho;
-        if (o.p) o.p[c] = pressure(pd, rho);
-    }
+    const double rho = pd.rho_ref + widen(drho);
+    if (o.rho) o.rho[c] = rho;
     if (o.uz) o.uz[c] = widen(uz);
     if (o.ur) o.ur[c] = widen(ur);
+    if (o.p) o.p[c] = pressure(pd, rho);
     if (o.u) {
         R* u = o.u + (j * p.pitch + k);
         u[0] = uz;
@@ -106,7 +104,9 @@ __device__ __forceinline__ int node_moments(const Params<double>& p, const doubl
 
 // Fields of an FP32 solve: 32 x TR nodes per block with 4 columns and rows of psi around them
 // gathered again (F needs psi_rr).  The velocity is k_update's, operation for operation.
-// 4096 x 2048: 598 us as k_density, k_update's moments form and four copies.
+// 4096 x 2048: 277 us, and 598 as k_density, k_update's moments form and four copies (density alone 117).
+// TR by size: the taller the tile, the less halo, and 32 rows beat 16 by 26 us there; 2048 x 1024 takes the
+// same 100 us either way, and below 152 blocks' worth of nodes 8 rows give every SM one.
 template <int TR>
 struct FieldsShape {
     static constexpr int TZ = 32, WP = TZ + 8, WD = TZ + 4;
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(256) k_fields(Params<float> p, Params<double> 
 }
 
 // Fields of an FP64 solve: k_phase_l's planes, then its velocity phase writing to the destination.
-// 1024 x 512: 437 us as k_density, k_update's moments form and four copies.
+// 1024 x 512: 210 us, and 437 as k_density, k_update's moments form and four copies.
 template <int TR, bool MP, bool AX>
 __global__ void __launch_bounds__(32 * TR) k_fields64(const PhaseOne<double> a, const FieldsOut<double> out,
                                                       const Params<double> pd) {
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(32 * TR) k_fields64(const PhaseOne<double> a, 
 
 // Sum of (j + 1/2) rho and of rho.  Summed over the deviations rho - rho_ref (one FP64 addition and
 // one fused multiply per node); the reference's share is nz nr rho_ref and nz nr^2/2 rho_ref.
-// 2048 x 1024: 78 us as k_density, k_mass and the final sum.
+// 2048 x 1024: 38 us, and 78 as k_density, k_mass and the final sum; 4096 x 2048: 97.
 template <typename R>
 __global__ void __launch_bounds__(256) k_mass(Params<R> p, const R* __restrict__ f, LinkPlanes<R> lk,
                                               double* __restrict__ partial, int* __restrict__ err) {
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(256) k_mass(Params<R> p, const R* __restrict__
 
 // Sums of P_k and node counts inside d < r_in and outside d > r_out.  The distance is compared in FP32
 // unless it is within 1e-5 of a radius (relative; FP32 errs by a few 1e-7), then in FP64 as before.
-// 2048 x 1024: 232 us with k_density and an FP64 root and quotient per node.
+// 2048 x 1024: 83 us, and 232 with k_density and an FP64 root and quotient per node.
 template <typename R>
 __global__ void __launch_bounds__(256) k_pjump(Params<R> p, Params<double> pd, const R* __restrict__ f,
                                                LinkPlanes<R> lk, double zc, double rc, double rin, double rout,

@@ -105,3 +105,24 @@ def test_fp64_edges_against_the_oracle(lbm, nz, nr, top, kappa, eos):
     s.close()
     assert rel_err(mg["rho"], mo["rho"]) <= 1e-12 and rel_err(mg["p"], mo["p"]) <= 1e-12
     assert all(e <= 1e-12 for e in component_errs(mg, mo).values())
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+def test_moments_to_an_unaligned_address(lbm, prec):
+    """Fields wanted at a device address that is no multiple of 8 come through the staging planes: the same bytes."""
+    import ctypes
+    import torch
+
+    nz, nr = 37, 18
+    rho = 1.0 + 0.1 * np.random.default_rng(7).uniform(size=(nr, nz))
+    s = lbm.Solver(nz, nr, 0.8, eos=lbm.make_eos(lbm.EOS_CS, 0.9), multiphase=0, precision=prec).init(rho)
+    s.step(2)
+    want = torch.zeros(nr, nz, dtype=torch.float64, device="cuda")
+    lbm.lbm_axi_moments_device(s.h, p=want)
+    got = torch.zeros(8 * nz * nr + 8, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    assert lbm.lib().lbm_axi_moments_device(s.h, None, None, None, ctypes.c_void_p(got.data_ptr() + 4)) == 0
+    raw = got.cpu().numpy()
+    assert raw[4:4 + 8 * nz * nr].tobytes() == want.cpu().numpy().tobytes()
+    assert not raw[:4].any() and not raw[-4:].any()
+    s.close()
