@@ -10,7 +10,7 @@
 namespace lbm {
 
 constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs (all that fit); fixed so reductions are reproducible
-constexpr int kStepMinRows = 16;    // the single-pass kernel needs single reflections at the walls
+constexpr int kStepMinRows = 16;    // the fused forms need single reflections at the walls
 // FP32 solves and batches up to this many nodes step by phases, larger ones by warps.  us per step, phases
 // and warps: 512 x 512 13.4 and 23.1, 1024 x 768 29.7 and 30.0, 1024 x 1024 38.5 and 37.1, 2048 x 1024 82.8
 // and 51.3; batches of 510k nodes 26.7 and 29.8, of 947k 47.0 and 36.9.
@@ -60,11 +60,9 @@ struct Ops {
     static size_t update_smem();
     // one-time kernel attributes (shared-memory opt-in); call outside stream capture
     static cudaError_t prepare();
-    // kernel (b'): the whole step in one pass (needs nr >= kStepMinRows); rows_per_cta
+    // kernel (b'): the whole step in one pass (needs nr >= kStepMinRows); rows_per_cta > 0
     // rows of each z-strip per CTA.
     static cudaError_t step(const Params<R>& p, const R* f, R* fout, int rows_per_cta, int* err, cudaStream_t s);
-    static size_t step_smem();
-    static int step_strip();  // z-columns per CTA of the single-pass kernel
     // Batched fused step: ncta CTAs, CTA c marching tiles first[c] .. first[c + 1] - 1
     // (device arrays planned by plan_tiles for this strip width); strip: kStripNarrow
     // or kStripWide z-columns per CTA.  FP32 only (cudaErrorNotSupported in FP64, like
@@ -102,7 +100,6 @@ struct Ops {
     static int phase_tile_z();
     static int phase_rows(long long nodes);
     static int batch_resident_ctas(int strip);
-    static size_t batch_smem(int strip);
 };
 
 template <>

@@ -44,13 +44,8 @@ struct StepTile<double> {
 };
 
 template <typename R>
-size_t Ops<R>::step_smem() {
+static size_t step_smem() {
     return sizeof(R) * (size_t)StepShape<StepTile<R>::TZ, StepTile<R>::RR>::elems;
-}
-
-template <typename R>
-int Ops<R>::step_strip() {
-    return StepTile<R>::TZ;
 }
 
 // The four compiled forms of the fused kernel (force on/off x axis terms on/off).
@@ -83,7 +78,7 @@ cudaError_t Ops<R>::prepare() {
     cudaError_t e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_update<R, T::TZ, T::TR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = set_step_attr<R>((int)step_smem());
+    if (e == cudaSuccess) e = set_step_attr<R>((int)step_smem<R>());
     // the marching forms (FP32): attributes and occupancy are settled here, outside any stream capture
     if constexpr (sizeof(R) == 4) {
         if (e == cudaSuccess && (batch_resident_ctas(kStripNarrow) <= 0 || batch_resident_ctas(kStripWide) <= 0))
@@ -95,39 +90,12 @@ cudaError_t Ops<R>::prepare() {
     return e;
 }
 
-// CTAs of the fused kernel that fit on the device at once (one wave).
-template <typename R>
-static int step_resident_ctas() {
-    static int cached = 0;
-    if (cached > 0) return cached;
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 152;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<R, true, true>(),
-                                                      StepShape<StepTile<R>::TZ, StepTile<R>::RR, StepTile<R>::CP>::NT,
-                                                      Ops<R>::step_smem()) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
-    cached = sms * per_sm;
-    return cached;
-}
-
 template <typename R>
 cudaError_t Ops<R>::step(const Params<R>& p, const R* f, R* fout, int rows_per_cta, int* err, cudaStream_t s) {
     constexpr int TZ = StepTile<R>::TZ, RR = StepTile<R>::RR, CP = StepTile<R>::CP;
     constexpr int NT = StepShape<TZ, RR, CP>::NT;
-    dim3 grid;
-    if (rows_per_cta > 0) {
-        grid = dim3((p.nz + TZ - 1) / TZ, (p.nr + rows_per_cta - 1) / rows_per_cta);
-    } else {
-        // balanced single wave; no CTA gets less than 16 rows of work
-        const long long total = (long long)((p.nz + TZ - 1) / TZ) * p.nr;
-        long long n = step_resident_ctas<R>();
-        if (n > (total + 15) / 16) n = (total + 15) / 16;
-        grid = dim3((unsigned)(n > 0 ? n : 1));
-    }
-    const size_t smem = step_smem();
+    const dim3 grid((p.nz + TZ - 1) / TZ, (p.nr + rows_per_cta - 1) / rows_per_cta);
+    const size_t smem = step_smem<R>();
     if (p.multiphase && p.axis)
         step_kernel<R, true, true>()<<<grid, NT, smem, s>>>(p, f, fout, rows_per_cta, err);
     else if (p.multiphase)
@@ -188,10 +156,6 @@ template <typename R>
 cudaError_t Ops<R>::take_error(int* err, int* host, cudaStream_t s) {
     return launch_early(k_take_error, 1, 1, s, err, host);
 }
-
-}  // namespace lbm
-
-namespace lbm {
 
 // Batched marching forms (FP32): strip width kStripNarrow or kStripWide (the autotuner picks), force and
 // axis terms compiled in or out.
@@ -290,11 +254,6 @@ cudaError_t Ops<R>::step_table(const BatchTable<R>& table, const Tile* tiles, co
     } else {
         return cudaErrorNotSupported;
     }
-}
-
-template <typename R>
-size_t Ops<R>::batch_smem(int strip) {
-    return strip == kStripNarrow ? BatchTile<R, kStripNarrow>::smem() : BatchTile<R, kStripWide>::smem();
 }
 
 template <typename R>

@@ -9,8 +9,9 @@
 // has to do, and every tile recomputes 12 extra rows.  Here every node of a
 // stage is independent, so a small grid fills the SMs and a step costs three
 // short launches.  us per step, marching kernel -> phases (GB300): FP32 64 x 64
-// 24.9 -> 6.1, 512 x 256 22.5 -> 9.4, 1023 x 511 (Guo) 32.4 -> 21.6; FP64 64 x 64
-// 182 -> 16.4, 500 x 250 212 -> 70, 1024 x 512 495 -> 282.
+// 24.9 -> 6.1, 512 x 256 22.5 -> 9.4, 1023 x 511 (Guo) 32.4 -> 20.4; FP64 64 x 64
+// 182 -> 15.7, 500 x 250 212 -> 70, 1024 x 512 495 -> 275.  (The smallest FP32
+// grids are faster still in one launch, lbm_tile.cuh.)
 //
 // FP32 runs node pairs with the arithmetic of march2 (the update of a node pair
 // in lbm_step.cuh), in the same order, so both give the same bits.  FP64 is

@@ -23,6 +23,11 @@
 // beyond a top wall are evaluated at their interior mirror row (already
 // behind the marching front) and given the field's parity; with periodic r
 // wrapped rows are evaluated in place.  Needs nr >= 16 (single reflections).
+//
+// Who marches this way: a large FP32 solve with the link source (k_step_single), a solve whose tuning
+// asks for fixed row chunks (k_step), an FP32 batch whose tuning asks for 64-column strips or a grid
+// (k_step_table, k_step_batch).  Every other call steps by tiles, phases or warps (lbm_tile.cuh,
+// lbm_phase.cuh, lbm_march.cuh), which are faster: 208 us here and 153 by warps on the 4096 x 2048 wave.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -153,13 +158,10 @@ __device__ __forceinline__ void link3(const Params<R>& p, const R* __restrict__ 
 }
 
 // One CTA marches z-strip `strip` over rows [j0, jend).  MP / AX: pseudopotential
-// force and axisymmetric terms compiled in or out.  FV: collision form (FV_GUO:
-// Guo forcing; FV_LINK: h_i as the link average, reading the previous step's
-// source planes from hsrc and writing this step's to hdst).
-template <typename R, int TZ, int RR, bool MP, bool AX, int FV = 0>
+// force and axisymmetric terms compiled in or out.
+template <typename R, int TZ, int RR, bool MP, bool AX>
 __device__ __forceinline__ void march(const Params<R>& p, const R* __restrict__ f, R* __restrict__ fout, int strip,
-                                      int j0, int jend, unsigned char* smem_raw, int& bad,
-                                      const R* __restrict__ hsrc = nullptr, R* __restrict__ hdst = nullptr) {
+                                      int j0, int jend, unsigned char* smem_raw, int& bad) {
     using S = StepShape<TZ, RR>;
     constexpr int WL = S::WL, WD = S::WD, WU = S::WU, LAG = S::LAG;
     constexpr int DP = S::DP, DD = S::DD, DJ = S::DJ, DU = S::DU;
@@ -218,18 +220,14 @@ __device__ __forceinline__ void march(const Params<R>& p, const R* __restrict__ 
     auto c_valid = [&](int row) { return row >= j0 && row < jend; };
 
     R lpf[Q], cpf[Q];  // populations gathered one iteration ahead (stage L, stage C)
-    R lpa[3] = {R(0), R(0), R(0)}, cpa[3] = {R(0), R(0), R(0)};  // link source planes, likewise
-    constexpr bool link = (FV & FV_LINK) != 0, guo = (FV & FV_GUO) != 0;
     {
         int sg;
         const int row = j0 - 6 + l_rr;
         const bool v = l_valid(row);
         const int jm = v ? lsrc(row, sg) : 0;
         prefetch(p, f, v, jm, lkc, lpf);
-        if (link && v) link3(p, hsrc, jm, lkc[1], lpa);
         const int crw = j0 - 6 - 3 * LAG + c_rr;
         prefetch(p, f, c_valid(crw), crw, ckc, cpf);
-        if (link && c_valid(crw)) link3(p, hsrc, crw, ckc[1], cpa);
     }
 
     for (int pb = j0 - 6; pb - 3 * LAG < jend; pb += RR) {
@@ -240,15 +238,9 @@ __device__ __forceinline__ void march(const Params<R>& p, const R* __restrict__ 
                 int sgn_r;
                 lsrc(row, sgn_r);
                 const R d1 = lpf[1] + lpf[5] + lpf[7], d2 = lpf[2] + lpf[6] + lpf[8];
-                R drho = lpf[0] + lpf[3] + lpf[4] + d1 + d2;
-                R jz = d1 - d2;
-                R jr = (lpf[3] + lpf[5] + lpf[8]) - (lpf[4] + lpf[6] + lpf[7]);
-                if (link) {
-                    // arrival halves h_i(y)/2: zeroth moment S0/2, first moment H/2
-                    drho += R(0.5) * lpa[0];
-                    jz += R(0.5) * lpa[1];
-                    jr += R(0.5) * lpa[2];
-                }
+                const R drho = lpf[0] + lpf[3] + lpf[4] + d1 + d2;
+                const R jz = d1 - d2;
+                const R jr = (lpf[3] + lpf[5] + lpf[8]) - (lpf[4] + lpf[6] + lpf[7]);
                 const R rho = p.rho_ref + drho;
                 if (mp) {
                     const R arg = rho * (R(1) / R(3)) - eos_p_fast(p, rho);
@@ -270,7 +262,6 @@ __device__ __forceinline__ void march(const Params<R>& p, const R* __restrict__ 
             const bool nv = l_valid(nrow);  // (inactive items sit far out of range: no map_row for them)
             const int njm = nv ? lsrc(nrow, sg) : 0;
             prefetch(p, f, nv, njm, lkc, lpf);
-            if (link && nv) link3(p, hsrc, njm, lkc[1], lpa);
         }
 
         // ---- stage D: rows pb-LAG ..: psi_z, psi_r (only with F_axis).
@@ -349,9 +340,7 @@ __device__ __forceinline__ void march(const Params<R>& p, const R* __restrict__ 
             R fi[Q];
 #pragma unroll
             for (int i = 0; i < Q; i++) fi[i] = cpf[i];
-            const R a0 = cpa[0], az = cpa[1], ar = cpa[2];
             prefetch(p, f, c_valid(row + RR), row + RR, ckc, cpf);  // next iteration's gather
-            if (link && c_valid(row + RR)) link3(p, hsrc, row + RR, ckc[1], cpa);
             if (c_valid(row)) {
                 const int c = cc + 2;
                 const int sj = (row & (DJ - 1)) * WU + c;
@@ -385,52 +374,19 @@ __device__ __forceinline__ void march(const Params<R>& p, const R* __restrict__ 
                 //          q(u) = 4.5 (c.u)^2 - 1.5 u.u
                 //   odd  = 3 w [rho ((c.u1) - (1 - omega)(c.u0)) + c.H]
                 const int o = row * p.pitch + k0 + cc;
-                // link-midpoint source: this node's arrival half of the previous step's
-                // h_i and the departure half of this step's; S0, H kept for the next step
-                const R hs = link ? R(0.5) : R(1);
-                const R hm0 = hs * m0, hHz = hs * Hz, hHr = hs * Hr;
-                if (link) {
+                const R u0sq = u0z * u0z + u0r * u0r, u1sq = u1z * u1z + u1r * u1r;
+                const R base = omega * drho + rho * (om1 * R(1.5) * u0sq - R(1.5) * u1sq);
+                fout[o] = om1 * fi[0] + w_of<R>(0) * (base + m0);
 #pragma unroll
-                    for (int i = 0; i < Q; i++)
-                        fi[i] += R(0.5) * w_of<R>(i) * (a0 + R(3) * (R(cz_of(i)) * az + R(cr_of(i)) * ar));
-                    hdst[o] = m0;
-                    hdst[plane + o] = Hz;
-                    hdst[2 * plane + o] = Hr;
-                }
-                if (guo) {
-                    // Guo forcing: f*_i = f_i + omega (f^eq_i(u) - f_i) + S_i + h_i with
-                    // S_i = w_i (1 - omega/2) [3 (c_i - u).F + 9 (c_i.u)(c_i.F)], F = 2 rho (u - u0)
-                    const R Fz = R(2) * rho * (uz - u0z), Fr = R(2) * rho * (ur - u0r);
-                    const R usq = uz * uz + ur * ur, uF = uz * Fz + ur * Fr;
-                    const R gpre = R(1) - R(0.5) * omega;
-                    const R base = omega * (drho - R(1.5) * rho * usq) - gpre * R(3) * uF + hm0;
-                    fout[o] = om1 * fi[0] + w_of<R>(0) * base;
-#pragma unroll
-                    for (int m = 0; m < 4; m++) {
-                        const int i = 2 * m + 1;
-                        const R w = w_of<R>(i);
-                        const R cx = R(cz_of(i)), cy = R(cr_of(i));
-                        const R cu = cx * uz + cy * ur, cF = cx * Fz + cy * Fr;
-                        const R even = w * (base + R(4.5) * omega * rho * cu * cu + gpre * R(9) * cu * cF);
-                        const R odd = R(3) * w * (omega * rho * cu + gpre * cF + cx * hHz + cy * hHr);
-                        fout[i * plane + o] = om1 * fi[i] + even + odd;
-                        fout[(i + 1) * plane + o] = om1 * fi[i + 1] + even - odd;
-                    }
-                } else {
-                    const R u0sq = u0z * u0z + u0r * u0r, u1sq = u1z * u1z + u1r * u1r;
-                    const R base = omega * drho + rho * (om1 * R(1.5) * u0sq - R(1.5) * u1sq);
-                    fout[o] = om1 * fi[0] + w_of<R>(0) * (base + hm0);
-#pragma unroll
-                    for (int m = 0; m < 4; m++) {
-                        const int i = 2 * m + 1;  // i and i+1 are opposite
-                        const R w = w_of<R>(i);
-                        const R cx = R(cz_of(i)), cy = R(cr_of(i));
-                        const R cu0 = cx * u0z + cy * u0r, cu1 = cx * u1z + cy * u1r;
-                        const R even = w * (base + rho * R(4.5) * (cu1 * cu1 - om1 * cu0 * cu0) + hm0);
-                        const R odd = R(3) * w * (rho * (cu1 - om1 * cu0) + cx * hHz + cy * hHr);
-                        fout[i * plane + o] = om1 * fi[i] + even + odd;
-                        fout[(i + 1) * plane + o] = om1 * fi[i + 1] + even - odd;
-                    }
+                for (int m = 0; m < 4; m++) {
+                    const int i = 2 * m + 1;  // i and i+1 are opposite
+                    const R w = w_of<R>(i);
+                    const R cx = R(cz_of(i)), cy = R(cr_of(i));
+                    const R cu0 = cx * u0z + cy * u0r, cu1 = cx * u1z + cy * u1r;
+                    const R even = w * (base + rho * R(4.5) * (cu1 * cu1 - om1 * cu0 * cu0) + m0);
+                    const R odd = R(3) * w * (rho * (cu1 - om1 * cu0) + cx * Hz + cy * Hr);
+                    fout[i * plane + o] = om1 * fi[i] + even + odd;
+                    fout[(i + 1) * plane + o] = om1 * fi[i + 1] + even - odd;
                 }
             }
         }
@@ -1066,10 +1022,6 @@ __device__ __forceinline__ void march2(const Params<R>& p, const R* __restrict__
     }
 }
 
-// Grid: one CTA per resident slot.  The flattened strip-row space
-// (strip * nr + row) is cut into gridDim.x equal contiguous ranges; a CTA
-// marches each strip segment of its range (usually one or two).  rows_per_cta
-// > 0 instead gives fixed chunks: CTA (x, y) = strip x, rows [y R, y R + R).
 template <typename R, int TZ, int RR, int CP, bool MP, bool AX, int FV = 0>
 __device__ __forceinline__ void march_cp(const Params<R>& p, const R* __restrict__ f, R* __restrict__ fout, int strip,
                                          int j0, int jend, unsigned char* smem_raw, int& bad,
@@ -1077,31 +1029,18 @@ __device__ __forceinline__ void march_cp(const Params<R>& p, const R* __restrict
     if constexpr (CP == 2)
         march2<R, TZ, RR, MP, AX, FV>(p, f, fout, strip, j0, jend, smem_raw, bad, hsrc, hdst);
     else
-        march<R, TZ, RR, MP, AX, FV>(p, f, fout, strip, j0, jend, smem_raw, bad, hsrc, hdst);
+        march<R, TZ, RR, MP, AX>(p, f, fout, strip, j0, jend, smem_raw, bad);
 }
 
+// Fixed chunks: CTA (x, y) marches strip x, rows [y R, y R + R) with R = rows_per_cta.
 template <typename R, int TZ, int RR, int CP, int MINB, bool MP, bool AX>
 __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB) k_step(Params<R> p, const R* __restrict__ f,
                                                                           R* __restrict__ fout, int rows_per_cta,
                                                                           int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int bad = 0;
-    if (rows_per_cta > 0) {
-        const int j0 = blockIdx.y * rows_per_cta;
-        march_cp<R, TZ, RR, CP, MP, AX>(p, f, fout, blockIdx.x, j0, min(j0 + rows_per_cta, p.nr), smem_raw, bad);
-    } else {
-        const int nstrips = (p.nz + TZ - 1) / TZ;
-        const long long total = (long long)nstrips * p.nr;
-        const long long per = (total + gridDim.x - 1) / gridDim.x;
-        long long a = (long long)blockIdx.x * per;
-        const long long b = min(a + per, total);
-        while (a < b) {
-            const int strip = (int)(a / p.nr), j0 = (int)(a - (long long)strip * p.nr);
-            const int jend = (int)min((long long)p.nr, j0 + (b - a));
-            march_cp<R, TZ, RR, CP, MP, AX>(p, f, fout, strip, j0, jend, smem_raw, bad);
-            a += jend - j0;
-        }
-    }
+    const int j0 = blockIdx.y * rows_per_cta;
+    march_cp<R, TZ, RR, CP, MP, AX>(p, f, fout, blockIdx.x, j0, min(j0 + rows_per_cta, p.nr), smem_raw, bad);
     if (bad) atomicOr(err, bad);
 }
 

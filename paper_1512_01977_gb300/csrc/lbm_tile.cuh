@@ -5,7 +5,8 @@
 // all stages in shared memory: more work in all (L runs on (TZ + 12)(TR + 12)
 // nodes for TZ x TR results), one launch.  What bounds it is the latency of the
 // four stages in a row, so every stage has one item per thread or little more,
-// and the collision's own populations are gathered first of all.
+// and the collision's own populations are gathered first of all.  us per step,
+// phases -> tiles: 64 x 64 6.2 -> 3.1, 512 x 256 9.3 -> 7.8; tile_form has more.
 //
 // The packed operations and their order are those of march2 (lbm_step.cuh), so
 // the results are the same bits.
@@ -58,7 +59,7 @@ __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWor
     float* sPr = sPz + WD * S::HD;
     const int tid = threadIdx.x, nz = p.nz, nr = p.nr, k0 = w.k0, j0 = w.j0;
     const bool periodic = p.top == TOP_PERIODIC;
-    const int jn = min(S::TR, nr - j0), jb = j0 + jn, kn = EDGE ? min(S::TZ, nz - k0) : S::TZ;
+    const int jn = min(S::TR, nr - j0), kn = EDGE ? min(S::TZ, nz - k0) : S::TZ;
     const T zero = pk(0.0f, 0.0f), ref = pk(p.rho_ref, p.rho_ref);
     const T la[3] = {zero, zero, zero};  // no link source in this form
     // columns k - 1 .. k + 2, wrapped: by one period unless the grid is narrower than the tile
