@@ -118,7 +118,7 @@ def _source_hash():
 def _ncu_traffic():
     """Per-launch DRAM bytes of the fused step kernel on this workload from the
     committed ncu summary, or None when the kernel sources changed since."""
-    path = os.path.join(ROOT, "profiles", "k_step_single_fp32_wave4096x2048.md")
+    path = os.path.join(ROOT, "profiles", "k_step_warp_fp32_wave4096x2048.md")
     try:
         vals = {}
         with open(path) as fh:
@@ -390,6 +390,9 @@ def run_ours(args):
         # the timed region ran this kernel alone, one launch per step: its average
         # launch duration over that region is the region's time per step
         t_a, t_b = 0.0, t_step
+    # launches per step: the fused step of the default grid is one (grids of at most 800,000 nodes take one
+    # or three, by size; counted as one)
+    per_step = 1 if path == lbm.PATH_FUSED else 2
     peak, peak_kind = _peaks()
     # algorithmic bytes of the kernel that ran: the fused kernel reads and writes the
     # 9 populations (72 B/node); kernel (b) of the split path 88 B/node
@@ -438,7 +441,7 @@ def run_ours(args):
                        "parallelism": "replicas only (independent solves per GPU)",
                        "device": props.name},
             "roofline": {"bound": "hbm",
-                         "kernel": "k_step_single (one-pass gather+psi+forces+EDM+source+collide; the single-solve form)"
+                         "kernel": "k_step_warp (one-pass gather+psi+forces+EDM+source+collide, one warp per strip)"
                          if path == lbm.PATH_FUSED else "k_update (forces+EDM+source+collide)",
                          "achieved": ach_b, "peak": peak, "unit": "GB/s", "frac": ach_b / peak,
                          "peak_source": peak_kind, "traffic": traffic,
@@ -448,7 +451,7 @@ def run_ours(args):
                          "avg_launch_source": "timed region / launches" if path == lbm.PATH_FUSED
                          else "CUDA events around each launch",
                          "isolated_launch_us": t_iso * 1e6,
-                         "launches_per_step": 1 if path == lbm.PATH_FUSED else 2,
+                         "launches_per_step": per_step,
                          "frac_of_nominal_7900_gbs": ach_b / 7900.0,
                          "two_kernel_equivalent": {
                              "bytes_per_node": BYTES_STEP,
@@ -459,7 +462,7 @@ def run_ours(args):
                     "d2h_bytes_per_step": 4 * 8 * n / args.steps,
                     "note": "one solve: init from pinned host fields, K steps, moments back to pinned host; "
                             "the copies are fixed per run, so the rate rises with K"},
-            "gpu_launches": (1 if path == lbm.PATH_FUSED else 2) * args.steps,
+            "gpu_launches": per_step * args.steps,
             "clocks": clocks,
             "mass_rweighted": mass_rw,
         }

@@ -194,13 +194,13 @@ int lbm_axi_sync(lbm_axi* h);
 int lbm_axi_time_kernels(lbm_axi* h, long long n, double* ms);
 
 /* Kernel configuration of a solve (performance only).
- *   path: LBM_PATH_FUSED -- one kernel per step (gather, moments, psi, forces,
- *         collision in a single pass over the populations, 72 B per node in FP32);
+ *   path: LBM_PATH_FUSED -- the whole update in one launch per step (FP32: tiles
+ *         held on chip for small grids, marching warps above 800,000 nodes, 72 B
+ *         per node) or in three (FP64, and FP32 in between), chosen by size;
  *         needs nr >= 16.  LBM_PATH_SPLIT -- kernel (a) (gather, rho, j, psi into
  *         field planes) then kernel (b) (forces + collision), 140 B per node.
- *   rows_per_cta: 0 -- one wave of CTAs, each marching an equal share of the
- *         (z-strip, row) space (default); > 0 -- fixed chunks of that many rows
- *         of one z-strip per CTA.
+ *   rows_per_cta: 0 -- the form the size chooses (default); > 0 -- one launch,
+ *         each CTA marching a fixed chunk of that many rows of one z-strip.
  * The default is FUSED (nr >= 16) with rows_per_cta = 0; a solve with
  * h_eval = LBM_H_LINK_AVG or forcing = LBM_FORCING_GUO defaults to FUSED only
  * when multiphase and axis_terms are both on (else SPLIT).  The paths agree to

@@ -2,10 +2,10 @@
  * lbm_axi_batch.h — batched stepping and autotuning on top of lbm_axi.h.
  *
  * Many independent solves (e.g. droplets of different sizes, temperatures and
- * relaxation times) advance together: each batch step is ONE launch of the
- * fused step kernel over a work list of tiles -- row ranges of the solves'
- * z-strips -- dealt to the CTAs by lbm_axi_tile_plan; steps are replayed from
- * a CUDA graph.  The update of every solve is exactly the single-solve update
+ * relaxation times) advance together: each batch step is ONE launch (three in
+ * FP64 and for FP32 batches of up to 800,000 nodes that do not fit the
+ * one-launch tiles) over a work list of tiles of all solves; steps are replayed
+ * from a CUDA graph.  The update of every solve is exactly the single-solve update
  * (Sec. II of arXiv:1512.01977); no arithmetic couples two solves, so a
  * solve's result is the same alone and in any batch.
  */
@@ -20,8 +20,10 @@ extern "C" {
 
 typedef struct lbm_axi_batch lbm_axi_batch;
 
-/* strip: z-columns per CTA, 64 or 112; grid: CTA slots the tiles are dealt to,
- * 0 = one wave of resident CTAs. */
+/* strip 112 with grid 0 (the default): the form the batch's size chooses.  Any
+ * other pair, FP32: CTAs marching strips of `strip` z-columns (64 or 112), their
+ * tiles dealt by lbm_axi_tile_plan to `grid` CTA slots (0 = one wave of resident
+ * CTAs).  FP64 has one form: the pair is kept but changes nothing. */
 typedef struct {
     int strip;
     int grid;
@@ -59,7 +61,7 @@ int lbm_axi_batch_get_tuning(const lbm_axi_batch* b, lbm_axi_batch_tuning* t);
 int lbm_axi_batch_set_tuning(lbm_axi_batch* b, const lbm_axi_batch_tuning* t);
 
 /* Autotuner: time `trials` launches of every candidate configuration (strip
- * 64 / 112 x tiles dealt to one or two resident waves) on this batch, keep the
+ * 64 / 112 x tiles dealt to one or two resident waves, the default form) on this batch, keep the
  * fastest and return it in *chosen (may be NULL).  Non-destructive: trial
  * launches read the current populations and write only the buffer the next
  * step overwrites; error words raised by trials are cleared.  Synchronous. */
@@ -71,8 +73,8 @@ int lbm_axi_batch_autotune(lbm_axi_batch* b, int trials, lbm_axi_batch_tuning* c
  * Non-destructive like lbm_axi_batch_autotune.  Synchronous. */
 int lbm_axi_autotune(lbm_axi* h, int trials, lbm_axi_tuning* chosen);
 
-/* Work plan of a batched launch (performance only; no counterpart in the
- * paper).  Every solve's (z-strip, row) space -- strip columns per strip,
+/* Work plan of a batched launch of marching CTAs (performance only; no
+ * counterpart in the paper).  Every solve's (z-strip, row) space -- strip columns per strip,
  * ceil(nz[i] / strip) strips -- is cut into tiles, rows [j0, jend) of one strip
  * of one solve, and the tiles are dealt to `slots` CTAs, largest first, each to
  * the CTA with the least work so far; a CTA marches its tiles one after
@@ -80,8 +82,8 @@ int lbm_axi_autotune(lbm_axi* h, int trials, lbm_axi_tuning* chosen);
  * above it and the 12-row lag between the kernel's first and last stage); of
  * the candidate cuts (whole strips, or the smallest chunk height of at least
  * 16 rows that fills 1..4 waves of slots) the one with the smallest largest
- * CTA cost is kept.  A single solve is planned the same way (wide strips, one
- * wave).  Host-only, no GPU.
+ * CTA cost is kept.  A large FP32 solve with the link source is planned the
+ * same way (wide strips, one wave).  Host-only, no GPU.
  *   nz, nr: n >= 1 grid sizes (host arrays); strip >= 1; slots >= 1;
  *   tiles_out: 4 ints per tile (solve, strip, j0, jend), grouped by CTA,
  *   max_tiles of room; first_out: the tiles of CTA c are first_out[c] ..

@@ -4,7 +4,7 @@ Requests (droplet oscillations and density waves of uneven grids, EOS kinds,
 temperatures and step counts) arrive on a schedule.  The server keeps every
 admitted solve's populations resident on the GPU, admits waiting requests in
 arrival order while the summed device footprint stays within a budget, and
-advances all active solves together -- one launch of the batched fused kernel
+advances all active solves together -- the batched step's one or three launches
 per time step -- in ticks that end when the next solve completes (or after
 `max_tick_steps`).  Finished solves are read back (rho, mass) and released,
 which frees room for the next admissions.  A request whose state goes
