@@ -29,7 +29,9 @@
 // by 5 262 (instruction fetch).
 //
 // The packed operations and their order are those of march2 (lbm_step.cuh), so
-// the results are the same bits.
+// the results are the same bits; with Guo forcing the compiler fuses a sum of
+// its longer collision differently here, and they agree to rounding (5e-7 after
+// 12 steps, relative).
 #pragma once
 
 #include <type_traits>

@@ -9,7 +9,9 @@
 // phases -> tiles: 64 x 64 6.2 -> 3.1, 512 x 256 9.3 -> 7.8; tile_form has more.
 //
 // The packed operations and their order are those of march2 (lbm_step.cuh), so
-// the results are the same bits.
+// the results are the same bits; with Guo forcing the compiler fuses a sum of
+// its longer collision differently here, and they agree to rounding (5e-7 after
+// 12 steps, relative).
 #pragma once
 
 #include "lbm_phase.cuh"
