@@ -82,8 +82,8 @@ int lbm_axi_autotune(lbm_axi* h, int trials, lbm_axi_tuning* chosen);
  * above it and the 12-row lag between the kernel's first and last stage); of
  * the candidate cuts (whole strips, or the smallest chunk height of at least
  * 16 rows that fills 1..4 waves of slots) the one with the smallest largest
- * CTA cost is kept.  A large FP32 solve with the link source is planned the
- * same way (wide strips, one wave).  Host-only, no GPU.
+ * CTA cost is kept.  A large FP32 solve with the link source or Guo
+ * forcing is planned the same way (wide strips, one wave).  Host-only, no GPU.
  *   nz, nr: n >= 1 grid sizes (host arrays); strip >= 1; slots >= 1;
  *   tiles_out: 4 ints per tile (solve, strip, j0, jend), grouped by CTA,
  *   max_tiles of room; first_out: the tiles of CTA c are first_out[c] ..

@@ -16,11 +16,11 @@ using TileB = Form<16, 16, 416>;
 using TileC = Form<32, 16, 320>;
 using TileD = Form<32, 8, 256>;
 
-template <typename F, bool AX, int FV>
+template <typename F, bool AX>
 cudaError_t one(const BatchSolve<float>& v, int parity, int* err, cudaStream_t s) {
     const int across = (v.p.nz + F::tz - 1) / F::tz;
     const unsigned grid = (unsigned)across * (unsigned)((v.p.nr + F::tr - 1) / F::tr);
-    return launch_early(k_tile<F::tz, F::tr, F::nt, true, AX, FV>, grid, F::nt, s,
+    return launch_early(k_tile<F::tz, F::tr, F::nt, true, AX>, grid, F::nt, s,
                         PhaseOne<float>{v, nullptr, nullptr, parity, across, err});
 }
 template <typename F, bool AX>
@@ -36,7 +36,7 @@ cudaError_t many(const PhaseMany<float>& a, int ntiles, cudaStream_t s) {
 // two of them, 16 x 16 while none has three, then the one with the least halo.  Axis terms off (psi one
 // row and column around): 500 x 500 11.7, 10.4, 7.9, 6.7, 9.8; 700 x 700 20, 18, 13.9, 11.1, 15.4.
 TileForm tile_form(const int* nz, const int* nr, int n, bool mp, bool ax, int fv) {
-    if (!mp || (fv & FV_LINK) || (fv && !ax)) return TILE_NONE;
+    if (!mp || fv) return TILE_NONE;
     constexpr long long kSms = 152, kMost = 200000;
     long long a = 0, b = 0, nodes = 0;
     for (int i = 0; i < n; i++) {
@@ -57,15 +57,10 @@ void tile_size(TileForm f, int* tz, int* tr) {
 }
 
 template <>
-cudaError_t Ops<float>::tile_step(TileForm f, const BatchSolve<float>& v, bool ax, int parity, int* err, cudaStream_t s,
-                                  int fv) {
-    if (!ax) return f == TILE_A ? one<TileA, false, 0>(v, parity, err, s) : one<TileD, false, 0>(v, parity, err, s);
-    if (fv == FV_GUO)
-        return f == TILE_A ? one<TileA, true, FV_GUO>(v, parity, err, s)
-                           : (f == TILE_B ? one<TileB, true, FV_GUO>(v, parity, err, s)
-                                          : one<TileC, true, FV_GUO>(v, parity, err, s));
-    return f == TILE_A ? one<TileA, true, 0>(v, parity, err, s)
-                       : (f == TILE_B ? one<TileB, true, 0>(v, parity, err, s) : one<TileC, true, 0>(v, parity, err, s));
+cudaError_t Ops<float>::tile_step(TileForm f, const BatchSolve<float>& v, bool ax, int parity, int* err, cudaStream_t s) {
+    if (!ax) return f == TILE_A ? one<TileA, false>(v, parity, err, s) : one<TileD, false>(v, parity, err, s);
+    return f == TILE_A ? one<TileA, true>(v, parity, err, s)
+                       : (f == TILE_B ? one<TileB, true>(v, parity, err, s) : one<TileC, true>(v, parity, err, s));
 }
 
 template <>

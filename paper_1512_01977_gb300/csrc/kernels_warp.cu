@@ -12,20 +12,18 @@ int kind_of(const Params<float>& p) {
 
 // One solve's kernel.  Without F_axis kappa is not used; without the force nor is the EOS.
 using One = void (*)(const BatchSolve<float>, const Tile*, int, int*);
-template <int FV>
 One one_mp_ax(int kind) {
     switch (kind) {
-        case WARP_CS: return k_step_warp<true, true, FV, WARP_CS>;
-        case WARP_CS_LATTICE: return k_step_warp<true, true, FV, WARP_CS_LATTICE>;
-        case WARP_VDW: return k_step_warp<true, true, FV, WARP_VDW>;
-        default: return k_step_warp<true, true, FV, WARP_VDW_LATTICE>;
+        case WARP_CS: return k_step_warp<true, true, WARP_CS>;
+        case WARP_CS_LATTICE: return k_step_warp<true, true, WARP_CS_LATTICE>;
+        case WARP_VDW: return k_step_warp<true, true, WARP_VDW>;
+        default: return k_step_warp<true, true, WARP_VDW_LATTICE>;
     }
 }
-One one(const Params<float>& p, int fv, bool mp, bool ax) {
-    if (fv == FV_GUO) return one_mp_ax<FV_GUO>(kind_of(p));
-    if (mp && ax) return one_mp_ax<0>(kind_of(p));
-    if (mp) return p.eos == EOS_VDW ? k_step_warp<true, false, 0, WARP_VDW> : k_step_warp<true, false, 0, WARP_CS>;
-    return ax ? k_step_warp<false, true, 0, WARP_CS> : k_step_warp<false, false, 0, WARP_CS>;
+One one(const Params<float>& p, bool mp, bool ax) {
+    if (mp && ax) return one_mp_ax(kind_of(p));
+    if (mp) return p.eos == EOS_VDW ? k_step_warp<true, false, WARP_VDW> : k_step_warp<true, false, WARP_CS>;
+    return ax ? k_step_warp<false, true, WARP_CS> : k_step_warp<false, false, WARP_CS>;
 }
 
 using Many = void (*)(const BatchTable<float>, const Tile*, int, int*);
@@ -52,17 +50,16 @@ int Ops<float>::warp_slots() {
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_warp<true, true, 0, WARP_CS>, 32, 0) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_warp<true, true, WARP_CS>, 32, 0) != cudaSuccess)
         return 0;
     return cached = sms * (per_sm > 0 ? per_sm : 1);
 }
 
 template <>
 cudaError_t Ops<float>::step_warp(const BatchSolve<float>& v, const Tile* tiles, int ntiles, bool mp, bool ax, int parity,
-                                  int* err, cudaStream_t s, int fv) {
+                                  int* err, cudaStream_t s) {
     if (ntiles <= 0) return cudaErrorInvalidConfiguration;
-    if (fv != 0 && !(fv == FV_GUO && mp && ax)) return cudaErrorInvalidValue;
-    one(v.p, fv, mp, ax)<<<ntiles, 32, 0, s>>>(v, tiles, parity, err);
+    one(v.p, mp, ax)<<<ntiles, 32, 0, s>>>(v, tiles, parity, err);
     return cudaGetLastError();
 }
 

@@ -45,11 +45,11 @@ static cudaError_t step_fused(lbm_axi* h, const Params<R>& p, int c) {
     const lbm::BatchSolve<R> s = lbm_handle_solve<R>(h, p, 0);
     const lbm::LinkSets<R> hs{static_cast<const R*>(h->hb[0]), static_cast<R*>(h->hb[1])};
     if constexpr (sizeof(R) == 4)
-        if (h->tile != lbm::TILE_NONE) return Ops<R>::tile_step(h->tile, s, ax, c, h->derr, h->stream, fv_of(h));
+        if (h->tile != lbm::TILE_NONE) return Ops<R>::tile_step(h->tile, s, ax, c, h->derr, h->stream);
     if (lbm_by_phases(h->precision, (long long)h->nz * h->nr))
         return Ops<R>::phase_step(s, hs, mp, ax, c, h->derr, h->stream, fv_of(h));
     if constexpr (sizeof(R) == 4)
-        if (!h->hb[0]) return Ops<R>::step_warp(s, h->d_tiles, h->ncta, mp, ax, c, h->derr, h->stream, fv_of(h));
+        if (fv_of(h) == 0) return Ops<R>::step_warp(s, h->d_tiles, h->ncta, mp, ax, c, h->derr, h->stream);
     return Ops<R>::step_single(s, hs, h->d_tiles, h->d_first, h->ncta, mp, ax, c, h->derr, h->stream, fv_of(h));
 }
 cudaError_t lbm_handle_step_fused(lbm_axi* h, int c) {
@@ -331,21 +331,22 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     h->mout = (double*)dev_alloc(4 * (size_t)nz * nr * sizeof(double));
     h->partial = (double*)dev_alloc(4 * lbm::kReduceBlocks * sizeof(double));
     h->derr = (int*)dev_alloc(sizeof(int));
-    // tile plan of the marching step: warps, or CTAs on wide strips with the link source
-    const bool link = o.h_eval == LBM_H_LINK_AVG && o.axis_terms;
+    // tile plan of the marching step: warps, or CTAs on wide strips with the link source or Guo forcing
+    // (4096 x 2048 Guo: 210 us per step by CTAs, 155 by warps, whose sums round differently)
+    const bool link = o.h_eval == LBM_H_LINK_AVG && o.axis_terms, ctas = link || guo_of(h);
     std::vector<lbm::Tile> tiles;
     std::vector<int> first;
     if (lbm_by_phases(o.precision, (long long)nz * nr)) {
         first.assign(1, 0);
     } else {
-        const int slots = link ? Ops<float>::batch_resident_ctas(lbm::kStripWide) : Ops<float>::warp_slots();
+        const int slots = ctas ? Ops<float>::batch_resident_ctas(lbm::kStripWide) : Ops<float>::warp_slots();
         int rc = LBM_ERR_CUDA;
         try {
-            if (link)
+            if (ctas)
                 rc = slots > 0 ? lbm::plan_tiles(&nz, &nr, 1, lbm::kStripWide, slots, tiles, first, nullptr) : rc;
             else
                 rc = slots > 0 ? lbm::plan_warp_tiles(&nz, &nr, 1, slots, tiles) : rc;
-            if (!link) first.assign(1, 0);
+            if (!ctas) first.assign(1, 0);
         } catch (...) {
             rc = LBM_ERR_OOM;
         }
@@ -355,7 +356,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
             return rc;
         }
     }
-    h->ncta = link ? (int)first.size() - 1 : (int)tiles.size();
+    h->ncta = ctas ? (int)first.size() - 1 : (int)tiles.size();
     h->d_tiles = (lbm::Tile*)dev_alloc(tiles.size() * sizeof(lbm::Tile));
     h->d_first = (int*)dev_alloc(first.size() * sizeof(int));
     h->bytes = lbm_axi_footprint(nz, nr, o.precision);

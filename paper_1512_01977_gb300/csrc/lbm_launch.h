@@ -69,15 +69,15 @@ struct Ops {
     // step_single and step_table: FP64 steps by phases).
     static cudaError_t step_batch(const BatchSolve<R>* solves, const Tile* tiles, const int* first, int ncta,
                                   bool mp, bool ax, int parity, int strip, int* err, cudaStream_t s);
-    // The fused step of one solve in a link-source form (fv has FV_LINK; mp && ax),
+    // The fused step of one solve with Guo forcing or the link source (fv; mp && ax),
     // descriptor by value, kStripWide tiles.
     static cudaError_t step_single(const BatchSolve<R>& solve, const LinkSets<R>& h, const Tile* tiles,
                                    const int* first, int ncta, bool mp, bool ax, int parity, int* err,
                                    cudaStream_t s, int fv = 0);
     // The fused step by warps (lbm_march.cuh; FP32 only): tile t on block t (plan_warp_tiles for warp_slots()),
-    // of one solve (fv: 0 or FV_GUO) or of the n solves of a table.
+    // of one solve or of the n solves of a table (EDM, h_i at the node).
     static cudaError_t step_warp(const BatchSolve<R>& solve, const Tile* tiles, int ntiles, bool mp, bool ax, int parity,
-                                 int* err, cudaStream_t s, int fv);
+                                 int* err, cudaStream_t s);
     static cudaError_t step_warp_table(const BatchTable<R>& table, int n, const Tile* tiles, int ntiles, bool mp,
                                        bool ax, int parity, int* err, cudaStream_t s);
     static int warp_slots();
@@ -93,8 +93,7 @@ struct Ops {
     // solve without a periodic top (axis terms on).
     static cudaError_t phase_step_many(const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles, int nghost,
                                        int rows, bool mp, bool ax, int parity, int* err, cudaStream_t s);
-    static cudaError_t tile_step(TileForm f, const BatchSolve<R>& solve, bool ax, int parity, int* err, cudaStream_t s,
-                                 int fv = 0);
+    static cudaError_t tile_step(TileForm f, const BatchSolve<R>& solve, bool ax, int parity, int* err, cudaStream_t s);
     static cudaError_t tile_step_many(TileForm f, const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles,
                                       bool ax, int parity, int* err, cudaStream_t s);
     static int phase_tile_z();
@@ -103,14 +102,14 @@ struct Ops {
 };
 
 template <>
-cudaError_t Ops<float>::tile_step(TileForm, const BatchSolve<float>&, bool, int, int*, cudaStream_t, int);
+cudaError_t Ops<float>::tile_step(TileForm, const BatchSolve<float>&, bool, int, int*, cudaStream_t);
 template <>
 cudaError_t Ops<float>::tile_step_many(TileForm, const BatchSolve<float>*, const PhaseTile*, int, bool, int, int*,
                                        cudaStream_t);
 template <>
 int Ops<float>::warp_slots();
 template <>
-cudaError_t Ops<float>::step_warp(const BatchSolve<float>&, const Tile*, int, bool, bool, int, int*, cudaStream_t, int);
+cudaError_t Ops<float>::step_warp(const BatchSolve<float>&, const Tile*, int, bool, bool, int, int*, cudaStream_t);
 template <>
 cudaError_t Ops<float>::step_warp_table(const BatchTable<float>&, int, const Tile*, int, bool, bool, int, int*,
                                         cudaStream_t);

@@ -190,7 +190,8 @@ template <typename R>
 static cudaError_t single_prepare() {
     const int smem = (int)BatchTile<R, kStripWide>::smem();
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const cudaError_t e = cudaFuncSetAttribute(single_kernel<R, FV_LINK>(), a, smem);
+    cudaError_t e = cudaFuncSetAttribute(single_kernel<R, FV_GUO>(), a, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(single_kernel<R, FV_LINK>(), a, smem);
     return e == cudaSuccess ? cudaFuncSetAttribute(single_kernel<R, FV_GUO | FV_LINK>(), a, smem) : e;
 }
 
@@ -304,8 +305,10 @@ cudaError_t Ops<R>::step_single(const BatchSolve<R>& solve, const LinkSets<R>& h
         using T = BatchTile<R, kStripWide>;
         if (ncta <= 0) return cudaErrorInvalidConfiguration;
         const size_t smem = T::smem();
-        if (!(fv & FV_LINK) || !(mp && ax)) return cudaErrorInvalidValue;
-        if (fv == FV_LINK)
+        if (fv == 0 || !(mp && ax)) return cudaErrorInvalidValue;
+        if (fv == FV_GUO)
+            single_kernel<R, FV_GUO>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
+        else if (fv == FV_LINK)
             single_kernel<R, FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);
         else
             single_kernel<R, FV_GUO | FV_LINK>()<<<ncta, T::NT, smem, s>>>(solve, h, tiles, first, parity, err);

@@ -29,9 +29,10 @@
 // by 5 262 (instruction fetch).
 //
 // The packed operations and their order are those of march2 (lbm_step.cuh), so
-// the results are the same bits; with Guo forcing the compiler fuses a sum of
-// its longer collision differently here, and they agree to rounding (5e-7 after
-// 12 steps, relative).
+// the results are the same bits.  (Not with Guo forcing: the compiler fuses a
+// sum of its longer collision differently here, which grows to 5e-5 of the
+// velocities in 200 steps; those solves step by phases and, when large, by
+// marching CTAs.)
 #pragma once
 
 #include <type_traits>
@@ -127,7 +128,7 @@ struct Column {
     __device__ __forceinline__ float2 operator[](int q) const { return a[q]; }
 };
 
-template <bool MP, bool AX, int FV, int EOS, bool LATTICE>
+template <bool MP, bool AX, int EOS, bool LATTICE>
 __device__ __forceinline__ void march_warp(const Params<float>& pp, const float* __restrict__ f, float* __restrict__ fout,
                                            int strip, int j0, int jend, float2* __restrict__ ring, int& bad) {
     using T = float2;
@@ -254,7 +255,7 @@ __device__ __forceinline__ void march_warp(const Params<float>& pp, const float*
                 source2(p, rho, cuz, cur, duz_dr, dur_dz, dur_dr, row, Hz, Hr, mir, rur);
             }
             float* out = fout + (row * p.pitch + k);
-            collide2<FV>(
+            collide2<0>(
                 p, cf, la, drho, o[32], o[64], cuz, cur, Hz, Hr, mir, rur,
                 [&](int q, T v) { cf[q] = v; }, [](int, T) {});
             if (stores && v1) {
@@ -294,7 +295,7 @@ __device__ __forceinline__ void march_warp(const Params<float>& pp, const float*
 enum WarpKind { WARP_CS = 0, WARP_CS_LATTICE = 1, WARP_VDW = 2, WARP_VDW_LATTICE = 3, WARP_MIXED = 4 };
 
 // One tile of one solve.
-template <bool MP, bool AX, int FV, int KIND>
+template <bool MP, bool AX, int KIND>
 __device__ __forceinline__ void march_tile(const BatchSolve<float>& s, const Tile& t, int parity, int* __restrict__ err) {
     __shared__ float2 ring[WarpShape::kRing * WarpShape::kRow];
     if (*static_cast<volatile const int*>(err)) return;  // the solve already went unphysical
@@ -302,19 +303,19 @@ __device__ __forceinline__ void march_tile(const BatchSolve<float>& s, const Til
     float* fo = parity ? const_cast<float*>(s.f_a) : s.f_b;
     int bad = 0;
     if constexpr (KIND != WARP_MIXED) {
-        march_warp<MP, AX, FV, (KIND & 2) ? EOS_VDW : EOS_CS, (KIND & 1) != 0>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
+        march_warp<MP, AX, (KIND & 2) ? EOS_VDW : EOS_CS, (KIND & 1) != 0>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
     } else {
         const bool lattice = s.p.kappa == KAPPA_LATTICE;
         if (s.p.eos == EOS_VDW) {
             if (lattice)
-                march_warp<MP, AX, FV, EOS_VDW, true>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
+                march_warp<MP, AX, EOS_VDW, true>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
             else
-                march_warp<MP, AX, FV, EOS_VDW, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
+                march_warp<MP, AX, EOS_VDW, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
         } else {
             if (lattice)
-                march_warp<MP, AX, FV, EOS_CS, true>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
+                march_warp<MP, AX, EOS_CS, true>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
             else
-                march_warp<MP, AX, FV, EOS_CS, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
+                march_warp<MP, AX, EOS_CS, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
         }
     }
     if (bad) atomicOr(err, bad);
@@ -328,10 +329,10 @@ __device__ __forceinline__ Tile warp_tile(const Tile* __restrict__ tiles) {
             __shfl_sync(0xffffffffu, t.j0, 0), __shfl_sync(0xffffffffu, t.jend, 0)};
 }
 
-template <bool MP, bool AX, int FV, int KIND>
+template <bool MP, bool AX, int KIND>
 __global__ void __launch_bounds__(32, WarpShape::kWarps)
     k_step_warp(const BatchSolve<float> s, const Tile* __restrict__ tiles, int parity, int* __restrict__ err) {
-    march_tile<MP, AX, FV, KIND>(s, warp_tile(tiles), parity, err);
+    march_tile<MP, AX, KIND>(s, warp_tile(tiles), parity, err);
 }
 
 // The tiles of many solves (at most BatchTable::N, a tile's solve counting from the table's first).
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(32, WarpShape::kWarps)
     k_step_warp_table(const __grid_constant__ BatchTable<float> tab, const Tile* __restrict__ tiles, int parity,
                       int* __restrict__ err) {
     const Tile t = warp_tile(tiles);
-    march_tile<MP, AX, 0, KIND>(tab.s[t.solve], t, parity, err + t.solve);
+    march_tile<MP, AX, KIND>(tab.s[t.solve], t, parity, err + t.solve);
 }
 
 }  // namespace lbm

@@ -24,7 +24,7 @@
 // behind the marching front) and given the field's parity; with periodic r
 // wrapped rows are evaluated in place.  Needs nr >= 16 (single reflections).
 //
-// Who marches this way: a large FP32 solve with the link source (k_step_single), a solve whose tuning
+// Who marches this way: a large FP32 solve with the link source or Guo forcing (k_step_single), a solve whose tuning
 // asks for fixed row chunks (k_step), an FP32 batch whose tuning asks for 64-column strips or a grid
 // (k_step_table, k_step_batch).  Every other call steps by tiles, phases or warps (lbm_tile.cuh,
 // lbm_phase.cuh, lbm_march.cuh), which are faster: 208 us here and 153 by warps on the 4096 x 2048 wave.
@@ -1103,7 +1103,7 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
     }
 }
 
-// The same step for a single solve in a link-source form (force and axis terms
+// The same step for a single solve with Guo forcing or the link source (force and axis terms
 // on), its descriptor passed by value: the parameters are read from the
 // kernel's constant bank instead of a shared-memory copy per tile.
 template <typename R, int TZ, int RR, int CP, int MINB, int FV>

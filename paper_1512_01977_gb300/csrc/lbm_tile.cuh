@@ -9,9 +9,10 @@
 // phases -> tiles: 64 x 64 6.2 -> 3.1, 512 x 256 9.3 -> 7.8; tile_form has more.
 //
 // The packed operations and their order are those of march2 (lbm_step.cuh), so
-// the results are the same bits; with Guo forcing the compiler fuses a sum of
-// its longer collision differently here, and they agree to rounding (5e-7 after
-// 12 steps, relative).
+// the results are the same bits.  (Not with Guo forcing: the compiler fuses a
+// sum of its longer collision differently here, which grows to 5e-5 of the
+// velocities in 200 steps; those solves step by phases and, when large, by
+// marching CTAs.)
 #pragma once
 
 #include "lbm_phase.cuh"
@@ -47,7 +48,7 @@ __device__ __forceinline__ void pull_pair(const Params<float>& p, const float* _
     }
 }
 
-template <typename S, bool MP, bool AX, int FV, bool EDGE>
+template <typename S, bool MP, bool AX, bool EDGE>
 __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWork<float>& w, float* smem, int failed) {
     using T = float2;
     constexpr int NT = S::NT, LZ = S::LZ, LR = S::LR, WL = S::WL, WD = S::WD, WU = S::WU;
@@ -173,7 +174,7 @@ __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWor
     }
     const int plane = (int)p.plane, k = k0 + cc;
     float* out = w.fout + (crow * p.pitch + k);
-    collide2<FV>(
+    collide2<0>(
         p, cf, la, drho, ld2<T>(sJz + o0, b), ld2<T>(sJr + o0, b), uz, ur, Hz, Hr, mir, rur,
         [&](int q, T v) {
             if (!EDGE || k + 1 < nz)
@@ -184,28 +185,28 @@ __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWor
         [](int, T) {});
 }
 
-template <typename S, bool MP, bool AX, int FV>
+template <typename S, bool MP, bool AX>
 __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWork<float>& w) {
     __shared__ __align__(16) float smem[S::elems];
     const int failed = *static_cast<volatile const int*>(w.err);
     if (w.k0 >= 8 && w.k0 + S::TZ + 8 <= p.nz)
-        tile_step<S, MP, AX, FV, false>(p, w, smem, failed);
+        tile_step<S, MP, AX, false>(p, w, smem, failed);
     else
-        tile_step<S, MP, AX, FV, true>(p, w, smem, failed);
+        tile_step<S, MP, AX, true>(p, w, smem, failed);
 }
 
-template <int TZ, int TR, int NT, bool MP, bool AX, int FV>
+template <int TZ, int TR, int NT, bool MP, bool AX>
 __global__ void __launch_bounds__(NT) k_tile(const PhaseOne<float> a) {
     const int ti = blockIdx.x / a.across, tk = blockIdx.x - ti * a.across;
     phase_wait();
-    tile_step<TileStep<TZ, TR, NT, AX>, MP, AX, FV>(a.s.p, phase_work(a.s, a.parity, a.err, tk * TZ, ti * TR));
+    tile_step<TileStep<TZ, TR, NT, AX>, MP, AX>(a.s.p, phase_work(a.s, a.parity, a.err, tk * TZ, ti * TR));
 }
 template <int TZ, int TR, int NT, bool MP, bool AX>
 __global__ void __launch_bounds__(NT) k_tile_many(const PhaseMany<float> a) {
     const PhaseTile tl = a.tiles[blockIdx.x];
     const Params<float> p = a.s[tl.solve].p;
     phase_wait();
-    tile_step<TileStep<TZ, TR, NT, AX>, MP, AX, 0>(p, phase_work(a.s[tl.solve], a.parity, a.err + tl.solve, tl.k0, tl.j0));
+    tile_step<TileStep<TZ, TR, NT, AX>, MP, AX>(p, phase_work(a.s[tl.solve], a.parity, a.err + tl.solve, tl.k0, tl.j0));
 }
 
 }  // namespace lbm

@@ -126,3 +126,21 @@ def test_moments_to_an_unaligned_address(lbm, prec):
     assert raw[4:4 + 8 * nz * nr].tobytes() == want.cpu().numpy().tobytes()
     assert not raw[:4].any() and not raw[-4:].any()
     s.close()
+
+
+@pytest.mark.parametrize("nz,nr", [(64, 16), (500, 250), (1001, 800)])
+def test_guo_steps_alike_at_every_size(lbm, nz, nr):
+    """Guo forcing, FP32: phases (64 x 16, 500 x 250) and marching CTAs (above 800,000 nodes) give one z-uniform
+    state, whatever the number of columns, the same bits as a narrow one."""
+    eos = lbm.make_eos(lbm.EOS_CS, 0.9)
+    rv, rl = lbm.lbm_eos_coexistence(eos)
+    column = rl - 0.05 * (rl - rv) * np.random.default_rng(3).uniform(size=(nr, 1))
+    got = []
+    for n in (32, nz):
+        s = lbm.Solver(n, nr, 0.9, eos=eos, precision=32, rho_ref=rl, forcing=lbm.FORCING_GUO)
+        s.init(np.repeat(column, n, axis=1)).step(5)
+        m = s.moments()
+        got.append([np.asarray(m[q]) for q in sorted(m)])
+        s.close()
+    for a, b in zip(*got):
+        assert np.array_equal(np.repeat(a[:, :1], nz, axis=1), b)
