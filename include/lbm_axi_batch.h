@@ -57,6 +57,8 @@ int lbm_axi_batch_status(lbm_axi_batch* b, int* status);
 /* Steps taken by the batch so far. */
 int lbm_axi_batch_steps(const lbm_axi_batch* b, long long* steps);
 
+/* Setting waits for the batch's stream and makes the new work lists; if that
+ * fails (LBM_ERR_CUDA) the batch keeps the tuning and the lists it had. */
 int lbm_axi_batch_get_tuning(const lbm_axi_batch* b, lbm_axi_batch_tuning* t);
 int lbm_axi_batch_set_tuning(lbm_axi_batch* b, const lbm_axi_batch_tuning* t);
 

@@ -2,7 +2,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "lbm_axi_batch.h"
@@ -22,6 +24,19 @@ struct WarpGroup {
     int s0, ns, t0, nt;
 };
 
+// The form of one (strip, grid) and the work lists it launches over.
+struct StepPlan {
+    int strip = lbm::kStripWide, grid = 0;
+    BatchForm form = FORM_MARCH;
+    lbm::TileForm tile = lbm::TILE_NONE;
+    std::vector<std::unique_ptr<WarpGroup>> groups;
+    lbm::PhaseTile* d_ptiles = nullptr;
+    int nptiles = 0, nghost = 0, prows = 0;
+    lbm::Tile* d_tiles = nullptr;  // tile plan for (strip, grid)
+    int* d_first = nullptr;        // [ncta + 1]
+    int ncta = 0;
+};
+
 struct lbm_axi_batch {
     int n;
     int precision;
@@ -31,23 +46,14 @@ struct lbm_axi_batch {
     std::vector<int> cur0;  // each solve's current buffer when the batch was made
     void* d_solves;         // BatchSolve<R>[n]
     lbm::BatchTable<float>* h_table;  // FP32, n <= BatchTable::N: the descriptors as one kernel argument
-    BatchForm form;         // of this tuning
-    lbm::TileForm tile;
-    std::vector<WarpGroup*> groups;
-    lbm::PhaseTile* d_ptiles;
-    int nptiles, nghost, prows;
-    lbm::Tile* d_tiles;     // tile plan for (strip, grid)
-    int* d_first;           // [ncta + 1]
-    int ncta;
+    StepPlan plan;          // replaced whole (replan), so it is always complete
     int* d_err;             // [n]
     int* h_err;             // pinned [n]
     cudaStream_t stream;
     bool own_stream;
     long long steps;  // batch steps taken; parity = steps & 1
-    int strip, grid;
-    cudaGraphExec_t graph;  // an even number of steps from parity 0
+    cudaGraphExec_t graph;  // an even number of steps from parity 0 of the plan
     int graph_steps;
-    int graph_strip, graph_grid;
     int pending;
 };
 
@@ -75,155 +81,162 @@ const Params<double>& params_of<double>(const lbm_axi* h) {
     return h->pdd;
 }
 
+template <typename R>
+BatchSolve<R> descriptor(const lbm_axi_batch* b, int i) {
+    return lbm_handle_solve<R>(b->solves[i], params_of<R>(b->solves[i]), b->cur0[i]);
+}
+
 // FP64 steps by phases at every tuning; FP32 at the default one (wide strips, grid
 // 0) by tiles or phases while the batch is small and by warps beyond, at the others by march2.
-BatchForm form_of(const lbm_axi_batch* b, long long nodes) {
+BatchForm form_of(const lbm_axi_batch* b, const StepPlan& p, long long nodes) {
     if (b->precision == 64) return FORM_PHASES;
-    if (b->strip != lbm::kStripWide || b->grid != 0) return FORM_MARCH;
-    if (b->tile != lbm::TILE_NONE) return FORM_TILES;
+    if (p.strip != lbm::kStripWide || p.grid != 0) return FORM_MARCH;
+    if (p.tile != lbm::TILE_NONE) return FORM_TILES;
     return lbm_by_phases(32, nodes) ? FORM_PHASES : FORM_WARPS;
 }
 
-void drop_groups(lbm_axi_batch* b) {
-    for (WarpGroup* g : b->groups) delete g;
-    b->groups.clear();
+void release(StepPlan& p) {
+    if (p.d_tiles) cudaFree(p.d_tiles);
+    if (p.d_first) cudaFree(p.d_first);
+    if (p.d_ptiles) cudaFree(p.d_ptiles);
+    p = StepPlan();
 }
 
+// The device's table of descriptors and the kernel argument that holds it when it fits (may throw).
 template <typename R>
-cudaError_t upload(lbm_axi_batch* b) {
+cudaError_t upload_solves(lbm_axi_batch* b) {
     std::vector<BatchSolve<R>> hs(b->n);
-    std::vector<int> nz(b->n), nr(b->n);
-    for (int i = 0; i < b->n; i++) {
-        lbm_axi* h = b->solves[i];
-        hs[i] = lbm_handle_solve<R>(h, params_of<R>(h), b->cur0[i]);
-        nz[i] = h->nz;
-        nr[i] = h->nr;
-    }
+    for (int i = 0; i < b->n; i++) hs[i] = descriptor<R>(b, i);
     if constexpr (sizeof(R) == 4) {
         if (b->h_table)
             for (int i = 0; i < b->n; i++) b->h_table->s[i] = hs[i];
     }
+    const cudaError_t e = cudaMemcpyAsync(b->d_solves, hs.data(), sizeof(BatchSolve<R>) * b->n, cudaMemcpyHostToDevice,
+                                          b->stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(b->stream) : e;
+}
+
+// Fill in the plan of p.strip and p.grid (may throw, device lists allocated so far in p).
+template <typename R>
+cudaError_t make_plan(const lbm_axi_batch* b, StepPlan& p) {
+    std::vector<int> nz(b->n), nr(b->n);
     long long nodes = 0;
-    for (int i = 0; i < b->n; i++) nodes += (long long)nz[i] * nr[i];
-    b->tile = b->precision == 32 ? lbm::tile_form(nz.data(), nr.data(), b->n, b->mp, b->ax, 0) : lbm::TILE_NONE;
-    b->form = form_of(b, nodes);
+    for (int i = 0; i < b->n; i++) {
+        nz[i] = b->solves[i]->nz;
+        nr[i] = b->solves[i]->nr;
+        nodes += (long long)nz[i] * nr[i];
+    }
+    p.tile = b->precision == 32 ? lbm::tile_form(nz.data(), nr.data(), b->n, b->mp, b->ax, 0) : lbm::TILE_NONE;
+    p.form = form_of(b, p, nodes);
     std::vector<lbm::Tile> tiles;
     std::vector<lbm::PhaseTile> ptiles;
     size_t inner = 0;  // tiles before the ghost rows'
     std::vector<int> first;
-    const bool node_tiles = b->form == FORM_PHASES || b->form == FORM_TILES;
+    const bool node_tiles = p.form == FORM_PHASES || p.form == FORM_TILES;
     if (node_tiles) {
         int tz = Ops<R>::phase_tile_z();
-        b->prows = Ops<R>::phase_rows(nodes);
-        if (b->form == FORM_TILES) lbm::tile_size(b->tile, &tz, &b->prows);
-        try {
-            for (int i = 0; i < b->n; i++)
-                for (int j = 0; j < nr[i]; j += b->prows)
-                    for (int k = 0; k < nz[i]; k += tz) ptiles.push_back(lbm::PhaseTile{i, k, j});
-            inner = ptiles.size();
-            for (int i = 0; i < b->n && b->ax && b->form == FORM_PHASES; i++)
-                for (int k = 0; k < nz[i] && b->solves[i]->opts.top_bc != LBM_TOP_PERIODIC; k += tz)
-                    ptiles.push_back(lbm::PhaseTile{i, k, -2});
-        } catch (...) {
-            return cudaErrorMemoryAllocation;
-        }
-    } else if (b->form == FORM_WARPS) {
-        drop_groups(b);
+        p.prows = Ops<R>::phase_rows(nodes);
+        if (p.form == FORM_TILES) lbm::tile_size(p.tile, &tz, &p.prows);
+        for (int i = 0; i < b->n; i++)
+            for (int j = 0; j < nr[i]; j += p.prows)
+                for (int k = 0; k < nz[i]; k += tz) ptiles.push_back(lbm::PhaseTile{i, k, j});
+        inner = ptiles.size();
+        for (int i = 0; i < b->n && b->ax && p.form == FORM_PHASES; i++)
+            for (int k = 0; k < nz[i] && b->solves[i]->opts.top_bc != LBM_TOP_PERIODIC; k += tz)
+                ptiles.push_back(lbm::PhaseTile{i, k, -2});
+    } else if (p.form == FORM_WARPS) {
         const int slots = Ops<float>::warp_slots();
         if (slots <= 0) return cudaErrorInvalidConfiguration;
-        try {
-            std::vector<lbm::Tile> part;
-            for (int s0 = 0; s0 < b->n; s0 += lbm::BatchTable<float>::N) {
-                const int ns = std::min(b->n - s0, (int)lbm::BatchTable<float>::N);
-                if (lbm::plan_warp_tiles(nz.data() + s0, nr.data() + s0, ns, slots, part) != LBM_OK)
-                    return cudaErrorMemoryAllocation;
-                b->groups.push_back(nullptr);
-                WarpGroup* g = b->groups.back() = new WarpGroup();
-                if constexpr (sizeof(R) == 4)
-                    for (int i = 0; i < ns; i++) g->table.s[i] = hs[s0 + i];
-                g->s0 = s0;
-                g->ns = ns;
-                g->t0 = (int)tiles.size();
-                g->nt = (int)part.size();
-                tiles.insert(tiles.end(), part.begin(), part.end());
-            }
-        } catch (...) {
-            return cudaErrorMemoryAllocation;
+        std::vector<lbm::Tile> part;
+        for (int s0 = 0; s0 < b->n; s0 += lbm::BatchTable<float>::N) {
+            const int ns = std::min(b->n - s0, (int)lbm::BatchTable<float>::N);
+            if (lbm::plan_warp_tiles(nz.data() + s0, nr.data() + s0, ns, slots, part) != LBM_OK)
+                return cudaErrorMemoryAllocation;
+            auto g = std::make_unique<WarpGroup>();
+            if constexpr (sizeof(R) == 4)
+                for (int i = 0; i < ns; i++) g->table.s[i] = descriptor<R>(b, s0 + i);
+            g->s0 = s0;
+            g->ns = ns;
+            g->t0 = (int)tiles.size();
+            g->nt = (int)part.size();
+            p.groups.push_back(std::move(g));
+            tiles.insert(tiles.end(), part.begin(), part.end());
         }
-        first.assign(1, 0);
     } else {
-        const int slots = b->grid > 0 ? b->grid : Ops<R>::batch_resident_ctas(b->strip);
+        const int slots = p.grid > 0 ? p.grid : Ops<R>::batch_resident_ctas(p.strip);
         if (slots <= 0) return cudaErrorInvalidConfiguration;
-        if (lbm::plan_tiles(nz.data(), nr.data(), b->n, b->strip, slots, tiles, first, nullptr) != LBM_OK)
+        if (lbm::plan_tiles(nz.data(), nr.data(), b->n, p.strip, slots, tiles, first, nullptr) != LBM_OK)
             return cudaErrorMemoryAllocation;
     }
-    // the graph holds the old plan's pointers
-    if (b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
-    cudaError_t e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return e;
-    if (b->d_tiles) cudaFree(b->d_tiles);
-    if (b->d_first) cudaFree(b->d_first);
-    if (b->d_ptiles) cudaFree(b->d_ptiles);
-    b->d_tiles = nullptr;
-    b->d_first = nullptr;
-    b->d_ptiles = nullptr;
-    b->ncta = b->nptiles = 0;
+    cudaError_t e = cudaSuccess;
     auto put = [&](void** d, const void* from, size_t bytes) {
+        if (bytes == 0) return;
         if (e == cudaSuccess) e = cudaMalloc(d, bytes);
         if (e == cudaSuccess) e = cudaMemcpyAsync(*d, from, bytes, cudaMemcpyHostToDevice, b->stream);
     };
-    if (node_tiles) {
-        put((void**)&b->d_ptiles, ptiles.data(), ptiles.size() * sizeof(lbm::PhaseTile));
-    } else {
-        put((void**)&b->d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile));
-        put((void**)&b->d_first, first.data(), first.size() * sizeof(int));
-    }
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->d_solves, hs.data(), sizeof(BatchSolve<R>) * b->n, cudaMemcpyHostToDevice,
-                            b->stream);
+    put((void**)&p.d_ptiles, ptiles.data(), ptiles.size() * sizeof(lbm::PhaseTile));
+    put((void**)&p.d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile));
+    put((void**)&p.d_first, first.data(), first.size() * sizeof(int));
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return e;
-    b->nptiles = (int)inner;
-    b->nghost = (int)(ptiles.size() - inner);
-    b->ncta = first.empty() ? 0 : (int)first.size() - 1;
+    p.nptiles = (int)inner;
+    p.nghost = (int)(ptiles.size() - inner);
+    p.ncta = first.empty() ? 0 : (int)first.size() - 1;
     return cudaSuccess;
 }
 
-cudaError_t upload_tables(lbm_axi_batch* b) {
-    return b->precision == 32 ? upload<float>(b) : upload<double>(b);
+// The plan of (strip, grid) in place of the present one, which stays if anything fails.
+cudaError_t replan(lbm_axi_batch* b, int strip, int grid) {
+    StepPlan p;
+    p.strip = strip;
+    p.grid = grid;
+    cudaError_t e;
+    try {
+        e = b->precision == 32 ? make_plan<float>(b, p) : make_plan<double>(b, p);
+    } catch (...) {
+        cudaStreamSynchronize(b->stream);  // copies from the lists that went away
+        e = cudaErrorMemoryAllocation;
+    }
+    if (e == cudaSuccess) {
+        if (b->graph) cudaGraphExecDestroy(b->graph);  // holds the old plan's pointers
+        b->graph = nullptr;
+        std::swap(b->plan, p);
+    }
+    release(p);
+    if (e != cudaSuccess) cudaGetLastError();  // not the next launch's error
+    return e;
 }
 
 cudaError_t launch(lbm_axi_batch* b, int parity) {
+    const StepPlan& p = b->plan;
+    if (!p.d_ptiles && !p.d_tiles) return cudaErrorInvalidConfiguration;
     if (b->precision == 64)
-        return Ops<double>::phase_step_many(static_cast<const BatchSolve<double>*>(b->d_solves), b->d_ptiles, b->nptiles,
-                                            b->nghost, b->prows, b->mp, b->ax, parity, b->d_err, b->stream);
+        return Ops<double>::phase_step_many(static_cast<const BatchSolve<double>*>(b->d_solves), p.d_ptiles, p.nptiles,
+                                            p.nghost, p.prows, b->mp, b->ax, parity, b->d_err, b->stream);
     const BatchSolve<float>* solves = static_cast<const BatchSolve<float>*>(b->d_solves);
-    if (b->form == FORM_WARPS) {
+    if (p.form == FORM_WARPS) {
         cudaError_t e = cudaSuccess;
-        for (size_t i = 0; i < b->groups.size() && e == cudaSuccess; i++) {
-            const WarpGroup& g = *b->groups[i];
-            e = Ops<float>::step_warp_table(g.table, g.ns, b->d_tiles + g.t0, g.nt, b->mp, b->ax, parity, b->d_err + g.s0,
+        for (size_t i = 0; i < p.groups.size() && e == cudaSuccess; i++) {
+            const WarpGroup& g = *p.groups[i];
+            e = Ops<float>::step_warp_table(g.table, g.ns, p.d_tiles + g.t0, g.nt, b->mp, b->ax, parity, b->d_err + g.s0,
                                             b->stream);
         }
         return e;
     }
-    if (b->form == FORM_TILES)
-        return Ops<float>::tile_step_many(b->tile, solves, b->d_ptiles, b->nptiles, b->ax, parity, b->d_err, b->stream);
-    if (b->form == FORM_PHASES)
-        return Ops<float>::phase_step_many(solves, b->d_ptiles, b->nptiles, b->nghost, b->prows, b->mp, b->ax, parity, b->d_err,
+    if (p.form == FORM_TILES)
+        return Ops<float>::tile_step_many(p.tile, solves, p.d_ptiles, p.nptiles, b->ax, parity, b->d_err, b->stream);
+    if (p.form == FORM_PHASES)
+        return Ops<float>::phase_step_many(solves, p.d_ptiles, p.nptiles, p.nghost, p.prows, b->mp, b->ax, parity, b->d_err,
                                            b->stream);
     if (b->h_table)  // n <= BatchTable::N: parameters through the constant bank
-        return Ops<float>::step_table(*b->h_table, b->d_tiles, b->d_first, b->ncta, b->mp, b->ax, parity, b->strip,
+        return Ops<float>::step_table(*b->h_table, p.d_tiles, p.d_first, p.ncta, b->mp, b->ax, parity, p.strip,
                                       b->d_err, b->stream);
-    return Ops<float>::step_batch(solves, b->d_tiles, b->d_first, b->ncta, b->mp, b->ax, parity, b->strip, b->d_err,
+    return Ops<float>::step_batch(solves, p.d_tiles, p.d_first, p.ncta, b->mp, b->ax, parity, p.strip, b->d_err,
                                   b->stream);
 }
 
 // Steps per graph replay: small batches take a few us per step, which a replay would otherwise spend on itself.
-int graph_steps_of(const lbm_axi_batch* b) { return b->form == FORM_TILES || b->form == FORM_PHASES ? 16 : 2; }
+int graph_steps_of(const lbm_axi_batch* b) { return b->plan.form == FORM_TILES || b->plan.form == FORM_PHASES ? 16 : 2; }
 
 int build_graph(lbm_axi_batch* b) {
     if (b->graph) {
@@ -247,8 +260,6 @@ int build_graph(lbm_axi_batch* b) {
         b->graph = nullptr;
         return LBM_ERR_CUDA;
     }
-    b->graph_strip = b->strip;
-    b->graph_grid = b->grid;
     return LBM_OK;
 }
 
@@ -260,14 +271,11 @@ void sync_handles(lbm_axi_batch* b) {
 void release(lbm_axi_batch* b) {
     if (b->graph) cudaGraphExecDestroy(b->graph);
     if (b->d_solves) cudaFree(b->d_solves);
-    if (b->d_tiles) cudaFree(b->d_tiles);
-    if (b->d_first) cudaFree(b->d_first);
-    if (b->d_ptiles) cudaFree(b->d_ptiles);
+    release(b->plan);
     if (b->d_err) cudaFree(b->d_err);
     if (b->h_err) cudaFreeHost(b->h_err);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b->h_table;
-    drop_groups(b);
 }
 
 // Time `trials` launches of fn on stream s (ms per launch), non-destructively.
@@ -319,23 +327,13 @@ int lbm_axi_batch_create(lbm_axi* const* solves, int n, void* stream, lbm_axi_ba
     b->device = dev;
     b->d_solves = nullptr;
     b->h_table = nullptr;
-    b->form = FORM_MARCH;
-    b->tile = lbm::TILE_NONE;
-    b->d_ptiles = nullptr;
-    b->nptiles = b->nghost = b->prows = 0;
-    b->d_tiles = nullptr;
-    b->d_first = nullptr;
-    b->ncta = 0;
     b->d_err = nullptr;
     b->h_err = nullptr;
     b->stream = nullptr;
     b->own_stream = false;
     b->steps = 0;
-    b->strip = lbm::kStripWide;
-    b->grid = 0;
     b->graph = nullptr;
     b->graph_steps = 0;
-    b->graph_strip = b->graph_grid = -1;
     b->pending = LBM_OK;
     try {
         b->solves.assign(solves, solves + n);
@@ -380,7 +378,12 @@ int lbm_axi_batch_create(lbm_axi* const* solves, int n, void* stream, lbm_axi_ba
         b->own_stream = true;
     }
     cudaError_t e = cudaMemsetAsync(b->d_err, 0, sizeof(int) * n, b->stream);
-    if (e == cudaSuccess) e = upload_tables(b);
+    try {
+        if (e == cudaSuccess) e = b->precision == 32 ? upload_solves<float>(b) : upload_solves<double>(b);
+    } catch (...) {
+        e = cudaErrorMemoryAllocation;
+    }
+    if (e == cudaSuccess) e = replan(b, lbm::kStripWide, 0);
     if (e != cudaSuccess) {
         release(b);
         delete b;
@@ -400,7 +403,7 @@ int lbm_axi_batch_step_async(lbm_axi_batch* b, long long nsteps) {
         nsteps--;
     }
     if (e == cudaSuccess && nsteps >= graph_steps_of(b)) {
-        if (!b->graph || b->graph_strip != b->strip || b->graph_grid != b->grid) {
+        if (!b->graph) {
             int rc = build_graph(b);
             if (rc != LBM_OK) return rc;
         }
@@ -463,8 +466,8 @@ int lbm_axi_batch_steps(const lbm_axi_batch* b, long long* steps) {
 
 int lbm_axi_batch_get_tuning(const lbm_axi_batch* b, lbm_axi_batch_tuning* t) {
     if (!b || !t) return LBM_ERR_INVALID_ARG;
-    t->strip = b->strip;
-    t->grid = b->grid;
+    t->strip = b->plan.strip;
+    t->grid = b->plan.grid;
     return LBM_OK;
 }
 
@@ -472,11 +475,8 @@ int lbm_axi_batch_set_tuning(lbm_axi_batch* b, const lbm_axi_batch_tuning* t) {
     if (!b || !t || (t->strip != lbm::kStripNarrow && t->strip != lbm::kStripWide) || t->grid < 0) return LBM_ERR_INVALID_ARG;
     DevGuard g(b->device);
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) return LBM_ERR_CUDA;
-    if (t->strip != b->strip || t->grid != b->grid || !(b->d_tiles || b->d_ptiles)) {
-        b->strip = t->strip;
-        b->grid = t->grid;
-        if (upload_tables(b) != cudaSuccess) return LBM_ERR_CUDA;
-    }
+    if ((t->strip != b->plan.strip || t->grid != b->plan.grid) && replan(b, t->strip, t->grid) != cudaSuccess)
+        return LBM_ERR_CUDA;
     return LBM_OK;
 }
 
@@ -485,7 +485,7 @@ int lbm_axi_batch_autotune(lbm_axi_batch* b, int trials, lbm_axi_batch_tuning* c
     DevGuard g(b->device);
     const int parity = (int)(b->steps & 1);
     float best = -1.f;
-    lbm_axi_batch_tuning bt = {b->strip, b->grid};
+    lbm_axi_batch_tuning bt = {b->plan.strip, b->plan.grid};
     const int strips[2] = {lbm::kStripNarrow, lbm::kStripWide};
     // the solves' error words before the trials (trial results are discarded; a
     // solve that had already failed stays failed, and skipped, afterwards)

@@ -1,0 +1,275 @@
+// A CUDA runtime and launchers that only keep books, so that the library's host code (lbm_axi.cu,
+// lbm_batch.cu) can be driven on the CPU through failures that a GPU must not be driven through: an
+// allocation that fails, a launch on a list that is gone.  Device memory is host memory; a launch checks
+// that the lists it is given lie in live allocations.  One program, one check per argument.
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include <stdio.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <map>
+#include <new>
+
+#include "lbm_axi.h"
+#include "lbm_axi_batch.h"
+#include "lbm_handle.h"
+#include "lbm_launch.h"
+
+namespace fake {
+std::map<uintptr_t, size_t>* live = nullptr;  // device allocations
+long long device_left = -1, host_left = -1;   // allocations until one fails (-1: none does)
+int launches = 0, violations = 0;
+bool track = false;
+
+bool inside(const void* p, size_t bytes) {
+    auto it = live->upper_bound((uintptr_t)p);
+    if (it == live->begin()) return false;
+    --it;
+    return (uintptr_t)p + bytes <= it->first + it->second;
+}
+cudaError_t launch(const void* list, size_t bytes, const void* list2 = nullptr, size_t bytes2 = 0) {
+    launches++;
+    if (!inside(list, bytes) || (bytes2 && !inside(list2, bytes2))) {
+        violations++;
+        return cudaErrorIllegalAddress;
+    }
+    return cudaSuccess;
+}
+}  // namespace fake
+
+void* operator new(size_t n) {
+    if (fake::host_left >= 0 && fake::track && fake::host_left-- == 0) throw std::bad_alloc();
+    void* p = malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+
+// ----------------------------------------------------------------- runtime --
+
+extern "C" {
+cudaError_t cudaMalloc(void** p, size_t n) {
+    if (fake::device_left >= 0 && fake::device_left-- == 0) return cudaErrorMemoryAllocation;
+    *p = malloc(n);
+    (*fake::live)[(uintptr_t)*p] = n;
+    return cudaSuccess;
+}
+cudaError_t cudaFree(void* p) {
+    fake::live->erase((uintptr_t)p);
+    free(p);
+    return cudaSuccess;
+}
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return *p = calloc(1, n), cudaSuccess; }
+cudaError_t cudaMallocHost(void** p, size_t n) { return *p = calloc(1, n), cudaSuccess; }
+cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
+cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return memcpy(d, s, n), cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    return memcpy(d, s, n), cudaSuccess;
+}
+cudaError_t cudaMemcpy2DAsync(void*, size_t, const void*, size_t, size_t, size_t, cudaMemcpyKind, cudaStream_t) {
+    return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
+    memset(a, 0, sizeof(*a));
+    if (fake::inside(p, 1)) a->type = cudaMemoryTypeDevice;
+    return cudaSuccess;
+}
+cudaError_t cudaEventCreate(cudaEvent_t* e) { return *e = nullptr, cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.0f, cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = (cudaStream_t)malloc(1), cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t s) { return free((void*)s), cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { return *g = (cudaGraph_t)malloc(1), cudaSuccess; }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) {
+    return *x = (cudaGraphExec_t)malloc(1), cudaSuccess;
+}
+cudaError_t cudaGraphDestroy(cudaGraph_t g) { return free((void*)g), cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { return free((void*)x), cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+}
+
+// --------------------------------------------------------------- launchers --
+
+namespace lbm {
+
+TileForm tile_form(const int*, const int*, int, bool, bool, int) { return TILE_NONE; }
+void tile_size(TileForm, int* tz, int* tr) { *tz = 16, *tr = 8; }
+
+template <typename R>
+cudaError_t Ops<R>::density(const Params<R>&, const R*, R*, int*, cudaStream_t, LinkPlanes<R>) { return cudaSuccess; }
+template <typename R>
+cudaError_t Ops<R>::update(const Params<R>&, const R*, R*, const R*, cudaStream_t, LinkPlanes<R>, bool) {
+    return cudaSuccess;
+}
+template <typename R>
+cudaError_t Ops<R>::fields(const BatchSolve<R>&, LinkPlanes<R>, const Params<double>&, int, double*, double*, double*,
+                           double*, R*, int*, cudaStream_t) {
+    return cudaSuccess;
+}
+template <typename R>
+cudaError_t Ops<R>::init(const Params<R>&, double, const double*, const double*, const double*, R*, cudaStream_t,
+                         const R*, const int*) {
+    return cudaSuccess;
+}
+template <typename R>
+cudaError_t Ops<R>::mass(const Params<R>&, const R*, LinkPlanes<R>, double*, double*, int*, cudaStream_t) {
+    return cudaSuccess;
+}
+template <typename R>
+cudaError_t Ops<R>::pjump(const Params<R>&, const Params<double>&, const R*, LinkPlanes<R>, double, double, double,
+                          double, double*, double*, int*, cudaStream_t) {
+    return cudaSuccess;
+}
+template <typename R>
+cudaError_t Ops<R>::take_error(int*, int*, cudaStream_t) { return cudaSuccess; }
+template <typename R>
+cudaError_t Ops<R>::prepare() { return cudaSuccess; }
+template <typename R>
+cudaError_t Ops<R>::step(const Params<R>&, const R*, R*, int, int*, cudaStream_t) { return cudaSuccess; }
+template <typename R>
+cudaError_t Ops<R>::step_batch(const BatchSolve<R>*, const Tile* tiles, const int* first, int ncta, bool, bool, int, int,
+                               int*, cudaStream_t) {
+    if (ncta <= 0) return cudaErrorInvalidConfiguration;
+    return fake::launch(first, (ncta + 1) * sizeof(int), tiles, sizeof(Tile));
+}
+template <typename R>
+cudaError_t Ops<R>::step_single(const BatchSolve<R>&, const LinkSets<R>&, const Tile* tiles, const int* first, int ncta,
+                                bool, bool, int, int*, cudaStream_t, int) {
+    if (ncta <= 0) return cudaErrorInvalidConfiguration;
+    return fake::launch(first, (ncta + 1) * sizeof(int), tiles, sizeof(Tile));
+}
+template <typename R>
+cudaError_t Ops<R>::step_table(const BatchTable<R>&, const Tile* tiles, const int* first, int ncta, bool, bool, int, int,
+                               int*, cudaStream_t) {
+    if (ncta <= 0) return cudaErrorInvalidConfiguration;
+    return fake::launch(first, (ncta + 1) * sizeof(int), tiles, sizeof(Tile));
+}
+template <typename R>
+cudaError_t Ops<R>::phase_step(const BatchSolve<R>&, const LinkSets<R>&, bool, bool, int, int*, cudaStream_t, int) {
+    return fake::launches++, cudaSuccess;
+}
+template <typename R>
+cudaError_t Ops<R>::phase_step_many(const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles, int nghost, int,
+                                    bool, bool, int, int*, cudaStream_t) {
+    if (ntiles <= 0) return cudaErrorInvalidConfiguration;
+    return fake::launch(tiles, (ntiles + nghost) * sizeof(PhaseTile), solves, sizeof(BatchSolve<R>));
+}
+template <typename R>
+int Ops<R>::phase_tile_z() { return 64; }
+template <typename R>
+int Ops<R>::phase_rows(long long) { return 8; }
+template <typename R>
+int Ops<R>::batch_resident_ctas(int) { return 608; }
+template <>
+cudaError_t Ops<float>::tile_step(TileForm, const BatchSolve<float>&, bool, int, int*, cudaStream_t) {
+    return fake::launches++, cudaSuccess;
+}
+template <>
+cudaError_t Ops<float>::tile_step_many(TileForm, const BatchSolve<float>*, const PhaseTile* tiles, int n, bool, int, int*,
+                                       cudaStream_t) {
+    return fake::launch(tiles, n * sizeof(PhaseTile));
+}
+template <>
+int Ops<float>::warp_slots() { return 1824; }
+template <>
+cudaError_t Ops<float>::step_warp(const BatchSolve<float>&, const Tile* tiles, int n, bool, bool, int, int*, cudaStream_t) {
+    return fake::launch(tiles, n * sizeof(Tile));
+}
+template <>
+cudaError_t Ops<float>::step_warp_table(const BatchTable<float>& t, int ns, const Tile* tiles, int n, bool, bool, int,
+                                        int*, cudaStream_t) {
+    if (n <= 0 || ns < 1) return cudaErrorInvalidConfiguration;
+    const cudaError_t e = fake::launch(tiles, n * sizeof(Tile));
+    for (int i = 0; e == cudaSuccess && i < n; i++)  // the list is this form's: strips of its width, its solves
+        if (tiles[i].solve < 0 || tiles[i].solve >= ns || tiles[i].strip * kWarpStrip >= t.s[tiles[i].solve].p.nz ||
+            tiles[i].jend > t.s[tiles[i].solve].p.nr)
+            fake::violations++;
+    return e;
+}
+template struct Ops<float>;
+template struct Ops<double>;
+
+}  // namespace lbm
+
+// ------------------------------------------------------------------ checks --
+
+#define CHECK(c)                                              \
+    do {                                                      \
+        if (!(c)) {                                           \
+            fprintf(stderr, "line %d: %s\n", __LINE__, #c);   \
+            exit(1);                                          \
+        }                                                     \
+    } while (0)
+
+static lbm_axi* solve(int nz, int nr, int precision, void* stream = nullptr) {
+    lbm_axi_opts o;
+    lbm_axi_default_opts(&o);
+    o.precision = precision;
+    o.stream = stream;
+    lbm_eos e = {LBM_EOS_CS, 0.9, 1.0, 4.0, 1.0, 0.01};
+    lbm_axi* h = nullptr;
+    CHECK(lbm_axi_create(nz, nr, 1.0, &e, -0.152, &o, &h) == LBM_OK);
+    double* rho = (double*)calloc((size_t)nz * nr, sizeof(double));
+    CHECK(lbm_axi_init(h, rho, nullptr, nullptr) == LBM_OK);
+    free(rho);
+    return h;
+}
+
+// A change of a batch's tuning that runs out of device or host memory, at any of its allocations: the call
+// reports it, the batch keeps the tuning it had and the next step launches over that tuning's lists.
+static void batch_retune(int nz, int nr, int n, int precision, bool device) {
+    lbm_axi* h[300];
+    for (int i = 0; i < n; i++) h[i] = solve(nz, nr, precision);
+    lbm_axi_batch* b = nullptr;
+    CHECK(lbm_axi_batch_create(h, n, nullptr, &b) == LBM_OK);
+    CHECK(lbm_axi_batch_step(b, 1) == LBM_OK);
+    const lbm_axi_batch_tuning to[4] = {{64, 0}, {112, 0}, {112, 300}, {112, 0}};
+    for (const lbm_axi_batch_tuning& t : to) {
+        lbm_axi_batch_tuning had, has;
+        lbm_axi_batch_get_tuning(b, &had);
+        int failures = 0;
+        for (int at = 0;; at++) {
+            (device ? fake::device_left : fake::host_left) = at;
+            fake::track = true;
+            const int rc = lbm_axi_batch_set_tuning(b, &t);
+            fake::track = false;
+            fake::device_left = fake::host_left = -1;
+            if (rc == LBM_OK) break;
+            failures++;
+            CHECK(rc == LBM_ERR_CUDA || rc == LBM_ERR_OOM);
+            lbm_axi_batch_get_tuning(b, &has);
+            CHECK(has.strip == had.strip && has.grid == had.grid);
+            CHECK(lbm_axi_batch_step(b, 1) == LBM_OK && lbm_axi_batch_step(b, 3) == LBM_OK);
+            CHECK(fake::violations == 0);
+        }
+        CHECK(failures > 0);
+        lbm_axi_batch_get_tuning(b, &has);
+        CHECK(has.strip == t.strip && has.grid == t.grid);
+        CHECK(lbm_axi_batch_step(b, 5) == LBM_OK && fake::violations == 0);
+    }
+    lbm_axi_batch_destroy(b);
+    for (int i = 0; i < n; i++) lbm_axi_destroy(h[i]);
+    CHECK(fake::live->empty());
+}
+
+int main(int argc, char** argv) {
+    fake::live = new std::map<uintptr_t, size_t>();
+    const char* what = argc > 1 ? argv[1] : "";
+    if (!strcmp(what, "retune_device_warps")) return batch_retune(1040, 400, 3, 32, true), 0;
+    if (!strcmp(what, "retune_host_warps")) return batch_retune(1040, 400, 3, 32, false), 0;
+    if (!strcmp(what, "retune_host_two_tables")) return batch_retune(64, 48, 280, 32, false), 0;
+    if (!strcmp(what, "retune_device_phases")) return batch_retune(100, 40, 3, 32, true), 0;
+    if (!strcmp(what, "retune_host_fp64")) return batch_retune(100, 40, 3, 64, false), 0;
+    fprintf(stderr, "unknown check %s\n", what);
+    return 2;
+}
