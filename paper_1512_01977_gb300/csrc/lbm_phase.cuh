@@ -71,11 +71,29 @@ struct PhaseWork {
     R* aux;
     R* u;  // u planes
     int* err;
-    int k0, j0;
+    int k0, j0, parity;
 };
 template <typename R>
 __device__ __forceinline__ PhaseWork<R> phase_work(const BatchSolve<R>& s, int parity, int* err, int k0, int j0) {
-    return {parity ? s.f_b : s.f_a, parity ? const_cast<R*>(s.f_a) : s.f_b, s.aux, s.stage, err, k0, j0};
+    return {parity ? s.f_b : s.f_a, parity ? const_cast<R*>(s.f_a) : s.f_b, s.aux, s.stage, err, k0, j0, parity};
+}
+
+// The error word of a solve that steps by phases: the bits of even steps in place, those of odd steps
+// above them.  So a phase knows an error of an earlier step, whose populations are void and left alone, from
+// one of its own step, which it finishes: the buffer that the step writes would otherwise go on holding
+// an older state that reads as a sound one.
+constexpr int kErrShift = 8;
+__device__ __forceinline__ int err_of_step(int bits, int parity) { return parity ? bits << kErrShift : bits; }
+__device__ __forceinline__ int earlier_error(const int* err, int parity) {
+    const int word = *static_cast<volatile const int*>(err);
+    return parity ? word & ((1 << kErrShift) - 1) : word >> kErrShift;
+}
+
+// Whether the gather leaves the step out; the step after it sees that by this step's mark.
+template <typename R>
+__device__ __forceinline__ bool left_alone(const PhaseWork<R>& w, int failed) {
+    if (failed && threadIdx.x == 0) atomicOr(w.err, err_of_step(failed, w.parity));
+    return failed != 0;
 }
 
 // u planes, in the staging planes of the moments pass (4 nz nr doubles, idle during a step): u_z, u_r
@@ -196,7 +214,7 @@ __device__ __forceinline__ void phase_l2(const Params<R>& p, const PhaseWork<R>&
     int bad = 0;
     moments2<LINK, R>(f, la, drho, jz, jr);
     const T psi = psi2<MP>(p, drho, k + 1 < p.nz, bad);
-    if (failed) return;
+    if (left_alone(w, failed)) return;
     // the second lane of an odd row's last pair goes to the row's padding
     R* o = w.aux + (row * p.pitch + k);
     const int plane = (int)p.plane;
@@ -204,7 +222,7 @@ __device__ __forceinline__ void phase_l2(const Params<R>& p, const PhaseWork<R>&
     st2(o + plane, 0, jz);
     st2(o + 2 * plane, 0, jr);
     if (MP) st2(o + 3 * plane, 0, psi);
-    if (bad) atomicOr(w.err, bad);
+    if (bad) atomicOr(w.err, err_of_step(bad, w.parity));
 }
 
 // Tile plus 4 columns and rows of psi (F on the tile needs psi_rr, which needs psi_r on a 2-ring).
@@ -459,14 +477,14 @@ __device__ __forceinline__ void phase_l1(const Params<double>& p, const PhaseWor
         if (!nonnegative(arg)) bad |= ERRBIT_PSI;
         psi = sqrt3(arg);
     }
-    if (failed) return;
+    if (left_alone(w, failed)) return;
     const int plane = (int)p.plane;
     double* o = w.aux + (row * p.pitch + k);
     o[0] = drho;
     o[plane] = jz;
     o[2 * plane] = jr;
     if (MP) o[3 * plane] = psi;
-    if (bad) atomicOr(w.err, bad);
+    if (bad) atomicOr(w.err, err_of_step(bad, w.parity));
 }
 
 // psi with 4 columns and rows around the tile, the column sums of its stencils, and psi_z, psi_r with 2.
@@ -674,12 +692,11 @@ __device__ __forceinline__ void phase_c1(const Params<double>& p, const PhaseWor
 
 // =============================================================== kernels ==
 
-// failed: the solve's error word was set before the phase (its populations are void and it is left
-// alone).  Read with the phase's other loads and looked at before the stores, so that a step's own
-// error stops its later phases too.
+// failed: an earlier step raised an error (the populations are void and left alone).  Read with the
+// phase's other loads and looked at before the stores.
 template <typename R, int TR, bool MP, bool LINK>
 __device__ __forceinline__ void phase_l(const Params<R>& p, const PhaseWork<R>& w, const R* h) {
-    const int failed = *static_cast<volatile const int*>(w.err);
+    const int failed = earlier_error(w.err, w.parity);
     if constexpr (sizeof(R) == 4) {
         if (phase_inner(p, w.k0))
             phase_l2<TR, MP, LINK, false>(p, w, h, failed);
@@ -691,7 +708,7 @@ __device__ __forceinline__ void phase_l(const Params<R>& p, const PhaseWork<R>& 
 }
 template <typename R, int TR, bool MP, bool AX>
 __device__ __forceinline__ void phase_u(const Params<R>& p, const PhaseWork<R>& w) {
-    const int failed = *static_cast<volatile const int*>(w.err);
+    const int failed = earlier_error(w.err, w.parity);
     if constexpr (sizeof(R) == 4) {
         __shared__ __align__(16) R smem[PhaseU2<TR>::elems];
         if (phase_inner(p, w.k0))
@@ -711,7 +728,7 @@ __device__ __forceinline__ void phase_u(const Params<R>& p, const PhaseWork<R>& 
 }
 template <typename R, int TR, bool AX, int FV>
 __device__ __forceinline__ void phase_c(const Params<R>& p, const PhaseWork<R>& w, const R* hs, R* hd) {
-    const int failed = *static_cast<volatile const int*>(w.err);
+    const int failed = earlier_error(w.err, w.parity);
     if constexpr (sizeof(R) == 4) {
         if (phase_inner(p, w.k0))
             phase_c2<TR, AX, FV, false>(p, w, hs, hd, failed);

@@ -144,3 +144,48 @@ def test_guo_steps_alike_at_every_size(lbm, nz, nr):
         s.close()
     for a, b in zip(*got):
         assert np.array_equal(np.repeat(a[:, :1], nz, axis=1), b)
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("nz,nr,forcing", [(64, 48, 0), (512, 500, 0), (600, 450, 1), (1040, 800, 0)])
+@pytest.mark.parametrize("steps", [1, 2, 3, 4])
+def test_a_failed_solve_does_not_read_as_an_older_state(lbm, prec, nz, nr, forcing, steps):
+    """Both population buffers hold a sound run's states when a start with NaN nodes fails in its first step: whatever
+    the number of steps asked for, the solve's reads report the failure (tiles, phases, warps; FP64)."""
+    c = Case(nz, nr, T_over_Tc=0.9, forcing=forcing)
+    rho, uz, ur = _fields(c, 3)
+    s = c.solver(prec, c.coexistence()[1] if prec == 32 else 0.0).init(rho, uz, ur).step(2)
+    bad = rho.copy()
+    bad[::7, ::5] = np.nan
+    s.init(bad, uz, ur)
+    for call in (lambda: s.step(steps), s.moments, s.mass, s.moments):
+        with pytest.raises(lbm.LbmError) as e:
+            call()
+        assert e.value.code == lbm.ERR_UNPHYSICAL
+    s.init(rho, uz, ur).step(3)  # and starts afresh
+    t = c.solver(prec, c.coexistence()[1] if prec == 32 else 0.0).init(rho, uz, ur).step(3)
+    assert s.save() == t.save()
+    s.close()
+    t.close()
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+def test_a_solve_that_failed_in_a_batch_does_not_read_as_an_older_state(lbm, prec):
+    cases = [Case(400, 300, T_over_Tc=0.9), Case(500, 400, T_over_Tc=0.9)]  # by phases in FP32 too
+    fields = [_fields(c, i) for i, c in enumerate(cases)]
+    solvers = [c.solver(prec, c.coexistence()[1] if prec == 32 else 0.0).init(*f).step(2) for c, f in zip(cases, fields)]
+    bad = fields[0][0].copy()
+    bad[::7, ::5] = np.nan
+    solvers[0].init(bad, *fields[0][1:])
+    b = lbm.Batch(solvers)
+    for n in (1, 1, 3):
+        b.step_async(n)
+        assert b.sync() == lbm.ERR_UNPHYSICAL and b.status() == [lbm.ERR_UNPHYSICAL, lbm.OK]
+        with pytest.raises(lbm.LbmError) as e:
+            solvers[0].moments()
+        assert e.value.code == lbm.ERR_UNPHYSICAL
+    b.close()
+    t = cases[1].solver(prec, cases[1].coexistence()[1] if prec == 32 else 0.0).init(*fields[1]).step(7)
+    assert solvers[1].save() == t.save()
+    for s in solvers + [t]:
+        s.close()
