@@ -412,7 +412,7 @@ static cudaError_t fields64(const BatchSolve<double>& v, const LinkPlanes<double
                             int parity, const FieldsOut<double>& out, int* err, cudaStream_t s) {
     const int across = (v.p.nz + PhaseShape<double>::TZ - 1) / PhaseShape<double>::TZ;
     const unsigned grid = (unsigned)across * (unsigned)((v.p.nr + TR - 1) / TR);
-    const PhaseOne<double> a{v, lk.src, lk.dst, parity, across, err};
+    const PhaseOne<double> a{v, lk.src, lk.dst, parity, across, err, true};
     const bool mp = v.p.multiphase != 0, ax = v.p.axis != 0;
     cudaError_t e;
     if (mp)

@@ -55,6 +55,7 @@ struct PhaseOne {
     int parity;
     int across;  // tiles along z
     int* err;
+    bool read = false;  // the gather of a field read: of the state as it is, failed or not
 };
 template <typename R>
 struct PhaseMany {
@@ -695,8 +696,8 @@ __device__ __forceinline__ void phase_c1(const Params<double>& p, const PhaseWor
 // failed: an earlier step raised an error (the populations are void and left alone).  Read with the
 // phase's other loads and looked at before the stores.
 template <typename R, int TR, bool MP, bool LINK>
-__device__ __forceinline__ void phase_l(const Params<R>& p, const PhaseWork<R>& w, const R* h) {
-    const int failed = earlier_error(w.err, w.parity);
+__device__ __forceinline__ void phase_l(const Params<R>& p, const PhaseWork<R>& w, const R* h, bool read = false) {
+    const int failed = read ? 0 : earlier_error(w.err, w.parity);
     if constexpr (sizeof(R) == 4) {
         if (phase_inner(p, w.k0))
             phase_l2<TR, MP, LINK, false>(p, w, h, failed);
@@ -756,7 +757,7 @@ __device__ __forceinline__ void phase_c(const Params<R>& p, const PhaseWork<R>& 
 template <typename R, int TR, bool MP, bool LINK>
 __global__ void __launch_bounds__(32 * TR) k_phase_l(const PhaseOne<R> a) {
     LBM_PHASE_ONE(a);
-    phase_l<R, TR, MP, LINK>(p, w, a.h_src);
+    phase_l<R, TR, MP, LINK>(p, w, a.h_src, a.read);
 }
 template <typename R, int TR, bool MP, bool AX>
 __global__ void __launch_bounds__(32 * TR) k_phase_u(const PhaseOne<R> a) {

@@ -189,3 +189,29 @@ def test_a_solve_that_failed_in_a_batch_does_not_read_as_an_older_state(lbm, pre
     assert solvers[1].save() == t.save()
     for s in solvers + [t]:
         s.close()
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("steps", [1, 2, 3])
+def test_fields_of_a_failed_solve_are_its_own(lbm, prec, steps):
+    """The first read after steps that nobody waited for gives the fields of the failed state, as the next one does."""
+    import torch
+
+    c = Case(130, 90, T_over_Tc=0.9)
+    rho, uz, ur = _fields(c, 3)
+    s = c.solver(prec, c.coexistence()[1] if prec == 32 else 0.0).init(rho, uz, ur).step(2)
+    bad = rho.copy()
+    bad[5, 7] = np.nan
+    s.init(bad, uz, ur)
+    lbm.lbm_axi_step_async(s.h, steps)
+    got = []
+    for _ in range(2):
+        out = torch.full((4, c.nr, c.nz), -1.0, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        with pytest.raises(lbm.LbmError) as e:
+            lbm.lbm_axi_moments_device(s.h, rho=out[0], u_z=out[1], u_r=out[2], p=out[3])
+        assert e.value.code == lbm.ERR_UNPHYSICAL
+        got.append(out.cpu().numpy())
+    assert not np.isnan(got[0][0][60:, 60:]).any()
+    np.testing.assert_array_equal(got[0], got[1])
+    s.close()
