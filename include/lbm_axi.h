@@ -178,7 +178,8 @@ int lbm_axi_init_physical_device(lbm_axi* h, const double* d_rho, const double* 
 int lbm_axi_step(lbm_axi* h, long long n);
 
 /* As lbm_axi_step, but only enqueues the work on the handle's stream; the
- * error status of the enqueued steps is returned by the next lbm_axi_sync. */
+ * error status of the enqueued steps is returned by the next lbm_axi_sync.
+ * A caller that captures the stream gets the steps' launches in its graph. */
 int lbm_axi_step_async(lbm_axi* h, long long n);
 
 /* Wait for the handle's stream; return the sticky error status of the steps

@@ -180,6 +180,12 @@ int chunk_steps(const lbm_axi* h) {
     return (int)(c & ~1LL);
 }
 
+// The caller is capturing the stream: steps go into that graph one by one.
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
 int read_error(lbm_axi* h) {
     // one launch that writes the pinned word and clears the device's (a copy and a memset take twice as long)
     if (Ops<float>::take_error(h->derr, h->herr, h->stream) != cudaSuccess) return LBM_ERR_CUDA;
@@ -489,7 +495,7 @@ int lbm_axi_step_async(lbm_axi* h, long long n) {
         n--;
     }
     const int chunk = chunk_steps(h);
-    if (e == cudaSuccess && n >= chunk) {
+    if (e == cudaSuccess && n >= chunk && !capturing(h->stream)) {
         if (!h->graph || h->graph_steps != chunk) {
             int rc = build_graph(h, chunk);
             if (rc != LBM_OK) return rc;

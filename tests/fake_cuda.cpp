@@ -21,6 +21,7 @@ std::map<uintptr_t, size_t>* live = nullptr;  // device allocations
 long long device_left = -1, host_left = -1;   // allocations until one fails (-1: none does)
 int launches = 0, violations = 0;
 bool track = false;
+cudaStream_t captured = nullptr;  // a stream that its owner is capturing
 
 bool inside(const void* p, size_t bytes) {
     auto it = live->upper_bound((uintptr_t)p);
@@ -88,14 +89,22 @@ cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = (cudaStream_t)malloc(1), cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { return free((void*)s), cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
+    return s == fake::captured ? cudaErrorIllegalState : cudaSuccess;
+}
+cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
+    *st = s == fake::captured ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { return *g = (cudaGraph_t)malloc(1), cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) {
     return *x = (cudaGraphExec_t)malloc(1), cudaSuccess;
 }
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { return free((void*)g), cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { return free((void*)x), cudaSuccess; }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t s) {
+    return s == fake::captured ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+}
 }
 
 // --------------------------------------------------------------- launchers --
@@ -262,6 +271,24 @@ static void batch_retune(int nz, int nr, int n, int precision, bool device) {
     CHECK(fake::live->empty());
 }
 
+// Steps enqueued while the caller captures the solve's stream: one launch each, whatever their number, before
+// and after the solve has built a graph of its own.
+static void step_under_capture(int precision) {
+    cudaStream_t s = (cudaStream_t)malloc(1);
+    lbm_axi* h = solve(64, 64, precision, s);
+    for (int round = 0; round < 2; round++) {
+        for (int n : {1, 31, 32, 64, 200, 255, 256, 400}) {
+            fake::captured = s;
+            fake::launches = 0;
+            CHECK(lbm_axi_step_async(h, n) == LBM_OK && fake::launches == n);
+            fake::captured = nullptr;
+        }
+        CHECK(lbm_axi_step_async(h, 600) == LBM_OK);
+    }
+    lbm_axi_destroy(h);
+    free((void*)s);
+}
+
 int main(int argc, char** argv) {
     fake::live = new std::map<uintptr_t, size_t>();
     const char* what = argc > 1 ? argv[1] : "";
@@ -270,6 +297,8 @@ int main(int argc, char** argv) {
     if (!strcmp(what, "retune_host_two_tables")) return batch_retune(64, 48, 280, 32, false), 0;
     if (!strcmp(what, "retune_device_phases")) return batch_retune(100, 40, 3, 32, true), 0;
     if (!strcmp(what, "retune_host_fp64")) return batch_retune(100, 40, 3, 64, false), 0;
+    if (!strcmp(what, "capture32")) return step_under_capture(32), 0;
+    if (!strcmp(what, "capture64")) return step_under_capture(64), 0;
     fprintf(stderr, "unknown check %s\n", what);
     return 2;
 }

@@ -215,3 +215,26 @@ def test_fields_of_a_failed_solve_are_its_own(lbm, prec, steps):
     assert not np.isnan(got[0][0][60:, 60:]).any()
     np.testing.assert_array_equal(got[0], got[1])
     s.close()
+
+
+@pytest.mark.parametrize("prec,nz,nr", [(32, 64, 64), (64, 64, 64), (32, 512, 500)])
+@pytest.mark.parametrize("steps", [20, 100])
+def test_steps_captured_by_the_caller(lbm, prec, nz, nr, steps):
+    """A caller's graph of a solve's steps, more and fewer than the solve's own graphs hold: the same bits."""
+    import torch
+
+    c = Case(nz, nr, T_over_Tc=0.9)
+    fields, ref = _fields(c, 4), c.coexistence()[1] if prec == 32 else 0.0
+    want = c.solver(prec, ref).init(*fields).step(steps)
+    stream = torch.cuda.Stream()
+    o = lbm.Solver(nz, nr, c.tau, eos=lbm.make_eos(c.eos, c.T_over_Tc), A=c.A, precision=prec, rho_ref=ref,
+                   stream=stream.cuda_stream).init(*fields)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        lbm.lbm_axi_step_async(o.h, steps)
+    with torch.cuda.stream(stream):
+        g.replay()
+    assert o.save() == want.save()
+    del g
+    o.close()
+    want.close()

@@ -1,6 +1,6 @@
 """The host code of the library (csrc/lbm_axi.cu, csrc/lbm_batch.cu) driven on
 the CPU over a CUDA runtime that only keeps books (tests/fake_cuda.cpp): what it
-launches after an allocation has failed."""
+launches after an allocation has failed or under a caller's stream capture."""
 import os
 import subprocess
 
@@ -31,4 +31,9 @@ def _run(program, what):
 @pytest.mark.parametrize("what", ["retune_device_warps", "retune_host_warps", "retune_host_two_tables",
                                   "retune_device_phases", "retune_host_fp64"])
 def test_batch_keeps_its_plan_when_a_new_one_fails(program, what):
+    _run(program, what)
+
+
+@pytest.mark.parametrize("what", ["capture32", "capture64"])
+def test_steps_can_be_captured(program, what):
     _run(program, what)
