@@ -1,5 +1,6 @@
 // C ABI of the engine (include/lbm_axi.h): handle lifetime, device memory,
 // the step loop (replayed as CUDA-graph chunks), moments and FP64 reductions.
+#include <cuda.h>
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
@@ -210,14 +211,37 @@ cudaError_t enqueue_init(lbm_axi* h, const double* rho, const double* uz, const 
                              static_cast<const double*>(phys), h->derr);
 }
 
-// Memory of this device that a kernel may write as doubles (a copy takes any address).
-bool writable_on(const void* p, int device) {
+// The allocation that a device address lies in (false: not known).
+bool allocation_of(const void* p, uintptr_t* base, size_t* size) {
+    using F = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const F range = [] {  // from the driver: the runtime has no call for it
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        if (!ok) cudaGetLastError();
+        return ok ? reinterpret_cast<F>(f) : nullptr;
+    }();
+    CUdeviceptr b = 0;
+    if (!range || range(&b, size, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
+    *base = static_cast<uintptr_t>(b);
+    return true;
+}
+
+// n doubles of this device's memory that a kernel may write: all of them in one allocation, as a copy would
+// check (and a copy takes any address).
+bool writable_on(const void* p, size_t n, int device) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return a.type == cudaMemoryTypeDevice && a.device == device && reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    if (a.type != cudaMemoryTypeDevice || a.device != device || at % sizeof(double) != 0) return false;
+    uintptr_t base = 0;
+    size_t size = 0;
+    return allocation_of(p, &base, &size) && at - base <= size && size - (at - base) >= n * sizeof(double);
 }
 
 struct DeviceGuard {
@@ -585,7 +609,7 @@ int lbm_axi_moments_device(lbm_axi* h, double* rho, double* uz, double* ur, doub
     double* dst[4] = {rho, uz, ur, p};
     double* to[4];
     for (int q = 0; q < 4; q++)
-        to[q] = !dst[q] || writable_on(dst[q], h->device) ? dst[q] : h->mout + q * n;
+        to[q] = !dst[q] || writable_on(dst[q], n, h->device) ? dst[q] : h->mout + q * n;
     cudaError_t e = enqueue_fields(h, to[0], to[1], to[2], to[3], nullptr);
     for (int q = 0; q < 4 && e == cudaSuccess; q++) {
         if (dst[q] && to[q] != dst[q])

@@ -2,6 +2,7 @@
 // lbm_batch.cu) can be driven on the CPU through failures that a GPU must not be driven through: an
 // allocation that fails, a launch on a list that is gone.  Device memory is host memory; a launch checks
 // that the lists it is given lie in live allocations.  One program, one check per argument.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdio.h>
@@ -21,6 +22,7 @@ std::map<uintptr_t, size_t>* live = nullptr;  // device allocations
 long long device_left = -1, host_left = -1;   // allocations until one fails (-1: none does)
 int launches = 0, violations = 0;
 bool track = false;
+const void* last_rho = nullptr;   // where the last read wrote its density
 cudaStream_t captured = nullptr;  // a stream that its owner is capturing
 
 bool inside(const void* p, size_t bytes) {
@@ -69,7 +71,23 @@ cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return memcpy(d, s, n), cudaSuccess; }
+static CUresult address_range(CUdeviceptr* base, size_t* size, CUdeviceptr p) {
+    auto it = fake::live->upper_bound(p);
+    if (it == fake::live->begin()) return CUDA_ERROR_NOT_FOUND;
+    --it;
+    *base = it->first, *size = it->second;
+    return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult* q) {
+    const bool known = !strcmp(name, "cuMemGetAddressRange");
+    *f = known ? (void*)address_range : nullptr;
+    *q = known ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+    return cudaSuccess;
+}
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    // to an address in device memory: refused unless it all fits
+    if (fake::inside(d, 1) && !fake::inside(d, n)) return cudaErrorInvalidValue;
     return memcpy(d, s, n), cudaSuccess;
 }
 cudaError_t cudaMemcpy2DAsync(void*, size_t, const void*, size_t, size_t, size_t, cudaMemcpyKind, cudaStream_t) {
@@ -121,8 +139,11 @@ cudaError_t Ops<R>::update(const Params<R>&, const R*, R*, const R*, cudaStream_
     return cudaSuccess;
 }
 template <typename R>
-cudaError_t Ops<R>::fields(const BatchSolve<R>&, LinkPlanes<R>, const Params<double>&, int, double*, double*, double*,
-                           double*, R*, int*, cudaStream_t) {
+cudaError_t Ops<R>::fields(const BatchSolve<R>& v, LinkPlanes<R>, const Params<double>&, int, double* rho, double* uz,
+                           double* ur, double* pk, R*, int*, cudaStream_t) {
+    for (double* q : {rho, uz, ur, pk})
+        if (q && !fake::inside(q, (size_t)v.p.nz * v.p.nr * sizeof(double))) fake::violations++;
+    fake::last_rho = rho;
     return cudaSuccess;
 }
 template <typename R>
@@ -289,6 +310,26 @@ static void step_under_capture(int precision) {
     free((void*)s);
 }
 
+// Fields wanted in device memory that is too short for them: refused, as the copy that checks it does, and no
+// kernel is given the address.  Memory that fits, from its start or within, is written directly.
+static void moments_to_short_memory(int precision) {
+    const int nz = 37, nr = 18, n = nz * nr;
+    lbm_axi* h = solve(nz, nr, precision);
+    double* d;
+    cudaMalloc((void**)&d, (2 * n + 1) * sizeof(double));
+    for (int at : {0, 1, n, n + 1}) {
+        CHECK(lbm_axi_moments_device(h, d + at, nullptr, nullptr, nullptr) == LBM_OK && fake::last_rho == d + at);
+        CHECK(fake::violations == 0);
+    }
+    for (int at : {n + 2, 2 * n}) {
+        CHECK(lbm_axi_moments_device(h, d + at, nullptr, nullptr, nullptr) == LBM_ERR_CUDA);
+        CHECK(lbm_axi_moments_device(h, nullptr, d, nullptr, d + at) == LBM_ERR_CUDA);
+        CHECK(fake::violations == 0);
+    }
+    cudaFree(d);
+    lbm_axi_destroy(h);
+}
+
 int main(int argc, char** argv) {
     fake::live = new std::map<uintptr_t, size_t>();
     const char* what = argc > 1 ? argv[1] : "";
@@ -299,6 +340,8 @@ int main(int argc, char** argv) {
     if (!strcmp(what, "retune_host_fp64")) return batch_retune(100, 40, 3, 64, false), 0;
     if (!strcmp(what, "capture32")) return step_under_capture(32), 0;
     if (!strcmp(what, "capture64")) return step_under_capture(64), 0;
+    if (!strcmp(what, "short32")) return moments_to_short_memory(32), 0;
+    if (!strcmp(what, "short64")) return moments_to_short_memory(64), 0;
     fprintf(stderr, "unknown check %s\n", what);
     return 2;
 }

@@ -1,6 +1,7 @@
 """The host code of the library (csrc/lbm_axi.cu, csrc/lbm_batch.cu) driven on
 the CPU over a CUDA runtime that only keeps books (tests/fake_cuda.cpp): what it
-launches after an allocation has failed or under a caller's stream capture."""
+launches after an allocation has failed, under a caller's stream capture, and
+on device memory that is too short."""
 import os
 import subprocess
 
@@ -36,4 +37,9 @@ def test_batch_keeps_its_plan_when_a_new_one_fails(program, what):
 
 @pytest.mark.parametrize("what", ["capture32", "capture64"])
 def test_steps_can_be_captured(program, what):
+    _run(program, what)
+
+
+@pytest.mark.parametrize("what", ["short32", "short64"])
+def test_fields_are_not_written_past_an_allocation(program, what):
     _run(program, what)
