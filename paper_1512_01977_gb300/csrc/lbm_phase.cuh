@@ -393,16 +393,19 @@ __device__ __forceinline__ double rcp3(double x) {
     const double e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
 }
-// sqrt(x), 0 for x <= 0: s = x y with y the approximate inverse root, e = 1 - s y,
-// s (1 + e/2 + 3 e^2/8), the series of (1 - e)^(-1/2).  The sign, zero and
-// subnormal cases go by the bits (an FP64 comparison costs as much as two operations).
+// sqrt(x), 0 for x <= 0: with y the approximate inverse root and s = x y, the root is s + r / (2 s) (1 - r /
+// (4 s^2)) for the remainder r = x - s^2, and with e = 1 - s y that is s + r (y/2) (1 + 3 e/4), 6 operations:
+// correctly rounded but for 6 roots in 10,000.  (The series of (1 - e)^(-1/2) alone, 5 operations, keeps half of
+// the rounding of s: a unit off in one root of eight.)  The sign, zero and subnormal cases go by the bits (an FP64
+// comparison costs as much as two operations).
 __device__ __forceinline__ double sqrt3(double x) {
     const int hi = __double2hiint(x);
     if (hi < 0x00100000) return hi < 0 ? 0.0 : sqrt(x);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double s = x * y, e = fma(-s, y, 1.0);
-    return fma(s * e, fma(e, 0.375, 0.5), s);
+    const double s = x * y, e = fma(-s, y, 1.0), r = fma(-s, s, x);
+    const double half_y = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
+    return fma(r * half_y, fma(0.75, e, 1.0), s);
 }
 // x > 0 and x >= 0 (NaN: false), by the bits.
 __device__ __forceinline__ bool positive(double x) {
