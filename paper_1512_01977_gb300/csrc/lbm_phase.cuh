@@ -386,8 +386,11 @@ __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, 
 
 // 1/x: the hardware's approximation y (relative error e below 2^-19.9) and one
 // third-order step, y (1 + e + e^2) with e = 1 - x y: within 1 ulp of the
-// quotient, 3 operations where a division takes the time of 17.
+// quotient, 3 operations where a division takes the time of 17.  Zeros, subnormal values and results, infinities
+// and NaN are left to the division.
 __device__ __forceinline__ double rcp3(double x) {
+    // by the bits: |x| in [2^-1022, 2^1020)
+    if ((unsigned)(__double2hiint(x) & 0x7fffffff) - 0x00100000u >= 0x7fa00000u) return 1.0 / x;
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x, y, 1.0);
@@ -396,11 +399,12 @@ __device__ __forceinline__ double rcp3(double x) {
 // sqrt(x), 0 for x <= 0: with y the approximate inverse root and s = x y, the root is s + r / (2 s) (1 - r /
 // (4 s^2)) for the remainder r = x - s^2, and with e = 1 - s y that is s + r (y/2) (1 + 3 e/4), 6 operations:
 // correctly rounded but for 6 roots in 10,000.  (The series of (1 - e)^(-1/2) alone, 5 operations, keeps half of
-// the rounding of s: a unit off in one root of eight.)  The sign, zero and subnormal cases go by the bits (an FP64
-// comparison costs as much as two operations).
+// the rounding of s: a unit off in one root of eight.)  Zeros, negative,
+// tiny and non-finite values are told by the bits (an FP64 comparison costs as much as two operations).
 __device__ __forceinline__ double sqrt3(double x) {
     const int hi = __double2hiint(x);
-    if (hi < 0x00100000) return hi < 0 ? 0.0 : sqrt(x);
+    // below 2^-959 the remainder would lose digits
+    if ((unsigned)hi - 0x04000000u >= 0x7ff00000u - 0x04000000u) return x > 0.0 ? sqrt(x) : 0.0;
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double s = x * y, e = fma(-s, y, 1.0), r = fma(-s, s, x);

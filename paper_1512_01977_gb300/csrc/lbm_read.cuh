@@ -34,7 +34,8 @@ __device__ __forceinline__ double pressure(const Params<double>& p, double rho) 
         return finite1(rho) ? fma(fma(-3.0, q, rho), 1.0 / 3.0, q) : q;
     }
     if (p.eos == EOS_VDW) {
-        const double d = 3.0 - rho, r = rcp3(d), n = 8.0 * p.T * rho, q0 = mul(n, r), q = fma(fma(-d, q0, n), r, q0);
+        const double d = 3.0 - rho, r = rcp3(d), n = 8.0 * p.T * rho, q0 = mul(n, r);
+        const double q = finite1(q0) ? fma(fma(-d, q0, n), r, q0) : q0;
         return mul(p.lambda, fma(-3.0 * rho, rho, q));
     }
     const double r = rcp3(fma(-0.25 * p.b, rho, 1.0)), r2 = mul(r, r), RT = p.Rg * p.T;

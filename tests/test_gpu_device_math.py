@@ -48,3 +48,16 @@ def test_rounding(rcp_sqrt, lo, hi):
     for got, want in ((r, 1.0 / x), (s, np.sqrt(x))):
         assert np.all(np.abs(got - want) <= np.spacing(want))
         assert np.mean(got != want) <= 0.024
+
+
+def test_special_values(rcp_sqrt):
+    """What the division and the root give for zeros, subnormal values and results, infinities and NaN (the root: 0 for
+    what is not positive)."""
+    tiny, big = np.finfo(float).tiny, np.finfo(float).max
+    x = np.array([0.0, np.inf, np.nan, 5e-324, 1e-310, np.nextafter(tiny, 0), tiny, np.nextafter(tiny, 1), 2.0 ** 1021,
+                  np.nextafter(2.0 ** 1021, 0), 2.0 ** 1022, 1.5 * 2.0 ** 1022, 2.0 ** 1023, big])
+    x = np.concatenate([x, -x])
+    r, s = rcp_sqrt(x)
+    with np.errstate(all="ignore"):
+        np.testing.assert_array_equal(r, 1.0 / x)
+        np.testing.assert_array_equal(s, np.where(x > 0, np.sqrt(x), 0.0))

@@ -276,3 +276,24 @@ def test_pressure_of_a_single_phase_run(lbm, prec):
     m = s.moments()
     s.close()
     np.testing.assert_array_equal(m["p"], m["rho"] / 3.0)
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("eos,pole", [(O.EOS_CS, 1.0), (O.EOS_VDW, 3.0)])
+def test_pressure_at_the_pole_of_the_eos(lbm, prec, eos, pole):
+    """A state at the EOS's largest density fails, and its P_k reads as the infinity that the formula gives there."""
+    import torch
+
+    c = Case(40, 24, T_over_Tc=0.9, eos=eos)
+    rho = np.full((c.nr, c.nz), c.coexistence()[1])
+    rho[3, 5] = pole
+    s = c.solver(prec, pole if prec == 32 else 0.0).init(rho)  # FP32: a deviation of 0 there
+    out = torch.zeros((2, c.nr, c.nz), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    with pytest.raises(lbm.LbmError) as e:
+        lbm.lbm_axi_moments_device(s.h, rho=out[0], p=out[1])
+    assert e.value.code == lbm.ERR_UNPHYSICAL
+    got = out.cpu().numpy()
+    s.close()
+    at = got[0] == pole
+    assert at[3, 5] and np.all(got[1][at] == np.inf) and np.all(np.isfinite(got[1][~at]))
