@@ -366,9 +366,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     const bool link = o.h_eval == LBM_H_LINK_AVG && o.axis_terms, ctas = link || guo_of(h);
     std::vector<lbm::Tile> tiles;
     std::vector<int> first;
-    if (lbm_by_phases(o.precision, (long long)nz * nr)) {
-        first.assign(1, 0);
-    } else {
+    if (!lbm_by_phases(o.precision, (long long)nz * nr)) {
         const int slots = ctas ? Ops<float>::batch_resident_ctas(lbm::kStripWide) : Ops<float>::warp_slots();
         int rc = LBM_ERR_CUDA;
         try {
@@ -376,7 +374,6 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
                 rc = slots > 0 ? lbm::plan_tiles(&nz, &nr, 1, lbm::kStripWide, slots, tiles, first, nullptr) : rc;
             else
                 rc = slots > 0 ? lbm::plan_warp_tiles(&nz, &nr, 1, slots, tiles) : rc;
-            if (!ctas) first.assign(1, 0);
         } catch (...) {
             rc = LBM_ERR_OOM;
         }
@@ -386,7 +383,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
             return rc;
         }
     }
-    h->ncta = ctas ? (int)first.size() - 1 : (int)tiles.size();
+    h->ncta = first.empty() ? (int)tiles.size() : (int)first.size() - 1;
     h->d_tiles = (lbm::Tile*)dev_alloc(tiles.size() * sizeof(lbm::Tile));
     h->d_first = (int*)dev_alloc(first.size() * sizeof(int));
     h->bytes = lbm_axi_footprint(nz, nr, o.precision);
@@ -427,7 +424,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     cudaError_t err = cudaSuccess;
     if (!tiles.empty()) {
         err = cudaMemcpy(h->d_tiles, tiles.data(), tiles.size() * sizeof(lbm::Tile), cudaMemcpyHostToDevice);
-        if (err == cudaSuccess)
+        if (err == cudaSuccess && !first.empty())
             err = cudaMemcpy(h->d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice);
     }
     if (err == cudaSuccess) err = cudaMemsetAsync(h->derr, 0, sizeof(int), h->stream);

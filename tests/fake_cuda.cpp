@@ -25,6 +25,12 @@ bool track = false;
 const void* last_rho = nullptr;   // where the last read wrote its density
 cudaStream_t captured = nullptr;  // a stream that its owner is capturing
 
+struct Untracked {  // the runtime's own bookkeeping does not count
+    const bool was = track;
+    Untracked() { track = false; }
+    ~Untracked() { track = was; }
+};
+
 bool inside(const void* p, size_t bytes) {
     auto it = live->upper_bound((uintptr_t)p);
     if (it == live->begin()) return false;
@@ -55,6 +61,7 @@ void operator delete(void* p, size_t) noexcept { free(p); }
 extern "C" {
 cudaError_t cudaMalloc(void** p, size_t n) {
     if (fake::device_left >= 0 && fake::device_left-- == 0) return cudaErrorMemoryAllocation;
+    fake::Untracked u;
     *p = malloc(n);
     (*fake::live)[(uintptr_t)*p] = n;
     return cudaSuccess;
@@ -330,6 +337,32 @@ static void moments_to_short_memory(int precision) {
     lbm_axi_destroy(h);
 }
 
+// A solve whose creation runs out of device or host memory, at any of its allocations: an error code, and nothing
+// stays allocated.
+static void create_out_of_memory(int nz, int nr, int precision, int forcing) {
+    lbm_axi_opts o;
+    lbm_axi_default_opts(&o);
+    o.precision = precision;
+    o.forcing = forcing;
+    lbm_eos e = {LBM_EOS_CS, 0.9, 1.0, 4.0, 1.0, 0.01};
+    for (bool device : {true, false})
+        for (int at = 0;; at++) {
+            lbm_axi* h = nullptr;
+            (device ? fake::device_left : fake::host_left) = at;
+            fake::track = true;
+            const int rc = lbm_axi_create(nz, nr, 1.0, &e, -0.152, &o, &h);
+            fake::track = false;
+            fake::device_left = fake::host_left = -1;
+            if (rc == LBM_OK) {
+                CHECK(h && at > 0);
+                lbm_axi_destroy(h);
+                CHECK(fake::live->empty());
+                break;
+            }
+            CHECK(rc == LBM_ERR_OOM && !h && fake::live->empty());
+        }
+}
+
 int main(int argc, char** argv) {
     fake::live = new std::map<uintptr_t, size_t>();
     const char* what = argc > 1 ? argv[1] : "";
@@ -342,6 +375,10 @@ int main(int argc, char** argv) {
     if (!strcmp(what, "capture64")) return step_under_capture(64), 0;
     if (!strcmp(what, "short32")) return moments_to_short_memory(32), 0;
     if (!strcmp(what, "short64")) return moments_to_short_memory(64), 0;
+    if (!strcmp(what, "create_phases")) return create_out_of_memory(64, 64, 32, 0), 0;
+    if (!strcmp(what, "create_fp64")) return create_out_of_memory(64, 64, 64, 0), 0;
+    if (!strcmp(what, "create_warps")) return create_out_of_memory(1040, 800, 32, 0), 0;
+    if (!strcmp(what, "create_ctas")) return create_out_of_memory(1040, 800, 32, 1), 0;
     fprintf(stderr, "unknown check %s\n", what);
     return 2;
 }

@@ -43,3 +43,8 @@ def test_steps_can_be_captured(program, what):
 @pytest.mark.parametrize("what", ["short32", "short64"])
 def test_fields_are_not_written_past_an_allocation(program, what):
     _run(program, what)
+
+
+@pytest.mark.parametrize("what", ["create_phases", "create_fp64", "create_warps", "create_ctas"])
+def test_creation_reports_that_memory_ran_out(program, what):
+    _run(program, what)
