@@ -26,19 +26,19 @@ One one(const Params<float>& p, bool mp, bool ax) {
     return ax ? k_step_warp<false, true, WARP_CS> : k_step_warp<false, false, WARP_CS>;
 }
 
-using Many = void (*)(const BatchTable<float>, const Tile*, int, int*);
+using Many = void (*)(const BatchSolve<float>*, const Tile*, int, int*);
 Many many(int kind, bool mp, bool ax) {
     if (mp && ax) {
         switch (kind) {
-            case WARP_CS: return k_step_warp_table<true, true, WARP_CS>;
-            case WARP_CS_LATTICE: return k_step_warp_table<true, true, WARP_CS_LATTICE>;
-            case WARP_VDW: return k_step_warp_table<true, true, WARP_VDW>;
-            case WARP_VDW_LATTICE: return k_step_warp_table<true, true, WARP_VDW_LATTICE>;
-            default: return k_step_warp_table<true, true, WARP_MIXED>;
+            case WARP_CS: return k_step_warp_many<true, true, WARP_CS>;
+            case WARP_CS_LATTICE: return k_step_warp_many<true, true, WARP_CS_LATTICE>;
+            case WARP_VDW: return k_step_warp_many<true, true, WARP_VDW>;
+            case WARP_VDW_LATTICE: return k_step_warp_many<true, true, WARP_VDW_LATTICE>;
+            default: return k_step_warp_many<true, true, WARP_MIXED>;
         }
     }
-    if (mp) return k_step_warp_table<true, false, WARP_MIXED>;
-    return ax ? k_step_warp_table<false, true, WARP_CS> : k_step_warp_table<false, false, WARP_CS>;
+    if (mp) return k_step_warp_many<true, false, WARP_MIXED>;
+    return ax ? k_step_warp_many<false, true, WARP_CS> : k_step_warp_many<false, false, WARP_CS>;
 }
 
 }  // namespace
@@ -64,13 +64,19 @@ cudaError_t Ops<float>::step_warp(const BatchSolve<float>& v, const Tile* tiles,
 }
 
 template <>
-cudaError_t Ops<float>::step_warp_table(const BatchTable<float>& tab, int n, const Tile* tiles, int ntiles, bool mp,
-                                        bool ax, int parity, int* err, cudaStream_t s) {
-    if (ntiles <= 0 || n < 1) return cudaErrorInvalidConfiguration;
-    int kind = kind_of(tab.s[0].p);
-    for (int i = 1; i < n; i++)
-        if (kind_of(tab.s[i].p) != kind) kind = WARP_MIXED;
-    many(kind, mp, ax)<<<ntiles, 32, 0, s>>>(tab, tiles, parity, err);
+int Ops<float>::warp_kind(const Params<float>& p) {
+    return kind_of(p);
+}
+template <>
+int Ops<float>::warp_kind(int a, int b) {
+    return a == b ? a : (int)WARP_MIXED;
+}
+
+template <>
+cudaError_t Ops<float>::step_warp_many(const BatchSolve<float>* solves, int kind, const Tile* tiles, int ntiles, bool mp,
+                                       bool ax, int parity, int* err, cudaStream_t s) {
+    if (ntiles <= 0) return cudaErrorInvalidConfiguration;
+    many(kind, mp, ax)<<<ntiles, 32, 0, s>>>(solves, tiles, parity, err);
     return cudaGetLastError();
 }
 

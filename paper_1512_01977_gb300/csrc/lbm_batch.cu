@@ -2,7 +2,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <memory>
 #include <new>
 #include <utility>
 #include <vector>
@@ -18,23 +17,17 @@ using lbm::Ops;
 // the marching kernel of the chosen strip width and CTA slots (lbm_step.cuh).
 enum BatchForm { FORM_TILES, FORM_PHASES, FORM_WARPS, FORM_MARCH };
 
-// The warp march of solves [s0, ...): their descriptors (a kernel argument) and tiles [t0, t0 + nt).
-struct WarpGroup {
-    lbm::BatchTable<float> table;
-    int s0, ns, t0, nt;
-};
-
 // The form of one (strip, grid) and the work lists it launches over.
 struct StepPlan {
     int strip = lbm::kStripWide, grid = 0;
     BatchForm form = FORM_MARCH;
     lbm::TileForm tile = lbm::TILE_NONE;
-    std::vector<std::unique_ptr<WarpGroup>> groups;
     lbm::PhaseTile* d_ptiles = nullptr;
     int nptiles = 0, nghost = 0, prows = 0;
     lbm::Tile* d_tiles = nullptr;  // tile plan for (strip, grid)
     int* d_first = nullptr;        // [ncta + 1]
-    int ncta = 0;
+    int ncta = 0, ntiles = 0;
+    int kind = 0;  // of the warp march
 };
 
 struct lbm_axi_batch {
@@ -81,11 +74,6 @@ const Params<double>& params_of<double>(const lbm_axi* h) {
     return h->pdd;
 }
 
-template <typename R>
-BatchSolve<R> descriptor(const lbm_axi_batch* b, int i) {
-    return lbm_handle_solve<R>(b->solves[i], params_of<R>(b->solves[i]), b->cur0[i]);
-}
-
 // FP64 steps by phases at every tuning; FP32 at the default one (wide strips, grid
 // 0) by tiles or phases while the batch is small and by warps beyond, at the others by march2.
 BatchForm form_of(const lbm_axi_batch* b, const StepPlan& p, long long nodes) {
@@ -106,7 +94,7 @@ void release(StepPlan& p) {
 template <typename R>
 cudaError_t upload_solves(lbm_axi_batch* b) {
     std::vector<BatchSolve<R>> hs(b->n);
-    for (int i = 0; i < b->n; i++) hs[i] = descriptor<R>(b, i);
+    for (int i = 0; i < b->n; i++) hs[i] = lbm_handle_solve<R>(b->solves[i], params_of<R>(b->solves[i]), b->cur0[i]);
     if constexpr (sizeof(R) == 4) {
         if (b->h_table)
             for (int i = 0; i < b->n; i++) b->h_table->s[i] = hs[i];
@@ -147,21 +135,9 @@ cudaError_t make_plan(const lbm_axi_batch* b, StepPlan& p) {
     } else if (p.form == FORM_WARPS) {
         const int slots = Ops<float>::warp_slots();
         if (slots <= 0) return cudaErrorInvalidConfiguration;
-        std::vector<lbm::Tile> part;
-        for (int s0 = 0; s0 < b->n; s0 += lbm::BatchTable<float>::N) {
-            const int ns = std::min(b->n - s0, (int)lbm::BatchTable<float>::N);
-            if (lbm::plan_warp_tiles(nz.data() + s0, nr.data() + s0, ns, slots, part) != LBM_OK)
-                return cudaErrorMemoryAllocation;
-            auto g = std::make_unique<WarpGroup>();
-            if constexpr (sizeof(R) == 4)
-                for (int i = 0; i < ns; i++) g->table.s[i] = descriptor<R>(b, s0 + i);
-            g->s0 = s0;
-            g->ns = ns;
-            g->t0 = (int)tiles.size();
-            g->nt = (int)part.size();
-            p.groups.push_back(std::move(g));
-            tiles.insert(tiles.end(), part.begin(), part.end());
-        }
+        if (lbm::plan_warp_tiles(nz.data(), nr.data(), b->n, slots, tiles) != LBM_OK) return cudaErrorMemoryAllocation;
+        p.kind = Ops<float>::warp_kind(b->solves[0]->pf);
+        for (int i = 1; i < b->n; i++) p.kind = Ops<float>::warp_kind(p.kind, Ops<float>::warp_kind(b->solves[i]->pf));
     } else {
         const int slots = p.grid > 0 ? p.grid : Ops<R>::batch_resident_ctas(p.strip);
         if (slots <= 0) return cudaErrorInvalidConfiguration;
@@ -182,6 +158,7 @@ cudaError_t make_plan(const lbm_axi_batch* b, StepPlan& p) {
     p.nptiles = (int)inner;
     p.nghost = (int)(ptiles.size() - inner);
     p.ncta = first.empty() ? 0 : (int)first.size() - 1;
+    p.ntiles = (int)tiles.size();
     return cudaSuccess;
 }
 
@@ -214,15 +191,8 @@ cudaError_t launch(lbm_axi_batch* b, int parity) {
         return Ops<double>::phase_step_many(static_cast<const BatchSolve<double>*>(b->d_solves), p.d_ptiles, p.nptiles,
                                             p.nghost, p.prows, b->mp, b->ax, parity, b->d_err, b->stream);
     const BatchSolve<float>* solves = static_cast<const BatchSolve<float>*>(b->d_solves);
-    if (p.form == FORM_WARPS) {
-        cudaError_t e = cudaSuccess;
-        for (size_t i = 0; i < p.groups.size() && e == cudaSuccess; i++) {
-            const WarpGroup& g = *p.groups[i];
-            e = Ops<float>::step_warp_table(g.table, g.ns, p.d_tiles + g.t0, g.nt, b->mp, b->ax, parity, b->d_err + g.s0,
-                                            b->stream);
-        }
-        return e;
-    }
+    if (p.form == FORM_WARPS)
+        return Ops<float>::step_warp_many(solves, p.kind, p.d_tiles, p.ntiles, b->mp, b->ax, parity, b->d_err, b->stream);
     if (p.form == FORM_TILES)
         return Ops<float>::tile_step_many(p.tile, solves, p.d_ptiles, p.nptiles, b->ax, parity, b->d_err, b->stream);
     if (p.form == FORM_PHASES)

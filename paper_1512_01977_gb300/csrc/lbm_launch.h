@@ -75,11 +75,14 @@ struct Ops {
                                    const int* first, int ncta, bool mp, bool ax, int parity, int* err,
                                    cudaStream_t s, int fv = 0);
     // The fused step by warps (lbm_march.cuh; FP32 only): tile t on block t (plan_warp_tiles for warp_slots()),
-    // of one solve or of the n solves of a table (EDM, h_i at the node).
+    // of one solve or of many (EDM, h_i at the node).  kind: what the parameters of many have in common
+    // (warp_kind of one, of two kinds).
     static cudaError_t step_warp(const BatchSolve<R>& solve, const Tile* tiles, int ntiles, bool mp, bool ax, int parity,
                                  int* err, cudaStream_t s);
-    static cudaError_t step_warp_table(const BatchTable<R>& table, int n, const Tile* tiles, int ntiles, bool mp,
-                                       bool ax, int parity, int* err, cudaStream_t s);
+    static cudaError_t step_warp_many(const BatchSolve<R>* solves, int kind, const Tile* tiles, int ntiles, bool mp,
+                                      bool ax, int parity, int* err, cudaStream_t s);
+    static int warp_kind(const Params<R>& p);
+    static int warp_kind(int a, int b);
     static int warp_slots();
     // The batched step with the descriptors as one kernel argument (FP32; n <=
     // BatchTable<R>::N solves; cudaErrorNotSupported in FP64).
@@ -111,7 +114,10 @@ int Ops<float>::warp_slots();
 template <>
 cudaError_t Ops<float>::step_warp(const BatchSolve<float>&, const Tile*, int, bool, bool, int, int*, cudaStream_t);
 template <>
-cudaError_t Ops<float>::step_warp_table(const BatchTable<float>&, int, const Tile*, int, bool, bool, int, int*,
-                                        cudaStream_t);
+cudaError_t Ops<float>::step_warp_many(const BatchSolve<float>*, int, const Tile*, int, bool, bool, int, int*, cudaStream_t);
+template <>
+int Ops<float>::warp_kind(const Params<float>&);
+template <>
+int Ops<float>::warp_kind(int, int);
 
 }  // namespace lbm

@@ -62,7 +62,7 @@ extern "C" {
 cudaError_t cudaMalloc(void** p, size_t n) {
     if (fake::device_left >= 0 && fake::device_left-- == 0) return cudaErrorMemoryAllocation;
     fake::Untracked u;
-    *p = malloc(n);
+    *p = calloc(n, 1);
     (*fake::live)[(uintptr_t)*p] = n;
     return cudaSuccess;
 }
@@ -223,16 +223,19 @@ cudaError_t Ops<float>::step_warp(const BatchSolve<float>&, const Tile* tiles, i
     return fake::launch(tiles, n * sizeof(Tile));
 }
 template <>
-cudaError_t Ops<float>::step_warp_table(const BatchTable<float>& t, int ns, const Tile* tiles, int n, bool, bool, int,
-                                        int*, cudaStream_t) {
-    if (n <= 0 || ns < 1) return cudaErrorInvalidConfiguration;
-    const cudaError_t e = fake::launch(tiles, n * sizeof(Tile));
-    for (int i = 0; e == cudaSuccess && i < n; i++)  // the list is this form's: strips of its width, its solves
-        if (tiles[i].solve < 0 || tiles[i].solve >= ns || tiles[i].strip * kWarpStrip >= t.s[tiles[i].solve].p.nz ||
-            tiles[i].jend > t.s[tiles[i].solve].p.nr)
+cudaError_t Ops<float>::step_warp_many(const BatchSolve<float>* solves, int, const Tile* tiles, int n, bool, bool, int, int*,
+                                       cudaStream_t) {
+    if (n <= 0) return cudaErrorInvalidConfiguration;
+    const cudaError_t e = fake::launch(tiles, n * sizeof(Tile), solves, sizeof(BatchSolve<float>));
+    for (int i = 0; e == cudaSuccess && i < n; i++)  // the list is this form's: strips of its width, rows of the solve
+        if (tiles[i].strip * kWarpStrip >= solves[tiles[i].solve].p.nz || tiles[i].jend > solves[tiles[i].solve].p.nr)
             fake::violations++;
     return e;
 }
+template <>
+int Ops<float>::warp_kind(const Params<float>&) { return 0; }
+template <>
+int Ops<float>::warp_kind(int a, int) { return a; }
 template struct Ops<float>;
 template struct Ops<double>;
 
@@ -297,6 +300,18 @@ static void batch_retune(int nz, int nr, int n, int precision, bool device) {
     lbm_axi_batch_destroy(b);
     for (int i = 0; i < n; i++) lbm_axi_destroy(h[i]);
     CHECK(fake::live->empty());
+}
+
+// A step of a large FP32 batch is one launch, whatever the number of solves.
+static void batch_launches(int nz, int nr, int n) {
+    lbm_axi* h[300];
+    for (int i = 0; i < n; i++) h[i] = solve(nz, nr, 32);
+    lbm_axi_batch* b = nullptr;
+    CHECK(lbm_axi_batch_create(h, n, nullptr, &b) == LBM_OK);
+    fake::launches = 0;
+    CHECK(lbm_axi_batch_step(b, 1) == LBM_OK && fake::launches == 1);
+    lbm_axi_batch_destroy(b);
+    for (int i = 0; i < n; i++) lbm_axi_destroy(h[i]);
 }
 
 // Steps enqueued while the caller captures the solve's stream: one launch each, whatever their number, before
@@ -368,7 +383,7 @@ int main(int argc, char** argv) {
     const char* what = argc > 1 ? argv[1] : "";
     if (!strcmp(what, "retune_device_warps")) return batch_retune(1040, 400, 3, 32, true), 0;
     if (!strcmp(what, "retune_host_warps")) return batch_retune(1040, 400, 3, 32, false), 0;
-    if (!strcmp(what, "retune_host_two_tables")) return batch_retune(64, 48, 280, 32, false), 0;
+    if (!strcmp(what, "retune_host_many")) return batch_retune(64, 48, 280, 32, false), 0;
     if (!strcmp(what, "retune_device_phases")) return batch_retune(100, 40, 3, 32, true), 0;
     if (!strcmp(what, "retune_host_fp64")) return batch_retune(100, 40, 3, 64, false), 0;
     if (!strcmp(what, "capture32")) return step_under_capture(32), 0;
@@ -379,6 +394,13 @@ int main(int argc, char** argv) {
     if (!strcmp(what, "create_fp64")) return create_out_of_memory(64, 64, 64, 0), 0;
     if (!strcmp(what, "create_warps")) return create_out_of_memory(1040, 800, 32, 0), 0;
     if (!strcmp(what, "create_ctas")) return create_out_of_memory(1040, 800, 32, 1), 0;
+    if (!strcmp(what, "launches")) {
+        batch_launches(1040, 400, 2);
+        batch_launches(64, 52, 256);
+        batch_launches(64, 52, 257);
+        batch_launches(64, 52, 300);
+        return 0;
+    }
     fprintf(stderr, "unknown check %s\n", what);
     return 2;
 }

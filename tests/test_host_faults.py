@@ -29,7 +29,7 @@ def _run(program, what):
     assert r.returncode == 0, (what, r.returncode, r.stderr)
 
 
-@pytest.mark.parametrize("what", ["retune_device_warps", "retune_host_warps", "retune_host_two_tables",
+@pytest.mark.parametrize("what", ["retune_device_warps", "retune_host_warps", "retune_host_many",
                                   "retune_device_phases", "retune_host_fp64"])
 def test_batch_keeps_its_plan_when_a_new_one_fails(program, what):
     _run(program, what)
@@ -48,3 +48,7 @@ def test_fields_are_not_written_past_an_allocation(program, what):
 @pytest.mark.parametrize("what", ["create_phases", "create_fp64", "create_warps", "create_ctas"])
 def test_creation_reports_that_memory_ran_out(program, what):
     _run(program, what)
+
+
+def test_a_step_of_a_large_batch_is_one_launch(program):
+    _run(program, "launches")
