@@ -196,8 +196,8 @@ int lbm_axi_time_kernels(lbm_axi* h, long long n, double* ms);
 
 /* Kernel configuration of a solve (performance only).
  *   path: LBM_PATH_FUSED -- the whole update in one launch per step (FP32: tiles
- *         held on chip for small grids, marching warps above 800,000 nodes, 72 B
- *         per node) or in three (FP64, and FP32 in between), chosen by size;
+ *         held on chip for small grids, marching warps above 800,000 nodes in
+ *         whole tiles of 64 x 8, 72 B per node) or in three (FP64, and FP32 in between), chosen by size;
  *         needs nr >= 16.  LBM_PATH_SPLIT -- kernel (a) (gather, rho, j, psi into
  *         field planes) then kernel (b) (forces + collision), 140 B per node.
  *   rows_per_cta: 0 -- the form the size chooses (default); > 0 -- one launch,

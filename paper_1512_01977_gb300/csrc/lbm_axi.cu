@@ -47,7 +47,7 @@ static cudaError_t step_fused(lbm_axi* h, const Params<R>& p, int c) {
     const lbm::LinkSets<R> hs{static_cast<const R*>(h->hb[0]), static_cast<R*>(h->hb[1])};
     if constexpr (sizeof(R) == 4)
         if (h->tile != lbm::TILE_NONE) return Ops<R>::tile_step(h->tile, s, ax, c, h->derr, h->stream);
-    if (lbm_by_phases(h->precision, (long long)h->nz * h->nr))
+    if (lbm_by_phases(h->precision, lbm::phase_nodes(h->nz, h->nr)))
         return Ops<R>::phase_step(s, hs, mp, ax, c, h->derr, h->stream, fv_of(h));
     if constexpr (sizeof(R) == 4)
         if (fv_of(h) == 0) return Ops<R>::step_warp(s, h->d_tiles, h->ncta, mp, ax, c, h->derr, h->stream);
@@ -366,7 +366,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     const bool link = o.h_eval == LBM_H_LINK_AVG && o.axis_terms, ctas = link || guo_of(h);
     std::vector<lbm::Tile> tiles;
     std::vector<int> first;
-    if (!lbm_by_phases(o.precision, (long long)nz * nr)) {
+    if (!lbm_by_phases(o.precision, lbm::phase_nodes(nz, nr))) {
         const int slots = ctas ? Ops<float>::batch_resident_ctas(lbm::kStripWide) : Ops<float>::warp_slots();
         int rc = LBM_ERR_CUDA;
         try {

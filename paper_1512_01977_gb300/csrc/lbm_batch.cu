@@ -76,11 +76,11 @@ const Params<double>& params_of<double>(const lbm_axi* h) {
 
 // FP64 steps by phases at every tuning; FP32 at the default one (wide strips, grid
 // 0) by tiles or phases while the batch is small and by warps beyond, at the others by march2.
-BatchForm form_of(const lbm_axi_batch* b, const StepPlan& p, long long nodes) {
+BatchForm form_of(const lbm_axi_batch* b, const StepPlan& p, long long phase_nodes) {
     if (b->precision == 64) return FORM_PHASES;
     if (p.strip != lbm::kStripWide || p.grid != 0) return FORM_MARCH;
     if (p.tile != lbm::TILE_NONE) return FORM_TILES;
-    return lbm_by_phases(32, nodes) ? FORM_PHASES : FORM_WARPS;
+    return lbm_by_phases(32, phase_nodes) ? FORM_PHASES : FORM_WARPS;
 }
 
 void release(StepPlan& p) {
@@ -108,14 +108,15 @@ cudaError_t upload_solves(lbm_axi_batch* b) {
 template <typename R>
 cudaError_t make_plan(const lbm_axi_batch* b, StepPlan& p) {
     std::vector<int> nz(b->n), nr(b->n);
-    long long nodes = 0;
+    long long nodes = 0, phase_nodes = 0;
     for (int i = 0; i < b->n; i++) {
         nz[i] = b->solves[i]->nz;
         nr[i] = b->solves[i]->nr;
         nodes += (long long)nz[i] * nr[i];
+        phase_nodes += lbm::phase_nodes(nz[i], nr[i]);
     }
     p.tile = b->precision == 32 ? lbm::tile_form(nz.data(), nr.data(), b->n, b->mp, b->ax, 0) : lbm::TILE_NONE;
-    p.form = form_of(b, p, nodes);
+    p.form = form_of(b, p, phase_nodes);
     std::vector<lbm::Tile> tiles;
     std::vector<lbm::PhaseTile> ptiles;
     size_t inner = 0;  // tiles before the ghost rows'

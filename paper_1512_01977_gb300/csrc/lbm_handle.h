@@ -74,9 +74,9 @@ inline bool unbatchable(const lbm_axi* h) { return fv_of(h) != 0; }
 cudaError_t lbm_handle_step_fused(lbm_axi* h, int c);
 
 // The step runs as three phase launches instead of a marching kernel: FP64
-// always, FP32 up to kPhaseMaxNodes nodes in all.
-inline bool lbm_by_phases(int precision, long long nodes) {
-    return precision == 64 || nodes <= lbm::kPhaseMaxNodes;
+// always, FP32 up to kPhaseMaxNodes nodes in all (counted by lbm::phase_nodes).
+inline bool lbm_by_phases(int precision, long long phase_nodes) {
+    return precision == 64 || phase_nodes <= lbm::kPhaseMaxNodes;
 }
 
 // A solve as the step kernels see it, reading f[a] on even steps.

@@ -11,9 +11,12 @@ namespace lbm {
 
 constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs (all that fit); fixed so reductions are reproducible
 constexpr int kStepMinRows = 16;    // the fused forms need single reflections at the walls
-// FP32 solves and batches up to this many nodes step by phases, larger ones by warps.  us per step, phases
-// and warps: 512 x 512 13.4 and 23.1, 1024 x 768 29.7 and 30.0, 1024 x 1024 38.5 and 37.1, 2048 x 1024 82.8
-// and 51.3; batches of 510k nodes 26.7 and 29.8, of 947k 47.0 and 36.9.
+// FP32 solves and batches up to this many nodes, counted in whole tiles (phase_nodes), step by phases, larger
+// ones by warps (with the link source or Guo forcing, a solve by CTAs).  us per step, phases and warps, by
+// such nodes: 256k (500 x 500) 14.0 and 23.2, 576k 22.5 and 28.2, 749k (800 x 900) 27.0 and 29.5, 768k (65 x
+// 6000) 28.8 and 29.6, 845k (900 x 880) 30.2 and 30.5, 1.15M (65 x 9000) 40.9 and 30.1, 1.28M (33 x 20000) 50 and
+// 39; batches: 707k (138 x 66 x 33) 29.4 and 25.0, 774k 33.6 and 29.6, 791k (386 x 64 x 32) 34.9 and 38.1,
+// 1.04M 42.8 and 31.3, 1.41M (276 x 66 x 33) 54.5 and 33.0.
 constexpr long long kPhaseMaxNodes = 800000;
 // z-columns per CTA of the two compiled forms of the batched kernel (the wide
 // one is the default; the autotuner may pick the narrow one for small grids).

@@ -31,7 +31,7 @@ template <typename R>
 struct PhaseShape;
 template <>
 struct PhaseShape<float> {
-    static constexpr int TZ = 64, CP = 2;  // one warp per tile row
+    static constexpr int TZ = kPhaseColumns, CP = 2;  // one warp per tile row
 };
 template <>
 struct PhaseShape<double> {

@@ -15,6 +15,13 @@ struct PhaseTile {
     int solve, k0, j0;
 };
 
+// Columns of an FP32 phase tile, and the nodes of a grid with its last tiles (of 8 rows) counted whole: what
+// the phases' time goes by, as a tile computes all its nodes.
+constexpr int kPhaseColumns = 64;
+inline long long phase_nodes(int nz, int nr) {
+    return (long long)((nz + kPhaseColumns - 1) / kPhaseColumns) * kPhaseColumns * ((nr + 7) / 8) * 8;
+}
+
 // Pipeline rows a tile costs beyond its own: 6 halo rows above it and the 12-row
 // lag between the first and the last marching stage.
 constexpr int kTileFillRows = 18;

@@ -21,6 +21,7 @@ namespace fake {
 std::map<uintptr_t, size_t>* live = nullptr;  // device allocations
 long long device_left = -1, host_left = -1;   // allocations until one fails (-1: none does)
 int launches = 0, violations = 0;
+const char* form = "";  // of the last step launched
 bool track = false;
 const void* last_rho = nullptr;   // where the last read wrote its density
 cudaStream_t captured = nullptr;  // a stream that its owner is capturing
@@ -176,28 +177,33 @@ cudaError_t Ops<R>::step(const Params<R>&, const R*, R*, int, int*, cudaStream_t
 template <typename R>
 cudaError_t Ops<R>::step_batch(const BatchSolve<R>*, const Tile* tiles, const int* first, int ncta, bool, bool, int, int,
                                int*, cudaStream_t) {
+    fake::form = "ctas";
     if (ncta <= 0) return cudaErrorInvalidConfiguration;
     return fake::launch(first, (ncta + 1) * sizeof(int), tiles, sizeof(Tile));
 }
 template <typename R>
 cudaError_t Ops<R>::step_single(const BatchSolve<R>&, const LinkSets<R>&, const Tile* tiles, const int* first, int ncta,
                                 bool, bool, int, int*, cudaStream_t, int) {
+    fake::form = "ctas";
     if (ncta <= 0) return cudaErrorInvalidConfiguration;
     return fake::launch(first, (ncta + 1) * sizeof(int), tiles, sizeof(Tile));
 }
 template <typename R>
 cudaError_t Ops<R>::step_table(const BatchTable<R>&, const Tile* tiles, const int* first, int ncta, bool, bool, int, int,
                                int*, cudaStream_t) {
+    fake::form = "ctas";
     if (ncta <= 0) return cudaErrorInvalidConfiguration;
     return fake::launch(first, (ncta + 1) * sizeof(int), tiles, sizeof(Tile));
 }
 template <typename R>
 cudaError_t Ops<R>::phase_step(const BatchSolve<R>&, const LinkSets<R>&, bool, bool, int, int*, cudaStream_t, int) {
+    fake::form = "phases";
     return fake::launches++, cudaSuccess;
 }
 template <typename R>
 cudaError_t Ops<R>::phase_step_many(const BatchSolve<R>* solves, const PhaseTile* tiles, int ntiles, int nghost, int,
                                     bool, bool, int, int*, cudaStream_t) {
+    fake::form = "phases";
     if (ntiles <= 0) return cudaErrorInvalidConfiguration;
     return fake::launch(tiles, (ntiles + nghost) * sizeof(PhaseTile), solves, sizeof(BatchSolve<R>));
 }
@@ -220,11 +226,13 @@ template <>
 int Ops<float>::warp_slots() { return 1824; }
 template <>
 cudaError_t Ops<float>::step_warp(const BatchSolve<float>&, const Tile* tiles, int n, bool, bool, int, int*, cudaStream_t) {
+    fake::form = "warps";
     return fake::launch(tiles, n * sizeof(Tile));
 }
 template <>
 cudaError_t Ops<float>::step_warp_many(const BatchSolve<float>* solves, int, const Tile* tiles, int n, bool, bool, int, int*,
                                        cudaStream_t) {
+    fake::form = "warps";
     if (n <= 0) return cudaErrorInvalidConfiguration;
     const cudaError_t e = fake::launch(tiles, n * sizeof(Tile), solves, sizeof(BatchSolve<float>));
     for (int i = 0; e == cudaSuccess && i < n; i++)  // the list is this form's: strips of its width, rows of the solve
@@ -251,11 +259,12 @@ template struct Ops<double>;
         }                                                     \
     } while (0)
 
-static lbm_axi* solve(int nz, int nr, int precision, void* stream = nullptr) {
+static lbm_axi* solve(int nz, int nr, int precision, void* stream = nullptr, int forcing = LBM_FORCING_EDM) {
     lbm_axi_opts o;
     lbm_axi_default_opts(&o);
     o.precision = precision;
     o.stream = stream;
+    o.forcing = forcing;
     lbm_eos e = {LBM_EOS_CS, 0.9, 1.0, 4.0, 1.0, 0.01};
     lbm_axi* h = nullptr;
     CHECK(lbm_axi_create(nz, nr, 1.0, &e, -0.152, &o, &h) == LBM_OK);
@@ -312,6 +321,31 @@ static void batch_launches(int nz, int nr, int n) {
     CHECK(lbm_axi_batch_step(b, 1) == LBM_OK && fake::launches == 1);
     lbm_axi_batch_destroy(b);
     for (int i = 0; i < n; i++) lbm_axi_destroy(h[i]);
+}
+
+// Which form a grid steps by: what counts is its nodes in whole tiles of 64 columns and 8 rows.
+static void forms() {
+    struct {
+        int nz, nr, n;
+        const char *edm, *other;  // other: Guo forcing, single solves only
+    } const cases[] = {{640, 1248, 1, "phases", "phases"}, {640, 1251, 1, "warps", "ctas"}, {65, 6248, 1, "phases", "phases"},
+                       {65, 6251, 1, "warps", "ctas"},     {65, 9000, 1, "warps", "ctas"},  {2, 12496, 1, "phases", "phases"},
+                       {2, 150000, 1, "warps", "ctas"},    {64, 32, 299, "phases", nullptr}, {66, 33, 156, "phases", nullptr},
+                       {66, 33, 157, "warps", nullptr}};
+    for (const auto& c : cases)
+        for (int forcing = 0; forcing < (c.other ? 2 : 1); forcing++) {
+            lbm_axi* h[300];
+            for (int i = 0; i < c.n; i++) h[i] = solve(c.nz, c.nr, 32, nullptr, forcing);
+            CHECK(lbm_axi_step(h[0], 1) == LBM_OK);
+            if (c.n == 1) CHECK(!strcmp(fake::form, forcing ? c.other : c.edm));
+            if (!forcing) {
+                lbm_axi_batch* b = nullptr;
+                CHECK(lbm_axi_batch_create(h, c.n, nullptr, &b) == LBM_OK && lbm_axi_batch_step(b, 1) == LBM_OK);
+                CHECK(!strcmp(fake::form, c.edm) && fake::violations == 0);
+                lbm_axi_batch_destroy(b);
+            }
+            for (int i = 0; i < c.n; i++) lbm_axi_destroy(h[i]);
+        }
 }
 
 // Steps enqueued while the caller captures the solve's stream: one launch each, whatever their number, before
@@ -394,6 +428,7 @@ int main(int argc, char** argv) {
     if (!strcmp(what, "create_fp64")) return create_out_of_memory(64, 64, 64, 0), 0;
     if (!strcmp(what, "create_warps")) return create_out_of_memory(1040, 800, 32, 0), 0;
     if (!strcmp(what, "create_ctas")) return create_out_of_memory(1040, 800, 32, 1), 0;
+    if (!strcmp(what, "forms")) return forms(), 0;
     if (!strcmp(what, "launches")) {
         batch_launches(1040, 400, 2);
         batch_launches(64, 52, 256);

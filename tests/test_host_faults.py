@@ -52,3 +52,7 @@ def test_creation_reports_that_memory_ran_out(program, what):
 
 def test_a_step_of_a_large_batch_is_one_launch(program):
     _run(program, "launches")
+
+
+def test_forms_go_by_whole_tiles(program):
+    _run(program, "forms")
