@@ -9,7 +9,7 @@ import pytest
 
 import oracle as O
 from paper_1512_01977_gb300 import inputs as I
-from tests._cases import Case, component_errs, rel_err, run_oracle
+from tests._cases import Case, component_errs, rel_err, run_oracle, vel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -297,3 +297,122 @@ def test_pressure_at_the_pole_of_the_eos(lbm, prec, eos, pole):
     s.close()
     at = got[0] == pole
     assert at[3, 5] and np.all(got[1][at] == np.inf) and np.all(np.isfinite(got[1][~at]))
+
+
+def _state(c, seed):
+    """Noise for a two-phase or a single-phase solve, and its reference density."""
+    if c.multiphase:
+        return _fields(c, seed), c.coexistence()[1]
+    rng = np.random.default_rng(seed)
+    _, uz, ur = I.random_state(c.nz, c.nr, 1.0, 0.0, 1e-3, seed)
+    return (1.0 + 0.05 * rng.uniform(size=(c.nr, c.nz)), uz, ur * (np.arange(c.nr) + 0.5)[:, None] / c.nr), 1.0
+
+
+@pytest.mark.parametrize("multiphase,top,axis", [(0, O.TOP_FREESLIP, 1), (0, O.TOP_NOSLIP, 1), (0, O.TOP_PERIODIC, 0),
+                                                 (0, O.TOP_PERIODIC, 1), (1, O.TOP_PERIODIC, 1)])
+@pytest.mark.parametrize("nz,nr", [(1, 16), (69, 23), (131, 18), (461, 301), (513, 401), (65, 3301), (1041, 801),
+                                   (1093, 799), (60, 14000)])
+def test_fp32_options_same_bits_as_marching(lbm, nz, nr, multiphase, top, axis):
+    """Single-phase runs and a periodic top with the axis terms on, in every form that a size chooses."""
+    c = Case(nz, nr, T_over_Tc=0.9, top=top, axis=axis, multiphase=multiphase)
+    fields, ref = _state(c, nz + nr)
+    got = []
+    for rows in (0, 1 << 20):
+        s = c.solver(32, ref)
+        lbm.lbm_axi_set_tuning(s.h, lbm.PATH_FUSED, rows)
+        s.init(*fields).step(5)
+        got.append(np.frombuffer(s.save()[192:], dtype=np.uint32))
+        s.close()
+    np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("multiphase", [0, 1])
+@pytest.mark.parametrize("nz,nr", [(1, 16), (33, 21), (65, 30)])
+def test_fp64_periodic_top_with_axis_terms(lbm, nz, nr, multiphase):
+    c = Case(nz, nr, T_over_Tc=0.9, top=O.TOP_PERIODIC, multiphase=multiphase)
+    fields, _ = _state(c, nz + nr)
+    mo = run_oracle(c, fields, 20).moments()
+    s = c.solver(64).init(*fields).step(20)
+    mg = s.moments()
+    s.close()
+    assert rel_err(mg["rho"], mo["rho"]) <= 1e-12 and rel_err(mg["p"], mo["p"]) <= 1e-12
+    assert all(e <= 1e-12 for e in component_errs(mg, mo).values())
+
+
+def test_fp64_infinite_density_of_a_single_phase_run(lbm):
+    rho = np.ones((20, 30))
+    rho[4, 5] = np.inf
+    s = lbm.Solver(30, 20, 1.0, multiphase=0).init(rho)
+    with pytest.raises(lbm.LbmError) as e:
+        s.step(1)
+    assert e.value.code == lbm.ERR_UNPHYSICAL
+    s.close()
+
+
+@pytest.mark.parametrize("forcing,h_eval", [(O.FORCING_GUO, O.H_LOCAL), (O.FORCING_EDM, O.H_LINK_AVG),
+                                            (O.FORCING_GUO, O.H_LINK_AVG)])
+@pytest.mark.parametrize("top", [O.TOP_FREESLIP, O.TOP_NOSLIP])
+@pytest.mark.parametrize("steps", [4, 5])
+def test_marching_ctas_repeat_a_narrow_solve(lbm, forcing, h_eval, top, steps):
+    """Guo forcing and the link source, FP32: a state of 40 columns, moving and with every node its own value, steps by
+    phases; repeated along z beyond 800,000 nodes it steps by marching CTAs, to the same bits in every column."""
+    nr, n, times = 800, 40, 26
+    got = []
+    for nz in (n, n * times):
+        c = Case(nz, nr, T_over_Tc=0.9, top=top, forcing=forcing, h_eval=h_eval)
+        rho, uz, ur = _fields(Case(n, nr, T_over_Tc=0.9), 11)
+        rho, uz, ur = (np.tile(a, (1, nz // n)) for a in (rho, uz + 0.01, ur))
+        s = c.solver(32, c.coexistence()[1]).init(rho, uz, ur).step(steps)
+        planes = np.frombuffer(s.save()[192:], dtype=np.uint32).reshape(-1, nr, nz)
+        got.append(planes)
+        s.close()
+    np.testing.assert_array_equal(np.tile(got[0], (1, 1, times)), got[1])
+
+
+@pytest.mark.parametrize("multiphase,axis,count,lo", [(1, 1, 60, 90), (0, 1, 60, 90), (0, 0, 60, 90), (0, 1, 90, 140),
+                                                      (1, 0, 90, 140)])
+def test_fp32_batch_forms_equal_alone(lbm, multiphase, axis, count, lo):
+    """Batches that step by phases (60 solves, 397,000 nodes) and by warps (90 solves, 1.4M), with walls of all
+    kinds: each solve the bits of its run alone."""
+    rng = np.random.default_rng(count)
+    cases = [Case(int(rng.integers(lo // 2, 2 * lo)), int(rng.integers(lo // 3, lo)), T_over_Tc=0.9, axis=axis,
+                  multiphase=multiphase, top=(O.TOP_FREESLIP, O.TOP_NOSLIP, O.TOP_PERIODIC)[i % 3]) for i in range(count)]
+    states = [_state(c, i) for i, c in enumerate(cases)]
+    solvers = [c.solver(32, ref).init(*f) for c, (f, ref) in zip(cases, states)]
+    b = lbm.Batch(solvers)
+    assert b.step(5) == lbm.OK
+    b.close()
+    for i in range(0, count, 7):
+        s = cases[i].solver(32, states[i][1]).init(*states[i][0]).step(5)
+        assert solvers[i].save() == s.save()
+        s.close()
+    for s in solvers:
+        s.close()
+
+
+@pytest.mark.parametrize("strip,grid", [(112, 300), (64, 0)])
+def test_marching_batch_beyond_one_table(lbm, strip, grid):
+    """More solves than a kernel argument holds, at a tuning that asks for marching CTAs (k_step_batch): the bits of
+    each solve alone by marching CTAs at 112 columns, FP32 rounding at 64."""
+    specs = I.batch_droplets(n=260, seed=9, lo=(24, 16), scale_max=1.6)
+    cases = [Case(q["nz"], q["nr"], T_over_Tc=0.85) for q in specs]
+    rv, rl = cases[0].coexistence()
+    fields = [I.droplet(c.nz, c.nr, min(q["R"], 6.0), rl, rv) for c, q in zip(cases, specs)]
+    solvers = [c.solver(32, rv).init(*f) for c, f in zip(cases, fields)]
+    b = lbm.Batch(solvers)
+    lbm.lbm_axi_batch_set_tuning(b.b, strip, grid)
+    assert b.step(21) == lbm.OK
+    b.close()
+    for i in range(0, 260, 37):
+        s = cases[i].solver(32, rv)
+        lbm.lbm_axi_set_tuning(s.h, lbm.PATH_FUSED, 1 << 20)
+        ref = s.init(*fields[i]).step(21).moments()
+        s.close()
+        m = solvers[i].moments()
+        if strip == 112:
+            for k in ("rho", "uz", "ur", "p"):
+                np.testing.assert_array_equal(m[k], ref[k])
+        else:
+            assert rel_err(m["rho"], ref["rho"]) <= 1e-6 and vel_err(m, ref) <= 1e-6
+    for s in solvers:
+        s.close()
