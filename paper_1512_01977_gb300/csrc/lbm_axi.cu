@@ -297,7 +297,8 @@ size_t lbm_axi_footprint(int nz, int nr, int precision) {
     if (nz < 1 || nr < 1) return 0;
     const size_t s = precision == 32 ? 4 : 8;
     const size_t plane = (size_t)pitch_of(nz) * nr;
-    return 2 * 9 * plane * s + 4 * plane * s + 4 * (size_t)nz * nr * 8 + 4 * lbm::kReduceBlocks * 8 + 64;
+    const size_t n = (size_t)nz * nr;
+    return 2 * 9 * plane * s + 4 * plane * s + 4 * n * 8 + 4 * (size_t)lbm::reduce_blocks((long long)n) * 8 + 64;
 }
 
 int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, const lbm_axi_opts* opts,
@@ -359,7 +360,7 @@ int lbm_axi_create(int nz, int nr, double tau, const lbm_eos* eos, double A, con
     h->f[1] = dev_alloc(9 * plane_bytes);
     h->aux = dev_alloc(4 * plane_bytes);
     h->mout = (double*)dev_alloc(4 * (size_t)nz * nr * sizeof(double));
-    h->partial = (double*)dev_alloc(4 * lbm::kReduceBlocks * sizeof(double));
+    h->partial = (double*)dev_alloc(4 * (size_t)lbm::reduce_blocks((long long)nz * nr) * sizeof(double));
     h->derr = (int*)dev_alloc(sizeof(int));
     // tile plan of the marching step: warps, or CTAs on wide strips with the link source or Guo forcing
     // (4096 x 2048 Guo: 210 us per step by CTAs, 155 by warps, whose sums round differently)

@@ -9,7 +9,9 @@
 
 namespace lbm {
 
-constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs (all that fit); fixed so reductions are reproducible
+// Blocks of 256 threads of a reduction over n nodes: 8 x 152 SMs (all that fit), fewer while that leaves some
+// without a node; by the size alone, so reductions are reproducible.
+constexpr int reduce_blocks(long long n) { return n > 1216 * 256 ? 1216 : (int)((n + 255) / 256); }
 constexpr int kStepMinRows = 16;    // the fused forms need single reflections at the walls
 // FP32 solves and batches up to this many nodes, counted in whole tiles (phase_nodes), step by phases, larger
 // ones by warps (with the link source or Guo forcing, a solve by CTAs).  us per step, phases and warps, by

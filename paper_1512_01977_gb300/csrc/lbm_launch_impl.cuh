@@ -138,8 +138,9 @@ cudaError_t Ops<R>::init(const Params<R>& p, double rho_ref, const double* rho, 
 template <typename R>
 cudaError_t Ops<R>::mass(const Params<R>& p, const R* f, LinkPlanes<R> lk, double* partial, double* out, int* err,
                          cudaStream_t s) {
-    k_mass<R><<<kReduceBlocks, 256, 0, s>>>(p, f, lk, partial, err);
-    k_reduce_final<2><<<1, 256, 0, s>>>(partial, kReduceBlocks, out);
+    const int blocks = reduce_blocks((long long)p.nz * p.nr);
+    k_mass<R><<<blocks, 256, 0, s>>>(p, f, lk, partial, err);
+    k_reduce_final<2><<<1, 256, 0, s>>>(partial, blocks, out);
     return cudaGetLastError();
 }
 
@@ -147,8 +148,9 @@ template <typename R>
 cudaError_t Ops<R>::pjump(const Params<R>& p, const Params<double>& pd, const R* f, LinkPlanes<R> lk, double zc,
                           double rc, double rin, double rout, double* partial, double* out, int* err,
                           cudaStream_t s) {
-    k_pjump<R><<<kReduceBlocks, 256, 0, s>>>(p, pd, f, lk, zc, rc, rin, rout, partial, err);
-    k_reduce_final<4><<<1, 256, 0, s>>>(partial, kReduceBlocks, out);
+    const int blocks = reduce_blocks((long long)p.nz * p.nr);
+    k_pjump<R><<<blocks, 256, 0, s>>>(p, pd, f, lk, zc, rc, rin, rout, partial, err);
+    k_reduce_final<4><<<1, 256, 0, s>>>(partial, blocks, out);
     return cudaGetLastError();
 }
 

@@ -83,3 +83,13 @@ def test_create_refuses_grids_beyond_32bit_offsets(lbm, nz, nr):
     with pytest.raises(lbm.LbmError) as e:
         lbm.lbm_axi_create(nz, nr, 1.0, lbm.make_eos(), -0.152)
     assert e.value.code == lbm.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("nz,nr", [(1, 1), (16, 16), (32, 32), (64, 64), (300, 250)])
+def test_footprint_of_a_small_solve_is_its_planes(lbm, nz, nr, prec):
+    """Beyond the 22 field planes and the staging: 304 x 4 partial sums (all there were) at most, one block of 256
+    nodes' 4 where there are fewer."""
+    pitch = (nz + 31) // 32 * 32
+    planes = 22 * pitch * nr * prec // 8 + 32 * nz * nr
+    assert lbm.lbm_axi_footprint(nz, nr, prec) - planes <= min(304, -(-nz * nr // 256)) * 32 + 64
