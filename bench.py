@@ -115,9 +115,27 @@ def _source_hash():
     return h.hexdigest()[:16]
 
 
-def _ncu_traffic():
-    """Per-launch DRAM bytes of the fused step kernel on this workload from the
-    committed ncu summary, or None when the kernel sources changed since."""
+# What the kernels of a step's main launch do (the names of lbm.lbm_axi_step_kernels).
+_KERNELS = {"k_step_warp": "one-pass gather+psi+forces+EDM+source+collide, one warp per strip",
+            "k_tile": "one-pass gather+psi+forces+EDM+source+collide over tiles held in shared memory",
+            "k_step": "one-pass gather+psi+forces+EDM+source+collide by CTAs marching fixed row chunks",
+            "k_phase_l": "gather+psi, forces+u, source+EDM+collide, one launch each",
+            "k_density": "forces+EDM+source+collide, after k_density"}
+
+
+def _step_form(kernels):
+    """(roofline label, launches per step, algorithmic bytes per node of what is timed) of a step of these kernels: the
+    whole step, whose populations are read and written once, or kernel (b) of the split path."""
+    split = kernels[0] == "k_density"
+    name = "k_update" if split else " + ".join(kernels)
+    return "%s (%s)" % (name, _KERNELS[kernels[0]]), len(kernels), BYTES_B if split else BYTES_FUSED
+
+
+def _ncu_traffic(kernels):
+    """Per-launch DRAM bytes of k_step_warp on the default grid from the committed ncu
+    summary, or None for another kernel or grid and when the kernel sources changed since."""
+    if kernels != ["k_step_warp"] or (NZ, NR) != (4096, 2048):
+        return None
     path = os.path.join(ROOT, "profiles", "k_step_warp_fp32_wave4096x2048.md")
     try:
         vals = {}
@@ -387,18 +405,14 @@ def run_ours(args):
     t_iso = t_b  # one launch bracketed by its own events
     t_step = ms * 1e-3 / args.steps
     if path == lbm.PATH_FUSED:
-        # the timed region ran this kernel alone, one launch per step: its average
-        # launch duration over that region is the region's time per step
+        # the timed region ran the step's kernels alone: their average duration per step
+        # over that region is the region's time per step
         t_a, t_b = 0.0, t_step
-    # launches per step: the fused step of the default grid is one (grids of at most 800,000 nodes take one
-    # or three, by size; counted as one)
-    per_step = 1 if path == lbm.PATH_FUSED else 2
+    kernels = lbm.lbm_axi_step_kernels(s.h)
+    label, per_step, bytes_main = _step_form(kernels)
     peak, peak_kind = _peaks()
-    # algorithmic bytes of the kernel that ran: the fused kernel reads and writes the
-    # 9 populations (72 B/node); kernel (b) of the split path 88 B/node
-    bytes_main = BYTES_FUSED if path == lbm.PATH_FUSED else BYTES_B
     ach_b = bytes_main * n / t_b / 1e9
-    traffic = _ncu_traffic() if path == lbm.PATH_FUSED else None  # the committed counters are the fused kernel's
+    traffic = _ncu_traffic(kernels)
 
     # ---- end to end through the C ABI: pinned host -> init -> K steps -> moments -> pinned host
     barrier()
@@ -441,13 +455,12 @@ def run_ours(args):
                        "parallelism": "replicas only (independent solves per GPU)",
                        "device": props.name},
             "roofline": {"bound": "hbm",
-                         "kernel": "k_step_warp (one-pass gather+psi+forces+EDM+source+collide, one warp per strip)"
-                         if path == lbm.PATH_FUSED else "k_update (forces+EDM+source+collide)",
+                         "kernel": label,
                          "achieved": ach_b, "peak": peak, "unit": "GB/s", "frac": ach_b / peak,
                          "peak_source": peak_kind, "traffic": traffic,
                          "algorithmic_bytes_per_node": bytes_main,
                          "traffic_bytes_per_node": traffic / n if traffic else None,
-                         "avg_launch_us": t_b * 1e6,
+                         "avg_launch_us": t_b * 1e6 / (per_step if path == lbm.PATH_FUSED else 1),
                          "avg_launch_source": "timed region / launches" if path == lbm.PATH_FUSED
                          else "CUDA events around each launch",
                          "isolated_launch_us": t_iso * 1e6,

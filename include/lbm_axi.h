@@ -217,6 +217,10 @@ typedef struct {
 int lbm_axi_get_tuning(const lbm_axi* h, lbm_axi_tuning* t);
 int lbm_axi_set_tuning(lbm_axi* h, const lbm_axi_tuning* t);
 
+/* The kernels that one step of this solve launches as it is tuned, in order,
+ * their names separated by commas (NULL for a NULL handle). */
+const char* lbm_axi_step_kernels(const lbm_axi* h);
+
 /* Macroscopic fields of the current state (host arrays, any may be NULL):
  * rho = sum_i f_i; physical velocity u = sum_i c_i f_i / rho + F / (2 rho)
  * (Sec. II.A); p = P_k(rho) (rho/3 for a single-phase run).  Synchronous. */

@@ -817,6 +817,16 @@ int lbm_axi_set_tuning(lbm_axi* h, const lbm_axi_tuning* t) {
     return LBM_OK;
 }
 
+// As enqueue_step and step_fused choose.
+const char* lbm_axi_step_kernels(const lbm_axi* h) {
+    if (!h) return nullptr;
+    if (h->path != LBM_PATH_FUSED) return "k_density,k_update";
+    if (h->rows_per_cta > 0) return "k_step";
+    if (h->tile != lbm::TILE_NONE) return "k_tile";
+    if (lbm_by_phases(h->precision, lbm::phase_nodes(h->nz, h->nr))) return "k_phase_l,k_phase_u,k_phase_c";
+    return fv_of(h) == 0 ? "k_step_warp" : "k_step_single";
+}
+
 int lbm_axi_temperature(const lbm_axi* h, double* T, double* Tc) {
     if (!h) return LBM_ERR_INVALID_ARG;
     if (T) *T = h->T;

@@ -83,6 +83,7 @@ _SIGS = {
     "lbm_axi_get_tuning": (C.c_int, [_H, C.POINTER(lbm_axi_tuning)]),
     "lbm_axi_set_tuning": (C.c_int, [_H, C.POINTER(lbm_axi_tuning)]),
     "lbm_axi_device_bytes": (C.c_int, [_H, C.POINTER(C.c_size_t)]),
+    "lbm_axi_step_kernels": (C.c_char_p, [_H]),
     "lbm_axi_footprint": (C.c_size_t, [C.c_int, C.c_int, C.c_int]),
     "lbm_eos_critical_temperature": (C.c_int, [C.POINTER(lbm_eos), _D]),
     "lbm_eos_coexistence": (C.c_int, [C.POINTER(lbm_eos), _D, _D]),
@@ -290,6 +291,11 @@ def lbm_axi_get_tuning(h):
 def lbm_axi_set_tuning(h, path, rows_per_cta):
     t = lbm_axi_tuning(path, rows_per_cta)
     _check(lib().lbm_axi_set_tuning(h, C.byref(t)), "lbm_axi_set_tuning")
+
+
+def lbm_axi_step_kernels(h):
+    """Names of the kernels that one step of the solve launches, in order."""
+    return lib().lbm_axi_step_kernels(h).decode().split(",")
 
 
 def lbm_axi_device_bytes(h):

@@ -337,7 +337,12 @@ static void forms() {
             lbm_axi* h[300];
             for (int i = 0; i < c.n; i++) h[i] = solve(c.nz, c.nr, 32, nullptr, forcing);
             CHECK(lbm_axi_step(h[0], 1) == LBM_OK);
-            if (c.n == 1) CHECK(!strcmp(fake::form, forcing ? c.other : c.edm));
+            if (c.n == 1) {
+                const char *form = forcing ? c.other : c.edm, *k = lbm_axi_step_kernels(h[0]);
+                CHECK(!strcmp(fake::form, form));
+                CHECK(!strcmp(k, !strcmp(form, "phases") ? "k_phase_l,k_phase_u,k_phase_c"
+                                                         : (!strcmp(form, "warps") ? "k_step_warp" : "k_step_single")));
+            }
             if (!forcing) {
                 lbm_axi_batch* b = nullptr;
                 CHECK(lbm_axi_batch_create(h, c.n, nullptr, &b) == LBM_OK && lbm_axi_batch_step(b, 1) == LBM_OK);

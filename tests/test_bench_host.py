@@ -24,3 +24,14 @@ def test_reference_arm_line_has_the_contract_keys():
     assert d["cpu_baseline"]["kind"] == "oracle" and d["cpu_baseline"]["cores"] >= 1
     assert d["e2e"]["h2d_bytes_per_step"] == 0 and d["e2e"]["d2h_bytes_per_step"] == 0
     assert "128x64" in json.dumps(d["config"])
+
+
+def test_roofline_names_the_kernels_that_ran():
+    import bench
+
+    label, launches, _ = bench._step_form(["k_phase_l", "k_phase_u", "k_phase_c"])
+    assert label.startswith("k_phase_l + k_phase_u + k_phase_c") and launches == 3
+    assert bench._step_form(["k_tile"])[1:] == (1, 72) and bench._step_form(["k_step_warp"])[1:] == (1, 72)
+    assert bench._step_form(["k_density", "k_update"])[0].startswith("k_update")
+    assert bench._step_form(["k_density", "k_update"])[1:] == (2, 88)
+    assert bench._ncu_traffic(["k_tile"]) is None  # the committed counters are k_step_warp's
