@@ -49,6 +49,23 @@ enum { KAPPA_THERMO = 0, KAPPA_LATTICE = 1, KAPPA_MIXED = 2 };
 // Error bits a kernel may raise in the device error word.
 enum : int { ERRBIT_RHO = 1, ERRBIT_PSI = 2, ERRBIT_NONFINITE = 4 };
 
+// The error word of a solve that steps: the bits of even steps (and of reads) in place, those of odd steps
+// above them.  So a launch knows an error of an earlier step, whose populations are void and left alone, from
+// one of its own step, which it finishes: the buffer that the step writes would otherwise go on holding,
+// where it was left out, an older state that reads as a sound one.
+constexpr int kErrShift = 8;
+__device__ __forceinline__ int err_of_step(int bits, int parity) { return parity ? bits << kErrShift : bits; }
+__device__ __forceinline__ int error_word(const int* err) { return *static_cast<volatile const int*>(err); }
+__device__ __forceinline__ int earlier_error(int word, int parity) {
+    return parity ? word & ((1 << kErrShift) - 1) : word >> kErrShift;
+}
+// Whether a step is left out for an earlier error (by one thread: marked, so that the next one is too).
+__device__ __forceinline__ int left_out(int* err, int parity) {
+    const int earlier = earlier_error(error_word(err), parity);
+    if (earlier) atomicOr(err, err_of_step(earlier, parity));
+    return earlier;
+}
+
 // ------------------------------------------------------------- parameters --
 template <typename R>
 struct Params {

@@ -298,11 +298,12 @@ enum WarpKind { WARP_CS = 0, WARP_CS_LATTICE = 1, WARP_VDW = 2, WARP_VDW_LATTICE
 template <bool MP, bool AX, int KIND>
 __device__ __forceinline__ void march_tile(const BatchSolve<float>& s, const Tile& t, int parity, int* __restrict__ err) {
     __shared__ float2 ring[WarpShape::kRing * WarpShape::kRow];
-    if (*static_cast<volatile const int*>(err)) return;  // the solve already went unphysical
+    int bad = earlier_error(error_word(err), parity);
     const float* f = parity ? s.f_b : s.f_a;
     float* fo = parity ? const_cast<float*>(s.f_a) : s.f_b;
-    int bad = 0;
-    if constexpr (KIND != WARP_MIXED) {
+    if (bad) {
+        // the solve already went unphysical: the step is left out, and so will the next one be
+    } else if constexpr (KIND != WARP_MIXED) {
         march_warp<MP, AX, (KIND & 2) ? EOS_VDW : EOS_CS, (KIND & 1) != 0>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
     } else {
         const bool lattice = s.p.kappa == KAPPA_LATTICE;
@@ -318,7 +319,7 @@ __device__ __forceinline__ void march_tile(const BatchSolve<float>& s, const Til
                 march_warp<MP, AX, EOS_CS, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
         }
     }
-    if (bad) atomicOr(err, bad);
+    if (bad) atomicOr(err, err_of_step(bad, parity));
 }
 
 // Block b marches tile b.  The tile is the same for the whole warp: said by a

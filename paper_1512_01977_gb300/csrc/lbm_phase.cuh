@@ -79,23 +79,8 @@ __device__ __forceinline__ PhaseWork<R> phase_work(const BatchSolve<R>& s, int p
     return {parity ? s.f_b : s.f_a, parity ? const_cast<R*>(s.f_a) : s.f_b, s.aux, s.stage, err, k0, j0, parity};
 }
 
-// The error word of a solve that steps by phases: the bits of even steps in place, those of odd steps
-// above them.  So a phase knows an error of an earlier step, whose populations are void and left alone, from
-// one of its own step, which it finishes: the buffer that the step writes would otherwise go on holding
-// an older state that reads as a sound one.
-constexpr int kErrShift = 8;
-__device__ __forceinline__ int err_of_step(int bits, int parity) { return parity ? bits << kErrShift : bits; }
-__device__ __forceinline__ int earlier_error(const int* err, int parity) {
-    const int word = *static_cast<volatile const int*>(err);
-    return parity ? word & ((1 << kErrShift) - 1) : word >> kErrShift;
-}
-
-// Whether the gather leaves the step out; the step after it sees that by this step's mark.
-template <typename R>
-__device__ __forceinline__ bool left_alone(const PhaseWork<R>& w, int failed) {
-    if (failed && threadIdx.x == 0) atomicOr(w.err, err_of_step(failed, w.parity));
-    return failed != 0;
-}
+// `word` below: the error word, read with a launch's other loads and looked at before its stores only.
+// The gather passes an earlier error on as its own step's, so that the next step sees it too.
 
 // u planes, in the staging planes of the moments pass (4 nz nr doubles, idle during a step): u_z, u_r
 // (and 1 / rho in FP64), each of nr + 2 rows, the first two being rows -2 and -1 (beyond the axis:
@@ -204,7 +189,7 @@ __device__ __forceinline__ bool phase_inner(const Params<R>& p, int k0) {
 }
 
 template <int TR, bool MP, bool LINK, bool EDGE, typename R>
-__device__ __forceinline__ void phase_l2(const Params<R>& p, const PhaseWork<R>& w, const R* h_src, int failed) {
+__device__ __forceinline__ void phase_l2(const Params<R>& p, const PhaseWork<R>& w, const R* h_src, int word) {
     using T = typename PairOf<R>::T;
     const int row = w.j0 + (threadIdx.x >> 5), k = w.k0 + 2 * (threadIdx.x & 31);
     if (row >= p.nr || k >= p.nz) return;
@@ -215,7 +200,10 @@ __device__ __forceinline__ void phase_l2(const Params<R>& p, const PhaseWork<R>&
     int bad = 0;
     moments2<LINK, R>(f, la, drho, jz, jr);
     const T psi = psi2<MP>(p, drho, k + 1 < p.nz, bad);
-    if (left_alone(w, failed)) return;
+    const int earlier = earlier_error(word, w.parity);
+    bad |= earlier;
+    if (bad) atomicOr(w.err, err_of_step(bad, w.parity));
+    if (earlier) return;
     // the second lane of an odd row's last pair goes to the row's padding
     R* o = w.aux + (row * p.pitch + k);
     const int plane = (int)p.plane;
@@ -223,7 +211,6 @@ __device__ __forceinline__ void phase_l2(const Params<R>& p, const PhaseWork<R>&
     st2(o + plane, 0, jz);
     st2(o + 2 * plane, 0, jr);
     if (MP) st2(o + 3 * plane, 0, psi);
-    if (bad) atomicOr(w.err, err_of_step(bad, w.parity));
 }
 
 // Tile plus 4 columns and rows of psi (F on the tile needs psi_rr, which needs psi_r on a 2-ring).
@@ -234,7 +221,7 @@ struct PhaseU2 {
 };
 
 template <int TR, bool MP, bool AX, bool EDGE, typename R>
-__device__ __forceinline__ void phase_u2(const Params<R>& p, const PhaseWork<R>& w, R* smem, int failed) {
+__device__ __forceinline__ void phase_u2(const Params<R>& p, const PhaseWork<R>& w, R* smem, int word) {
     using T = typename PairOf<R>::T;
     using S = PhaseU2<TR>;
     constexpr int TZ = S::TZ, WP = S::WP, WD = S::WD, NT = 32 * TR;
@@ -286,7 +273,7 @@ __device__ __forceinline__ void phase_u2(const Params<R>& p, const PhaseWork<R>&
         }
         __syncthreads();
     }
-    if (!mine || failed) return;
+    if (!mine || earlier_error(word, w.parity)) return;
     if (row < 0) jr = psub(pk(R(0), R(0)), jr);
     const T rho = padd(drho, pk(p.rho_ref, p.rho_ref));
     T fz = pmul(rho, pk(p.gz, p.gz)), fr = pk(R(0), R(0));
@@ -311,7 +298,7 @@ __device__ __forceinline__ void phase_u2(const Params<R>& p, const PhaseWork<R>&
 
 template <int TR, bool AX, int FV, bool EDGE, typename R>
 __device__ __forceinline__ void phase_c2(const Params<R>& p, const PhaseWork<R>& w, const R* h_src, R* h_dst,
-                                         int failed) {
+                                         int word) {
     using T = typename PairOf<R>::T;
     constexpr bool link = (FV & FV_LINK) != 0;
     const int row = w.j0 + (threadIdx.x >> 5), k = w.k0 + 2 * (threadIdx.x & 31);
@@ -362,7 +349,7 @@ __device__ __forceinline__ void phase_c2(const Params<R>& p, const PhaseWork<R>&
     }
     moments2<link, R>(f, la, drho, jz, jr);
     if (AX) source2(p, padd(drho, pk(p.rho_ref, p.rho_ref)), uz, ur, duz_dr, dur_dz, dur_dr, row, Hz, Hr, mir, rur);
-    if (failed) return;
+    if (earlier_error(word, w.parity)) return;
     const int plane = (int)p.plane;
     R* o = w.fout + (row * p.pitch + k);
     R* hq = link ? h_dst + (row * p.pitch + k) : nullptr;
@@ -463,7 +450,7 @@ __device__ __forceinline__ bool finite1(double x) { return (__double2hiint(x) & 
 
 template <int TR, bool MP, bool LINK>
 __device__ __forceinline__ void phase_l1(const Params<double>& p, const PhaseWork<double>& w, const double* h_src,
-                                         int failed) {
+                                         int word) {
     const int row = w.j0 + (threadIdx.x >> 5), k = w.k0 + (threadIdx.x & 31);
     if (row >= p.nr || k >= p.nz) return;
     double f[Q];
@@ -485,14 +472,16 @@ __device__ __forceinline__ void phase_l1(const Params<double>& p, const PhaseWor
         if (!nonnegative(arg)) bad |= ERRBIT_PSI;
         psi = sqrt3(arg);
     }
-    if (left_alone(w, failed)) return;
+    const int earlier = earlier_error(word, w.parity);
+    bad |= earlier;
+    if (bad) atomicOr(w.err, err_of_step(bad, w.parity));
+    if (earlier) return;
     const int plane = (int)p.plane;
     double* o = w.aux + (row * p.pitch + k);
     o[0] = drho;
     o[plane] = jz;
     o[2 * plane] = jr;
     if (MP) o[3 * plane] = psi;
-    if (bad) atomicOr(w.err, err_of_step(bad, w.parity));
 }
 
 // psi with 4 columns and rows around the tile, the column sums of its stencils, and psi_z, psi_r with 2.
@@ -505,7 +494,7 @@ struct PhaseU1 {
 // put(row, k, drho, u_z, u_r, 1/rho) takes the results.
 template <int TR, bool MP, bool AX, typename P>
 __device__ __forceinline__ void phase_u1(const Params<double>& p, const PhaseWork<double>& w, double* smem,
-                                         int failed, P&& put) {
+                                         int word, P&& put) {
     using S = PhaseU1<TR>;
     constexpr int TZ = S::TZ, WP = S::WP, WD = S::WD, NT = 32 * TR, NC = WP * (TR + 4);
     double* sPsi = smem;
@@ -564,7 +553,7 @@ __device__ __forceinline__ void phase_u1(const Params<double>& p, const PhaseWor
             __syncthreads();
         }
     }
-    if (!mine || failed) return;
+    if (!mine || earlier_error(word, w.parity)) return;
     const double rho = p.rho_ref + drho;
     double fz = mul(rho, p.gz), fr = 0.0;
     if (MP) {
@@ -596,7 +585,7 @@ __device__ __forceinline__ void phase_u1(const Params<double>& p, const PhaseWor
 
 template <int TR, bool AX, int FV>
 __device__ __forceinline__ void phase_c1(const Params<double>& p, const PhaseWork<double>& w, const double* h_src,
-                                         double* h_dst, int failed) {
+                                         double* h_dst, int word) {
     constexpr bool link = (FV & FV_LINK) != 0, guo = (FV & FV_GUO) != 0;
     const int row = w.j0 + (threadIdx.x >> 5), k = w.k0 + (threadIdx.x & 31), nz = p.nz;
     if (row >= p.nr || k >= nz) return;
@@ -643,7 +632,7 @@ __device__ __forceinline__ void phase_c1(const Params<double>& p, const PhaseWor
         Hr = mul(fma(2.0 * mu, fma(p.hr_sign * ir, ur, dur_dr), -mul(rur, ur)), ir);
         m0 = mul(-rur, ir);
     }
-    if (failed) return;
+    if (earlier_error(word, w.parity)) return;
     const double om = p.tau_inv, om1 = 1.0 - p.tau_inv;
     const int plane = (int)p.plane;
     double* o = w.fout + (row * p.pitch + k);
@@ -700,33 +689,31 @@ __device__ __forceinline__ void phase_c1(const Params<double>& p, const PhaseWor
 
 // =============================================================== kernels ==
 
-// failed: an earlier step raised an error (the populations are void and left alone).  Read with the
-// phase's other loads and looked at before the stores.
 template <typename R, int TR, bool MP, bool LINK>
 __device__ __forceinline__ void phase_l(const Params<R>& p, const PhaseWork<R>& w, const R* h, bool read = false) {
-    const int failed = read ? 0 : earlier_error(w.err, w.parity);
+    const int word = read ? 0 : error_word(w.err);
     if constexpr (sizeof(R) == 4) {
         if (phase_inner(p, w.k0))
-            phase_l2<TR, MP, LINK, false>(p, w, h, failed);
+            phase_l2<TR, MP, LINK, false>(p, w, h, word);
         else
-            phase_l2<TR, MP, LINK, true>(p, w, h, failed);
+            phase_l2<TR, MP, LINK, true>(p, w, h, word);
     } else {
-        phase_l1<TR, MP, LINK>(p, w, h, failed);
+        phase_l1<TR, MP, LINK>(p, w, h, word);
     }
 }
 template <typename R, int TR, bool MP, bool AX>
 __device__ __forceinline__ void phase_u(const Params<R>& p, const PhaseWork<R>& w) {
-    const int failed = earlier_error(w.err, w.parity);
+    const int word = error_word(w.err);
     if constexpr (sizeof(R) == 4) {
         __shared__ __align__(16) R smem[PhaseU2<TR>::elems];
         if (phase_inner(p, w.k0))
-            phase_u2<TR, MP, AX, false>(p, w, smem, failed);
+            phase_u2<TR, MP, AX, false>(p, w, smem, word);
         else
-            phase_u2<TR, MP, AX, true>(p, w, smem, failed);
+            phase_u2<TR, MP, AX, true>(p, w, smem, word);
     } else {
         __shared__ __align__(16) R smem[PhaseU1<TR>::elems];
         const long long n = u_plane<double>(p.nz, p.nr);
-        phase_u1<TR, MP, AX>(p, w, smem, failed, [&](int row, int k, double, double uz, double ur, double irho) {
+        phase_u1<TR, MP, AX>(p, w, smem, word, [&](int row, int k, double, double uz, double ur, double irho) {
             double* o = w.u + ((long long)(row + kGhostRows) * u_stride<double>(p.nz) + k);
             o[0] = uz;
             o[n] = ur;
@@ -736,14 +723,14 @@ __device__ __forceinline__ void phase_u(const Params<R>& p, const PhaseWork<R>& 
 }
 template <typename R, int TR, bool AX, int FV>
 __device__ __forceinline__ void phase_c(const Params<R>& p, const PhaseWork<R>& w, const R* hs, R* hd) {
-    const int failed = earlier_error(w.err, w.parity);
+    const int word = error_word(w.err);
     if constexpr (sizeof(R) == 4) {
         if (phase_inner(p, w.k0))
-            phase_c2<TR, AX, FV, false>(p, w, hs, hd, failed);
+            phase_c2<TR, AX, FV, false>(p, w, hs, hd, word);
         else
-            phase_c2<TR, AX, FV, true>(p, w, hs, hd, failed);
+            phase_c2<TR, AX, FV, true>(p, w, hs, hd, word);
     } else {
-        phase_c1<TR, AX, FV>(p, w, hs, hd, failed);
+        phase_c1<TR, AX, FV>(p, w, hs, hd, word);
     }
 }
 

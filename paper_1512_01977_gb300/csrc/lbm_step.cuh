@@ -1063,7 +1063,7 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
         __syncthreads();  // everyone is done with the previous tile's parameters
         if (threadIdx.x == 0) {
             sp = solves[tl.solve].p;
-            skip = *static_cast<volatile const int*>(err + tl.solve);
+            skip = left_out(err + tl.solve, parity);
         }
         __syncthreads();  // parameters and the skip decision are the same for the whole CTA
         const R* fin = parity ? solves[tl.solve].f_b : solves[tl.solve].f_a;
@@ -1071,7 +1071,7 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
         if (!skip) {
             int bad = 0;
             march_cp<R, TZ, RR, CP, MP, AX>(sp, fin, fo, tl.strip, tl.j0, tl.jend, smem_raw, bad);
-            if (bad) atomicOr(&err[tl.solve], bad);
+            if (bad) atomicOr(&err[tl.solve], err_of_step(bad, parity));
         }
     }
 }
@@ -1090,7 +1090,7 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
     for (int t = first[blockIdx.x]; t < t1; t++) {
         const Tile tl = tiles[t];
         __syncthreads();  // everyone is done with the previous tile
-        if (threadIdx.x == 0) skip = *static_cast<volatile const int*>(err + tl.solve);
+        if (threadIdx.x == 0) skip = left_out(err + tl.solve, parity);
         __syncthreads();
         const BatchSolve<R>& s = tab.s[tl.solve];
         const R* fin = parity ? s.f_b : s.f_a;
@@ -1098,7 +1098,7 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
         if (!skip) {
             int bad = 0;
             march_cp<R, TZ, RR, CP, MP, AX>(s.p, fin, fo, tl.strip, tl.j0, tl.jend, smem_raw, bad);
-            if (bad) atomicOr(&err[tl.solve], bad);
+            if (bad) atomicOr(&err[tl.solve], err_of_step(bad, parity));
         }
     }
 }
@@ -1120,12 +1120,12 @@ __global__ void __launch_bounds__(StepShape<TZ, RR, CP>::NT, MINB)
     for (int t = first[blockIdx.x]; t < t1; t++) {
         const Tile tl = tiles[t];
         __syncthreads();  // everyone is done with the previous tile
-        if (threadIdx.x == 0) skip = *static_cast<volatile const int*>(err);
+        if (threadIdx.x == 0) skip = left_out(err, parity);
         __syncthreads();
         if (!skip) {
             int bad = 0;
             march_cp<R, TZ, RR, CP, true, true, FV>(s.p, fin, fo, tl.strip, tl.j0, tl.jend, smem_raw, bad, hin, ho);
-            if (bad) atomicOr(err, bad);
+            if (bad) atomicOr(err, err_of_step(bad, parity));
         }
     }
 }

@@ -49,7 +49,7 @@ __device__ __forceinline__ void pull_pair(const Params<float>& p, const float* _
 }
 
 template <typename S, bool MP, bool AX, bool EDGE>
-__device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWork<float>& w, float* smem, int failed) {
+__device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWork<float>& w, float* smem, int word) {
     using T = float2;
     constexpr int NT = S::NT, LZ = S::LZ, LR = S::LR, WL = S::WL, WD = S::WD, WU = S::WU;
     float* sPsi = smem;
@@ -148,8 +148,10 @@ __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWor
     }
     __syncthreads();
     // ---- collide
-    if (bad) atomicOr(w.err, bad);
-    if (!collides || failed) return;
+    const int earlier = earlier_error(word, w.parity);
+    bad |= earlier;
+    if (bad) atomicOr(w.err, err_of_step(bad, w.parity));
+    if (!collides || earlier) return;
     const int b = cc + S::U;
     const int o0 = (ct + S::U) * WU;
     const T drho = ld2<T>(sRho + o0, b), uz = ld2<T>(sUz + o0, b), ur = ld2<T>(sUr + o0, b);
@@ -188,11 +190,11 @@ __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWor
 template <typename S, bool MP, bool AX>
 __device__ __forceinline__ void tile_step(const Params<float>& p, const PhaseWork<float>& w) {
     __shared__ __align__(16) float smem[S::elems];
-    const int failed = *static_cast<volatile const int*>(w.err);
+    const int word = error_word(w.err);
     if (w.k0 >= 8 && w.k0 + S::TZ + 8 <= p.nz)
-        tile_step<S, MP, AX, false>(p, w, smem, failed);
+        tile_step<S, MP, AX, false>(p, w, smem, word);
     else
-        tile_step<S, MP, AX, true>(p, w, smem, failed);
+        tile_step<S, MP, AX, true>(p, w, smem, word);
 }
 
 template <int TZ, int TR, int NT, bool MP, bool AX>

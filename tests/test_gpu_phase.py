@@ -416,3 +416,25 @@ def test_marching_batch_beyond_one_table(lbm, strip, grid):
             assert rel_err(m["rho"], ref["rho"]) <= 1e-6 and vel_err(m, ref) <= 1e-6
     for s in solvers:
         s.close()
+
+
+@pytest.mark.parametrize("nz,nr,axis", [(64, 48, 1), (500, 390, 1), (800, 900, 0), (512, 500, 1), (1040, 800, 1), (4100, 1000, 1)])
+def test_a_failing_step_is_finished(lbm, nz, nr, axis):
+    """A step that fails early, at one node in the first tile, writes the same populations as the kernel that never
+    looks at the error word (chunked rows): tiles, phases and warps of one launch and of several waves of blocks."""
+    c = Case(nz, nr, T_over_Tc=0.9, axis=axis)
+    rho, uz, ur = _fields(c, 3)
+    bad = rho.copy()
+    bad[0, 0] = np.nan
+    got = []
+    for rows in (0, 1 << 20):
+        s = c.solver(32, c.coexistence()[1])
+        lbm.lbm_axi_set_tuning(s.h, lbm.PATH_FUSED, rows)
+        s.init(*_fields(c, 4)).step(2)
+        s.init(bad, uz, ur)
+        with pytest.raises(lbm.LbmError) as e:
+            s.step(1)
+        assert e.value.code == lbm.ERR_UNPHYSICAL
+        got.append(np.frombuffer(s.save()[192:], dtype=np.float32))
+        s.close()
+    np.testing.assert_array_equal(got[0], got[1])
