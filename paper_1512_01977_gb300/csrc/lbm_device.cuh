@@ -59,13 +59,6 @@ __device__ __forceinline__ int error_word(const int* err) { return *static_cast<
 __device__ __forceinline__ int earlier_error(int word, int parity) {
     return parity ? word & ((1 << kErrShift) - 1) : word >> kErrShift;
 }
-// Whether a step is left out for an earlier error (by one thread: marked, so that the next one is too).
-__device__ __forceinline__ int left_out(int* err, int parity) {
-    const int earlier = earlier_error(error_word(err), parity);
-    if (earlier) atomicOr(err, err_of_step(earlier, parity));
-    return earlier;
-}
-
 // ------------------------------------------------------------- parameters --
 template <typename R>
 struct Params {

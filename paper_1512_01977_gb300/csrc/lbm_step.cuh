@@ -35,6 +35,13 @@
 
 namespace lbm {
 
+// Whether a step is left out for an earlier error (by one thread: marked, so that the next one is too).
+__device__ __forceinline__ int left_out(int* err, int parity) {
+    const int earlier = earlier_error(error_word(err), parity);
+    if (earlier) atomicOr(err, err_of_step(earlier, parity));
+    return earlier;
+}
+
 template <typename R>
 __device__ __forceinline__ R rcp(R x) {
     return R(1) / x;
