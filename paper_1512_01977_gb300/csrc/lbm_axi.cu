@@ -181,10 +181,14 @@ int chunk_steps(const lbm_axi* h) {
     return (int)(c & ~1LL);
 }
 
-// The caller is capturing the stream: steps go into that graph one by one.
-bool capturing(cudaStream_t s) {
+// Steps go to the stream one by one where no graph of them can be made or launched: the legacy stream, which
+// cannot be captured, and a stream that the caller is capturing.
+bool one_by_one(cudaStream_t s) {
+    if (s == cudaStreamLegacy) return true;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // not the next launch's error
+    return false;
 }
 
 int read_error(lbm_axi* h) {
@@ -517,7 +521,7 @@ int lbm_axi_step_async(lbm_axi* h, long long n) {
         n--;
     }
     const int chunk = chunk_steps(h);
-    if (e == cudaSuccess && n >= chunk && !capturing(h->stream)) {
+    if (e == cudaSuccess && n >= chunk && !one_by_one(h->stream)) {
         if (!h->graph || h->graph_steps != chunk) {
             int rc = build_graph(h, chunk);
             if (rc != LBM_OK) return rc;

@@ -116,7 +116,7 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = (
 cudaError_t cudaStreamDestroy(cudaStream_t s) { return free((void*)s), cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
-    return s == fake::captured ? cudaErrorIllegalState : cudaSuccess;
+    return s == fake::captured || s == cudaStreamLegacy ? cudaErrorIllegalState : cudaSuccess;
 }
 cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
     *st = s == fake::captured ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
@@ -417,6 +417,18 @@ static void create_out_of_memory(int nz, int nr, int precision, int forcing) {
         }
 }
 
+// A solve on the legacy stream, which cannot be captured.
+static void step_on_the_legacy_stream() {
+    for (int precision : {32, 64}) {
+        lbm_axi* h = solve(64, 64, precision, cudaStreamLegacy);
+        for (int n : {1, 31, 32, 100, 255, 256, 700}) {
+            fake::launches = 0;
+            CHECK(lbm_axi_step(h, n) == LBM_OK && fake::launches == n);
+        }
+        lbm_axi_destroy(h);
+    }
+}
+
 int main(int argc, char** argv) {
     fake::live = new std::map<uintptr_t, size_t>();
     const char* what = argc > 1 ? argv[1] : "";
@@ -433,6 +445,7 @@ int main(int argc, char** argv) {
     if (!strcmp(what, "create_fp64")) return create_out_of_memory(64, 64, 64, 0), 0;
     if (!strcmp(what, "create_warps")) return create_out_of_memory(1040, 800, 32, 0), 0;
     if (!strcmp(what, "create_ctas")) return create_out_of_memory(1040, 800, 32, 1), 0;
+    if (!strcmp(what, "legacy_stream")) return step_on_the_legacy_stream(), 0;
     if (!strcmp(what, "forms")) return forms(), 0;
     if (!strcmp(what, "launches")) {
         batch_launches(1040, 400, 2);

@@ -438,3 +438,15 @@ def test_a_failing_step_is_finished(lbm, nz, nr, axis):
         got.append(np.frombuffer(s.save()[192:], dtype=np.float32))
         s.close()
     np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("stream", [1, 2])  # cudaStreamLegacy, cudaStreamPerThread
+def test_steps_on_the_default_streams(lbm, prec, stream):
+    c = Case(64, 64, T_over_Tc=0.9)
+    fields, ref = _fields(c, 4), c.coexistence()[1] if prec == 32 else 0.0
+    want = c.solver(prec, ref).init(*fields).step(100)
+    s = lbm.Solver(64, 64, c.tau, eos=lbm.make_eos(c.eos, c.T_over_Tc), A=c.A, precision=prec, rho_ref=ref, stream=stream)
+    assert s.init(*fields).step(100).save() == want.save()
+    s.close()
+    want.close()

@@ -56,3 +56,7 @@ def test_a_step_of_a_large_batch_is_one_launch(program):
 
 def test_forms_go_by_whole_tiles(program):
     _run(program, "forms")
+
+
+def test_steps_on_the_legacy_stream(program):
+    _run(program, "legacy_stream")
