@@ -85,9 +85,3 @@ inline lbm::BatchSolve<R> lbm_handle_solve(const lbm_axi* h, const Params<R>& p,
     return {p, static_cast<const R*>(h->f[a]), static_cast<R*>(h->f[a ^ 1]), static_cast<R*>(h->aux),
             reinterpret_cast<R*>(h->mout)};
 }
-
-// Step parity bookkeeping used by the batch API: after n steps run outside
-// the handle's own step loop, its current buffer flips when n is odd.
-inline void lbm_handle_advance(lbm_axi* h, long long n) {
-    if (n & 1) h->cur ^= 1;
-}

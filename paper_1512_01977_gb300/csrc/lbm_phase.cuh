@@ -31,11 +31,11 @@ template <typename R>
 struct PhaseShape;
 template <>
 struct PhaseShape<float> {
-    static constexpr int TZ = kPhaseColumns, CP = 2;  // one warp per tile row
+    static constexpr int TZ = kPhaseColumns;  // a node pair per lane: one warp per tile row
 };
 template <>
 struct PhaseShape<double> {
-    static constexpr int TZ = 32, CP = 1;
+    static constexpr int TZ = 32;  // a node per lane
 };
 
 // The launches carry the programmatic attribute but no trigger: a trigger at the start lets the next
@@ -188,7 +188,7 @@ __device__ __forceinline__ bool phase_inner(const Params<R>& p, int k0) {
     return k0 >= 4 && k0 + PhaseShape<R>::TZ + 4 <= p.nz;
 }
 
-template <int TR, bool MP, bool LINK, bool EDGE, typename R>
+template <bool MP, bool LINK, bool EDGE, typename R>
 __device__ __forceinline__ void phase_l2(const Params<R>& p, const PhaseWork<R>& w, const R* h_src, int word) {
     using T = typename PairOf<R>::T;
     const int row = w.j0 + (threadIdx.x >> 5), k = w.k0 + 2 * (threadIdx.x & 31);
@@ -296,7 +296,7 @@ __device__ __forceinline__ void phase_u2(const Params<R>& p, const PhaseWork<R>&
     st2(o + u_plane<R>(nz, nr), 0, vr);
 }
 
-template <int TR, bool AX, int FV, bool EDGE, typename R>
+template <bool AX, int FV, bool EDGE, typename R>
 __device__ __forceinline__ void phase_c2(const Params<R>& p, const PhaseWork<R>& w, const R* h_src, R* h_dst,
                                          int word) {
     using T = typename PairOf<R>::T;
@@ -448,7 +448,7 @@ __device__ __forceinline__ void moments1(const double (&f)[Q], double& drho, dou
 }
 __device__ __forceinline__ bool finite1(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
-template <int TR, bool MP, bool LINK>
+template <bool MP, bool LINK>
 __device__ __forceinline__ void phase_l1(const Params<double>& p, const PhaseWork<double>& w, const double* h_src,
                                          int word) {
     const int row = w.j0 + (threadIdx.x >> 5), k = w.k0 + (threadIdx.x & 31);
@@ -583,7 +583,7 @@ __device__ __forceinline__ void phase_u1(const Params<double>& p, const PhaseWor
     put(row, k0 + c, drho, mul(fma(0.5, fz, jz), irho), mul(fma(0.5, fr, row < 0 ? -jr : jr), irho), irho);
 }
 
-template <int TR, bool AX, int FV>
+template <bool AX, int FV>
 __device__ __forceinline__ void phase_c1(const Params<double>& p, const PhaseWork<double>& w, const double* h_src,
                                          double* h_dst, int word) {
     constexpr bool link = (FV & FV_LINK) != 0, guo = (FV & FV_GUO) != 0;
@@ -689,16 +689,16 @@ __device__ __forceinline__ void phase_c1(const Params<double>& p, const PhaseWor
 
 // =============================================================== kernels ==
 
-template <typename R, int TR, bool MP, bool LINK>
+template <typename R, bool MP, bool LINK>
 __device__ __forceinline__ void phase_l(const Params<R>& p, const PhaseWork<R>& w, const R* h, bool read = false) {
     const int word = read ? 0 : error_word(w.err);
     if constexpr (sizeof(R) == 4) {
         if (phase_inner(p, w.k0))
-            phase_l2<TR, MP, LINK, false>(p, w, h, word);
+            phase_l2<MP, LINK, false>(p, w, h, word);
         else
-            phase_l2<TR, MP, LINK, true>(p, w, h, word);
+            phase_l2<MP, LINK, true>(p, w, h, word);
     } else {
-        phase_l1<TR, MP, LINK>(p, w, h, word);
+        phase_l1<MP, LINK>(p, w, h, word);
     }
 }
 template <typename R, int TR, bool MP, bool AX>
@@ -721,16 +721,16 @@ __device__ __forceinline__ void phase_u(const Params<R>& p, const PhaseWork<R>& 
         });
     }
 }
-template <typename R, int TR, bool AX, int FV>
+template <typename R, bool AX, int FV>
 __device__ __forceinline__ void phase_c(const Params<R>& p, const PhaseWork<R>& w, const R* hs, R* hd) {
     const int word = error_word(w.err);
     if constexpr (sizeof(R) == 4) {
         if (phase_inner(p, w.k0))
-            phase_c2<TR, AX, FV, false>(p, w, hs, hd, word);
+            phase_c2<AX, FV, false>(p, w, hs, hd, word);
         else
-            phase_c2<TR, AX, FV, true>(p, w, hs, hd, word);
+            phase_c2<AX, FV, true>(p, w, hs, hd, word);
     } else {
-        phase_c1<TR, AX, FV>(p, w, hs, hd, word);
+        phase_c1<AX, FV>(p, w, hs, hd, word);
     }
 }
 
@@ -751,7 +751,7 @@ __device__ __forceinline__ void phase_c(const Params<R>& p, const PhaseWork<R>& 
 template <typename R, int TR, bool MP, bool LINK>
 __global__ void __launch_bounds__(32 * TR) k_phase_l(const PhaseOne<R> a) {
     LBM_PHASE_ONE(a);
-    phase_l<R, TR, MP, LINK>(p, w, a.h_src, a.read);
+    phase_l<R, MP, LINK>(p, w, a.h_src, a.read);
 }
 template <typename R, int TR, bool MP, bool AX>
 __global__ void __launch_bounds__(32 * TR) k_phase_u(const PhaseOne<R> a) {
@@ -761,12 +761,12 @@ __global__ void __launch_bounds__(32 * TR) k_phase_u(const PhaseOne<R> a) {
 template <typename R, int TR, bool AX, int FV>
 __global__ void __launch_bounds__(32 * TR) k_phase_c(const PhaseOne<R> a) {
     LBM_PHASE_ONE(a);
-    phase_c<R, TR, AX, FV>(p, w, a.h_src, a.h_dst);
+    phase_c<R, AX, FV>(p, w, a.h_src, a.h_dst);
 }
 template <typename R, int TR, bool MP>
 __global__ void __launch_bounds__(32 * TR) k_phase_l_many(const PhaseMany<R> a) {
     LBM_PHASE_MANY(a);
-    phase_l<R, TR, MP, false>(p, w, nullptr);
+    phase_l<R, MP, false>(p, w, nullptr);
 }
 template <typename R, int TR, bool MP, bool AX>
 __global__ void __launch_bounds__(32 * TR) k_phase_u_many(const PhaseMany<R> a) {
@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(32 * TR) k_phase_u_many(const PhaseMany<R> a) 
 template <typename R, int TR, bool AX>
 __global__ void __launch_bounds__(32 * TR) k_phase_c_many(const PhaseMany<R> a) {
     LBM_PHASE_MANY(a);
-    phase_c<R, TR, AX, 0>(p, w, nullptr, nullptr);
+    phase_c<R, AX, 0>(p, w, nullptr, nullptr);
 }
 #undef LBM_PHASE_ONE
 #undef LBM_PHASE_MANY
