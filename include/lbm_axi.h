@@ -162,9 +162,8 @@ int lbm_axi_init_device(lbm_axi* h, const double* d_rho, const double* d_u_z, co
  * flow); lbm_axi_init instead leaves a spurious F/(2 rho) in every interface
  * at t = 0.  F is evaluated on f^eq(rho, u) (density rho up to rounding).
  * rho is required; u_z and u_r may be NULL (zero).  Host arrays, nz*nr
- * doubles; a temporary device copy is made.  Synchronous.  Returns
- * LBM_ERR_UNPHYSICAL (populations then hold f^eq(rho, u)) when psi^2 < 0 or
- * rho <= 0 somewhere, LBM_ERR_OOM when the temporary copy cannot be made. */
+ * doubles.  Synchronous.  Returns LBM_ERR_UNPHYSICAL (populations then hold
+ * f^eq(rho, u)) when psi^2 < 0 or rho <= 0 somewhere. */
 int lbm_axi_init_physical(lbm_axi* h, const double* rho, const double* u_z, const double* u_r);
 
 /* Same as lbm_axi_init_physical with device arrays (nz*nr doubles,
@@ -197,8 +196,8 @@ int lbm_axi_time_kernels(lbm_axi* h, long long n, double* ms);
 /* Kernel configuration of a solve (performance only).
  *   path: LBM_PATH_FUSED -- the whole update in one launch per step (FP32: tiles
  *         held on chip for small grids, marching warps above 800,000 nodes in
- *         whole tiles of 64 x 8, 72 B per node) or in three (FP64, and FP32 in between), chosen by size;
- *         needs nr >= 16.  LBM_PATH_SPLIT -- kernel (a) (gather, rho, j, psi into
+ *         whole tiles of 64 x 8, 72 B per node) or in three (FP64, and FP32 in
+ *         between), chosen by size; needs nr >= 16.  LBM_PATH_SPLIT -- kernel (a) (gather, rho, j, psi into
  *         field planes) then kernel (b) (forces + collision), 140 B per node.
  *   rows_per_cta: 0 -- the form the size chooses (default); > 0 -- one launch,
  *         each CTA marching a fixed chunk of that many rows of one z-strip.

@@ -4,10 +4,11 @@
  * Many independent solves (e.g. droplets of different sizes, temperatures and
  * relaxation times) advance together: each batch step is ONE launch (three in
  * FP64 and for FP32 batches of up to 800,000 nodes, in whole tiles of 64 x 8,
- * that do not fit the one-launch tiles) over a work list of tiles of all solves; steps are replayed
- * from a CUDA graph.  The update of every solve is exactly the single-solve update
- * (Sec. II of arXiv:1512.01977); no arithmetic couples two solves, so a
- * solve's result is the same alone and in any batch.
+ * that do not fit the one-launch tiles) over a work list of tiles of all
+ * solves; steps are replayed from a CUDA graph.  The update of every solve is
+ * exactly the single-solve update (Sec. II of arXiv:1512.01977); no arithmetic
+ * couples two solves, so a solve's result is the same bits alone and in any
+ * batch (FP32 batches tuned to 64-column strips: to FP32 rounding).
  */
 #ifndef LBM_AXI_BATCH_H
 #define LBM_AXI_BATCH_H

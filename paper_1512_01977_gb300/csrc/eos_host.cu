@@ -136,7 +136,7 @@ bool coexistence(const lbm_eos& e, double T, double* rv_out, double* rl_out) {
     }
     // ... and Newton steps on the quadrature, which keeps its relative precision near the critical point,
     // where the closed form's two values cancel; d/dps of the area is 1/rho_l - 1/rho_v.  (Bisection on
-    // the quadrature alone took 4.7 ms, this 0.3 ms.)
+    // the quadrature alone took 4.8 to 5.4 ms on the Grace host, this 0.14 to 0.23 ms.)
     double ps = 0.5 * (lo + hi);
     for (int it = 0; it < 4; it++) {
         densities(ps);

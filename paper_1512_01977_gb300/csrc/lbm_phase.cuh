@@ -10,16 +10,17 @@
 // stage is independent, so a small grid fills the SMs and a step costs three
 // short launches.  us per step, marching kernel -> phases (GB300): FP32 64 x 64
 // 24.9 -> 6.1, 512 x 256 22.5 -> 9.4, 1023 x 511 (Guo) 32.4 -> 20.4; FP64 64 x 64
-// 182 -> 15.7, 500 x 250 212 -> 70, 1024 x 512 495 -> 275.  (The smallest FP32
+// 182 -> 16.3, 500 x 250 212 -> 70, 1024 x 512 495 -> 275.  (The smallest FP32
 // grids are faster still in one launch, lbm_tile.cuh.)
 //
 // FP32 runs node pairs with the arithmetic of march2 (the update of a node pair
 // in lbm_step.cuh), in the same order, so both give the same bits.  FP64 is
 // bound by its arithmetic rate (1.9 DFMA lanes per clock and SM measured), so
 // its kernels run one node per lane on the expressions with the fewest
-// operations (33 + 116 + 104 FP64 instructions per node in the three phases,
-// 437 in the marching kernel) and take reciprocals and roots from the hardware
-// approximation and one third-order correction instead of a division.
+// operations (34 + 116 + 104 FP64 instructions per node in the three phases,
+// 437 in the marching kernel) and take reciprocals and roots from the hardware's
+// FP64 approximations (rcp.approx.ftz.f64, rsqrt.approx.ftz.f64) and one
+// correction each instead of a division.
 #pragma once
 
 #include "lbm_step.cuh"

@@ -566,8 +566,10 @@ __device__ __forceinline__ T kappa2(const Params<R>& p, T rho) {
 
 // ------------------------------------------- the update of a node pair --
 // The arithmetic of one step for two adjacent nodes, shared by every kernel
-// that steps in FP32 (march2, the phase kernels): the same packed operations in
-// the same order, so all of them give the same bits.
+// that steps in FP32: the same packed operations in the same order, so the forms
+// that a solve may take give the same bits.  (But for H with the link source: the
+// tiles at the z edges of k_phase_c differ in the last place of about one stored
+// value in a million.)
 
 // rho - rho_ref, j_z, j_r of the arrived populations (la: the link source's
 // arrival planes; its halves h_i/2 have zeroth moment S0/2, first moment H/2).

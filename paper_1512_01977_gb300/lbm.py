@@ -418,7 +418,7 @@ def lbm_axi_tile_plan(sizes, strip, slots):
 
 
 class Batch:
-    """Solves advanced together (one to three launches per step).  Borrows the Solver objects."""
+    """Solves advanced together (one or three launches per step).  Borrows the Solver objects."""
 
     def __init__(self, solvers, stream=None):
         self.solvers = list(solvers)
