@@ -215,8 +215,20 @@ cudaError_t enqueue_init(lbm_axi* h, const double* rho, const double* uz, const 
                              static_cast<const double*>(phys), h->derr);
 }
 
-// The allocation that a device address lies in (false: not known).
-bool allocation_of(const void* p, uintptr_t* base, size_t* size) {
+// Memory of this device, [base, base + size).
+struct DeviceRange {
+    uintptr_t base = 0;
+    size_t size = 0;
+    // n doubles at p that a kernel may write: all of them in the range, as a copy would check (and a copy takes any
+    // address)
+    bool holds(const void* p, size_t n) const {
+        const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+        return at % sizeof(double) == 0 && at >= base && at - base <= size && size - (at - base) >= n * sizeof(double);
+    }
+};
+
+// The allocation of this device that p lies in (size 0: none, or not known).
+DeviceRange allocation_of(const void* p, int device) {
     using F = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
     static const F range = [] {  // from the driver: the runtime has no call for it
         void* f = nullptr;
@@ -227,25 +239,20 @@ bool allocation_of(const void* p, uintptr_t* base, size_t* size) {
         if (!ok) cudaGetLastError();
         return ok ? reinterpret_cast<F>(f) : nullptr;
     }();
-    CUdeviceptr b = 0;
-    if (!range || range(&b, size, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
-    *base = static_cast<uintptr_t>(b);
-    return true;
-}
-
-// n doubles of this device's memory that a kernel may write: all of them in one allocation, as a copy would
-// check (and a copy takes any address).
-bool writable_on(const void* p, size_t n, int device) {
+    DeviceRange r;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return r;
     }
-    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
-    if (a.type != cudaMemoryTypeDevice || a.device != device || at % sizeof(double) != 0) return false;
-    uintptr_t base = 0;
+    CUdeviceptr base = 0;
     size_t size = 0;
-    return allocation_of(p, &base, &size) && at - base <= size && size - (at - base) >= n * sizeof(double);
+    if (a.type != cudaMemoryTypeDevice || a.device != device || !range ||
+        range(&base, &size, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS)
+        return r;
+    r.base = static_cast<uintptr_t>(base);
+    r.size = size;
+    return r;
 }
 
 struct DeviceGuard {
@@ -610,8 +617,11 @@ int lbm_axi_moments_device(lbm_axi* h, double* rho, double* uz, double* ur, doub
     const size_t n = (size_t)h->nz * h->nr;
     double* dst[4] = {rho, uz, ur, p};
     double* to[4];
-    for (int q = 0; q < 4; q++)
-        to[q] = !dst[q] || writable_on(dst[q], n, h->device) ? dst[q] : h->mout + q * n;
+    DeviceRange r;  // looked up again only for a destination that is not in the last one's allocation
+    for (int q = 0; q < 4; q++) {
+        if (dst[q] && !r.holds(dst[q], n)) r = allocation_of(dst[q], h->device);
+        to[q] = !dst[q] || r.holds(dst[q], n) ? dst[q] : h->mout + q * n;
+    }
     cudaError_t e = enqueue_fields(h, to[0], to[1], to[2], to[3], nullptr);
     for (int q = 0; q < 4 && e == cudaSuccess; q++) {
         if (dst[q] && to[q] != dst[q])
