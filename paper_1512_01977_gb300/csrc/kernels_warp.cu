@@ -7,7 +7,7 @@ namespace lbm {
 namespace {
 
 int kind_of(const Params<float>& p) {
-    return (p.eos == EOS_VDW ? WARP_VDW : WARP_CS) | (p.kappa == KAPPA_LATTICE ? 1 : 0);
+    return (p.eos == EOS_VDW ? WARP_VDW : WARP_CS) | (p.axis && p.kappa == KAPPA_LATTICE ? 1 : 0);
 }
 
 // One solve's kernel.  Without F_axis kappa is not used; without the force nor is the EOS.
@@ -37,7 +37,8 @@ Many many(int kind, bool mp, bool ax) {
             default: return k_step_warp_many<true, true, WARP_MIXED>;
         }
     }
-    if (mp) return k_step_warp_many<true, false, WARP_MIXED>;
+    if (mp && kind == WARP_MIXED) return k_step_warp_many<true, false, WARP_MIXED>;
+    if (mp) return kind == WARP_VDW ? k_step_warp_many<true, false, WARP_VDW> : k_step_warp_many<true, false, WARP_CS>;
     return ax ? k_step_warp_many<false, true, WARP_CS> : k_step_warp_many<false, false, WARP_CS>;
 }
 

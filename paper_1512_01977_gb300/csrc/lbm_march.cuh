@@ -134,7 +134,7 @@ __device__ __forceinline__ void march_warp(const Params<float>& pp, const float*
     using T = float2;
     using S = WarpShape;
     Params<float> p = pp;  // with what the compiler is to know
-    p.eos = EOS;
+    if (EOS >= 0) p.eos = EOS;
     if (LATTICE) p.kappa = KAPPA_LATTICE;
     const int lane = threadIdx.x & 31, nz = p.nz, nr = p.nr, plane = (int)p.plane;
     const int k = strip * S::TZ + 2 * (lane - S::kFirst);  // the lane's first column, not wrapped
@@ -290,8 +290,11 @@ __device__ __forceinline__ void march_warp(const Params<float>& pp, const float*
     }
 }
 
-// What a kernel knows of its solves' parameters: the EOS and whether kappa is the lattice constant.  One
-// kind per kernel is 8 % faster than the choice by tile (153 and 167 us on 4096 x 2048).
+// What a kernel knows of its solves' parameters: the EOS and whether kappa is the lattice constant.
+// With axis terms WARP_MIXED knows neither and asks in the loop, which costs 0 to 3 % (100 solves of 1.1M nodes
+// 39.8 us per step with mixed EOS and 39.0 with one); a copy of the loop for each kind costs more as soon as their
+// warps meet on an SM, whose instruction cache does not hold them: 76.6.  Without axis terms (a shorter loop) two
+// copies are better: 256 solves of 6.3M nodes 157 us, 173 asking in the loop, 139 with one EOS.
 enum WarpKind { WARP_CS = 0, WARP_CS_LATTICE = 1, WARP_VDW = 2, WARP_VDW_LATTICE = 3, WARP_MIXED = 4 };
 
 // One tile of one solve.
@@ -305,19 +308,12 @@ __device__ __forceinline__ void march_tile(const BatchSolve<float>& s, const Til
         // the solve already went unphysical: the step is left out, and so will the next one be
     } else if constexpr (KIND != WARP_MIXED) {
         march_warp<MP, AX, (KIND & 2) ? EOS_VDW : EOS_CS, (KIND & 1) != 0>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
+    } else if constexpr (AX) {
+        march_warp<MP, AX, -1, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
+    } else if (s.p.eos == EOS_VDW) {
+        march_warp<MP, AX, EOS_VDW, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
     } else {
-        const bool lattice = s.p.kappa == KAPPA_LATTICE;
-        if (s.p.eos == EOS_VDW) {
-            if (lattice)
-                march_warp<MP, AX, EOS_VDW, true>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
-            else
-                march_warp<MP, AX, EOS_VDW, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
-        } else {
-            if (lattice)
-                march_warp<MP, AX, EOS_CS, true>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
-            else
-                march_warp<MP, AX, EOS_CS, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
-        }
+        march_warp<MP, AX, EOS_CS, false>(s.p, f, fo, t.strip, t.j0, t.jend, ring, bad);
     }
     if (bad) atomicOr(err, err_of_step(bad, parity));
 }
