@@ -9,8 +9,12 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
+#include <chrono>
 #include <map>
 #include <new>
+#include <tuple>
+#include <vector>
 
 #include "lbm_axi.h"
 #include "lbm_axi_batch.h"
@@ -429,6 +433,40 @@ static void step_on_the_legacy_stream() {
     }
 }
 
+// The warps' plan against the general one on the same strips: the same tiles, the tallest first, and no slower than
+// the general plan of a march on wide strips.
+static void warp_plan() {
+    unsigned seed = 1;
+    auto rnd = [&](int lo, int hi) { return lo + (int)((seed = seed * 1664525u + 1013904223u) >> 8) % (hi - lo + 1); };
+    auto key = [](const lbm::Tile& t) { return std::make_tuple(t.solve, t.strip, t.j0, t.jend); };
+    for (int round = 0; round < 120; round++) {
+        const int n = round < 40 ? 1 : rnd(2, 300), slots = round % 3 ? 1824 : rnd(1, 4000);
+        std::vector<int> nz(n), nr(n), first;
+        for (int i = 0; i < n; i++) nz[i] = rnd(1, n == 1 ? 5000 : 600), nr[i] = rnd(16, n == 1 ? 100000 : 400);
+        std::vector<lbm::Tile> a, b;
+        CHECK(lbm::plan_warp_tiles(nz.data(), nr.data(), n, slots, a) == LBM_OK);
+        CHECK(lbm::plan_tiles(nz.data(), nr.data(), n, lbm::kWarpStrip, slots, b, first, nullptr, lbm::kWarpFillRows) == LBM_OK);
+        for (size_t i = 1; i < a.size(); i++) CHECK(a[i - 1].jend - a[i - 1].j0 >= a[i].jend - a[i].j0);
+        auto less = [&](const lbm::Tile& x, const lbm::Tile& y) { return key(x) < key(y); };
+        std::sort(a.begin(), a.end(), less);
+        std::sort(b.begin(), b.end(), less);
+        CHECK(a.size() == b.size());
+        for (size_t i = 0; i < a.size(); i++) CHECK(key(a[i]) == key(b[i]));
+    }
+    const int nz = 4096, nr = 2048;
+    double best[2] = {1e9, 1e9};
+    for (int i = 0; i < 20; i++)
+        for (int which = 0; which < 2; which++) {
+            std::vector<lbm::Tile> t;
+            std::vector<int> first;
+            const auto t0 = std::chrono::steady_clock::now();
+            if (which) lbm::plan_warp_tiles(&nz, &nr, 1, 1824, t);
+            else lbm::plan_tiles(&nz, &nr, 1, lbm::kStripWide, 608, t, first, nullptr);
+            best[which] = std::min(best[which], std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count());
+        }
+    CHECK(best[1] <= best[0]);
+}
+
 int main(int argc, char** argv) {
     fake::live = new std::map<uintptr_t, size_t>();
     const char* what = argc > 1 ? argv[1] : "";
@@ -446,6 +484,7 @@ int main(int argc, char** argv) {
     if (!strcmp(what, "create_warps")) return create_out_of_memory(1040, 800, 32, 0), 0;
     if (!strcmp(what, "create_ctas")) return create_out_of_memory(1040, 800, 32, 1), 0;
     if (!strcmp(what, "legacy_stream")) return step_on_the_legacy_stream(), 0;
+    if (!strcmp(what, "warp_plan")) return warp_plan(), 0;
     if (!strcmp(what, "forms")) return forms(), 0;
     if (!strcmp(what, "launches")) {
         batch_launches(1040, 400, 2);

@@ -60,3 +60,7 @@ def test_forms_go_by_whole_tiles(program):
 
 def test_steps_on_the_legacy_stream(program):
     _run(program, "legacy_stream")
+
+
+def test_plan_of_the_warp_march(program):
+    _run(program, "warp_plan")
